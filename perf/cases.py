@@ -204,7 +204,7 @@ def prepare(case, seed):
         miss[at] = nxt[np.roll(at, 1)]
         wd = _weights(draft, seed + 1, miss)
     eng = binding.Engine(target, w, P, draft, wd, device="cuda:0")
-    state = dict(case=case, eng=eng)
+    state = dict(case=case, eng=eng, next=nxt)
     if kind in ("prefill", "vanilla", "generate"):
         state["prompt"] = _prompt(rs, nxt, case["prompt"])
         return state
@@ -268,6 +268,107 @@ def run(state):
         n, chosen, accurate, accepted = eng.verify_step()
     end = case["cache"] + n
     return {"accepted": np.array(accepted[:n]), "logits": logits, "k": T.k_cache[:, :end], "v": T.v_cache[:, :end]}
+
+
+# ------------------------------------------------------------------------- the same in 64 bits
+
+def _norm64(x, gain, eps):
+    return gain.double() * x / (x.square().mean(-1, keepdim=True) + eps).sqrt()
+
+
+def _rope64(x, pos, theta):
+    half = x.shape[-1] // 2
+    inv = theta ** (-torch.arange(half, dtype=torch.float64, device=x.device) / half)
+    angle = pos.double()[:, None, None] * inv
+    a, b = x[..., :half], x[..., half:]
+    return torch.cat([a * angle.cos() - b * angle.sin(), b * angle.cos() + a * angle.sin()], -1)
+
+
+def _matmul64(x, w):
+    """x w^T, the bf16 or fp32 weights widened a slab at a time."""
+    return torch.cat([x @ part.double().T for part in w.split(8192)], -1)
+
+
+def _attend64(q, k, v, hidden):
+    """q [rows, heads, h]; k, v [keys, kv heads, h]; hidden [rows, rows] for the last keys (the block's own)."""
+    group = q.shape[1] // k.shape[1]
+    out = torch.empty_like(q)
+    for j in range(k.shape[1]):
+        s = torch.einsum("rah,kh->ark", q[:, j * group: (j + 1) * group], k[:, j]) / math.sqrt(q.shape[-1])
+        s[..., s.shape[-1] - len(hidden):].masked_fill_(hidden, -math.inf)
+        out[:, j * group: (j + 1) * group] = torch.einsum("ark,kh->rah", s.softmax(-1), v[:, j])
+    return out
+
+
+def _forward64(m, w, tokens, pos, hidden, before, logits=True):
+    """Keys and values of a block in every layer ([layers, rows, kv heads, h] each), and its logits.  `before`: the cached
+    keys and values in front of it, or None."""
+    device = w["embed"].device
+    pos = torch.as_tensor(np.asarray(pos), device=device)
+    x = w["embed"][torch.as_tensor(np.asarray(tokens), dtype=torch.int64, device=device)].double()
+    rows = len(pos)
+    ks, vs = [], []
+    for layer in range(m.n_layers):
+        lw = w["layers"][layer]
+        n1 = _norm64(x, lw["attn_norm"], m.rms_eps)
+        q = _rope64(_matmul64(n1, lw["wq"]).view(rows, m.n_heads, m.head_dim), pos, m.rope_theta)
+        k = _rope64(_matmul64(n1, lw["wk"]).view(rows, m.n_kv_heads, m.head_dim), pos, m.rope_theta)
+        v = _matmul64(n1, lw["wv"]).view(rows, m.n_kv_heads, m.head_dim)
+        ks.append(k)
+        vs.append(v)
+        if before is not None:
+            k, v = torch.cat([before[0][layer].double(), k]), torch.cat([before[1][layer].double(), v])
+        x = x + _matmul64(_attend64(q, k, v, hidden).reshape(rows, -1), lw["wo"])
+        n2 = _norm64(x, lw["ffn_norm"], m.rms_eps)
+        gate = _matmul64(n2, lw["w_gate"])
+        x = x + _matmul64(gate * gate.sigmoid() * _matmul64(n2, lw["w_up"]), lw["w_down"])
+    return torch.stack(ks), torch.stack(vs), _matmul64(_norm64(x, w["final_norm"], m.rms_eps), w["lm_head"]) if logits else None
+
+
+def _causal(n):
+    return torch.ones(n, n, dtype=torch.bool, device="cuda").triu(1)
+
+
+def exact(case, seed):
+    """Token choices have wide margins, so keys and values are those of one causal forward over the greedy text."""
+    state = prepare(case, seed)
+    torch.cuda.synchronize()
+    if case["kind"] == "lm_head":
+        return {"argmax": None, "logits": _matmul64(state["x"].double(), state["w"]) if case["logits"] else None}
+    kind, eng, nxt = case["kind"], state["eng"], state["next"]
+    if kind in ("prefill", "vanilla", "generate"):
+        text = [int(t) for t in state["prompt"]]
+        if kind != "prefill":
+            text += _follow(nxt, text[-1], case["new"])
+        text = text[:-1]
+        k, v, _ = _forward64(eng.target_desc, eng.tm.w, text, range(len(text)), _causal(len(text)), None, logits=False)
+        return {"k": k, "v": v} if kind == "prefill" else {"tokens": None, "k": k, "v": v}
+    L, P = case["cache"], eng.params
+    mem, m = (eng.dm, eng.draft_desc) if kind == "draft" else (eng.tm, eng.target_desc)
+    before = mem.k_cache[:, :L], mem.v_cache[:, :L]
+    if kind == "draft":
+        text = [state["pending"]] + _follow(nxt, state["pending"], P.gamma - 1)
+        logits = None
+    else:
+        # accepted: the draft's right tokens and, behind a whole draft, the right phrase's, then one of the target's own
+        matched = case["hits"]
+        if matched == P.gamma and case["phrases"] > 0:
+            matched += P.S
+        text = [state["pending"]] + _follow(nxt, state["pending"], matched)
+        logits = None
+        if case["logits"]:
+            draft = [int(t) for t in eng.draft_tokens[: P.gamma]]
+            suffixes = eng.suffix[: int(eng.count) * P.S].view(-1, P.S).tolist()
+            trunk = 1 + P.gamma
+            tokens = [state["pending"]] + draft + sum(suffixes, [])
+            pos = list(range(L, L + trunk)) + list(range(L + trunk, L + trunk + P.S)) * len(suffixes)
+            hidden = _causal(len(tokens))
+            group = torch.as_tensor([0] * trunk + [1 + j for j in range(len(suffixes)) for _ in range(P.S)], device="cuda")
+            hidden |= (group[None, :] != group[:, None]) & (group[None, :] != 0)
+            logits = _forward64(m, mem.w, tokens, pos, hidden, before)[2]
+    k, v, _ = _forward64(m, mem.w, text, range(L, L + len(text)), _causal(len(text)), before, logits=False)
+    k, v = (torch.cat([old.double(), new], 1) for old, new in zip(before, (k, v)))
+    return {"tokens": None, "k": k, "v": v} if kind == "draft" else {"accepted": None, "logits": logits, "k": k, "v": v}
 
 
 # -------------------------------------------------------------------------------- least work, tolerance
