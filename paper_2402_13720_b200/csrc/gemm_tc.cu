@@ -71,6 +71,7 @@ struct GemmParams {
   int mode;
   int tiles;          // total tiles
   int kb;             // k-blocks per tile (K / 64)
+  int splitters;      // CTAs that share the remainder tiles (see weight_stream.cuh); -1: the whole grid
   int t_pad;          // tokens padded to a multiple of 16 (MMA N)
   int rows;           // valid tokens (an upper bound when rows_dev is set)
   const int *rows_dev;  // NULL, or where the block's true row count sits in device memory: the host then sizes the
@@ -219,7 +220,8 @@ constexpr int STAGE_BYTES = STAGE_TOK * STAGE_PITCH * 4;
 
 // The schedule of this launch for CTA blockIdx.x (see weight_stream.cuh).
 struct SpanWalker : ws::SpanWalker {
-  __device__ SpanWalker(const GemmParams &p) : ws::SpanWalker(p.tiles, p.kb, (int)gridDim.x, (int)blockIdx.x) {}
+  __device__ SpanWalker(const GemmParams &p)
+      : ws::SpanWalker(p.tiles, p.kb, (int)gridDim.x, p.splitters < 0 ? (int)gridDim.x : p.splitters, (int)blockIdx.x) {}
 };
 
 // Locates a tile: which stacked matrix, its first row there, and the first output column.
@@ -1159,6 +1161,7 @@ static void flush_chain(ouro_ctx *c) {
 static void push_gemm(ouro_ctx *c, GemmParams &p, int kind, const CUtensorMap *xmaps, int K, int rows, bool last) {
   FastState &s = c->fast->s;
   p.kb = K / BLOCK_K;
+  p.splitters = -1;
   p.rows = rows;
   p.t_pad = (rows + 15) & ~15;
   p.b = xmaps[p.t_pad / 16 - 1];
@@ -1410,9 +1413,9 @@ int ouro_fast_head(ouro_ctx *c, int which, int rows, float *logits, int32_t *arg
 // (cudaGetSymbolAddress) with the right device current; that is done once per device by the first call.
 // ===================================================================================================
 namespace {
-constexpr int NA_GRID = 32;                        // CTAs of the static-scratch launch (slots are per CTA)
+constexpr int NA_SPLITTERS = 32;                   // CTAs that may leave partial tiles (two slots each)
 constexpr int NA_MAX_TILES = 512;                  // vocabulary <= 65536
-constexpr size_t NA_SLOT_BYTES = (size_t)NA_GRID * 2 * SLOT_FLOATS * sizeof(float);
+constexpr size_t NA_SLOT_BYTES = (size_t)NA_SPLITTERS * 2 * SLOT_FLOATS * sizeof(float);
 constexpr size_t NA_OFF_COUNTERS = NA_SLOT_BYTES;
 constexpr size_t NA_OFF_STATUS = NA_OFF_COUNTERS + 2 * NA_MAX_TILES * sizeof(int);   // published + finished counters
 constexpr size_t NA_OFF_TMAX = NA_OFF_STATUS + 256;
@@ -1427,6 +1430,7 @@ static __device__ __align__(256) unsigned char g_static_scratch[NA_BYTES];
 namespace {
 unsigned char *g_na_ptr[NA_MAX_DEVICES] = {};      // device address of g_static_scratch, per device
 int g_na_smem[NA_MAX_DEVICES] = {};
+int g_na_sms[NA_MAX_DEVICES] = {};
 
 // Once per device, with that device current: resolve the array's device address and size the kernel's
 // shared memory.  Returns OURO_OK or an error with a text for ouro_last_error(NULL).
@@ -1438,8 +1442,9 @@ int na_setup(int dev) {
     ouro_set_global_error(std::string("cudaGetSymbolAddress(static scratch): ") + cudaGetErrorString(e));
     return OURO_ECUDA;
   }
-  int smem = 0;
+  int smem = 0, sms = 0;
   if ((e = cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
       (e = cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) {
     ouro_set_global_error(std::string("static-scratch set-up: ") + cudaGetErrorString(e));
     return OURO_ECUDA;
@@ -1454,6 +1459,7 @@ int na_setup(int dev) {
     g_encode = (EncodeTiledFn)fn;
   }
   g_na_smem[dev] = smem;
+  g_na_sms[dev] = sms;
   g_na_ptr[dev] = (unsigned char *)ptr;
   return OURO_OK;
 }
@@ -1507,8 +1513,20 @@ extern "C" int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, i
   p.counters = (int *)(base + NA_OFF_COUNTERS);
   p.gen = 1;                                   // the words were cleared just above
   p.status = (int *)(base + NA_OFF_STATUS);
-  const int total = tiles * p.kb;
-  gemm_tc_kernel<<<total < NA_GRID ? total : NA_GRID, THREADS, g_na_smem[dev], s>>>(cp);
+  // One CTA per SM streams whole tiles, which need no scratch.  The remainder (all tiles of a small vocabulary) is cut
+  // along K over the CTAs that have slots while it has no more tiles than those: beyond that, as many CTAs stream when
+  // each takes a tile whole.  Bound by the weight stream: 32000 x 4096 with 37 rows took 208 us on 32 CTAs (1.3 TB/s, what
+  // 32 rings can ask for) and takes 95 us on all SMs.
+  const int total = tiles * p.kb, sms = std::min(g_na_sms[dev], MAX_GRID), rest = tiles % sms;
+  int grid;
+  if (tiles <= NA_SPLITTERS) {
+    grid = std::min(total, NA_SPLITTERS);
+    p.splitters = -1;
+  } else {
+    grid = std::min(tiles, sms);
+    p.splitters = tiles > sms && rest <= NA_SPLITTERS ? NA_SPLITTERS : 0;
+  }
+  gemm_tc_kernel<<<grid, THREADS, g_na_smem[dev], s>>>(cp);
   argmax_tiles_kernel<<<rows, 128, 0, s>>>(p.tile_max, p.tile_arg, tiles, argmax_dev);
   int status = 0;
   if ((e = cudaGetLastError()) != cudaSuccess ||

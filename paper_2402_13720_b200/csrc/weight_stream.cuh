@@ -16,16 +16,18 @@ struct Span {  // one piece of a CTA's work: k-blocks [kb0, kb1) of `tile`
 
 // Work of one CTA.  The last R = tiles mod grid tiles are cut stream-K fashion into equal contiguous spans of
 // the (tile, k-block) space and come first, so that their partial sums are added up while the whole tiles
-// (tile c, c + grid, ...) that follow are still streaming.  Depends on (tiles, kb, grid) only.
+// (tile c, c + grid, ...) that follow are still streaming.  Depends on (tiles, kb, grid, splitters) only.
+// `splitters` is the number of CTAs that share the remainder: all of them where scratch memory holds two partial tiles
+// per CTA, fewer (or none: the remainder is then handled whole as well) where it does not.
 struct SpanWalker {
   int kb, per, t0, it, end, whole, grid, cta;
-  __device__ SpanWalker(int tiles, int kb_, int grid_, int cta_) {
+  __device__ SpanWalker(int tiles, int kb_, int grid_, int splitters, int cta_) {
     kb = kb_;
     grid = grid_;
     cta = cta_;
-    t0 = (tiles / grid) * grid;                              // tiles [0, t0) are handled whole
+    t0 = splitters ? (tiles / grid) * grid : tiles;          // tiles [0, t0) are handled whole
     int total = (tiles - t0) * kb;
-    per = (total + grid - 1) / grid;
+    per = splitters ? (total + splitters - 1) / splitters : 0;
     it = min(total, cta * per);
     end = min(total, it + per);
     whole = cta;

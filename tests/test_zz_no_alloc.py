@@ -63,6 +63,20 @@ def test_static_scratch_head_equals_the_definition_twice(d_model, vocab):
         assert torch.equal(arg2, arg)
 
 
+@pytest.mark.parametrize("d_model,vocab", [(64, 18944), (192, 19080), (128, 23048), (128, 23176), (64, 65536)])
+def test_static_scratch_head_over_all_sms(d_model, vocab):
+    """One CTA per SM (148): 148 tiles exactly, 150 (two left over, cut over the CTAs that have slots), 181 (33 left over
+    with a ragged last tile: whole), 182, and the largest vocabulary (512 tiles: 68 left over, whole)."""
+    build.build()
+    head = synth.tensor(41, 3, (vocab, d_model), 0.02, torch.bfloat16, "cuda:0")
+    for call, rows in enumerate((1, 37, 128)):
+        x = synth.tensor(42 + call, 4, (rows, d_model), 1.0, torch.bfloat16, "cuda:0")
+        arg, logits = binding.lm_head_static(x, head, want_logits=True)
+        _check_against_definition(x, head, arg, logits)
+        few, _ = binding.lm_head_static(x[:1].contiguous(), head)
+        assert torch.equal(few, arg[:1])                         # a row's choice does not depend on the others
+
+
 def test_static_scratch_head_matches_verify_forward_twice():
     build.build()
     desc = synth.ModelDesc(1, 256, 4, 4, 64, 256, 4104, 192, "bf16")
