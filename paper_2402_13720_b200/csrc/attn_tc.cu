@@ -51,6 +51,8 @@ constexpr int THREADS = WARPS * 32;
 // instruction fetches.  A row's arithmetic does not involve its tile's index or the other rows, so both sizes give the
 // same bits.
 
+constexpr int SHORT_ROUNDS = 2 * 148;   // CTAs of 16-row rounds that are resident at once (74 KB of shared memory each)
+
 struct AttnParams {
   const __nv_bfloat16 *q;          // [rows][H*HD] rotated queries
   const __nv_bfloat16 *k, *v;      // this layer's cache: [max_seq][Hkv*HD]
@@ -458,10 +460,15 @@ bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_
   p.scale_log2 = 1.4426950408889634f / sqrtf((float)d.head_dim);
   p.part = part;
   p.out = (__nv_bfloat16 *)out;
-  const int m_all = (d.n_heads / d.n_kv_heads) * rows;      // query rows per kv head, served 64 per CTA
-  const int mt = m_all <= 16 ? 1 : 4, qr = 16 * mt;         // rows per round (m_all is an upper bound when the count is on the device)
-  dim3 grid((n_vis_max + SPAN - 1) / SPAN, d.n_kv_heads, (m_all + qr - 1) / qr);
-  p.direct = n_vis_max <= SPAN;                             // a single span: nothing to fold
+  const int m_all = (d.n_heads / d.n_kv_heads) * rows;      // query rows per kv head (an upper bound when the count is on the device)
+  // A round of 16 query rows takes 9-11 us (its chain of latencies over four chunks), one of 64 rows 14-27 us, and the
+  // rounds of a short block run side by side: 16 rows each while all CTAs are resident at once.  (1.1B draft, 19 rows x 8
+  // heads over 540 keys: 27.0 us on 24 CTAs of 64 rows, 11.3 us on 80 CTAs of 16.)  Beyond that, larger rounds read the
+  // keys less often.
+  const int n_spans = (n_vis_max + SPAN - 1) / SPAN;
+  const int mt = n_spans * d.n_kv_heads * ((m_all + 15) / 16) <= SHORT_ROUNDS ? 1 : 4, qr = 16 * mt;
+  dim3 grid(n_spans, d.n_kv_heads, (m_all + qr - 1) / qr);
+  p.direct = n_spans <= 1;                                  // a single span: nothing to fold
   if (d.head_dim == 128) {
     if (mt == 1) launch_pdl(attn_span_kernel<128, 1>, grid, THREADS, Smem<128, 1>::BYTES, s, p);
     else launch_pdl(attn_span_kernel<128, 4>, grid, THREADS, Smem<128, 4>::BYTES, s, p);
