@@ -15,71 +15,66 @@ namespace fold {
 constexpr int SPAN_KEYS = 512;
 
 struct Params {
-  const float *part;               // [rows][H][cap][HD + 2]; NULL: nothing to fold
+  const float *part;               // [rows][H][cap][PIECE]; NULL: nothing to fold
   __nv_bfloat16 *out;              // [rows][H * HD]
   const int32_t *lin_end, *seg_len;   // per block row: keys seen = lin_end + seg_len
   const int *rows_dev;             // NULL, or the block's true row count in device memory
   int rows, H, cap, head_dim;
 };
 
-// Pairs first, first + step, .. (pair = row * H + head), two per pass so that their loads overlap.  Lane c fetches span
-// c's maximum and sum (cap <= 32), then every lane fetches its dims of every span before the first is used.
+// A piece: the span's score maximum and sum in front, two words of padding, then the output, so that a lane fetches its
+// dims of a piece with one 16-byte (head dim 64: 8-byte) load.
+template <int HD> constexpr int PIECE = HD + 4;
+template <int HD> struct Dims { typedef float4 V; };
+template <> struct Dims<64> { typedef float2 V; };
+__device__ __forceinline__ void add_scaled(float4 &a, const float4 &o, float w) { a.x += o.x * w; a.y += o.y * w; a.z += o.z * w; a.w += o.w * w; }
+__device__ __forceinline__ void add_scaled(float2 &a, const float2 &o, float w) { a.x += o.x * w; a.y += o.y * w; }
+__device__ __forceinline__ void store_bf16(__nv_bfloat16 *dst, const float4 &a, float s) {
+  __nv_bfloat162 lo = __floats2bfloat162_rn(a.x * s, a.y * s), hi = __floats2bfloat162_rn(a.z * s, a.w * s);
+  *reinterpret_cast<uint2 *>(dst) = make_uint2(*(uint32_t *)&lo, *(uint32_t *)&hi);
+}
+__device__ __forceinline__ void store_bf16(__nv_bfloat16 *dst, const float2 &a, float s) {
+  *reinterpret_cast<__nv_bfloat162 *>(dst) = __floats2bfloat162_rn(a.x * s, a.y * s);
+}
+
+// Pairs first, first + step, .. (pair = row * H + head).  Lane c fetches span c's maximum and sum (cap <= 32) while every
+// lane fetches its dims of up to UNR spans: one round trip to L2 up to 16 spans (8192 keys), two beyond.
 template <int HD>
 __device__ __forceinline__ void pairs(const Params &p, int rows, int first, int step, int lane) {
-  constexpr int PW = HD + 2, DPL = HD / 32, UNR = 12;
+  typedef typename Dims<HD>::V V;
+  constexpr int PW = PIECE<HD>, DPL = HD / 32, UNR = 16;
   const int n_pairs = rows * p.H;
-  for (int q0 = first; q0 < n_pairs; q0 += 2 * step) {
-    const float *src[2];
-    int ns[2];
-    float m_l[2], l_l[2];
+#pragma unroll 1
+  for (int q = first; q < n_pairs; q += step) {
+    const int r = q / p.H, ns = (p.lin_end[r] + p.seg_len[r] + SPAN_KEYS - 1) / SPAN_KEYS;
+    const float *src = p.part + (size_t)q * p.cap * PW;
+    float2 ml = make_float2(-INFINITY, 0.f);
+    if (lane < ns) ml = __ldcg(reinterpret_cast<const float2 *>(src + (size_t)lane * PW));
+    float mx = -INFINITY, w_l = 0.f, l = 0.f;
+    V acc{};
+#pragma unroll 1
+    for (int c0 = 0; c0 < ns; c0 += UNR) {
+      V o[UNR];
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int q = q0 + k * step;
-      ns[k] = 0;
-      src[k] = p.part;
-      if (q < n_pairs) {
-        const int r = q / p.H;
-        ns[k] = (p.lin_end[r] + p.seg_len[r] + SPAN_KEYS - 1) / SPAN_KEYS;
-        src[k] = p.part + (size_t)q * p.cap * PW;
+      for (int cc = 0; cc < UNR; ++cc) {
+        o[cc] = V{};
+        if (c0 + cc < ns) o[cc] = __ldcg(reinterpret_cast<const V *>(src + (size_t)(c0 + cc) * PW + 4 + DPL * lane));
       }
-      m_l[k] = -INFINITY;
-      l_l[k] = 0.f;
-      if (lane < ns[k]) {
-        m_l[k] = __ldcg(src[k] + (size_t)lane * PW);
-        l_l[k] = __ldcg(src[k] + (size_t)lane * PW + 1);
+      if (c0 == 0) {
+        mx = ml.x;
+#pragma unroll
+        for (int s = 16; s; s >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
+        w_l = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - mx);          // mx is finite: the first span holds a visible key
+      }
+#pragma unroll
+      for (int cc = 0; cc < UNR; ++cc) {
+        if (c0 + cc >= ns) break;                                    // uniform in the warp
+        const float w = __shfl_sync(0xffffffffu, w_l, c0 + cc);
+        l += __shfl_sync(0xffffffffu, ml.y, c0 + cc) * w;
+        add_scaled(acc, o[cc], w);
       }
     }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      if (ns[k] == 0) continue;                                    // uniform in the warp
-      float mx = m_l[k];
-#pragma unroll
-      for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const float w_l = (m_l[k] == -INFINITY) ? 0.f : exp2f(m_l[k] - mx);   // mx is finite: the first span holds a visible key
-      float l = 0.f, acc[DPL];
-#pragma unroll
-      for (int i = 0; i < DPL; ++i) acc[i] = 0.f;
-      for (int c0 = 0; c0 < ns[k]; c0 += UNR) {
-        float o[UNR][DPL];
-#pragma unroll
-        for (int cc = 0; cc < UNR; ++cc)
-#pragma unroll
-          for (int i = 0; i < DPL; ++i)
-            o[cc][i] = c0 + cc < ns[k] ? __ldcg(src[k] + (size_t)(c0 + cc) * PW + 2 + lane + 32 * i) : 0.f;
-#pragma unroll
-        for (int cc = 0; cc < UNR; ++cc) {
-          if (c0 + cc >= ns[k]) break;                              // uniform in the warp
-          const float w = __shfl_sync(0xffffffffu, w_l, c0 + cc);
-          l += __shfl_sync(0xffffffffu, l_l[k], c0 + cc) * w;
-#pragma unroll
-          for (int i = 0; i < DPL; ++i) acc[i] += o[cc][i] * w;
-        }
-      }
-      const float inv = 1.0f / l;
-      __nv_bfloat16 *dst = p.out + (size_t)(q0 + k * step) * HD;
-#pragma unroll
-      for (int i = 0; i < DPL; ++i) dst[lane + 32 * i] = __float2bfloat16_rn(acc[i] * inv);
-    }
+    store_bf16(p.out + (size_t)q * HD + DPL * lane, acc, 1.0f / l);
   }
 }
 

@@ -20,6 +20,7 @@
 // (virtual position -> key) and on fixed chunk, span and warp boundaries, never on the other rows of the block:
 // a token gets bit-identical attention whether it is verified inside a candidate block or decoded alone.
 #include "ouro_internal.h"
+#include "attn_fold.cuh"
 
 // Optional timeline (compile with -DOURO_TRACE): see gemm_tc.cu.
 #ifdef OURO_TRACE
@@ -59,7 +60,7 @@ struct AttnParams {
   const int32_t *lin_end, *seg_start, *seg_len, *group;
   int rows, H, Hkv, L, cap;        // L: cache length before the block; cap: span slots per (row, head)
   float scale_log2;
-  float *part;                     // [rows][H][cap][HD+2]: max (log2 domain), sum, unnormalised output
+  float *part;                     // [rows][H][cap][PIECE]: max (log2 domain), sum, -, -, unnormalised output
   __nv_bfloat16 *out;              // [rows][H*HD]
   int direct;                      // every row's keys lie in span 0: the span kernel normalises and writes `out` itself
   const int *rows_dev;             // NULL, or the block's true row count in device memory (`rows` is then an upper bound)
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
   constexpr int QR = S::QR;
   constexpr int CPR = HD / 8;                  // 16-byte pieces per row
   constexpr int ROWB = S::ROWB;
-  constexpr int PW = HD + 2;
+  constexpr int PW = fold::PIECE<HD>;
   constexpr int DW = HD / WARPS;               // output dims per warp in the P V phase (16 or 8)
   constexpr int NT2 = DW / 8;                  // 8-dim MMA tiles per warp
   extern __shared__ __align__(128) uint8_t smem[];
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
 #pragma unroll
       for (int nt = 0; nt < NT2; ++nt) {
         int d = warp * DW + 8 * nt + 2 * (lane & 3);
-        *reinterpret_cast<float2 *>(dst + 2 + d) = make_float2(o[i >> 1][nt][2 * (i & 1)], o[i >> 1][nt][2 * (i & 1) + 1]);
+        *reinterpret_cast<float2 *>(dst + 4 + d) = make_float2(o[i >> 1][nt][2 * (i & 1)], o[i >> 1][nt][2 * (i & 1) + 1]);
       }
     }
     TRACE(5);
@@ -433,7 +434,7 @@ bool attention_tc_supported(const ouro_model_desc &d) {
 size_t attention_tc_scratch_bytes(const ouro_model_desc &d) {
   if (!attention_tc_supported(d)) return 0;
   size_t cap = (d.max_seq + SPAN - 1) / SPAN;
-  return (size_t)OURO_MAX_ROWS * d.n_heads * cap * (d.head_dim + 2) * sizeof(float);
+  return (size_t)OURO_MAX_ROWS * d.n_heads * cap * (d.head_dim + 4) * sizeof(float);
 }
 
 template <int HD, int MT>

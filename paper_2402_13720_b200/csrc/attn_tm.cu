@@ -30,6 +30,7 @@
 #include <cuda.h>
 
 #include "ouro_internal.h"
+#include "attn_fold.cuh"
 
 // Optional timeline (compile with -DOURO_TRACE): see gemm_tc.cu.
 #ifdef OURO_TRACE
@@ -52,9 +53,10 @@ namespace {
 constexpr int HD = 128;
 constexpr int CH = 128;            // keys per chunk
 constexpr int SC = 4;              // chunks per span
-constexpr int SPAN = CH * SC;      // must equal the span of the merge kernel
+constexpr int SPAN = CH * SC;
+static_assert(SPAN == fold::SPAN_KEYS, "the fold's spans");
 constexpr int QR = 128;            // query rows per round = TMEM lanes
-constexpr int PW = HD + 2;
+constexpr int PW = fold::PIECE<HD>;
 constexpr int ROW_THREADS = 256;  // two threads per query row
 constexpr int THREADS = 64 + ROW_THREADS;
 constexpr uint32_t SPIN_LIMIT = 1u << 22;
@@ -94,7 +96,7 @@ struct TmParams {
   int rows, H, Hkv, L, cap, row0;  // row0: first row of this layer in the tensor maps
   int n_spans;
   float scale_log2;
-  float *part;                     // [rows][H][cap][HD+2]: max (log2 domain), sum, unnormalised output
+  float *part;                     // [rows][H][cap][PIECE]: max (log2 domain), sum, -, -, unnormalised output
   __nv_bfloat16 *out;              // [rows][H*HD], written here only when `direct`
   int direct;                      // every row's keys lie in span 0: normalise and write `out`, no folding needed
   int *status;
@@ -650,7 +652,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
         float *dst = p.part + (((size_t)r * p.H + kvh * g + hq) * p.cap + sc) * PW;
         if (h == 0) *reinterpret_cast<float2 *>(dst) = make_float2(m_run, lsum[t] + lsum[QR + t]);
 #pragma unroll
-        for (int d = 0; d < HD / 2; d += 2) *reinterpret_cast<float2 *>(dst + 2 + h * 64 + d) = make_float2(o_reg[d], o_reg[d + 1]);
+        for (int d = 0; d < HD / 2; d += 4)
+          *reinterpret_cast<float4 *>(dst + 4 + h * 64 + d) = make_float4(o_reg[d], o_reg[d + 1], o_reg[d + 2], o_reg[d + 3]);
       }
     }
   }

@@ -10,16 +10,20 @@
 //     (stream-K), so every SM streams the same number of bytes whatever N and K are;
 //   * a span that covers only part of a tile's K range leaves a partial tile in scratch memory.  After its last
 //     MMA every contributor of a tile adds up a share of the tile's tokens (token t belongs to contributor
-//     t mod n) in ascending K order and runs the epilogue on them.  A CTA waits for the others' partials only
+//     t mod n) in ascending K order and runs the epilogue on them.  The partial sums carry their own arrival (see
+//     EMPTY).  A CTA waits for the others' partials only
 //     after it has published all of its own, so the waits cannot form a cycle (and they are bounded); the
 //     result does not depend on arrival order;
 //   * warp 0 issues TMA loads into a ring of shared-memory stages (128-byte swizzle), warp 1 issues
-//     tcgen05.mma and releases stages with tcgen05.commit, warps 2-5 drain TMEM (double buffered) and run the
+//     tcgen05.mma and releases stages with tcgen05.commit, warps 2-9 drain TMEM (double buffered) and run the
 //     epilogue: plain store, residual add, or SiLU(gate)*up for the stacked gate/up matrices.
 // The span boundaries depend on N, K and the grid only, never on the number of rows, and an output element
 // is a function of its own row of X: a token's result is bitwise the same in a 1-row and in a 128-row call.
 // Every mbarrier wait is bounded; on expiry the CTA raises the context's status word and drains.
 #include <cuda.h>
+
+#include <atomic>
+#include <type_traits>
 
 #include "ouro_internal.h"
 #include "weight_stream.cuh"
@@ -51,7 +55,10 @@ using ws::BLOCK_K;
 using ws::TILE_N;
 using ws::Span;
 constexpr int A_BYTES = TILE_N * BLOCK_K * 2;
-constexpr int THREADS = 224;      // warp 0 weight TMA, warp 1 MMA, warps 2..5 epilogue, warp 6 activation TMA
+constexpr int EPI_WARPS = 8;      // two per TMEM lane quarter
+constexpr int EPI_THREADS = 32 * EPI_WARPS;
+constexpr int ACT_WARP = 2 + EPI_WARPS;
+constexpr int THREADS = 32 * (ACT_WARP + 1);   // warp 0 weight TMA, warp 1 MMA, warps 2..9 epilogue, warp 10 activation TMA
 constexpr int W_PRODUCERS = 2;    // lanes of warp 0 that issue the weight copies, stage by stage in turn (a power of two, smaller than the ring)
 constexpr int MAX_GRID = 160;
 constexpr int SLOT_FLOATS = TILE_N * OURO_MAX_ROWS;
@@ -62,16 +69,18 @@ constexpr unsigned long long HINT_EVICT_LAST = 0x14F0000000000000ull;
 enum { MODE_STORE = 0, MODE_RESIDUAL = 1, MODE_SWIGLU = 2, MODE_HEAD = 3, MODE_QKV = 4 };
 // HEAD: per-tile row maxima (+ optional logits).  QKV: rotary positions on q and k, q to its buffer, k and v appended to the cache.
 
-struct GemmParams {
+struct GemmMaps {
   CUtensorMap a[3];   // weight matrices stacked along the output dimension (q|k|v), or gate and up
   CUtensorMap b;      // activations, box = 64 x t_pad
+};
+struct GemmParams {
   int a_tiles[3];     // tiles of each stacked matrix (MODE_STORE / MODE_RESIDUAL)
   int a_rows[3];      // output features of each stacked matrix
   int a_count;
   int mode;
   int tiles;          // total tiles
   int kb;             // k-blocks per tile (K / 64)
-  int splitters;      // CTAs that share the remainder tiles (see weight_stream.cuh); -1: the whole grid
+  int t0, per;        // tiles below t0 are handled whole; the others are cut into spans of `per` k-blocks (ws::cut)
   int t_pad;          // tokens padded to a multiple of 16 (MMA N)
   int rows;           // valid tokens (an upper bound when rows_dev is set)
   const int *rows_dev;  // NULL, or where the block's true row count sits in device memory: the host then sizes the
@@ -97,10 +106,7 @@ struct GemmParams {
   const float *ss_in;         // other modes: sums of squares of the activation rows (NULL: no scaling)
   int ss_tiles;
   float ss_inv_d, eps;
-  float *scratch;     // [grid][2][t][128] partial tiles
-  int *counters;      // [tiles] partial tiles published, as (gen << 8) + count: a word left by an earlier GEMM is
-                      // smaller than this GEMM's (gen << 8), so nothing has to be cleared between GEMMs or launches
-  int gen;            // this GEMM's generation number (1 .. 2^22, grows with every GEMM the context runs)
+  float *scratch;     // [grid][2][t][128] partial tiles; a word that holds no partial sum holds EMPTY
   int *status;        // context status word
   int trace_id;           // which GEMM of the layer this is (timeline builds only)
   uint32_t wait_limit;    // polls of a partial-tile wait before it gives up (1 << 22 unless a test shortens it)
@@ -112,7 +118,7 @@ struct GemmParams {
 // a counter in global memory (one per chain position, counting finished tiles, never reset: the host passes the value
 // it will have reached).  All GEMMs of a chain have the same rows / t_pad / stages.
 constexpr int MAX_CHAIN = 4;
-struct ChainParams {
+struct ChainArgs {
   GemmParams g[MAX_CHAIN];
   int n;
   int *finished;            // [MAX_CHAIN + 1] tiles finished, per chain position (monotonic); last: CTAs done folding
@@ -133,7 +139,12 @@ struct ChainParams {
     int rows, d;
   } embed;
 };
+struct ChainParams {
+  GemmMaps maps[MAX_CHAIN];
+  ChainArgs args;
+};
 static_assert(sizeof(ChainParams) <= 4096, "kernel parameters");
+constexpr int MISC_BYTES = 1536;   // barriers, flags, per-token factors and positions
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -211,9 +222,38 @@ __device__ __forceinline__ float ordered_f32(uint32_t u) {
 }
 // x * sigmoid(x) with the fast exponential and reciprocal (the result is rounded to bf16 right after)
 __device__ __forceinline__ float silu(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
-__device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-// one half (64 threads) of the epilogue warps; grp = 0 or 1
-__device__ __forceinline__ void group_barrier(int grp) { asm volatile("bar.sync %0, 64;" ::"r"(2 + grp) : "memory"); }
+__device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory"); }
+// one half of the epilogue warps; grp = 0 or 1
+__device__ __forceinline__ void group_barrier(int grp) { asm volatile("bar.sync %0, %1;" ::"r"(2 + grp), "n"(EPI_THREADS / 2) : "memory"); }
+// Partial sums travel between CTAs without flags: a scratch word is EMPTY until its contributor has stored the sum, and
+// whoever fetches it (exactly one thread of one CTA) empties it again.  The fetching thread polls the words themselves, so
+// a partial tile costs one store and one load latency; with a fence, an arrival counter and a poll of that in between it
+// was 4.5 us from the last contraction to the sum (7B output projection, 37 rows), now 3.3.  EMPTY is a NaN the tensor
+// cores do not produce (theirs is 0x7fffffff).  A GEMM's stores into a slot come after the hand-over of the GEMM before it (or the
+// end of the launch before it), which the fetching threads signal after having emptied their words.
+constexpr uint32_t EMPTY = 0xffffffffu;
+__device__ __forceinline__ void part_store(float *dst, float v) {
+  const uint32_t u = __float_as_uint(v);
+  asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(dst), "r"(u == EMPTY ? 0x7fffffffu : u) : "memory");
+}
+// Predicated inside the assembly: several of these in a row are in flight together, where a branch around each would wait
+// for one before the next is requested.  A load that is left out gives zeros.
+__device__ __forceinline__ uint4 part_load(const float *src, bool wanted) {
+  uint4 v;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "mov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\tmov.b32 %3, 0;\n\t"
+      "@p ld.relaxed.gpu.global.v4.b32 {%0, %1, %2, %3}, [%4];\n\t}"
+      : "=&r"(v.x), "=&r"(v.y), "=&r"(v.z), "=&r"(v.w)
+      : "l"(src), "r"((uint32_t)wanted)
+      : "memory");
+  return v;
+}
+__device__ __forceinline__ bool part_there(const uint4 &v) { return v.x != EMPTY && v.y != EMPTY && v.z != EMPTY && v.w != EMPTY; }
+__device__ __forceinline__ void part_empty(float *src) {
+  asm volatile("st.relaxed.gpu.global.v4.b32 [%0], {%1, %1, %1, %1};" ::"l"(src), "r"(EMPTY) : "memory");
+}
 constexpr int STAGE_TOK = 64;     // tokens of a whole tile parked in shared memory at a time
 constexpr int STAGE_PITCH = TILE_N + 4;   // floats per parked token: 16-byte aligned rows that start 4 banks apart
 constexpr int STAGE_BYTES = STAGE_TOK * STAGE_PITCH * 4;
@@ -221,7 +261,7 @@ constexpr int STAGE_BYTES = STAGE_TOK * STAGE_PITCH * 4;
 // The schedule of this launch for CTA blockIdx.x (see weight_stream.cuh).
 struct SpanWalker : ws::SpanWalker {
   __device__ SpanWalker(const GemmParams &p)
-      : ws::SpanWalker(p.tiles, p.kb, (int)gridDim.x, p.splitters < 0 ? (int)gridDim.x : p.splitters, (int)blockIdx.x) {}
+      : ws::SpanWalker(p.tiles, p.kb, p.t0, p.per, (int)gridDim.x, (int)blockIdx.x) {}
 };
 
 // Locates a tile: which stacked matrix, its first row there, and the first output column.
@@ -249,16 +289,17 @@ __device__ __forceinline__ bool counter_wait(const int *counter, int target, con
   }
   return false;
 }
-__device__ __forceinline__ bool chain_wait(const ChainParams &cp, int i) {
+__device__ __forceinline__ bool chain_wait(const ChainArgs &cp, int i) {
   return counter_wait(cp.finished + i, cp.target[i], cp.g[0].status, 1u << 22);
 }
 
-__global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_constant__ ChainParams cp) {
+__global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_constant__ ChainParams kp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const ChainArgs &cp = kp.args;
   const GemmParams &p0 = cp.g[0];                 // rows, t_pad and stages are common to the chain
-  const int n_stages = p0.stages;
-  const int b_bytes = p0.t_pad * BLOCK_K * 2;
+  const int n_stages = p0.stages, t_pad = p0.t_pad;
+  const int b_bytes = t_pad * BLOCK_K * 2;
   const int stage_bytes = A_BYTES + b_bytes;
   uint8_t *ring = smem;
   float *xchg = (float *)(ring + (size_t)n_stages * stage_bytes);          // [64 tokens][128] accumulators of a whole tile
@@ -266,15 +307,14 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
   uint64_t *full = bars, *empty = bars + 16, *acc_full = bars + 32, *acc_empty = bars + 34;
   uint32_t *tmem_base_p = (uint32_t *)(bars + 36);
   volatile int *abort_flag = (volatile int *)(bars + 37);
-  volatile int *wait_flag = (volatile int *)(bars + 39);   // [0..1]: outcome of an accumulator wait; [2]: a fix-up gave up; [4..5]: outcome of a fix-up group's wait
+  volatile int *wait_flag = (volatile int *)(bars + 39);   // [0..1]: outcome of an accumulator wait; [2]: a fix-up gave up
   uint64_t *drain_bar = bars + 44;                          // give-up path: "every contraction issued so far has completed"
   float *rs = (float *)(bars + 48);                         // [128] per-token factor 1/rms of the consumed activations
   int *spos = (int *)(rs + OURO_MAX_ROWS);                  // [128] token positions (rotary table rows), QKV epilogue
 
   pdl_trigger();
-  if (threadIdx.x == 0) { const GemmParams &p = p0; TRACE(0); }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int acc_cols = p0.t_pad <= 32 ? 32 : p0.t_pad <= 64 ? 64 : 128;   // columns per accumulator buffer
+  const int acc_cols = t_pad <= 32 ? 32 : t_pad <= 64 ? 64 : 128;   // columns per accumulator buffer
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < n_stages; ++s) {
@@ -283,7 +323,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], 4);
+      mbar_init(&acc_empty[a], EPI_WARPS);
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
@@ -298,13 +338,14 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem_base = *tmem_base_p;
+  if (threadIdx.x == 0) { const GemmParams &p = p0; TRACE(0); }
   uint32_t n_issued = 0;                           // producer lanes: stages they have issued copies into
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
     if (lane < W_PRODUCERS) {
       // The weights do not depend on the previous kernel, so this warp never waits for it: the ring fills with
-      // weight tiles while the predecessor drains.  The activation tiles come from warp 6, after its wait.
+      // weight tiles while the predecessor drains.  The activation tiles come from another warp, after its wait.
       // One thread runs this loop once per 16 KB stage; at 40 GB/s per SM that is every 0.4 us, so the loop carries
       // no division and nothing that is constant over a span: stage index and ring round are counted along.
       uint32_t n = 0, round = 0;
@@ -318,7 +359,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       while (ok && w.next(s)) {
         int seg = 0, row0 = s.tile * 64, col0, valid;
         if (!swiglu) locate(p, s.tile, seg, row0, col0, valid);
-        const CUtensorMap *m0 = &p.a[seg];
+        const CUtensorMap *m0 = &kp.maps[ci].a[seg];
         uint8_t *sa = ring + (size_t)st * stage_bytes;
         for (int kb = s.kb0; kb < s.kb1; ++kb, ++n) {
           if ((n & (W_PRODUCERS - 1)) == (uint32_t)lane) {           // the lanes take the stages in turn
@@ -328,8 +369,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
             }
             mbar_expect_tx(&full[st], A_BYTES);
             if (swiglu) {
-              tma_load_2d(sa, &p.a[0], &full[st], kb * BLOCK_K, row0, HINT_EVICT_FIRST);
-              tma_load_2d(sa + A_BYTES / 2, &p.a[1], &full[st], kb * BLOCK_K, row0, HINT_EVICT_FIRST);
+              tma_load_2d(sa, &kp.maps[ci].a[0], &full[st], kb * BLOCK_K, row0, HINT_EVICT_FIRST);
+              tma_load_2d(sa + A_BYTES / 2, &kp.maps[ci].a[1], &full[st], kb * BLOCK_K, row0, HINT_EVICT_FIRST);
             } else {
               tma_load_2d(sa, m0, &full[st], kb * BLOCK_K, row0, HINT_EVICT_FIRST);
             }
@@ -343,7 +384,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       if (!ok) { *abort_flag = 1; atomicExch(p0.status, 1); }
       n_issued = n;
     }
-  } else if (warp == 6) {
+  } else if (warp == ACT_WARP) {
     // ---------------------------------------------------------------- activation producer
     if (lane == 0) {
       pdl_wait();                                  // the first GEMM's activations are the previous kernel's output
@@ -374,7 +415,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
               if (!ok) break;
             }
             mbar_expect_tx(&full[st], b_bytes);
-            tma_load_2d(sb, &p.b, &full[st], kb * BLOCK_K, 0, HINT_EVICT_LAST);
+            tma_load_2d(sb, &kp.maps[ci].b, &full[st], kb * BLOCK_K, 0, HINT_EVICT_LAST);
             sb += stage_bytes;
             if (++st == n_stages) { st = 0; ++round; sb = ring + A_BYTES; }
           }
@@ -428,18 +469,19 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
     pdl_wait();
     const int q = warp & 3;                      // TMEM lane quarter this warp may read
     const int nl = q * 32 + lane;                // row of the tile held by this thread
-    const int et = threadIdx.x - 64;             // 0..127 among the epilogue threads
+    const int et = threadIdx.x - 64;             // 0..255 among the epilogue threads
+    const int wh = (warp - 2) >> 2;              // which of the two warps of its lane quarter this is
     uint32_t item = 0;
     bool ok = true;
     float v[16];
     if (cp.fold.part || cp.embed.table) {
-      const int gw = (int)blockIdx.x * 4 + (warp - 2), nw = (int)gridDim.x * 4;
+      const int gw = (int)blockIdx.x * EPI_WARPS + (warp - 2), nw = (int)gridDim.x * EPI_WARPS;
       if (cp.fold.part) {
         fold::run(cp.fold, gw, nw, lane);
       } else {
         // Embedding rows into the residual stream, plus what the first norm's consumer needs: bf16(gain * x) and the
         // sums of squares per 128-column tile.  One warp per (row, tile): four columns per lane.
-        const ChainParams::Embed &e = cp.embed;
+        const ChainArgs::Embed &e = cp.embed;
         const int rows = e.rows_dev ? min(e.rows, __ldg(e.rows_dev)) : e.rows, tiles = (e.d + TILE_N - 1) / TILE_N;
         for (int it = gw; it < rows * tiles; it += nw) {
           const int r = it / tiles, col = (it - r * tiles) * TILE_N + 4 * lane;
@@ -479,277 +521,213 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
     const int rows = p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows;
     SpanWalker w(p);
     Span s;
-    int pend_tile[2], pend_n[2], pend_first[2], n_pend = 0;     // partial tiles this CTA contributed to (<= 2)
+    int pend_tile[2] = {0, 0}, pend_n[2] = {1, 1}, pend_first[2] = {0, 0}, n_pend = 0;     // partial tiles this CTA contributed to (<= 2)
     float *stage = xchg;                                         // [STAGE_TOK tokens][STAGE_PITCH] fp32, 128 tile rows each
 
     // Finishing tokens of a tile.  Whatever produced the accumulator values - this CTA's own whole tile, parked
     // in shared memory token-major, or the partial tiles of all contributors in scratch - the last step is the
     // same: a group of G threads walks over "its" tokens, a warp's 32 lanes holding the tile's 128 rows (= output
     // columns) four apiece, so every global access is a 16-byte piece of a contiguous 512-byte row.
-    //   whole tile:  stg != NULL; tokens t_base + tg + TG j below t_lim (one staged chunk of tokens)
-    //   split tile:  stg == NULL; tokens my + n (tg + TG j): contributor `my` of n takes the tokens t = my (mod n)
-    //                and adds the partials up in ascending K order; it first waits (bounded) until all n have
-    //                published, and fetches what the epilogue itself reads (residual stream, rotary table) for its
-    //                first tokens before that wait.
-    // Returns false when the wait gave up.
-    auto others_there = [&](int tile, int n, int gi, int grp, int G) -> bool {
-      if (gi == 0) {
-        wait_flag[4 + grp] = counter_wait(p.counters + tile, (p.gen << 8) + n, p.status, p.wait_limit) && !*abort_flag;
-        TRACE(6);
-      }
-      // The polling thread's acquire and the barrier order the others' reads of the partial sums behind the
-      // contributors' releases; those reads go to L2 (ld.global.cg), so no fence of their own is needed.
-      if (G == 128) epi_barrier(); else group_barrier(grp);
-      if (gi == 0 && grp == 0) TRACE(9);
-      return wait_flag[4 + grp] != 0;
-    };
-
-    auto finish_plain = [&](int tile, int gi, int G, int grp, int my, int n, int first, const float *stg, int t_base,
-                            int t_lim) -> bool {
-      int seg, row0, col0, valid;
-      locate(p, tile, seg, row0, col0, valid);
+    //   whole tile:  tokens t_base + tg + TG i below t_lim (one staged chunk of tokens)
+    //   split tile:  contributor `my` of n takes the tokens t = my (mod n), that is my + n (tg + TG i), and adds the
+    //                partials up in ascending K order as they arrive
+    // Returns false (warp-uniform) when the wait for a partial gave up.
+    auto finish = [&](auto split_c, int tile, int gi, int G, int my, int n, int first, float *stg, int t_base, int t_lim) -> bool {
+      constexpr bool SPLIT = decltype(split_c)::value;
+      const bool swiglu = p.mode == MODE_SWIGLU;                     // tile rows 0..63: gate of 64 features, 64..127: up
+      int seg = 0, row0 = 0, col0 = 0, valid = TILE_N;
+      if (!swiglu) locate(p, tile, seg, row0, col0, valid);
       const int ng = gi & 31, tg = gi >> 5, TG = G >> 5;
       const int col = col0 + 4 * ng;
       // Every matrix has a multiple of 8 output features (the shape checks see to it), so a thread's four columns are
       // inside the matrix together or not at all.
       const bool full4 = 4 * ng < valid;
-      const int js = n * TG;                                         // token step inside a batch of four
+      const int js = n * TG;                                         // step between this warp's tokens
       const int cm = row0 + 4 * ng;                                  // first of this thread's 4 columns inside q, k or v
       const int half = p.head_dim >> 1;
-      const bool upper = (cm & half) != 0;
       const bool res_norm = p.mode == MODE_RESIDUAL && p.gain != nullptr;
       const bool rope = p.mode == MODE_QKV && seg != 2;
-      float gn[4] = {0.f, 0.f, 0.f, 0.f};
-      if (res_norm) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) gn[e] = full4 ? __bfloat162float(p.gain[col + e]) : 0.f;
-      }
-      // what the epilogue reads besides the accumulators, for the four tokens of a batch at once
-      auto load_ops = [&](int tb, float4 *oa, float4 *ob) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int t = tb + j * js;
-          oa[j] = ob[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (t >= t_lim) continue;
-          if (res_norm) {
-            const float *y = p.out_f32 + (size_t)t * p.ldo + col;
-            if (full4) oa[j] = *reinterpret_cast<const float4 *>(y);
-          } else if (rope) {
-            const size_t ti = (size_t)spos[t] * half + (cm & (half - 1));
-            oa[j] = *reinterpret_cast<const float4 *>(p.cos_t + ti);
-            ob[j] = *reinterpret_cast<const float4 *>(p.sin_t + ti);
-          }
-        }
-      };
-      const int tb0 = t_base + my + n * tg;
-      float4 oa[4], ob[4];
-      if (tb0 < t_lim) load_ops(tb0, oa, ob);
-      if (!stg && !others_there(tile, n, gi, grp, G)) return false;
-      for (int tb = tb0; tb < t_lim; tb += 4 * js) {                 // tokens are uniform inside a warp
-        if (tb != tb0) load_ops(tb, oa, ob);
-        float4 acc[4];
-        if (stg) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int t = tb + j * js;
-            acc[j] = t < t_lim ? *reinterpret_cast<const float4 *>(stg + (size_t)(t - t_base) * STAGE_PITCH + 4 * ng)
-                               : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-          for (int c0 = 0; c0 < n; c0 += 4) {
-            float4 tmp[4][4];
-#pragma unroll
-            for (int cc = 0; cc < 4; ++cc) {
-              const int owner = first + c0 + cc;
-              const float *src = p.scratch + ((size_t)owner * 2 + w.owner_slot(tile, owner)) * SLOT_FLOATS + 4 * ng;
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const int t = tb + j * js;
-                tmp[cc][j] = (c0 + cc < n && t < t_lim) ? __ldcg((const float4 *)(src + (size_t)t * TILE_N))
-                                                         : make_float4(0.f, 0.f, 0.f, 0.f);
-              }
-            }
-#pragma unroll
-            for (int cc = 0; cc < 4; ++cc)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                acc[j].x += tmp[cc][j].x; acc[j].y += tmp[cc][j].y; acc[j].z += tmp[cc][j].z; acc[j].w += tmp[cc][j].w;
-              }
-          }
-        }
-        if (!stg && tb == tb0 && gi == 0 && grp == 0) {
-          if (acc[0].x == 1.2345e-30f) TRACE(14);                    // (keeps the partial sums live up to here)
-          TRACE(12);
-        }
+      uint2 graw = make_uint2(0, 0);
+      if (res_norm && full4) graw = *reinterpret_cast<const uint2 *>(p.gain + col);
+
+      auto finish_token = [&](int t, const float4 acc) {
         if (res_norm) {
           // new residual stream, its bf16(gain * x) image for the next GEMM, and this tile's sums of squares
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int t = tb + j * js;
-            if (t >= t_lim) continue;                                // uniform inside the warp
-            float *y = p.out_f32 + (size_t)t * p.ldo + col;
-            const float yn[4] = {oa[j].x + acc[j].x, oa[j].y + acc[j].y, oa[j].z + acc[j].z, oa[j].w + acc[j].w};
-            float sq = 0.f;
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              if (full4) sq += yn[e] * yn[e];
-            if (full4) {
-              *reinterpret_cast<float4 *>(y) = make_float4(yn[0], yn[1], yn[2], yn[3]);
-              __nv_bfloat162 lo = __floats2bfloat162_rn(gn[0] * yn[0], gn[1] * yn[1]);
-              __nv_bfloat162 hi = __floats2bfloat162_rn(gn[2] * yn[2], gn[3] * yn[3]);
-              *reinterpret_cast<uint2 *>(p.xb + (size_t)t * p.ldo + col) = make_uint2(*(uint32_t *)&lo, *(uint32_t *)&hi);
-            }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-            if (lane == 0) p.ss_out[(size_t)tile * OURO_MAX_ROWS + t] = sq;
+          float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (full4) {
+            float *x = p.out_f32 + (size_t)t * p.ldo + col;
+            y = acc;
+            if (!SPLIT) { const float4 x4 = *reinterpret_cast<const float4 *>(x); y.x += x4.x; y.y += x4.y; y.z += x4.z; y.w += x4.w; }
+            *reinterpret_cast<float4 *>(x) = y;
+            const __nv_bfloat162 g01 = *reinterpret_cast<const __nv_bfloat162 *>(&graw.x), g23 = *reinterpret_cast<const __nv_bfloat162 *>(&graw.y);
+            __nv_bfloat162 lo = __floats2bfloat162_rn(__low2float(g01) * y.x, __high2float(g01) * y.y);
+            __nv_bfloat162 hi = __floats2bfloat162_rn(__low2float(g23) * y.z, __high2float(g23) * y.w);
+            *reinterpret_cast<uint2 *>(p.xb + (size_t)t * p.ldo + col) = make_uint2(*(uint32_t *)&lo, *(uint32_t *)&hi);
           }
-          continue;
+          float sq = 0.f;
+          sq += y.x * y.x; sq += y.y * y.y; sq += y.z * y.z; sq += y.w * y.w;
+#pragma unroll
+          for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+          if (lane == 0) p.ss_out[(size_t)tile * OURO_MAX_ROWS + t] = sq;
+          return;
         }
-        if (p.mode == MODE_QKV) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int t = tb + j * js;
-            if (t >= t_lim) continue;                                // uniform inside the warp
-            const float r = rs[t];
-            const float vals[4] = {acc[j].x * r, acc[j].y * r, acc[j].z * r, acc[j].w * r};
-            float other[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) other[e] = __shfl_xor_sync(0xffffffffu, vals[e], half >> 2);
-            const float cs[4] = {oa[j].x, oa[j].y, oa[j].z, oa[j].w}, sn[4] = {ob[j].x, ob[j].y, ob[j].z, ob[j].w};
-            float rv[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              rv[e] = seg == 2 ? vals[e] : (upper ? vals[e] * cs[e] + other[e] * sn[e] : vals[e] * cs[e] - other[e] * sn[e]);
-            __nv_bfloat16 *dst = seg == 0 ? p.q_out + (size_t)t * p.dq + cm
-                               : seg == 1 ? p.k_out + (size_t)(p.L + t) * p.dkv + cm
-                                          : p.v_out + (size_t)(p.L + t) * p.dkv + cm;
-            if (full4) {
-              __nv_bfloat162 lo = __floats2bfloat162_rn(rv[0], rv[1]), hi = __floats2bfloat162_rn(rv[2], rv[3]);
-              *reinterpret_cast<uint2 *>(dst) = make_uint2(*(uint32_t *)&lo, *(uint32_t *)&hi);
+        const float r = rs[t];
+        float4 v4 = make_float4(acc.x * r, acc.y * r, acc.z * r, acc.w * r);
+        if (swiglu || p.mode == MODE_QKV) {
+          __nv_bfloat16 *dst;
+          bool store = full4;
+          if (swiglu || rope) {
+            // the other half of the pair sits in another lane: gate with up, or dimension i with i + head_dim/2
+            const int x = swiglu ? 16 : half >> 2;
+            const float4 o4 = make_float4(__shfl_xor_sync(0xffffffffu, v4.x, x), __shfl_xor_sync(0xffffffffu, v4.y, x),
+                                          __shfl_xor_sync(0xffffffffu, v4.z, x), __shfl_xor_sync(0xffffffffu, v4.w, x));
+            if (swiglu) {
+              const int feat = tile * 64 + 4 * ng;
+              v4 = make_float4(silu(v4.x) * o4.x, silu(v4.y) * o4.y, silu(v4.z) * o4.z, silu(v4.w) * o4.w);
+              dst = p.out_bf16 + (size_t)t * p.a_rows[0] + feat;
+              store = ng < 16 && feat < p.a_rows[0];
+            } else {
+              const size_t ti = (size_t)spos[t] * half + (cm & (half - 1));
+              const float4 cs = *reinterpret_cast<const float4 *>(p.cos_t + ti);
+              float4 sn = *reinterpret_cast<const float4 *>(p.sin_t + ti);
+              if ((cm & half) == 0) sn = make_float4(-sn.x, -sn.y, -sn.z, -sn.w);     // lower half: a cos - b sin
+              v4 = make_float4(v4.x * cs.x + o4.x * sn.x, v4.y * cs.y + o4.y * sn.y, v4.z * cs.z + o4.z * sn.z, v4.w * cs.w + o4.w * sn.w);
+              dst = seg == 0 ? p.q_out + (size_t)t * p.dq + cm : p.k_out + (size_t)(p.L + t) * p.dkv + cm;
             }
+          } else {
+            dst = p.v_out + (size_t)(p.L + t) * p.dkv + cm;                          // v goes to the cache as it is
           }
-          continue;
+          if (store) {
+            __nv_bfloat162 lo = __floats2bfloat162_rn(v4.x, v4.y), hi = __floats2bfloat162_rn(v4.z, v4.w);
+            *reinterpret_cast<uint2 *>(dst) = make_uint2(*(uint32_t *)&lo, *(uint32_t *)&hi);
+          }
+          return;
         }
+        if (p.mode == MODE_HEAD) {                                   // the warp's 32 lanes hold the tile's 128 columns
+          const float vals[4] = {v4.x, v4.y, v4.z, v4.w};
+          uint32_t bu = 0;
+          int bi = col;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int t = tb + j * js;
-          if (t >= t_lim) continue;                                  // uniform inside the warp
-          const float r = rs[t];
-          const float vals[4] = {acc[j].x * r, acc[j].y * r, acc[j].z * r, acc[j].w * r};
-          if (p.mode == MODE_HEAD && !stg) {                         // the warp's 32 lanes hold the tile's 128 columns
-            uint32_t bu = 0;
-            int bi = col;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              uint32_t uo = ordered_u32(vals[e]);
-              if (full4 && uo > bu) { bu = uo; bi = col + e; }
-            }
-            const uint32_t mx = __reduce_max_sync(0xffffffffu, bu);
-            const int src_lane = __ffs(__ballot_sync(0xffffffffu, bu == mx)) - 1;   // lowest lane = smallest index
-            bi = __shfl_sync(0xffffffffu, bi, src_lane);
-            if (lane == 0) {
-              p.tile_max[(size_t)tile * OURO_MAX_ROWS + t] = ordered_f32(mx);
-              p.tile_arg[(size_t)tile * OURO_MAX_ROWS + t] = bi;
-            }
+          for (int e = 0; e < 4; ++e) {
+            const uint32_t uo = ordered_u32(vals[e]);
+            if (full4 && uo > bu) { bu = uo; bi = col + e; }
           }
-          if (p.out_f32) {
-            float *y = p.out_f32 + (size_t)t * p.ldo + col;
-            const bool add = p.mode == MODE_RESIDUAL;
-            if (full4) {                                              // the row pitch is a multiple of 4 as well
-              float4 o4 = make_float4(vals[0], vals[1], vals[2], vals[3]);
-              if (add) { const float4 y4 = *reinterpret_cast<const float4 *>(y); o4.x += y4.x; o4.y += y4.y; o4.z += y4.z; o4.w += y4.w; }
-              *reinterpret_cast<float4 *>(y) = o4;
-            }
+          const uint32_t mx = __reduce_max_sync(0xffffffffu, bu);
+          const int src_lane = __ffs(__ballot_sync(0xffffffffu, bu == mx)) - 1;      // lowest lane = smallest index
+          bi = __shfl_sync(0xffffffffu, bi, src_lane);
+          if (lane == 0) {
+            p.tile_max[(size_t)tile * OURO_MAX_ROWS + t] = ordered_f32(mx);
+            p.tile_arg[(size_t)tile * OURO_MAX_ROWS + t] = bi;
           }
         }
-      }
-      return true;
-    };
+        if (p.out_f32 && full4) {                                    // the row pitch is a multiple of 4 as well
+          float *y = p.out_f32 + (size_t)t * p.ldo + col;
+          if (p.mode == MODE_RESIDUAL) { const float4 y4 = *reinterpret_cast<const float4 *>(y); v4.x += y4.x; v4.y += y4.y; v4.z += y4.z; v4.w += y4.w; }
+          *reinterpret_cast<float4 *>(y) = v4;
+        }
+      };
 
-    // SiLU(gate) * up: a tile holds 64 output features, gate in tile rows 0..63 and up in rows 64..127
-    auto finish_swiglu = [&](int tile, int gi, int G, int grp, int my, int n, int first, const float *stg, int t_base,
-                             int t_lim) -> bool {
-      const int F = p.a_rows[0];
-      const int ng = gi & 15, tg = gi >> 4, TG = G >> 4;             // 4 features; tokens my + n (tg + TG j)
-      const int feat = tile * 64 + 4 * ng;
-      const int js = n * TG;
-      if (!stg && !others_there(tile, n, gi, grp, G)) return false;
-      for (int tb = t_base + my + n * tg; tb < t_lim; tb += 4 * js) {
-        float4 g[4], u[4];
-        if (stg) {
+      if constexpr (!SPLIT) {
+#pragma unroll 1
+        for (int t = t_base + tg; t < t_lim; t += TG)                // tokens are uniform inside a warp
+          finish_token(t, *reinterpret_cast<const float4 *>(stg + (size_t)(t - t_base) * STAGE_PITCH + 4 * ng));
+        return true;
+      } else {
+        // Sixteen pieces are under way together: one token of sixteen contributors where a warp has a single token or there
+        // are many contributors (1.1B draft at one row: 4323 -> 4198 us), else four tokens of four (7B prefill: 18.9 -> 18.0
+        // ms).  They are fetched without asking first whether they are there: a probe in front is one more round trip to L2
+        // between two GEMMs.  What the epilogue reads besides comes after them, which keeps the code short: with everything
+        // requested up front and the tokens unrolled the routine is twice as long and 3 % slower, all of it waiting for
+        // instructions that a GEMM executes once.
+        const int tbn = n <= 4 || (n <= 8 && t_lim > js) ? 4 : 1;
+        float *slot = stg + (size_t)(warp - 2) * 4 * TILE_N + 4 * lane;       // this thread's 16 bytes of four parked tokens
+        auto gather = [&](auto tb_c, int tb) -> bool {
+          constexpr int TB = decltype(tb_c)::value, CB = 16 / TB;
+          float4 acc[TB];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int t = tb + j * js;
-            g[j] = u[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (t < t_lim) {
-              g[j] = *reinterpret_cast<const float4 *>(stg + (size_t)(t - t_base) * STAGE_PITCH + 4 * ng);
-              u[j] = *reinterpret_cast<const float4 *>(stg + (size_t)(t - t_base) * STAGE_PITCH + 64 + 4 * ng);
+          for (int j = 0; j < TB; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int c0 = 0; c0 < n; c0 += CB) {
+            uint4 tmp[CB][TB];
+            bool there = false;
+            for (uint32_t spin = 0; spin < p.wait_limit; ++spin) {
+              there = true;
+#pragma unroll
+              for (int cc = 0; cc < CB; ++cc) {
+                const int owner = first + c0 + cc;
+                const float *src = p.scratch + ((size_t)owner * 2 + w.owner_slot(tile, owner)) * SLOT_FLOATS + (size_t)tb * TILE_N + 4 * ng;
+#pragma unroll
+                for (int j = 0; j < TB; ++j)
+                  tmp[cc][j] = part_load(src + (size_t)(j * js) * TILE_N, c0 + cc < n && tb + j * js < t_lim);
+              }
+#pragma unroll
+              for (int cc = 0; cc < CB; ++cc)
+#pragma unroll
+                for (int j = 0; j < TB; ++j) there = there && part_there(tmp[cc][j]);
+              there = __all_sync(0xffffffffu, there);
+              if (there) break;
+              if ((spin & 15) == 15 && __any_sync(0xffffffffu, *abort_flag || *(volatile const int *)p.status != 0)) break;   // some CTA has given up
             }
-          }
-        } else {
+            if (!there) return false;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) g[j] = u[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-          for (int c0 = 0; c0 < n; c0 += 4) {
-            float4 tg4[4][4], tu4[4][4];
-#pragma unroll
-            for (int cc = 0; cc < 4; ++cc) {
+            for (int cc = 0; cc < CB; ++cc) {
               const int owner = first + c0 + cc;
-              const float *src = p.scratch + ((size_t)owner * 2 + w.owner_slot(tile, owner)) * SLOT_FLOATS + 4 * ng;
+              float *src = p.scratch + ((size_t)owner * 2 + w.owner_slot(tile, owner)) * SLOT_FLOATS + (size_t)tb * TILE_N + 4 * ng;
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const int t = tb + j * js;
-                const bool in = c0 + cc < n && t < t_lim;
-                tg4[cc][j] = in ? __ldcg((const float4 *)(src + (size_t)t * TILE_N)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                tu4[cc][j] = in ? __ldcg((const float4 *)(src + (size_t)t * TILE_N + 64)) : make_float4(0.f, 0.f, 0.f, 0.f);
+              for (int j = 0; j < TB; ++j) {
+                if (c0 + cc < n && tb + j * js < t_lim) part_empty(src + (size_t)(j * js) * TILE_N);
+                acc[j].x += __uint_as_float(tmp[cc][j].x); acc[j].y += __uint_as_float(tmp[cc][j].y);
+                acc[j].z += __uint_as_float(tmp[cc][j].z); acc[j].w += __uint_as_float(tmp[cc][j].w);
               }
             }
+          }
+          if (res_norm) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll
-            for (int cc = 0; cc < 4; ++cc)
+            for (int j = 0; j < TB; ++j) {
+              const float4 x = *reinterpret_cast<const float4 *>(slot + j * TILE_N);
+              acc[j].x += x.x; acc[j].y += x.y; acc[j].z += x.z; acc[j].w += x.w;
+            }
+          }
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                g[j].x += tg4[cc][j].x; g[j].y += tg4[cc][j].y; g[j].z += tg4[cc][j].z; g[j].w += tg4[cc][j].w;
-                u[j].x += tu4[cc][j].x; u[j].y += tu4[cc][j].y; u[j].z += tu4[cc][j].z; u[j].w += tu4[cc][j].w;
-              }
+          for (int j = 0; j < TB; ++j) *reinterpret_cast<float4 *>(slot + j * TILE_N) = acc[j];
+          return true;
+        };
+        for (int tb = my + n * tg; tb < t_lim; tb += tbn * js) {
+          if (res_norm && full4) {
+            for (int j = 0; j < tbn && tb + j * js < t_lim; ++j)
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(slot + j * TILE_N)),
+                           "l"(p.out_f32 + (size_t)(tb + j * js) * p.ldo + col) : "memory");
+          }
+          if (!(tbn == 4 ? gather(std::integral_constant<int, 4>{}, tb)
+                         : gather(std::integral_constant<int, 1>{}, tb)))
+            return false;
+          if (gi == 0) TRACE(12);
+#pragma unroll 1
+          for (int j = 0; j < tbn; ++j) {
+            const int t = tb + j * js;
+            if (t < t_lim) finish_token(t, *reinterpret_cast<const float4 *>(slot + j * TILE_N));
           }
         }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int t = tb + j * js;
-          if (t < t_lim && feat < F) {
-            const float r = rs[t];
-            g[j].x *= r; g[j].y *= r; g[j].z *= r; g[j].w *= r;
-            u[j].x *= r; u[j].y *= r; u[j].z *= r; u[j].w *= r;
-            __nv_bfloat162 lo = __floats2bfloat162_rn(silu(g[j].x) * u[j].x, silu(g[j].y) * u[j].y);
-            __nv_bfloat162 hi = __floats2bfloat162_rn(silu(g[j].z) * u[j].z, silu(g[j].w) * u[j].w);
-            *(uint2 *)(p.out_bf16 + (size_t)t * F + feat) = make_uint2(*(uint32_t *)&lo, *(uint32_t *)&hi);
-          }
-        }
+        return true;
       }
-      return true;
     };
 
     // Partial tiles.  Called once this CTA has published all its own partials, so waiting for the others cannot
     // form a cycle.  The (at most two) tiles are finished side by side, each by one half of the epilogue threads.
     auto run_fixups = [&]() {
-      const int grp = et >> 6, gi = et & 63;
-      bool mine = true;
+      const int grp = et / (EPI_THREADS / 2), gi = et % (EPI_THREADS / 2);
       if (grp < n_pend) {
-        const int tile = pend_tile[grp], n = pend_n[grp], first = pend_first[grp], my = (int)blockIdx.x - first;
-        mine = p.mode == MODE_SWIGLU ? finish_swiglu(tile, gi, 64, grp, my, n, first, nullptr, 0, rows)
-                                     : finish_plain(tile, gi, 64, grp, my, n, first, nullptr, 0, rows);
+        const int first = pend_first[grp];
+        if (!finish(std::true_type{}, pend_tile[grp], gi, EPI_THREADS / 2, (int)blockIdx.x - first, pend_n[grp], first, stage, 0, rows))
+          wait_flag[2] = 1;
         if (gi == 0 && grp == 0) TRACE(10);
-        if (mine) {
-          if (publish) __threadfence();                                // this thread's outputs, before the tile counts as finished
-          group_barrier(grp);
-          // every contributor counts towards the hand-over itself: the GEMM is finished once all shares of all tiles
-          // are (the host passes the total), and nobody has to learn that it was the last of its tile
-          if (gi == 0 && publish) atomicAdd(cp.finished + ci, 1);
-        }
+        if (publish) __threadfence();                                // this thread's outputs, before the tile counts as finished
+        group_barrier(grp);
+        // every contributor counts towards the hand-over itself: the GEMM is finished once all shares of all tiles
+        // are (the host passes the total), and nobody has to learn that it was the last of its tile
+        if (gi == 0 && publish && !wait_flag[2]) atomicAdd(cp.finished + ci, 1);
       }
       if (gi == 0 && grp == 0) TRACE(11);
-      if (!mine) wait_flag[2] = 1;
       epi_barrier();
       if (wait_flag[2]) ok = false;
       n_pend = 0;
@@ -777,13 +755,15 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
     if (et == 0) wait_flag[2] = 0;
     epi_barrier();
 
-    while (w.next(s)) {
-      int a = item & 1;
+    for (;;) {
+      const bool more = w.next(s);
+      const int a = item & 1;
       // the stream-K spans come first: once the whole tiles start, this CTA has published all its partials and
-      // can add up its shares while the tensor cores work on the whole tile
-      if (s.n_contrib == 1 && n_pend > 0) run_fixups();
-      if (!ok) break;
-      // one thread waits (bounded) and tells the others, so that all 128 leave the loop together
+      // can add up its shares while the tensor cores work on the whole tile  (one call site: the routine is inlined)
+      if (!more && et == 0) TRACE(5);
+      if (n_pend > 0 && (!more || s.n_contrib == 1)) run_fixups();
+      if (!ok || !more) break;
+      // one thread waits (bounded) and tells the others, so that all leave the loop together
       if (et == 0) wait_flag[a] = mbar_wait(&acc_full[a], (item >> 1) & 1, abort_flag) && !*abort_flag;
       epi_barrier();
       ok = wait_flag[a] != 0;
@@ -796,7 +776,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
         // from there; the TMEM buffer is handed back as soon as it has been read
         for (int c0 = 0; c0 < p.t_pad; c0 += STAGE_TOK) {
           const int c1 = min(p.t_pad, c0 + STAGE_TOK);
-          for (int t0 = c0; t0 < c1; t0 += 16) {
+          for (int t0 = c0 + 16 * wh; t0 < c1; t0 += 32) {           // the quarter's two warps take 16 tokens in turn
             tmem_ld16(taddr + t0, v);
 #pragma unroll
             for (int i = 0; i < 16; ++i) stage[(t0 - c0 + i) * STAGE_PITCH + nl] = v[i];
@@ -807,64 +787,23 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
             if (lane == 0) mbar_arrive(&acc_empty[a]);
           }
           epi_barrier();
-          const int lim = min(c1, rows);
-          if (p.mode == MODE_SWIGLU) {
-            finish_swiglu(s.tile, et, 128, 0, 0, 1, 0, stage, c0, lim);
-          } else if (p.mode == MODE_HEAD) {
-            // greedy choice inside the tile: two threads per token scan 64 parked logits each in ascending index
-            // order (a strict comparison keeps the smallest index among equals), then the halves are compared
-            int seg, row0, col0, valid;
-            locate(p, s.tile, seg, row0, col0, valid);
-            const int t = c0 + (et >> 1), h = et & 1;
-            uint32_t bu = 0;
-            int bi = col0 + 64 * h;
-            if (t < lim) {
-              const float r = rs[t];
-              const float *row = stage + (size_t)(t - c0) * STAGE_PITCH + 64 * h;
-#pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                const float4 x4 = *reinterpret_cast<const float4 *>(row + 4 * i);
-                const float xs[4] = {x4.x * r, x4.y * r, x4.z * r, x4.w * r};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  const int cidx = 64 * h + 4 * i + e;
-                  const uint32_t uo = ordered_u32(xs[e]);
-                  if (cidx < valid && uo > bu) { bu = uo; bi = col0 + cidx; }
-                }
-              }
-            }
-            const uint32_t ou = __shfl_xor_sync(0xffffffffu, bu, 1);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, 1);
-            if (ou > bu || (ou == bu && oi < bi)) { bu = ou; bi = oi; }
-            if (t < lim && h == 0) {
-              p.tile_max[(size_t)s.tile * OURO_MAX_ROWS + t] = ordered_f32(bu);
-              p.tile_arg[(size_t)s.tile * OURO_MAX_ROWS + t] = bi;
-            }
-          }
-          // one call site for every other mode (the routine is inlined: a second site would be a second copy of it)
-          if (p.mode != MODE_SWIGLU && (p.mode != MODE_HEAD || p.out_f32)) finish_plain(s.tile, et, 128, 0, 0, 1, 0, stage, c0, lim);
+          finish(std::false_type{}, s.tile, et, EPI_THREADS, 0, 1, 0, stage, c0, min(c1, rows));
           if (publish && c1 == p.t_pad) __threadfence();
           epi_barrier();
           if (publish && c1 == p.t_pad && et == 0) atomicAdd(cp.finished + ci, 1);
         }
       } else {
-        // partial tile: park it in this CTA's slot and announce it; the partials are added up after the loop
+        // partial tile: parked in this CTA's slot, for its contributors to fetch; added up after the loop
         float *mine = p.scratch + ((size_t)blockIdx.x * 2 + s.slot) * SLOT_FLOATS;
-        for (int t0 = 0; t0 < p.t_pad; t0 += 16) {
+        for (int t0 = 16 * wh; t0 < rows; t0 += 32) {
           tmem_ld16(taddr + t0, v);
 #pragma unroll
           for (int i = 0; i < 16; ++i)
-            if (t0 + i < rows) __stcg(mine + (size_t)(t0 + i) * TILE_N + nl, v[i]);
+            if (t0 + i < rows) part_store(mine + (size_t)(t0 + i) * TILE_N + nl, v[i]);
         }
         fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[a]);
-        __threadfence();
-        epi_barrier();
-        if (et == 0) {                             // first of this generation to get here: replaces what an earlier GEMM left
-          atomicMax(p.counters + s.tile, p.gen << 8);
-          atomicAdd(p.counters + s.tile, 1);
-        }
         pend_tile[n_pend] = s.tile;
         pend_n[n_pend] = s.n_contrib;
         pend_first[n_pend] = s.first_owner;
@@ -872,8 +811,6 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       }
       ++item;
     }
-    if (et == 0) TRACE(5);
-    if (ok) run_fixups();
     if (et == 0) TRACE(7);
     }
     if (!ok && et == 0) { *abort_flag = 1; atomicExch(p0.status, 1); }
@@ -881,7 +818,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
   // ------------------------------------------------------------------ teardown
   fence_before_sync();
   __syncthreads();
-  if (*abort_flag && ((warp == 0 && lane < W_PRODUCERS) || (warp == 6 && lane == 0))) {
+  if (*abort_flag && ((warp == 0 && lane < W_PRODUCERS) || (warp == ACT_WARP && lane == 0))) {
     // Somebody gave up: copies this lane issued may still be landing in this CTA's shared memory.  Wait (bounded) for
     // the last one of every stage before the CTA leaves; a stage whose other half was never requested cannot
     // complete its phase, which the limit covers (the bytes themselves arrive within microseconds).
@@ -934,7 +871,6 @@ struct FastState {
   int grid = 0;
   int smem_max = 0;
   float *slots = nullptr;
-  int *counters = nullptr;
   float *attn_part = nullptr;   // per-chunk softmax pieces of the split attention
   float *tile_max = nullptr;    // LM head: per-tile best logit and index of every token
   int *tile_arg = nullptr;
@@ -945,12 +881,11 @@ struct FastState {
   int chain_kind[MAX_CHAIN] = {0, 0, 0, 0};
   bool fuse = true;             // run consecutive GEMMs as one launch
   long pf_ffn_rows = 0;         // rows of gate and of up the attention kernel prefetches into L2 besides the output projection (< 0: nothing)
-  int gen_next = 1;             // generation number of the next GEMM (tile counters carry it, see GemmParams::counters)
   bool dirty = false;           // a bounded wait gave up: counters must be cleared before the next launch
   uint32_t wait_limit = 1u << 22;   // polls of a partial-tile wait (ouro_debug_set_wait_limit)
 };
 constexpr int MAX_TILES = 4096;
-constexpr int SPARE_BYTES = 2048;          // behind the tile counters: chain counters [0, 64), attention arrival counters [64, 512)
+constexpr int CHAIN_BYTES = 256;           // the chain counters
 
 size_t slots_bytes() { return (size_t)MAX_GRID * 2 * SLOT_FLOATS * sizeof(float); }
 size_t tile_best_bytes() { return (size_t)MAX_TILES * OURO_MAX_ROWS * 4; }
@@ -959,7 +894,7 @@ size_t ss_bytes() { return (size_t)MAX_SS_TILES * OURO_MAX_ROWS * sizeof(float);
 
 int stages_for(int t_pad, int smem_max) {
   int stage = A_BYTES + t_pad * BLOCK_K * 2;
-  int fixed = 1024 + STAGE_BYTES + 1536;  // alignment slack, parked whole tile, barriers, flags, per-token factors and positions
+  int fixed = 1024 + STAGE_BYTES + MISC_BYTES;  // alignment slack, parked whole tile, the rest
   int s = (smem_max - fixed) / stage;
   return s > 12 ? 12 : s;
 }
@@ -971,7 +906,7 @@ struct ouro_fast { FastState s; };
 size_t ouro_scratch_bytes(const ouro_model_desc *t, const ouro_model_desc *d) {
   size_t attn = attention_tc_scratch_bytes(*t);
   if (d && attention_tc_scratch_bytes(*d) > attn) attn = attention_tc_scratch_bytes(*d);
-  return slots_bytes() + 2 * MAX_TILES * sizeof(int) + SPARE_BYTES + 2 * tile_best_bytes() + ss_bytes() + attn;
+  return slots_bytes() + CHAIN_BYTES + 2 * tile_best_bytes() + ss_bytes() + attn;
 }
 
 static bool shape_ok(const ouro_model_desc &d) {
@@ -1004,21 +939,19 @@ int ouro_fast_setup(ouro_ctx *c) {
   f->s.grid = sms < MAX_GRID ? sms : MAX_GRID;
   f->s.smem_max = smem;
   f->s.slots = c->a.scratch;
-  f->s.counters = (int *)((char *)c->a.scratch + slots_bytes());
-  f->s.finished = f->s.counters + 2 * MAX_TILES;               // inside the spare words behind the tile counters
+  f->s.finished = (int *)((char *)c->a.scratch + slots_bytes());
   {
     const char *e = getenv("OURO_FUSE");                       // OURO_FUSE=0: every GEMM is a launch of its own
     f->s.fuse = !(e && e[0] == '0');
     const char *pf = getenv("OURO_PF_ROWS");
     if (pf) f->s.pf_ffn_rows = atol(pf);
-    const char *g0 = getenv("OURO_GEN_START");                  // test aid: first generation number of the tile counters
-    if (g0 && atoi(g0) > 0 && atoi(g0) < (1 << 22)) f->s.gen_next = atoi(g0);
   }
-  f->s.tile_max = (float *)((char *)c->a.scratch + slots_bytes() + 2 * MAX_TILES * sizeof(int) + SPARE_BYTES);
+  f->s.tile_max = (float *)((char *)c->a.scratch + slots_bytes() + CHAIN_BYTES);
   f->s.tile_arg = (int *)((char *)f->s.tile_max + tile_best_bytes());
   f->s.ss = (float *)((char *)f->s.tile_arg + tile_best_bytes());
   f->s.attn_part = (float *)((char *)f->s.ss + ss_bytes());
-  if (cudaMemsetAsync(f->s.counters, 0, 2 * MAX_TILES * sizeof(int) + SPARE_BYTES, c->stream) != cudaSuccess ||
+  if (cudaMemsetAsync(f->s.slots, 0xff, slots_bytes(), c->stream) != cudaSuccess ||
+      cudaMemsetAsync(f->s.finished, 0, CHAIN_BYTES, c->stream) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       attention_tc_setup() != OURO_OK || attention_tm_setup() != OURO_OK) {
     delete f;
@@ -1111,8 +1044,9 @@ static WeightSide weight_side(const ouro_model_desc &d, const FastModel &fm, int
   }
   return w;
 }
-static void set_weights(GemmParams &p, const WeightSide &w) {
-  for (int i = 0; i < 3; ++i) { p.a[i] = w.a[i]; p.a_tiles[i] = w.a_tiles[i]; p.a_rows[i] = w.a_rows[i]; }
+struct Gemm : GemmParams { GemmMaps m; };
+static void set_weights(Gemm &p, const WeightSide &w) {
+  for (int i = 0; i < 3; ++i) { p.m.a[i] = w.a[i]; p.a_tiles[i] = w.a_tiles[i]; p.a_rows[i] = w.a_rows[i]; }
   p.a_count = w.a_count;
   p.tiles = w.tiles;
 }
@@ -1122,35 +1056,32 @@ static int grid_for(const FastState &s, int tiles, int kb) {
 }
 // What the hand-over counter of a GEMM reaches: one count per whole tile and one per contributor of a split tile
 // (the schedule of weight_stream.cuh, worked out on the host).
-static int finish_units(int tiles, int kb, int grid) {
-  const int t0 = (tiles / grid) * grid, rem = tiles - t0;
-  if (rem == 0) return tiles;
-  const int total = rem * kb, per = (total + grid - 1) / grid;
-  int units = t0;
-  for (int rel = 0; rel < rem; ++rel) units += (rel * kb + kb - 1) / per - (rel * kb) / per + 1;
+static int finish_units(const GemmParams &g) {
+  int units = g.t0;
+  for (int rel = 0; rel < g.tiles - g.t0; ++rel) units += (rel * g.kb + g.kb - 1) / g.per - (rel * g.kb) / g.per + 1;
   return units;
 }
 // Launches the GEMMs collected so far as one chain.
 static void flush_chain(ouro_ctx *c) {
   FastState &s = c->fast->s;
-  ChainParams &cp = s.chain;
+  ChainArgs &cp = s.chain.args;
   if (cp.n == 0) return;
   OURO_COUNT_LAUNCH();
   int grid = 1;
   for (int i = 0; i < cp.n; ++i) grid = std::max(grid, grid_for(s, cp.g[i].tiles, cp.g[i].kb));
   cp.finished = s.finished;
-  if (s.gen_next + MAX_CHAIN >= (1 << 22)) {                 // generation numbers used up: start over on cleared words
-    cudaMemsetAsync(s.counters, 0, MAX_TILES * sizeof(int), c->stream);
-    s.gen_next = 1;
+  for (int i = 0; i < cp.n; ++i) {
+    const ws::Cut cut = ws::cut(cp.g[i].tiles, cp.g[i].kb, grid, grid);
+    cp.g[i].t0 = cut.t0;
+    cp.g[i].per = cut.per;
   }
-  for (int i = 0; i < cp.n; ++i) cp.g[i].gen = s.gen_next++;
-  for (int i = 0; i + 1 < cp.n; ++i) cp.target[i] = (s.finished_host[i] += finish_units(cp.g[i].tiles, cp.g[i].kb, grid));
+  for (int i = 0; i + 1 < cp.n; ++i) cp.target[i] = (s.finished_host[i] += finish_units(cp.g[i]));
   if (cp.fold.part || cp.embed.table) cp.fold_target = (s.finished_host[MAX_CHAIN] += grid);
   const bool per_kind = cp.n == 1 && c->prof_class >= OURO_PROF_QKV && c->prof_class <= OURO_PROF_HEAD;
   static const int kind_class[5] = {OURO_PROF_QKV, OURO_PROF_WO, OURO_PROF_GATEUP, OURO_PROF_DOWN, OURO_PROF_HEAD};
   {
     ProfScope ps(c, per_kind ? kind_class[s.chain_kind[0]] : OURO_PROF_GEMM);
-    launch_pdl(gemm_tc_kernel, grid, THREADS, (size_t)s.smem_max, c->stream, cp);
+    launch_pdl(gemm_tc_kernel, grid, THREADS, (size_t)s.smem_max, c->stream, s.chain);
   }
   cp.n = 0;
   cp.fold.part = nullptr;
@@ -1158,39 +1089,39 @@ static void flush_chain(ouro_ctx *c) {
 }
 
 // Adds a GEMM to the chain under construction; `last` launches the chain (something other than a GEMM follows).
-static void push_gemm(ouro_ctx *c, GemmParams &p, int kind, const CUtensorMap *xmaps, int K, int rows, bool last) {
+static void push_gemm(ouro_ctx *c, Gemm &p, int kind, const CUtensorMap *xmaps, int K, int rows, bool last) {
   FastState &s = c->fast->s;
   p.kb = K / BLOCK_K;
-  p.splitters = -1;
   p.rows = rows;
   p.t_pad = (rows + 15) & ~15;
-  p.b = xmaps[p.t_pad / 16 - 1];
+  p.m.b = xmaps[p.t_pad / 16 - 1];
   p.stages = stages_for(p.t_pad, s.smem_max);
   p.scratch = s.slots;
-  p.counters = s.counters;
   p.status = &c->st->status;
   p.rows_dev = c->cur_rows_dev;
   p.trace_id = kind;
   p.wait_limit = s.wait_limit;
-  if (s.chain.n > 0 && s.chain.g[0].rows != rows) flush_chain(c);   // cannot happen inside one forward
-  s.chain_kind[s.chain.n] = kind;
-  s.chain.g[s.chain.n++] = p;
+  ChainArgs &cp = s.chain.args;
+  if (cp.n > 0 && cp.g[0].rows != rows) flush_chain(c);             // cannot happen inside one forward
+  s.chain_kind[cp.n] = kind;
+  s.chain.maps[cp.n] = p.m;
+  cp.g[cp.n++] = p;
   // one launch per GEMM when asked for, and while a single kind of GEMM is being timed
   const bool split = !s.fuse || (c->prof_class >= OURO_PROF_QKV && c->prof_class <= OURO_PROF_HEAD);
-  if (last || split || s.chain.n == MAX_CHAIN) flush_chain(c);
+  if (last || split || cp.n == MAX_CHAIN) flush_chain(c);
 }
 
-// Clears what an aborted launch may have left behind (tile counters, chain counters).
+// Clears what an aborted launch may have left behind (partial tiles nobody fetched, chain counters).
 void ouro_fast_reset(ouro_ctx *c, bool force) {
   if (!c->fast) return;
   FastState &s = c->fast->s;
-  s.chain.n = 0;
-  s.chain.fold.part = nullptr;
-  s.chain.embed.table = nullptr;
+  s.chain.args.n = 0;
+  s.chain.args.fold.part = nullptr;
+  s.chain.args.embed.table = nullptr;
   if (!force && !s.dirty) return;
-  cudaMemsetAsync(s.counters, 0, 2 * MAX_TILES * sizeof(int) + SPARE_BYTES, c->stream);
+  cudaMemsetAsync(s.slots, 0xff, slots_bytes(), c->stream);
+  cudaMemsetAsync(s.finished, 0, CHAIN_BYTES, c->stream);
   for (int &v : s.finished_host) v = 0;
-  s.gen_next = 1;
   s.dirty = false;
 }
 void ouro_fast_mark_dirty(ouro_ctx *c) {
@@ -1215,10 +1146,10 @@ bool ouro_fast_available(ouro_ctx *c, int which) {
 int ouro_fast_embed(ouro_ctx *c, int which, int rows) {
   if (!c->fast || !c->fast->s.m[which].ok) return OURO_ESTATE;
   ModelRt &M = c->m[which];
-  ChainParams &cp = c->fast->s.chain;
+  ChainArgs &cp = c->fast->s.chain.args;
   cp.n = 0;
   cp.fold.part = nullptr;
-  ChainParams::Embed &e = cp.embed;
+  ChainArgs::Embed &e = cp.embed;
   e.table = (const __nv_bfloat16 *)M.embed;
   e.tok = M.blk.tok;
   e.gain = (const __nv_bfloat16 *)M.attn_norm[0];
@@ -1247,7 +1178,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows) {
   auto consume = [&](GemmParams &p) { p.ss_in = ss; p.ss_tiles = ss_tiles; p.ss_inv_d = 1.0f / (float)d.d_model; p.eps = d.rms_eps; };
   auto produce = [&](GemmParams &p, const void *gain) { p.gain = (const __nv_bfloat16 *)gain; p.xb = (__nv_bfloat16 *)a.xn; p.ss_out = ss; };
   {
-    GemmParams p{};
+    Gemm p{};
     set_weights(p, weight_side(d, fm, l, G_QKV));
     consume(p);
     const bool fused_rope = d.head_dim == 64 || d.head_dim == 128;   // tiles then hold whole heads
@@ -1291,7 +1222,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows) {
     else
       launch_attention_simple(d, a.q, M.k_cache, M.v_cache, M.blk, rows, l, a.att, s);
     if (pieces) {                    // folded by the output projection's launch, all its CTAs taking part
-      fold::Params &f = c->fast->s.chain.fold;
+      fold::Params &f = c->fast->s.chain.args.fold;
       f.part = c->fast->s.attn_part;
       f.out = (__nv_bfloat16 *)a.att;
       f.lin_end = M.blk.lin_end;
@@ -1304,7 +1235,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows) {
     }
   }
   {
-    GemmParams p{};
+    Gemm p{};
     set_weights(p, weight_side(d, fm, l, G_WO));
     p.mode = MODE_RESIDUAL;
     p.out_f32 = a.x;
@@ -1313,7 +1244,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows) {
     push_gemm(c, p, G_WO, fm.x_q, dq, rows, false);
   }
   {
-    GemmParams p{};
+    Gemm p{};
     set_weights(p, weight_side(d, fm, l, G_GATEUP));
     p.mode = MODE_SWIGLU;
     p.out_bf16 = (__nv_bfloat16 *)a.act;
@@ -1321,7 +1252,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows) {
     push_gemm(c, p, G_GATEUP, fm.x_d, d.d_model, rows, false);
   }
   {
-    GemmParams p{};
+    Gemm p{};
     set_weights(p, weight_side(d, fm, l, G_DOWN));
     p.mode = MODE_RESIDUAL;
     p.out_f32 = a.x;
@@ -1375,7 +1306,7 @@ int ouro_fast_head(ouro_ctx *c, int which, int rows, float *logits, int32_t *arg
   FastModel &fm = c->fast->s.m[which];
   const ouro_model_desc &d = M.d;
   {
-    GemmParams p{};
+    Gemm p{};
     set_weights(p, weight_side(d, fm, 0, G_HEAD));
     p.mode = MODE_HEAD;
     p.out_f32 = logits;
@@ -1416,8 +1347,7 @@ namespace {
 constexpr int NA_SPLITTERS = 32;                   // CTAs that may leave partial tiles (two slots each)
 constexpr int NA_MAX_TILES = 512;                  // vocabulary <= 65536
 constexpr size_t NA_SLOT_BYTES = (size_t)NA_SPLITTERS * 2 * SLOT_FLOATS * sizeof(float);
-constexpr size_t NA_OFF_COUNTERS = NA_SLOT_BYTES;
-constexpr size_t NA_OFF_STATUS = NA_OFF_COUNTERS + 2 * NA_MAX_TILES * sizeof(int);   // published + finished counters
+constexpr size_t NA_OFF_STATUS = NA_SLOT_BYTES;
 constexpr size_t NA_OFF_TMAX = NA_OFF_STATUS + 256;
 constexpr size_t NA_OFF_TARG = NA_OFF_TMAX + (size_t)NA_MAX_TILES * OURO_MAX_ROWS * sizeof(float);
 constexpr size_t NA_BYTES = NA_OFF_TARG + (size_t)NA_MAX_TILES * OURO_MAX_ROWS * sizeof(int);
@@ -1431,6 +1361,7 @@ namespace {
 unsigned char *g_na_ptr[NA_MAX_DEVICES] = {};      // device address of g_static_scratch, per device
 int g_na_smem[NA_MAX_DEVICES] = {};
 int g_na_sms[NA_MAX_DEVICES] = {};
+std::atomic<bool> g_na_ready[NA_MAX_DEVICES] = {};  // the slots are empty and the status word is zero
 
 // Once per device, with that device current: resolve the array's device address and size the kernel's
 // shared memory.  Returns OURO_OK or an error with a text for ouro_last_error(NULL).
@@ -1487,13 +1418,19 @@ extern "C" int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, i
   cudaStream_t s = (cudaStream_t)cuda_stream;
   unsigned char *base = g_na_ptr[dev];
   const int tiles = (vocab + TILE_N - 1) / TILE_N;
-  // the array keeps whatever the last call left: counters and status must start at zero
-  cudaError_t e = cudaMemsetAsync(base + NA_OFF_COUNTERS, 0, NA_OFF_TMAX - NA_OFF_COUNTERS, s);
-  ChainParams cp{};
+  // the slots are empty (see EMPTY): cleared by the first call on the device, and every call leaves them so
+  cudaError_t e = cudaSuccess;
+  if (!g_na_ready[dev].load(std::memory_order_acquire)) {
+    e = cudaMemsetAsync(base, 0xff, NA_SLOT_BYTES, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(base + NA_OFF_STATUS, 0, NA_OFF_TMAX - NA_OFF_STATUS, s);
+  }
+  ChainParams kp{};
+  ChainArgs &cp = kp.args;
   cp.n = 1;
   GemmParams &p = cp.g[0];
+  GemmMaps &m = kp.maps[0];
   const int t_pad = (rows + 15) & ~15;
-  if (e != cudaSuccess || !make_map(&p.a[0], lm_head_dev, vocab, d_model, TILE_N) || !make_map(&p.b, x_dev, rows, d_model, t_pad)) {
+  if (e != cudaSuccess || !make_map(&m.a[0], lm_head_dev, vocab, d_model, TILE_N) || !make_map(&m.b, x_dev, rows, d_model, t_pad)) {
     ouro_set_global_error("ouro_lm_head_static: could not describe the operands to the copy engine");
     return OURO_ECUDA;
   }
@@ -1510,23 +1447,17 @@ extern "C" int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, i
   p.tile_arg = (int *)(base + NA_OFF_TARG);
   p.wait_limit = 1u << 22;
   p.scratch = (float *)base;
-  p.counters = (int *)(base + NA_OFF_COUNTERS);
-  p.gen = 1;                                   // the words were cleared just above
   p.status = (int *)(base + NA_OFF_STATUS);
   // One CTA per SM streams whole tiles, which need no scratch.  The remainder (all tiles of a small vocabulary) is cut
   // along K over the CTAs that have slots while it has no more tiles than those: beyond that, as many CTAs stream when
   // each takes a tile whole.  Bound by the weight stream: 32000 x 4096 with 37 rows took 208 us on 32 CTAs (1.3 TB/s, what
   // 32 rings can ask for) and takes 95 us on all SMs.
   const int total = tiles * p.kb, sms = std::min(g_na_sms[dev], MAX_GRID), rest = tiles % sms;
-  int grid;
-  if (tiles <= NA_SPLITTERS) {
-    grid = std::min(total, NA_SPLITTERS);
-    p.splitters = -1;
-  } else {
-    grid = std::min(tiles, sms);
-    p.splitters = tiles > sms && rest <= NA_SPLITTERS ? NA_SPLITTERS : 0;
-  }
-  gemm_tc_kernel<<<grid, THREADS, g_na_smem[dev], s>>>(cp);
+  const int grid = tiles <= NA_SPLITTERS ? std::min(total, NA_SPLITTERS) : std::min(tiles, sms);
+  const ws::Cut cut = ws::cut(tiles, p.kb, grid, rest <= NA_SPLITTERS ? std::min(total, NA_SPLITTERS) : 0);
+  p.t0 = cut.t0;
+  p.per = cut.per;
+  gemm_tc_kernel<<<grid, THREADS, g_na_smem[dev], s>>>(kp);
   argmax_tiles_kernel<<<rows, 128, 0, s>>>(p.tile_max, p.tile_arg, tiles, argmax_dev);
   int status = 0;
   if ((e = cudaGetLastError()) != cudaSuccess ||
@@ -1535,6 +1466,7 @@ extern "C" int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, i
     ouro_set_global_error(std::string("ouro_lm_head_static: ") + cudaGetErrorString(e));
     return OURO_ECUDA;
   }
+  g_na_ready[dev].store(status == 0, std::memory_order_release);   // after a give-up the next call clears the array
   if (status != 0) {
     ouro_set_global_error("ouro_lm_head_static: a bounded device-side wait gave up");
     return OURO_ETIMEOUT;

@@ -17,17 +17,17 @@ struct Span {  // one piece of a CTA's work: k-blocks [kb0, kb1) of `tile`
 // Work of one CTA.  The last R = tiles mod grid tiles are cut stream-K fashion into equal contiguous spans of
 // the (tile, k-block) space and come first, so that their partial sums are added up while the whole tiles
 // (tile c, c + grid, ...) that follow are still streaming.  Depends on (tiles, kb, grid, splitters) only.
-// `splitters` is the number of CTAs that share the remainder: all of them where scratch memory holds two partial tiles
-// per CTA, fewer (or none: the remainder is then handled whole as well) where it does not.
+// The host works the cut out (GemmParams::t0, ::per): a walker is built by four warps of every CTA for every GEMM, and
+// each integer division by a run-time number there is 0.1 us in front of the first load.
 struct SpanWalker {
   int kb, per, t0, it, end, whole, grid, cta;
-  __device__ SpanWalker(int tiles, int kb_, int grid_, int splitters, int cta_) {
+  __device__ SpanWalker(int tiles, int kb_, int t0_, int per_, int grid_, int cta_) {
     kb = kb_;
     grid = grid_;
     cta = cta_;
-    t0 = splitters ? (tiles / grid) * grid : tiles;          // tiles [0, t0) are handled whole
-    int total = (tiles - t0) * kb;
-    per = splitters ? (total + splitters - 1) / splitters : 0;
+    t0 = t0_;                                                // tiles [0, t0) are handled whole
+    per = per_;                                              // k-blocks per CTA of the others' (0: there are none)
+    const int total = (tiles - t0) * kb;
     it = min(total, cta * per);
     end = min(total, it + per);
     whole = cta;
@@ -58,5 +58,18 @@ struct SpanWalker {
     return false;
   }
 };
+
+// The cut of `tiles` tiles of kb k-blocks for a launch of `grid` CTAs.  `splitters` CTAs share the remainder: all of them
+// where scratch memory holds two partial tiles per CTA, fewer (or none: the remainder is then handled whole as well)
+// where it does not.
+struct Cut { int t0, per; };
+inline Cut cut(int tiles, int kb, int grid, int splitters) {
+  Cut c{tiles, 0};
+  if (splitters > 0 && tiles % grid != 0) {
+    c.t0 = tiles / grid * grid;
+    c.per = ((tiles - c.t0) * kb + splitters - 1) / splitters;
+  }
+  return c;
+}
 
 }  // namespace ws
