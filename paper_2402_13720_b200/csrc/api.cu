@@ -85,7 +85,9 @@ static size_t carve(ouro_ctx *c, char *base, const ouro_model_desc *t, const our
   size_t F = mx([](const ouro_model_desc *m) { return (size_t)m->d_ffn; });
   size_t V = mx([](const ouro_model_desc *m) { return (size_t)m->vocab; });
   Activations a{};
-  a.x = cv.take<float>(R * dm);
+  // rows of a block: R, and OURO_TEXT_ROWS = 2 R where blocks of known text run on the tensor cores (16-bit activations then
+  // fill the same space)
+  a.x = cv.take<float>(OURO_TEXT_ROWS * dm);
   a.xn = cv.take<float>(R * dm);
   a.qkv = cv.take<float>(R * dqkv);
   a.q = cv.take<float>(R * dq);
@@ -96,7 +98,7 @@ static size_t carve(ouro_ctx *c, char *base, const ouro_model_desc *t, const our
   a.scratch_bytes = ouro_scratch_bytes(t, d);
   a.scratch = cv.take<float>(a.scratch_bytes / 4);
   DevState *st = cv.take<DevState>(1);
-  int32_t *seq_dev = cv.take<int32_t>((size_t)t->max_seq + OURO_MAX_ROWS);
+  int32_t *seq_dev = cv.take<int32_t>((size_t)t->max_seq + OURO_TEXT_ROWS);
   int S = p->beta - 1;
   int32_t *cand_suffix = cv.take<int32_t>((size_t)std::max(1, p->K * S));
   int32_t *cand_count = cv.take<int32_t>(1);
@@ -115,13 +117,13 @@ static size_t carve(ouro_ctx *c, char *base, const ouro_model_desc *t, const our
   float *rc[2]{}, *rs[2]{};
   for (int w = 0; w < 2; ++w) {
     if (!ds[w]) continue;
-    blk[w].tok = cv.take<int32_t>(R);
-    blk[w].pos = cv.take<int32_t>(R);
-    blk[w].group = cv.take<int32_t>(R);
-    blk[w].lin_end = cv.take<int32_t>(R);
-    blk[w].seg_start = cv.take<int32_t>(R);
-    blk[w].seg_len = cv.take<int32_t>(R);
-    blk[w].mask = cv.take<u64>(2 * R);
+    blk[w].tok = cv.take<int32_t>(OURO_TEXT_ROWS);
+    blk[w].pos = cv.take<int32_t>(OURO_TEXT_ROWS);
+    blk[w].group = cv.take<int32_t>(OURO_TEXT_ROWS);
+    blk[w].lin_end = cv.take<int32_t>(OURO_TEXT_ROWS);
+    blk[w].seg_start = cv.take<int32_t>(OURO_TEXT_ROWS);
+    blk[w].seg_len = cv.take<int32_t>(OURO_TEXT_ROWS);
+    blk[w].mask = cv.take<u64>(2 * OURO_TEXT_ROWS);
     size_t nt = (size_t)ds[w]->max_seq * (ds[w]->head_dim / 2);
     rc[w] = cv.take<float>(nt);
     rs[w] = cv.take<float>(nt);
@@ -312,11 +314,8 @@ extern "C" int ouro_set_drafter(ouro_ctx *c, ouro_drafter_fn fn, void *user) {
 }
 
 // ------------------------------------------------------------------------------------ blocks
-extern "C" int ouro_assemble_causal(ouro_ctx *c, int which, const int32_t *tokens_dev, int32_t n) {
-  if (!c || which < 0 || which > 1 || !tokens_dev) return OURO_EINVAL;
+static int assemble_causal(ouro_ctx *c, int which, const int32_t *tokens_dev, int32_t n) {
   ModelRt &M = c->m[which];
-  if (!M.present) return fail(c, OURO_ESTATE, "model not present");
-  if (n < 1 || n > OURO_MAX_ROWS) return fail(c, OURO_ECAPACITY, "block rows outside 1..OURO_MAX_ROWS");
   if (M.L + n > M.d.max_seq) return fail(c, OURO_ECAPACITY, "cache length + block rows exceeds max_seq");
   launch_assemble_causal(M.blk, tokens_dev, n, M.L, c->stream);
   CKL();
@@ -325,6 +324,13 @@ extern "C" int ouro_assemble_causal(ouro_ctx *c, int which, const int32_t *token
   M.blk_L = M.L;
   M.blk_is_candidate = false;
   return OURO_OK;
+}
+
+extern "C" int ouro_assemble_causal(ouro_ctx *c, int which, const int32_t *tokens_dev, int32_t n) {
+  if (!c || which < 0 || which > 1 || !tokens_dev) return OURO_EINVAL;
+  if (!c->m[which].present) return fail(c, OURO_ESTATE, "model not present");
+  if (n < 1 || n > OURO_MAX_ROWS) return fail(c, OURO_ECAPACITY, "block rows outside 1..OURO_MAX_ROWS");
+  return assemble_causal(c, which, tokens_dev, n);
 }
 
 // Waits for a kernel to post sequence number `seq` in a mailbox slot.  The wait is bounded: after two seconds
@@ -433,9 +439,11 @@ extern "C" int ouro_profile_read(ouro_ctx *c, float *ms_total, int32_t *launches
 
 // ----------------------------------------------------------------------------------- forward
 int ouro_fast_embed(ouro_ctx *c, int which, int rows);                     // embedding + first norm's inputs
-int ouro_fast_layer(ouro_ctx *c, int which, int layer, int rows);          // tensor-core layer; OURO_ESTATE = not available
+int ouro_fast_layer(ouro_ctx *c, int which, int layer, int rows, bool kv_only);   // tensor-core layer; OURO_ESTATE = not available
 int ouro_fast_head(ouro_ctx *c, int which, int rows, float *logits, int32_t *argmax_dev);   // tensor-core LM head + argmax
 
+// argmax_dev NULL: a block of known text, of which only the keys and values are wanted; the last layer then ends with
+// them and there is no LM head.
 static int forward(ouro_ctx *c, int which, int32_t *argmax_dev, float *logits_dev) {
   ModelRt &M = c->m[which];
   if (!M.present) return fail(c, OURO_ESTATE, "model not present");
@@ -452,7 +460,8 @@ static int forward(ouro_ctx *c, int which, int32_t *argmax_dev, float *logits_de
     launch_embed(dt, M.embed, M.blk.tok, rows, d.d_model, a.x, s);
   }
   for (int l = 0; l < d.n_layers; ++l) {
-    int rc = ouro_fast_layer(c, which, l, rows);
+    const bool kv_only = !argmax_dev && l + 1 == d.n_layers;
+    int rc = ouro_fast_layer(c, which, l, rows, kv_only);
     if (rc == OURO_OK) continue;
     if (rc != OURO_ESTATE) return rc;
     { ProfScope ps(c, OURO_PROF_NORM); launch_rmsnorm(dt, a.x, M.attn_norm[l], rows, d.d_model, d.rms_eps, a.xn, s); }
@@ -462,6 +471,7 @@ static int forward(ouro_ctx *c, int which, int32_t *argmax_dev, float *logits_de
       launch_gemm_simple(dt, a.xn, qkv, rows, d.d_model, a.qkv, dq + 2 * dkv, EPI_STORE, s);
     }
     { ProfScope ps(c, OURO_PROF_ROPE); launch_rope_append(d, a.qkv, M.blk.pos, M.rope_cos, M.rope_sin, rows, L, l, a.q, M.k_cache, M.v_cache, s); }
+    if (kv_only) break;
     { ProfScope ps(c, OURO_PROF_ATTENTION); launch_attention_simple(d, a.q, M.k_cache, M.v_cache, M.blk, rows, l, a.att, s); }
     {
       ProfScope ps(c, OURO_PROF_WO);
@@ -475,6 +485,10 @@ static int forward(ouro_ctx *c, int which, int32_t *argmax_dev, float *logits_de
       GemmSegs wd{{M.w_down[l], nullptr, nullptr}, {d.d_model, 0, 0}, 1};
       launch_gemm_simple(dt, a.act, wd, rows, d.d_ffn, a.x, d.d_model, EPI_RESIDUAL, s);
     }
+  }
+  if (!argmax_dev) {
+    CKL();
+    return OURO_OK;
   }
   int rc = ouro_fast_head(c, which, rows, logits_dev, argmax_dev);
   if (rc == OURO_ESTATE) {
@@ -508,17 +522,22 @@ extern "C" int ouro_advance(ouro_ctx *c, int which, int32_t n) {
   return OURO_OK;
 }
 
-// Runs model `which` over text positions [M.L, upto) taken from seq_dev, in chunks; the outputs of the last
-// chunk stay in a.argmax (row index of the last position returned through last_row).
+// Runs model `which` over text positions [M.L, upto) taken from seq_dev, in blocks.  With last_row the outputs of the
+// last block stay in a.argmax (row index of the last position returned through last_row); the others only leave their
+// keys and values, and are as wide as the kernels take: streaming the weights once for 256 rows costs a third more than
+// for 128.
 static int feed_text(ouro_ctx *c, int which, int upto, int *last_row) {
   ModelRt &M = c->m[which];
+  const int widest = ouro_fast_available(c, which) ? OURO_TEXT_ROWS : OURO_MAX_ROWS;
   while (M.L < upto) {
-    int n = std::min<int>(OURO_MAX_ROWS, upto - M.L);
-    TRY(ouro_assemble_causal(c, which, c->seq_dev + M.L, n));
-    TRY(forward(c, which, c->a.argmax, nullptr));
+    const int left = upto - M.L;
+    const bool outputs = last_row && left <= OURO_MAX_ROWS;
+    const int n = outputs ? left : std::min(widest, last_row ? left - 1 : left);
+    TRY(assemble_causal(c, which, c->seq_dev + M.L, n));
+    TRY(forward(c, which, outputs ? c->a.argmax : nullptr, nullptr));
     M.L += n;
     M.blk_rows = 0;
-    if (last_row) *last_row = n - 1;
+    if (outputs) *last_row = n - 1;
   }
   return OURO_OK;
 }

@@ -19,6 +19,8 @@
 // tile and the other rows masked out (an exact no-op for them).  The value computed for a query depends only on
 // (virtual position -> key) and on fixed chunk, span and warp boundaries, never on the other rows of the block:
 // a token gets bit-identical attention whether it is verified inside a candidate block or decoded alone.
+#include <algorithm>
+
 #include "ouro_internal.h"
 #include "attn_fold.cuh"
 
@@ -59,6 +61,7 @@ struct AttnParams {
   const __nv_bfloat16 *k, *v;      // this layer's cache: [max_seq][Hkv*HD]
   const int32_t *lin_end, *seg_start, *seg_len, *group;
   int rows, H, Hkv, L, cap;        // L: cache length before the block; cap: span slots per (row, head)
+  int rounds;                      // rounds of query rows per 128 block rows
   float scale_log2;
   float *part;                     // [rows][H][cap][PIECE]: max (log2 domain), sum, -, -, unnormalised output
   __nv_bfloat16 *out;              // [rows][H*HD]
@@ -150,13 +153,17 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sc = blockIdx.x, kvh = blockIdx.y;
   const int g = p.H / p.Hkv, dkv = p.Hkv * HD;
-  const int rows = p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows;   // written before the forward pass began
+  // a block of more than 128 rows (known text: one group, rows in order) is handled 128 rows at a time, the cache in front
+  // of a part being the cache in front of the block and the rows before the part
+  const int zb = (int)blockIdx.z / p.rounds * OURO_MAX_ROWS, L = p.L + zb;
+  const int rows = min(OURO_MAX_ROWS, (p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows) - zb);   // written before the forward pass began
+  const int32_t *group = p.group + zb, *lin_end = p.lin_end + zb, *seg_start = p.seg_start + zb, *seg_len = p.seg_len + zb;
   const int M_all = g * rows;
 
   int nv_max = 0;
   for (int r = threadIdx.x; r < rows; r += THREADS) {
-    s_nvis[r] = p.lin_end[r] + p.seg_len[r];
-    s_grp[r] = p.group[r];
+    s_nvis[r] = lin_end[r] + seg_len[r];
+    s_grp[r] = group[r];
   }
   __syncthreads();
   for (int r = 0; r < rows; ++r) nv_max = max(nv_max, s_nvis[r]);
@@ -169,7 +176,7 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
     for (int idx = threadIdx.x; idx < CH * CPR; idx += THREADS) {
       int row = idx / CPR, ch = idx % CPR, pos = c0 + row;
       uint32_t off = buf * S::KV + row * ROWB + ((ch ^ (row & 7)) << 4);
-      if (pos < p.L) {
+      if (pos < L) {
         size_t src = (size_t)pos * dkv + kvh * HD + ch * 8;
         cp_async16(sm_u + off, p.k + src);
         cp_async16(sm_u + S::OFF_V + off, p.v + src);
@@ -183,7 +190,7 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
 
   {
     // ---------------------------------------------------------------- this CTA's round of up to 64 query rows
-    const int m0 = blockIdx.z * QR;
+    const int m0 = (int)blockIdx.z % p.rounds * QR;
     // Query rows are ordered group by group (a group's rows for head 0, then for head 1, ..), so that the 64 rows
     // of a round belong to few groups and the chunk that holds block keys needs few passes.  Rows of this thread
     // in row tile mt: lane/4 and +8.
@@ -210,15 +217,16 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
     if (!__syncthreads_or(any_row)) return;            // nobody in this round reaches the span
     const int n_mt = (min(QR, M_all - m0) + 15) >> 4;  // row tiles that hold query rows; the others are skipped
 
-    stage_common(0, 0);                                 // chunk 0 (its rows below the cache length) is on its way ...
+    if (zb == 0) stage_common(0, 0);                    // chunk 0 (its rows below the cache length) is on its way ...
     TRACE(1);
     pdl_wait();                                         // ... while the previous kernel finishes
+    if (zb != 0) stage_common(0, 0);
     TRACE(2);
     for (int idx = threadIdx.x; idx < QR * CPR; idx += THREADS) {
       int row = idx / CPR, ch = idx % CPR, m = m0 + row;
       uint32_t off = S::OFF_Q + row * ROWB + ((ch ^ (row & 7)) << 4);
       if (m < M_all)
-        cp_async16(sm_u + off, p.q + (size_t)(s_map[row] & 0xffff) * p.H * HD + (kvh * g + (s_map[row] >> 16)) * HD + ch * 8);
+        cp_async16(sm_u + off, p.q + (size_t)(zb + (s_map[row] & 0xffff)) * p.H * HD + (kvh * g + (s_map[row] >> 16)) * HD + ch * 8);
       else
         *reinterpret_cast<uint4 *>(smem + off) = make_uint4(0, 0, 0, 0);
     }
@@ -237,7 +245,7 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
       if (ci + 1 < n_chunks) { stage_common(ci + 1, buf ^ 1); cp_wait_but_one(); } else { cp_wait_all(); }
       __syncthreads();
       if (ci == 0) TRACE(3);
-      const bool common = c0 + CH <= p.L;
+      const bool common = c0 + CH <= L;
       int g_begin = 0;
       while (g_begin < rows) {
         // -------------------------------------------------------------- one pass over the chunk
@@ -248,7 +256,7 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
           while (g_end < rows && s_grp[g_end] == gid) ++g_end;
           const int last = g_end - 1, nvg = s_nvis[last];
           int lin_g = INT_MAX, seg_g = 0;
-          if (p.seg_len[last] > 0) { lin_g = p.lin_end[last]; seg_g = p.seg_start[last]; }
+          if (seg_len[last] > 0) { lin_g = lin_end[last]; seg_g = seg_start[last]; }
           bool mine = false;
 #pragma unroll
           for (int i = 0; i < 2 * MT; ++i) mine = mine || (gr[i] == gid && nv[i] > c0);
@@ -256,7 +264,7 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
           // swap in the group's own keys: virtual positions [max(c0, L), min(c0 + CH, nvg))
           for (int idx = threadIdx.x; idx < CH * CPR; idx += THREADS) {
             int row = idx / CPR, ch = idx % CPR, pos = c0 + row;
-            if (pos >= p.L && pos < nvg) {
+            if (pos >= L && pos < nvg) {
               int slot = pos < lin_g ? pos : seg_g + (pos - lin_g);
               uint32_t off = buf * S::KV + row * ROWB + ((ch ^ (row & 7)) << 4);
               size_t src = (size_t)slot * dkv + kvh * HD + ch * 8;
@@ -408,12 +416,12 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
 #pragma unroll
         for (int nt = 0; nt < NT2; ++nt) {
           int d = warp * DW + 8 * nt + 2 * (lane & 3);
-          *reinterpret_cast<__nv_bfloat162 *>(p.out + ((size_t)rr[i] * p.H + hh[i]) * HD + d) =
+          *reinterpret_cast<__nv_bfloat162 *>(p.out + ((size_t)(zb + rr[i]) * p.H + hh[i]) * HD + d) =
               __floats2bfloat162_rn(o[i >> 1][nt][2 * (i & 1)] * inv, o[i >> 1][nt][2 * (i & 1) + 1] * inv);
         }
         continue;
       }
-      float *dst = p.part + (((size_t)rr[i] * p.H + hh[i]) * p.cap + sc) * PW;
+      float *dst = p.part + (((size_t)(zb + rr[i]) * p.H + hh[i]) * p.cap + sc) * PW;
       if (warp == 0 && (lane & 3) == 0) { dst[0] = m_run[i]; dst[1] = l_run[i]; }
 #pragma unroll
       for (int nt = 0; nt < NT2; ++nt) {
@@ -434,7 +442,7 @@ bool attention_tc_supported(const ouro_model_desc &d) {
 size_t attention_tc_scratch_bytes(const ouro_model_desc &d) {
   if (!attention_tc_supported(d)) return 0;
   size_t cap = (d.max_seq + SPAN - 1) / SPAN;
-  return (size_t)OURO_MAX_ROWS * d.n_heads * cap * (d.head_dim + 4) * sizeof(float);
+  return (size_t)OURO_TEXT_ROWS * d.n_heads * cap * (d.head_dim + 4) * sizeof(float);
 }
 
 template <int HD, int MT>
@@ -461,14 +469,16 @@ bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_
   p.scale_log2 = 1.4426950408889634f / sqrtf((float)d.head_dim);
   p.part = part;
   p.out = (__nv_bfloat16 *)out;
-  const int m_all = (d.n_heads / d.n_kv_heads) * rows;      // query rows per kv head (an upper bound when the count is on the device)
+  const int parts = (rows + OURO_MAX_ROWS - 1) / OURO_MAX_ROWS;
+  const int m_all = (d.n_heads / d.n_kv_heads) * std::min<int>(rows, OURO_MAX_ROWS);   // query rows per kv head (an upper bound when the count is on the device)
   // A round of 16 query rows takes 9-11 us (its chain of latencies over four chunks), one of 64 rows 14-27 us, and the
   // rounds of a short block run side by side: 16 rows each while all CTAs are resident at once.  (1.1B draft, 19 rows x 8
   // heads over 540 keys: 27.0 us on 24 CTAs of 64 rows, 11.3 us on 80 CTAs of 16.)  Beyond that, larger rounds read the
   // keys less often.
   const int n_spans = (n_vis_max + SPAN - 1) / SPAN;
-  const int mt = n_spans * d.n_kv_heads * ((m_all + 15) / 16) <= SHORT_ROUNDS ? 1 : 4, qr = 16 * mt;
-  dim3 grid(n_spans, d.n_kv_heads, (m_all + qr - 1) / qr);
+  const int mt = parts * n_spans * d.n_kv_heads * ((m_all + 15) / 16) <= SHORT_ROUNDS ? 1 : 4, qr = 16 * mt;
+  p.rounds = (m_all + qr - 1) / qr;
+  dim3 grid(n_spans, d.n_kv_heads, parts * p.rounds);
   p.direct = n_spans <= 1;                                  // a single span: nothing to fold
   if (d.head_dim == 128) {
     if (mt == 1) launch_pdl(attn_span_kernel<128, 1>, grid, THREADS, Smem<128, 1>::BYTES, s, p);

@@ -29,6 +29,8 @@
 // Every mbarrier wait is bounded; on expiry the CTA raises the context's status word, stops waiting and drains.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "ouro_internal.h"
 #include "attn_fold.cuh"
 
@@ -215,13 +217,17 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
   // blockIdx.x walks (span, kv head) with the last span of every head first: it holds the block's own keys and
   // takes one pass per group, so it should not be what the grid ends on
   const int sc = p.n_spans - 1 - blockIdx.x / p.Hkv, kvh = blockIdx.x % p.Hkv, m0 = blockIdx.y * QR;
-  const int rows = p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows;   // written before the forward pass began
+  // a block of more than 128 rows (known text: one group, rows in order) is handled 128 rows at a time, the cache in front
+  // of a part being the cache in front of the block and the rows before the part
+  const int zb = blockIdx.z * OURO_MAX_ROWS, L = p.L + zb;
+  const int rows = min(OURO_MAX_ROWS, (p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows) - zb);   // written before the forward pass began
+  const int32_t *group = p.group + zb, *lin_end = p.lin_end + zb, *seg_start = p.seg_start + zb, *seg_len = p.seg_len + zb;
   const int g = p.H / p.Hkv, dkv = p.Hkv * HD, M_all = g * rows, span0 = sc * SPAN;
 
   if (tid == 0) TRACE(0);
   if (tid == 32) {
     // the weights the next kernels start with do not depend on anything computed here: ask for this CTA's share now
-    const uint32_t u = blockIdx.y * gridDim.x + blockIdx.x, U = gridDim.x * gridDim.y;
+    const uint32_t u = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x, U = gridDim.x * gridDim.y * gridDim.z;
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
       const uint32_t bytes = p.pf_bytes[r];
@@ -264,9 +270,9 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
   if (tid < 128) {
     int lin = 0, len = 0;
     if (tid < rows) {
-      start = tid == 0 || p.group[tid] != p.group[tid - 1];
-      lin = p.lin_end[tid];
-      len = p.seg_len[tid];
+      start = tid == 0 || group[tid] != group[tid - 1];
+      lin = lin_end[tid];
+      len = seg_len[tid];
     }
     ms->lin[tid] = lin;
     ms->len[tid] = len;
@@ -313,7 +319,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
       const int nch = min(SC, (rmax - span0 + CH - 1) / CH);
       for (int ci = 0; ci < nch; ++ci) {
         const int c0 = span0 + ci * CH;
-        if (c0 + CH <= p.L) {
+        if (c0 + CH <= L) {
           ms->items[n++] = ci | (63 << 3);
         } else {
           // the chunk's tile is fetched into both stages once; later passes only patch their rows over it
@@ -345,7 +351,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
   int early = 0;                                       // passes whose tile was requested before the wait
   if (warp == 0) {
     const int n = ms->n_items;
-    while (early < 2 && early < n && ((ms->items[early] >> 3) & 63) == 63) {
+    while (early < 2 && early < n && ((ms->items[early] >> 3) & 63) == 63 && span0 + (ms->items[early] & 7) * CH + CH <= p.L) {
       if (lane == 0) request_tile(early, ms->items[early] & 7);
       ++early;
     }
@@ -366,7 +372,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
         const int info = ms->map[t];
         if (info >= 0) {
           const int r = info & 0xff, hq = (info >> 8) & 0xff;
-          val[i] = __ldg(reinterpret_cast<const uint4 *>(p.q + ((size_t)r * p.H + kvh * g + hq) * HD + ch * 8));
+          val[i] = __ldg(reinterpret_cast<const uint4 *>(p.q + ((size_t)(zb + r) * p.H + kvh * g + hq) * HD + ch * 8));
         }
       }
     }
@@ -401,7 +407,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
           // a candidate's pass: its suffix rows go over the tile the TMA fetched (slots = positions up to the trunk)
           mbar_wait(&ms->full[st], (i >> 1) & 1, ms, p.status);
           const int c0 = span0 + ci * CH, last = ms->gs[go + 1] - 1;
-          const int lin_g = ms->lin[last], seg_g = p.seg_start[last], len_g = ms->len[last];
+          const int lin_g = ms->lin[last], seg_g = seg_start[last], len_g = ms->len[last];
           const int lo = max(c0, lin_g), hi = min(c0 + CH, lin_g + len_g);
           for (int idx = lane; idx < (hi - lo) * 32; idx += 32) {
             const int pos = lo + (idx >> 5), w = idx & 31, ch = w & 15, trow = pos - c0;
@@ -640,7 +646,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
       if (has && nv > span0 && p.direct) {
         // what the merge kernel would compute from this single span: weight exp2(0) = 1, then o * (1 / l)
         const float inv = 1.0f / (lsum[t] + lsum[QR + t]);
-        __nv_bfloat16 *dst = p.out + ((size_t)r * p.H + kvh * g + hq) * HD + h * 64;
+        __nv_bfloat16 *dst = p.out + ((size_t)(zb + r) * p.H + kvh * g + hq) * HD + h * 64;
 #pragma unroll
         for (int d = 0; d < HD / 2; d += 8) {
           uint32_t w[4];
@@ -649,7 +655,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
           *reinterpret_cast<uint4 *>(dst + d) = make_uint4(w[0], w[1], w[2], w[3]);
         }
       } else if (has && nv > span0) {
-        float *dst = p.part + (((size_t)r * p.H + kvh * g + hq) * p.cap + sc) * PW;
+        float *dst = p.part + (((size_t)(zb + r) * p.H + kvh * g + hq) * p.cap + sc) * PW;
         if (h == 0) *reinterpret_cast<float2 *>(dst) = make_float2(m_run, lsum[t] + lsum[QR + t]);
 #pragma unroll
         for (int d = 0; d < HD / 2; d += 4)
@@ -707,9 +713,9 @@ bool launch_attention_tm(const ouro_model_desc &d, const void *q, const void *km
   p.direct = n_vis_max <= SPAN;
   p.status = status;
   p.rows_dev = rows_dev;
-  const int m_all = (d.n_heads / d.n_kv_heads) * rows;
+  const int m_all = (d.n_heads / d.n_kv_heads) * std::min<int>(rows, OURO_MAX_ROWS);
   p.n_spans = (n_vis_max + SPAN - 1) / SPAN;
-  dim3 grid(p.n_spans * d.n_kv_heads, (m_all + QR - 1) / QR);
+  dim3 grid(p.n_spans * d.n_kv_heads, (m_all + QR - 1) / QR, (rows + OURO_MAX_ROWS - 1) / OURO_MAX_ROWS);
   launch_pdl(attn_tm_kernel, grid, THREADS, SMEM_BYTES, s, p);
   return !p.direct;
 }

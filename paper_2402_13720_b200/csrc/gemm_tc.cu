@@ -1,6 +1,6 @@
 // Weight-streaming GEMM for a few dozen tokens on sm_100a tensor cores (tcgen05 + TMEM), fed by TMA.
 //
-//   Y[t, n] = sum_k X[t, k] * W[n, k]      X: [rows <= 128, K] bf16 activations, W: [N, K] bf16 weights
+//   Y[t, n] = sum_k X[t, k] * W[n, k]      X: [rows <= 256, K] bf16 activations, W: [N, K] bf16 weights
 //
 // The verification forward is bound by the one pass over the weights (the paper's premise: checking dozens
 // of tokens costs about as much as one, Section 3.2), so the kernel is organised around the weight stream:
@@ -61,7 +61,6 @@ constexpr int ACT_WARP = 2 + EPI_WARPS;
 constexpr int THREADS = 32 * (ACT_WARP + 1);   // warp 0 weight TMA, warp 1 MMA, warps 2..9 epilogue, warp 10 activation TMA
 constexpr int W_PRODUCERS = 2;    // lanes of warp 0 that issue the weight copies, stage by stage in turn (a power of two, smaller than the ring)
 constexpr int MAX_GRID = 160;
-constexpr int SLOT_FLOATS = TILE_N * OURO_MAX_ROWS;
 constexpr uint32_t SPIN_LIMIT = 1u << 24;
 constexpr unsigned long long HINT_EVICT_FIRST = 0x12F0000000000000ull;
 constexpr unsigned long long HINT_EVICT_LAST = 0x14F0000000000000ull;
@@ -102,11 +101,11 @@ struct GemmParams {
   int head_dim, dq, dkv, L;
   const __nv_bfloat16 *gain;  // MODE_RESIDUAL: gain of the norm that follows (NULL: plain residual add)
   __nv_bfloat16 *xb;          // MODE_RESIDUAL: bf16(gain * x_new), [rows, ldo]
-  float *ss_out;              // MODE_RESIDUAL: [tiles][128] per-tile sums of squares of x_new
+  float *ss_out;              // MODE_RESIDUAL: [tiles][256] per-tile sums of squares of x_new
   const float *ss_in;         // other modes: sums of squares of the activation rows (NULL: no scaling)
   int ss_tiles;
   float ss_inv_d, eps;
-  float *scratch;     // [grid][2][t][128] partial tiles; a word that holds no partial sum holds EMPTY
+  float *scratch;     // [grid][2][128, or 256 in a wide launch][128] partial tiles; a word that holds no partial sum holds EMPTY
   int *status;        // context status word
   int trace_id;           // which GEMM of the layer this is (timeline builds only)
   uint32_t wait_limit;    // polls of a partial-tile wait before it gives up (1 << 22 unless a test shortens it)
@@ -134,7 +133,7 @@ struct ChainArgs {
     const __nv_bfloat16 *gain;    // first norm's gain [d]
     float *x;                     // residual stream [rows][d]
     __nv_bfloat16 *xb;            // bf16(gain * x) [rows][d]
-    float *ss;                    // [d / 128][128] sums of squares per 128-column tile
+    float *ss;                    // [d / 128][256] sums of squares per 128-column tile
     const int *rows_dev;
     int rows, d;
   } embed;
@@ -144,7 +143,7 @@ struct ChainParams {
   ChainArgs args;
 };
 static_assert(sizeof(ChainParams) <= 4096, "kernel parameters");
-constexpr int MISC_BYTES = 1536;   // barriers, flags, per-token factors and positions
+constexpr int MISC_BYTES = 512 + 2 * OURO_TEXT_ROWS * 4;   // barriers, flags, per-token factors and positions
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -254,9 +253,10 @@ __device__ __forceinline__ bool part_there(const uint4 &v) { return v.x != EMPTY
 __device__ __forceinline__ void part_empty(float *src) {
   asm volatile("st.relaxed.gpu.global.v4.b32 [%0], {%1, %1, %1, %1};" ::"l"(src), "r"(EMPTY) : "memory");
 }
-constexpr int STAGE_TOK = 64;     // tokens of a whole tile parked in shared memory at a time
+// Tokens of a whole tile parked in shared memory at a time: fewer where the activation tiles are so large that a fourth
+// stage of the ring hangs on it.
+__host__ __device__ constexpr int stage_tokens(int rows) { return rows > OURO_MAX_ROWS ? 32 : 64; }
 constexpr int STAGE_PITCH = TILE_N + 4;   // floats per parked token: 16-byte aligned rows that start 4 banks apart
-constexpr int STAGE_BYTES = STAGE_TOK * STAGE_PITCH * 4;
 
 // The schedule of this launch for CTA blockIdx.x (see weight_stream.cuh).
 struct SpanWalker : ws::SpanWalker {
@@ -293,6 +293,11 @@ __device__ __forceinline__ bool chain_wait(const ChainArgs &cp, int i) {
   return counter_wait(cp.finished + i, cp.target[i], cp.g[0].status, 1u << 22);
 }
 
+// The kernel by the block's size.  What a GEMM executes once per CTA it mostly waits for as instructions, so that the
+// short blocks' kernel is kept short (and free of spills: a hundred bytes of them cost 4 % of a decoding step).
+enum { FEW = 0, SOME = 1, MANY = 2 };      // up to FEW_ROWS, up to 128, up to 256 rows (known text)
+constexpr int FEW_ROWS = 48;
+template <int SIZE>
 __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_constant__ ChainParams kp) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -300,21 +305,24 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
   const GemmParams &p0 = cp.g[0];                 // rows, t_pad and stages are common to the chain
   const int n_stages = p0.stages, t_pad = p0.t_pad;
   const int b_bytes = t_pad * BLOCK_K * 2;
+  constexpr int MAX_ROWS = SIZE == MANY ? OURO_TEXT_ROWS : OURO_MAX_ROWS, stage_tok = stage_tokens(MAX_ROWS);
+  constexpr int slot_floats = MAX_ROWS * TILE_N;  // (all slots together stay below 2^31 bytes)
   const int stage_bytes = A_BYTES + b_bytes;
   uint8_t *ring = smem;
-  float *xchg = (float *)(ring + (size_t)n_stages * stage_bytes);          // [64 tokens][128] accumulators of a whole tile
-  uint64_t *bars = (uint64_t *)((uint8_t *)xchg + STAGE_BYTES);
+  float *xchg = (float *)(ring + (size_t)n_stages * stage_bytes);          // [stage_tok tokens][128] accumulators of a whole tile
+  uint64_t *bars = (uint64_t *)((uint8_t *)xchg + stage_tok * STAGE_PITCH * 4);
   uint64_t *full = bars, *empty = bars + 16, *acc_full = bars + 32, *acc_empty = bars + 34;
   uint32_t *tmem_base_p = (uint32_t *)(bars + 36);
   volatile int *abort_flag = (volatile int *)(bars + 37);
   volatile int *wait_flag = (volatile int *)(bars + 39);   // [0..1]: outcome of an accumulator wait; [2]: a fix-up gave up
+  volatile int *pend = (volatile int *)(bars + 50);         // [2][4]: tile, contributors, first contributor
   uint64_t *drain_bar = bars + 44;                          // give-up path: "every contraction issued so far has completed"
-  float *rs = (float *)(bars + 48);                         // [128] per-token factor 1/rms of the consumed activations
-  int *spos = (int *)(rs + OURO_MAX_ROWS);                  // [128] token positions (rotary table rows), QKV epilogue
+  float *rs = (float *)(bars + 56);                         // [256] per-token factor 1/rms of the consumed activations
+  int *spos = (int *)(rs + OURO_TEXT_ROWS);                 // [256] token positions (rotary table rows), QKV epilogue
 
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int acc_cols = t_pad <= 32 ? 32 : t_pad <= 64 ? 64 : 128;   // columns per accumulator buffer
+  const int acc_cols = t_pad <= 32 ? 32 : t_pad <= 64 ? 64 : t_pad <= 128 ? 128 : 256;   // columns per accumulator buffer
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < n_stages; ++s) {
@@ -500,7 +508,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
           }
 #pragma unroll
           for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-          if (lane == 0) e.ss[(size_t)(it - r * tiles) * OURO_MAX_ROWS + r] = sq;
+          if (lane == 0) e.ss[(size_t)(it - r * tiles) * OURO_TEXT_ROWS + r] = sq;
         }
       }
       __threadfence();
@@ -521,8 +529,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
     const int rows = p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows;
     SpanWalker w(p);
     Span s;
-    int pend_tile[2] = {0, 0}, pend_n[2] = {1, 1}, pend_first[2] = {0, 0}, n_pend = 0;     // partial tiles this CTA contributed to (<= 2)
-    float *stage = xchg;                                         // [STAGE_TOK tokens][STAGE_PITCH] fp32, 128 tile rows each
+    int n_pend = 0;                                              // partial tiles this CTA contributed to (<= 2), see pend
+    float *stage = xchg;                                         // [stage_tok tokens][STAGE_PITCH] fp32, 128 tile rows each
 
     // Finishing tokens of a tile.  Whatever produced the accumulator values - this CTA's own whole tile, parked
     // in shared memory token-major, or the partial tiles of all contributors in scratch - the last step is the
@@ -568,7 +576,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
           sq += y.x * y.x; sq += y.y * y.y; sq += y.z * y.z; sq += y.w * y.w;
 #pragma unroll
           for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-          if (lane == 0) p.ss_out[(size_t)tile * OURO_MAX_ROWS + t] = sq;
+          if (lane == 0) p.ss_out[(size_t)tile * OURO_TEXT_ROWS + t] = sq;
           return;
         }
         const float r = rs[t];
@@ -633,16 +641,15 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
           finish_token(t, *reinterpret_cast<const float4 *>(stg + (size_t)(t - t_base) * STAGE_PITCH + 4 * ng));
         return true;
       } else {
-        // Sixteen pieces are under way together: one token of sixteen contributors where a warp has a single token or there
-        // are many contributors (1.1B draft at one row: 4323 -> 4198 us), else four tokens of four (7B prefill: 18.9 -> 18.0
-        // ms).  They are fetched without asking first whether they are there: a probe in front is one more round trip to L2
-        // between two GEMMs.  What the epilogue reads besides comes after them, which keeps the code short: with everything
-        // requested up front and the tokens unrolled the routine is twice as long and 3 % slower, all of it waiting for
-        // instructions that a GEMM executes once.
-        const int tbn = n <= 4 || (n <= 8 && t_lim > js) ? 4 : 1;
+        // Twelve pieces are under way together: one token of twelve contributors, or, where there are more tokens than warps
+        // and few contributors, four tokens of three (7B prefill 13.2 -> 11.9 ms, 69 rows of the 34B shape 2.155 -> 2.130 ms;
+        // up to 48 rows the shorter code is as fast or faster: 1.1B draft 4.07 -> 3.98 ms, 37 rows of 7B 3.49 ms either way).
+        // With sixteen pieces the registers spill.  They are fetched without asking first whether they are there: a probe in
+        // front is one more round trip to L2 between two GEMMs.
+        const int tbn = SIZE != FEW && (n <= 4 || (n <= 8 && t_lim > js)) ? 4 : 1;
         float *slot = stg + (size_t)(warp - 2) * 4 * TILE_N + 4 * lane;       // this thread's 16 bytes of four parked tokens
         auto gather = [&](auto tb_c, int tb) -> bool {
-          constexpr int TB = decltype(tb_c)::value, CB = 16 / TB;
+          constexpr int TB = decltype(tb_c)::value, CB = 12 / TB;
           float4 acc[TB];
 #pragma unroll
           for (int j = 0; j < TB; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -654,10 +661,10 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
 #pragma unroll
               for (int cc = 0; cc < CB; ++cc) {
                 const int owner = first + c0 + cc;
-                const float *src = p.scratch + ((size_t)owner * 2 + w.owner_slot(tile, owner)) * SLOT_FLOATS + (size_t)tb * TILE_N + 4 * ng;
+                const float *src = p.scratch + ((owner * 2 + w.owner_slot(tile, owner)) * slot_floats + tb * TILE_N + 4 * ng);
 #pragma unroll
                 for (int j = 0; j < TB; ++j)
-                  tmp[cc][j] = part_load(src + (size_t)(j * js) * TILE_N, c0 + cc < n && tb + j * js < t_lim);
+                  tmp[cc][j] = part_load(src + j * js * TILE_N, c0 + cc < n && tb + j * js < t_lim);
               }
 #pragma unroll
               for (int cc = 0; cc < CB; ++cc)
@@ -671,10 +678,10 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
 #pragma unroll
             for (int cc = 0; cc < CB; ++cc) {
               const int owner = first + c0 + cc;
-              float *src = p.scratch + ((size_t)owner * 2 + w.owner_slot(tile, owner)) * SLOT_FLOATS + (size_t)tb * TILE_N + 4 * ng;
+              float *src = p.scratch + ((owner * 2 + w.owner_slot(tile, owner)) * slot_floats + tb * TILE_N + 4 * ng);
 #pragma unroll
               for (int j = 0; j < TB; ++j) {
-                if (c0 + cc < n && tb + j * js < t_lim) part_empty(src + (size_t)(j * js) * TILE_N);
+                if (c0 + cc < n && tb + j * js < t_lim) part_empty(src + j * js * TILE_N);
                 acc[j].x += __uint_as_float(tmp[cc][j].x); acc[j].y += __uint_as_float(tmp[cc][j].y);
                 acc[j].z += __uint_as_float(tmp[cc][j].z); acc[j].w += __uint_as_float(tmp[cc][j].w);
               }
@@ -698,8 +705,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
               asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(slot + j * TILE_N)),
                            "l"(p.out_f32 + (size_t)(tb + j * js) * p.ldo + col) : "memory");
           }
-          if (!(tbn == 4 ? gather(std::integral_constant<int, 4>{}, tb)
-                         : gather(std::integral_constant<int, 1>{}, tb)))
+          if (!(SIZE != FEW && tbn == 4 ? gather(std::integral_constant<int, SIZE == FEW ? 1 : 4>{}, tb)
+                                        : gather(std::integral_constant<int, 1>{}, tb)))
             return false;
           if (gi == 0) TRACE(12);
 #pragma unroll 1
@@ -716,9 +723,10 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
     // form a cycle.  The (at most two) tiles are finished side by side, each by one half of the epilogue threads.
     auto run_fixups = [&]() {
       const int grp = et / (EPI_THREADS / 2), gi = et % (EPI_THREADS / 2);
+      epi_barrier();
       if (grp < n_pend) {
-        const int first = pend_first[grp];
-        if (!finish(std::true_type{}, pend_tile[grp], gi, EPI_THREADS / 2, (int)blockIdx.x - first, pend_n[grp], first, stage, 0, rows))
+        const int tile = pend[4 * grp], n = pend[4 * grp + 1], first = pend[4 * grp + 2];
+        if (!finish(std::true_type{}, tile, gi, EPI_THREADS / 2, (int)blockIdx.x - first, n, first, stage, 0, rows))
           wait_flag[2] = 1;
         if (gi == 0 && grp == 0) TRACE(10);
         if (publish) __threadfence();                                // this thread's outputs, before the tile counts as finished
@@ -742,11 +750,12 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       if (!ok) break;
       __threadfence();
     }
-    if (et < OURO_MAX_ROWS) {
+    static_assert(EPI_THREADS >= OURO_TEXT_ROWS, "one thread per token");
+    if (et < OURO_TEXT_ROWS) {
       float r = 1.0f;
       if (p.ss_in && et < rows) {
         float sum = 0.f;
-        for (int i = 0; i < p.ss_tiles; ++i) sum += p.ss_in[(size_t)i * OURO_MAX_ROWS + et];
+        for (int i = 0; i < p.ss_tiles; ++i) sum += p.ss_in[(size_t)i * OURO_TEXT_ROWS + et];
         r = 1.0f / sqrtf(sum * p.ss_inv_d + p.eps);
       }
       rs[et] = r;
@@ -772,29 +781,29 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       fence_after_sync();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + a * acc_cols;
       if (s.n_contrib == 1) {
-        // whole tile: the accumulators go to shared memory token-major, STAGE_TOK tokens at a time, and are finished
+        // whole tile: the accumulators go to shared memory token-major, stage_tok tokens at a time, and are finished
         // from there; the TMEM buffer is handed back as soon as it has been read
-        for (int c0 = 0; c0 < p.t_pad; c0 += STAGE_TOK) {
-          const int c1 = min(p.t_pad, c0 + STAGE_TOK);
+        for (int c0 = 0; c0 < t_pad; c0 += stage_tok) {
+          const int c1 = min(t_pad, c0 + stage_tok);
           for (int t0 = c0 + 16 * wh; t0 < c1; t0 += 32) {           // the quarter's two warps take 16 tokens in turn
             tmem_ld16(taddr + t0, v);
 #pragma unroll
             for (int i = 0; i < 16; ++i) stage[(t0 - c0 + i) * STAGE_PITCH + nl] = v[i];
           }
-          if (c1 == p.t_pad) {
+          if (c1 == t_pad) {
             fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[a]);
           }
           epi_barrier();
           finish(std::false_type{}, s.tile, et, EPI_THREADS, 0, 1, 0, stage, c0, min(c1, rows));
-          if (publish && c1 == p.t_pad) __threadfence();
+          if (publish && c1 == t_pad) __threadfence();
           epi_barrier();
-          if (publish && c1 == p.t_pad && et == 0) atomicAdd(cp.finished + ci, 1);
+          if (publish && c1 == t_pad && et == 0) atomicAdd(cp.finished + ci, 1);
         }
       } else {
         // partial tile: parked in this CTA's slot, for its contributors to fetch; added up after the loop
-        float *mine = p.scratch + ((size_t)blockIdx.x * 2 + s.slot) * SLOT_FLOATS;
+        float *mine = p.scratch + ((int)blockIdx.x * 2 + s.slot) * slot_floats;
         for (int t0 = 16 * wh; t0 < rows; t0 += 32) {
           tmem_ld16(taddr + t0, v);
 #pragma unroll
@@ -804,9 +813,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
         fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[a]);
-        pend_tile[n_pend] = s.tile;
-        pend_n[n_pend] = s.n_contrib;
-        pend_first[n_pend] = s.first_owner;
+        if (et == 0) { pend[4 * n_pend] = s.tile; pend[4 * n_pend + 1] = s.n_contrib; pend[4 * n_pend + 2] = s.first_owner; }
         ++n_pend;
       }
       ++item;
@@ -864,7 +871,7 @@ struct FastModel {
   CUtensorMap head;
   CUtensorMap kmap, vmap;               // K and V caches as [layers * max_seq][kv width], box 64 x 128 (tcgen05 attention)
   bool kv_maps = false;
-  CUtensorMap x_d[8], x_q[8], x_f[8];   // activations normed [128, d], attention out [128, dq], SwiGLU out [128, F]; box rows 16, 32, .., 128
+  CUtensorMap x_d[16], x_q[16], x_f[16];   // activations normed [256, d], attention out [256, dq], SwiGLU out [256, F]; box rows 16, 32, .., 256
 };
 struct FastState {
   FastModel m[2];
@@ -887,14 +894,14 @@ struct FastState {
 constexpr int MAX_TILES = 4096;
 constexpr int CHAIN_BYTES = 256;           // the chain counters
 
-size_t slots_bytes() { return (size_t)MAX_GRID * 2 * SLOT_FLOATS * sizeof(float); }
+size_t slots_bytes() { return (size_t)MAX_GRID * 2 * TILE_N * OURO_TEXT_ROWS * sizeof(float); }
 size_t tile_best_bytes() { return (size_t)MAX_TILES * OURO_MAX_ROWS * 4; }
 constexpr int MAX_SS_TILES = 64;           // d_model <= 8192
-size_t ss_bytes() { return (size_t)MAX_SS_TILES * OURO_MAX_ROWS * sizeof(float); }
+size_t ss_bytes() { return (size_t)MAX_SS_TILES * OURO_TEXT_ROWS * sizeof(float); }
 
 int stages_for(int t_pad, int smem_max) {
   int stage = A_BYTES + t_pad * BLOCK_K * 2;
-  int fixed = 1024 + STAGE_BYTES + MISC_BYTES;  // alignment slack, parked whole tile, the rest
+  int fixed = 1024 + stage_tokens(t_pad) * STAGE_PITCH * 4 + MISC_BYTES;  // alignment slack, parked whole tile, the rest
   int s = (smem_max - fixed) / stage;
   return s > 12 ? 12 : s;
 }
@@ -952,7 +959,9 @@ int ouro_fast_setup(ouro_ctx *c) {
   f->s.attn_part = (float *)((char *)f->s.ss + ss_bytes());
   if (cudaMemsetAsync(f->s.slots, 0xff, slots_bytes(), c->stream) != cudaSuccess ||
       cudaMemsetAsync(f->s.finished, 0, CHAIN_BYTES, c->stream) != cudaSuccess ||
-      cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      cudaFuncSetAttribute(gemm_tc_kernel<FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      cudaFuncSetAttribute(gemm_tc_kernel<SOME>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      cudaFuncSetAttribute(gemm_tc_kernel<MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       attention_tc_setup() != OURO_OK || attention_tm_setup() != OURO_OK) {
     delete f;
     c->err = "tensor-core GEMM set-up failed";
@@ -978,10 +987,10 @@ int ouro_fast_setup(ouro_ctx *c) {
       ok = make_map(&fm.kmap, M.k_cache, d.n_layers * d.max_seq, dkv, 128) && make_map(&fm.vmap, M.v_cache, d.n_layers * d.max_seq, dkv, 128);
       fm.kv_maps = ok;
     }
-    for (int i = 0; i < 8 && ok; ++i)
-      ok = make_map(&fm.x_d[i], c->a.xn, OURO_MAX_ROWS, d.d_model, 16 * (i + 1)) &&
-           make_map(&fm.x_q[i], c->a.att, OURO_MAX_ROWS, dq, 16 * (i + 1)) &&
-           make_map(&fm.x_f[i], c->a.act, OURO_MAX_ROWS, d.d_ffn, 16 * (i + 1));
+    for (int i = 0; i < 16 && ok; ++i)
+      ok = make_map(&fm.x_d[i], c->a.xn, OURO_TEXT_ROWS, d.d_model, 16 * (i + 1)) &&
+           make_map(&fm.x_q[i], c->a.att, OURO_TEXT_ROWS, dq, 16 * (i + 1)) &&
+           make_map(&fm.x_f[i], c->a.act, OURO_TEXT_ROWS, d.d_ffn, 16 * (i + 1));
     if (!ok) {
       delete f;
       c->err = "cuTensorMapEncodeTiled failed";
@@ -1081,7 +1090,8 @@ static void flush_chain(ouro_ctx *c) {
   static const int kind_class[5] = {OURO_PROF_QKV, OURO_PROF_WO, OURO_PROF_GATEUP, OURO_PROF_DOWN, OURO_PROF_HEAD};
   {
     ProfScope ps(c, per_kind ? kind_class[s.chain_kind[0]] : OURO_PROF_GEMM);
-    launch_pdl(gemm_tc_kernel, grid, THREADS, (size_t)s.smem_max, c->stream, s.chain);
+    const int t_pad = cp.g[0].t_pad;
+    launch_pdl(t_pad > OURO_MAX_ROWS ? gemm_tc_kernel<MANY> : t_pad > FEW_ROWS ? gemm_tc_kernel<SOME> : gemm_tc_kernel<FEW>, grid, THREADS, (size_t)s.smem_max, c->stream, s.chain);
   }
   cp.n = 0;
   cp.fold.part = nullptr;
@@ -1162,8 +1172,9 @@ int ouro_fast_embed(ouro_ctx *c, int which, int rows) {
   return OURO_OK;
 }
 
-// One decoder layer with the tensor-core GEMMs; OURO_ESTATE when the model does not qualify.
-int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows) {
+// One decoder layer with the tensor-core GEMMs (kv_only: up to its keys and values); OURO_ESTATE when the model does not
+// qualify.
+int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
   if (!c->fast || !c->fast->s.m[which].ok) return OURO_ESTATE;
   ModelRt &M = c->m[which];
   FastModel &fm = c->fast->s.m[which];
@@ -1201,7 +1212,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows) {
       launch_rope_append(d, a.qkv, M.blk.pos, M.rope_cos, M.rope_sin, rows, M.L, l, a.q, M.k_cache, M.v_cache, s);
     }
   }
-  {
+  if (!kv_only) {
     ProfScope ps(c, OURO_PROF_ATTENTION);
     bool pieces = false;             // the attention output is still in per-span pieces
     if (c->fast->s.m[which].kv_maps) {
@@ -1234,7 +1245,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows) {
       f.head_dim = d.head_dim;
     }
   }
-  {
+  if (!kv_only) {
     Gemm p{};
     set_weights(p, weight_side(d, fm, l, G_WO));
     p.mode = MODE_RESIDUAL;
@@ -1243,7 +1254,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows) {
     produce(p, M.ffn_norm[l]);
     push_gemm(c, p, G_WO, fm.x_q, dq, rows, false);
   }
-  {
+  if (!kv_only) {
     Gemm p{};
     set_weights(p, weight_side(d, fm, l, G_GATEUP));
     p.mode = MODE_SWIGLU;
@@ -1251,7 +1262,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows) {
     consume(p);
     push_gemm(c, p, G_GATEUP, fm.x_d, d.d_model, rows, false);
   }
-  {
+  if (!kv_only) {
     Gemm p{};
     set_weights(p, weight_side(d, fm, l, G_DOWN));
     p.mode = MODE_RESIDUAL;
@@ -1346,7 +1357,7 @@ int ouro_fast_head(ouro_ctx *c, int which, int rows, float *logits, int32_t *arg
 namespace {
 constexpr int NA_SPLITTERS = 32;                   // CTAs that may leave partial tiles (two slots each)
 constexpr int NA_MAX_TILES = 512;                  // vocabulary <= 65536
-constexpr size_t NA_SLOT_BYTES = (size_t)NA_SPLITTERS * 2 * SLOT_FLOATS * sizeof(float);
+constexpr size_t NA_SLOT_BYTES = (size_t)NA_SPLITTERS * 2 * TILE_N * OURO_MAX_ROWS * sizeof(float);
 constexpr size_t NA_OFF_STATUS = NA_SLOT_BYTES;
 constexpr size_t NA_OFF_TMAX = NA_OFF_STATUS + 256;
 constexpr size_t NA_OFF_TARG = NA_OFF_TMAX + (size_t)NA_MAX_TILES * OURO_MAX_ROWS * sizeof(float);
@@ -1376,7 +1387,7 @@ int na_setup(int dev) {
   int smem = 0, sms = 0;
   if ((e = cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess ||
       (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) {
+      (e = cudaFuncSetAttribute(gemm_tc_kernel<SOME>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) {
     ouro_set_global_error(std::string("static-scratch set-up: ") + cudaGetErrorString(e));
     return OURO_ECUDA;
   }
@@ -1457,7 +1468,7 @@ extern "C" int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, i
   const ws::Cut cut = ws::cut(tiles, p.kb, grid, rest <= NA_SPLITTERS ? std::min(total, NA_SPLITTERS) : 0);
   p.t0 = cut.t0;
   p.per = cut.per;
-  gemm_tc_kernel<<<grid, THREADS, g_na_smem[dev], s>>>(kp);
+  gemm_tc_kernel<SOME><<<grid, THREADS, g_na_smem[dev], s>>>(kp);
   argmax_tiles_kernel<<<rows, 128, 0, s>>>(p.tile_max, p.tile_arg, tiles, argmax_dev);
   int status = 0;
   if ((e = cudaGetLastError()) != cudaSuccess ||

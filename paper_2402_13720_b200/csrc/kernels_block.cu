@@ -254,8 +254,8 @@ __global__ void assemble_causal_kernel(BlockDev b, const int32_t *tokens, int n,
   b.lin_end[r] = L + r + 1;
   b.seg_start[r] = 0;
   b.seg_len[r] = 0;
-  u64 m0 = 0, m1 = 0;
-  for (int c = 0; c <= r; ++c) (c < 64 ? m0 : m1) |= 1ull << (c & 63);
+  u64 m0 = 0, m1 = 0;                      // (a block of known text may be longer than the masks, which nobody reads then)
+  for (int c = 0; c <= min(r, OURO_MAX_ROWS - 1); ++c) (c < 64 ? m0 : m1) |= 1ull << (c & 63);
   b.mask[2 * r] = m0;
   b.mask[2 * r + 1] = m1;
 }
@@ -272,7 +272,7 @@ void launch_lookup_assemble(const PoolDev &P, const BlockDev &b, DevState *st, c
 }
 void launch_assemble_causal(const BlockDev &b, const int32_t *tokens, int n, int L, cudaStream_t s) {
   OURO_COUNT_LAUNCH();
-  assemble_causal_kernel<<<1, OURO_MAX_ROWS, 0, s>>>(b, tokens, n, L);
+  assemble_causal_kernel<<<1, OURO_TEXT_ROWS, 0, s>>>(b, tokens, n, L);
 }
 
 // ------------------------------------------------------------------------------- acceptance

@@ -39,6 +39,10 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 #endif
 
+// Rows of a block whose outputs nobody reads: long stretches of known text on the tensor-core path.  The weights are
+// streamed once for all of them, and 256 is the widest tcgen05 tile.
+enum { OURO_TEXT_ROWS = 2 * OURO_MAX_ROWS };
+
 // Device-resident scalars of one decoding stream.
 struct DevState {
   int32_t pending;   // last accepted token; its K/V is not cached yet (block row 0 of the next step)

@@ -928,3 +928,50 @@ def test_lookahead_window_bf16_self_draft():
     assert res[1]["target_calls"] <= res[0]["target_calls"]
     with pytest.raises(binding.OuroError):              # a window together with phrase-level drafting is refused
         binding.Engine(MIDB, w, dataclasses.replace(P1, draft_phrases=True), MIDB, w)
+
+
+# ------------------------------------------------------------ wide blocks of known text
+
+@pytest.mark.parametrize("heads,kv,hd", [(4, 2, 128), (8, 2, 64)])
+def test_prefill_in_wide_blocks_is_bit_identical_to_short_blocks(heads, kv, hd):
+    """Prompts beyond 128 tokens are prefilled up to 256 rows at a time, without the LM head and the last layer's second
+    half.  A token's keys and values must not show it: they equal, bit for bit, those left by blocks of 1 to 100 rows.
+    Lengths around the block edges, one that ends a span of 512 keys, and one with a one-row rest."""
+    desc = synth.ModelDesc(3, 512, heads, kv, hd, 704, 1024, 900, "bf16")
+    P = synth.DecodeParams(3, 4, 2, 16, 8, seed_prompt=False)
+    eng, _ = make(desc, P, 6)
+    rng = np.random.default_rng(6)
+    text = rng.integers(0, desc.vocab, 780).astype(np.int32)
+    eng.reset()
+    at = 0
+    for n in (1, 100, 47, 100, 3, 96, 100, 100, 100, 100, 32):
+        eng.assemble_causal(binding.OURO_TARGET, text[at: at + n])
+        eng.verify_forward()
+        eng.advance(binding.OURO_TARGET, n)
+        at += n
+    torch.cuda.synchronize()
+    want = [c[:, :at].clone() for c in (eng.tm.k_cache, eng.tm.v_cache)]
+    assert bool(torch.isfinite(want[0].float()).all()) and float(want[1].float().abs().max()) > 0
+    for n in (129, 130, 256, 257, 258, 385, 513, 514, 600, 770):
+        eng.reset()
+        eng.tm.k_cache.zero_(); eng.tm.v_cache.zero_()
+        eng.prefill(text[:n])                                      # caches n - 1 positions
+        for got, ref in zip((eng.tm.k_cache, eng.tm.v_cache), want):
+            assert torch.equal(got[:, : n - 1], ref[:, : n - 1]), n
+            assert not bool(got[:, n - 1:].any()), n               # and nothing behind them
+    eng.close()
+
+
+def test_draft_catches_up_on_a_long_prompt():
+    """The draft model's first block is the whole prompt, the last 128 rows of it or fewer with outputs: its drafts equal
+    those of the same model as the target (self-draft), which accepts every one of them."""
+    desc = synth.ModelDesc(2, 512, 8, 2, 64, 704, 1024, 700, "bf16")
+    P = synth.DecodeParams(4, 5, 2, 16, 8)
+    w = synth.model_weights(desc, 8, device="cuda:0")
+    eng = binding.Engine(desc, w, P, desc, w)
+    for n in (130, 200, 257, 385, 400):
+        prompt = synth.prompt(n, desc.vocab, n, 0.4, 4, 8)
+        van, _ = eng.generate_vanilla(prompt, 24)
+        out, st = eng.generate(prompt, 24)
+        assert np.array_equal(out, van) and st["full_accepts"] == st["target_calls"]
+    eng.close()
