@@ -102,6 +102,7 @@ static size_t carve(ouro_ctx *c, char *base, const ouro_model_desc *t, const our
   int S = p->beta - 1;
   int32_t *cand_suffix = cv.take<int32_t>((size_t)std::max(1, p->K * S));
   int32_t *cand_count = cv.take<int32_t>(1);
+  int *arrived = cv.take<int>(1);
   int32_t *draft_dev = cv.take<int32_t>(p->gamma);
   int32_t *win_dev = cv.take<int32_t>(OURO_MAX_WINDOW);
   PoolDev pool{};
@@ -134,6 +135,7 @@ static size_t carve(ouro_ctx *c, char *base, const ouro_model_desc *t, const our
     c->seq_dev = seq_dev;
     c->cand_suffix = cand_suffix;
     c->cand_count = cand_count;
+    c->arrived_dev = arrived;
     c->draft_dev = draft_dev;
     c->win_dev = win_dev;
     c->pool = pool;
@@ -180,6 +182,7 @@ int ouro_fast_setup(ouro_ctx *c);  // tensor maps etc. of the tensor-core paths 
 void ouro_fast_reset(ouro_ctx *c, bool force);   // clears split-K / chain counters (always, or only after a device-side give-up)
 void ouro_fast_mark_dirty(ouro_ctx *c);
 bool ouro_fast_available(ouro_ctx *c, int which);   // model `which` runs on the tensor-core kernels
+bool ouro_fast_layers(ouro_ctx *c, int which);      // its GEMMs do
 
 extern "C" int ouro_create(const ouro_model_desc *t, const ouro_model_mem *tm, const ouro_model_desc *d,
                            const ouro_model_mem *dm, const ouro_params *p, void *ws, size_t ws_bytes, void *stream,
@@ -239,6 +242,10 @@ extern "C" int ouro_create(const ouro_model_desc *t, const ouro_model_mem *tm, c
           (e = cudaMemsetAsync(n->m[w].v_cache, 0, bytes, n->stream)) != cudaSuccess)
         return bail(OURO_ECUDA, std::string("clearing the KV cache: ") + cudaGetErrorString(e));
     }
+  int dev = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&n->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+      (e = cudaMemsetAsync(n->arrived_dev, 0, sizeof(int), n->stream)) != cudaSuccess)
+    return bail(OURO_ECUDA, std::string("device set-up: ") + cudaGetErrorString(e));
   launch_pool_clear(n->pool, n->st, n->stream);
   launch_set_state(n->st, n->seq_dev, 1, 0, 1, n->stream);
   int rc = ouro_fast_setup(n);
@@ -276,6 +283,8 @@ extern "C" int ouro_reset(ouro_ctx *c, int keep_pool) {
   c->seq.assign(1, 0);
   c->step = 0;
   ouro_fast_reset(c, true);
+  CK(cudaMemsetAsync(c->arrived_dev, 0, sizeof(int), c->stream));      // a barrier that gave up leaves the count short
+  c->arrived_host = 0;
   launch_set_state(c->st, c->seq_dev, 1, 0, 1, c->stream);
   if (!keep_pool) launch_pool_clear(c->pool, c->st, c->stream);
   CKL();
@@ -349,6 +358,13 @@ static int mbox_wait(ouro_ctx *c, int slot, int32_t seq) {
   return OURO_OK;
 }
 
+// The whole forward runs as one launch (and reads the block's row count from device memory).  Single kernels are timed as
+// kernels of their own.
+static bool small_forward(ouro_ctx *c, int which) {
+  const bool timed = c->prof_class >= OURO_PROF_EMBED && c->prof_class <= OURO_PROF_ARGMAX;
+  return !ouro_fast_available(c, which) && !ouro_fast_layers(c, which) && forward_small_supported(c->m[which].d) && !timed;
+}
+
 extern "C" int ouro_assemble_candidates(ouro_ctx *c, const int32_t *draft_dev, const int32_t *suffix_dev,
                                         const int32_t *count_dev) {
   if (!c || !draft_dev || ((suffix_dev == nullptr) != (count_dev == nullptr))) return OURO_EINVAL;
@@ -360,8 +376,8 @@ extern "C" int ouro_assemble_candidates(ouro_ctx *c, const int32_t *draft_dev, c
   else
     launch_assemble_candidates(M.blk, c->st, draft_dev, suffix_dev, count_dev, M.L, gamma, S, K, c->stream);
   CKL();
-  if (ouro_fast_available(c, OURO_TARGET)) {
-    // The tensor-core kernels read the block's row count from device memory: the forward is launched for the largest
+  if (ouro_fast_available(c, OURO_TARGET) || small_forward(c, OURO_TARGET)) {
+    // The tensor-core kernels and the one-launch forward read the block's row count from device memory: the forward is launched for the largest
     // block these parameters allow and the host never waits for the lookup.
     M.blk_rows = 1 + gamma + K * S;
     M.blk_rows_dev = true;
@@ -447,14 +463,25 @@ int ouro_fast_head(ouro_ctx *c, int which, int rows, float *logits, int32_t *arg
 static int forward(ouro_ctx *c, int which, int32_t *argmax_dev, float *logits_dev) {
   ModelRt &M = c->m[which];
   if (!M.present) return fail(c, OURO_ESTATE, "model not present");
+  if (M.blk_rows == 0 || M.blk_L != M.L) return fail(c, OURO_ESTATE, "no block assembled for the current cache length");
+  if (M.blk_rows_dev && !ouro_fast_available(c, which) && !small_forward(c, which)) {   // timing was switched on in between
+    CK(cudaMemcpyAsync(c->pin, &c->st->n_rows, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    M.blk_rows = c->pin[0];
+    M.blk_rows_dev = false;
+  }
   const int rows = M.blk_rows, L = M.L;
-  if (rows == 0 || M.blk_L != L) return fail(c, OURO_ESTATE, "no block assembled for the current cache length");
   const ouro_model_desc &d = M.d;
   const int dt = d.dtype, dq = d.n_heads * d.head_dim, dkv = d.n_kv_heads * d.head_dim;
   cudaStream_t s = c->stream;
   Activations &a = c->a;
   ProfScope whole(c, OURO_PROF_FORWARD);
   c->cur_rows_dev = M.blk_rows_dev ? &c->st->n_rows : nullptr;
+  if (small_forward(c, which)) {
+    TRY(launch_forward_small(c, which, rows, c->cur_rows_dev, argmax_dev, logits_dev ? logits_dev : a.logits));
+    CKL();
+    return OURO_OK;
+  }
   if (ouro_fast_embed(c, which, rows) == OURO_ESTATE) {
     ProfScope ps(c, OURO_PROF_EMBED);
     launch_embed(dt, M.embed, M.blk.tok, rows, d.d_model, a.x, s);

@@ -1,0 +1,367 @@
+// One forward of a small generic model (fp32, or bf16 shapes the tensor-core kernels do not take) as ONE launch.
+//
+// Such a model's weights are read in microseconds; what a forward costs is its chain of dependent steps, eight launches a
+// layer as kernels of their own (5.6 us each on the fp32 pair of 128-wide layers).  Here one CTA per SM stays for the
+// whole forward and the steps are separated by grid barriers (1 us).  A warp takes a unit of a step: one or two output
+// columns for a tile of rows, or one (row, head) of the attention.  RMSNorm has no step of its own: the warp that
+// contracts a row with the weights has just read the row, and sums its squares first.
+//
+// The rule of kernels_layer.cu holds: a value depends on its own row and on the keys that row sees, in fixed groups.
+//
+// The barriers are bounded: on expiry the CTA raises the context's status word and leaves, and so do the others.
+#include <algorithm>
+
+#include "ouro_internal.h"
+#include "generic.cuh"
+
+namespace {
+
+constexpr int THREADS = 256;
+constexpr int WARPS = THREADS / 32;
+constexpr int RT = 4;                    // rows of a unit
+constexpr int MAX_LAYERS = 40;           // layer pointers travel as kernel parameters
+constexpr uint32_t BARRIER_LIMIT = 1u << 22;
+
+struct LayerPtrs { const void *attn_norm, *wq, *wk, *wv, *wo, *ffn_norm, *w_gate, *w_up, *w_down; };
+struct SmallParams {
+  LayerPtrs layer[MAX_LAYERS];
+  const void *embed, *final_norm, *lm_head;
+  void *k_cache, *v_cache;
+  const float *cos_t, *sin_t;
+  BlockDev b;
+  int n_layers, d, H, Hkv, h, F, V, max_seq, L;
+  float eps, scale;
+  int rows;
+  const int *rows_dev;     // NULL, or the block's true row count in device memory (`rows` is then an upper bound)
+  float *x;                // residual stream [rows][d]
+  void *q, *att, *act;     // [rows][dq], [rows][dq], [rows][F]
+  float *logits;           // [rows][V]
+  int32_t *argmax;         // [rows]; NULL: the last layer ends with its keys and values
+  int *arrived;            // CTAs arrived at barriers, ever
+  int base;                // what it holds when the launch begins
+  int *status;
+};
+static_assert(sizeof(SmallParams) <= 4096, "kernel parameters");
+
+// All CTAs of the grid (one per SM, launched cooperatively) meet; writes before are visible after.  False: given up.
+__device__ __forceinline__ bool grid_barrier(const SmallParams &p, int &target, int *flag) {
+  target += gridDim.x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.arrived) : "memory");
+    int ok = 0;
+    for (uint32_t spin = 0; spin < BARRIER_LIMIT; ++spin) {
+      int seen;
+      asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(p.arrived) : "memory");
+      if (seen - target >= 0) { ok = 1; break; }
+      if ((spin & 63) == 63 && *(volatile const int *)p.status != 0) break;
+    }
+    if (!ok) atomicExch(p.status, 1);
+    *flag = ok;
+  }
+  __syncthreads();
+  return *flag != 0;
+}
+
+// Contractions of a tile of rows with C weight rows, the rows normalised on the way (gain != NULL):
+//   acc[c][i] = sum_k T(gain[k] * x[i][k] / rms(x[i])) * w[c][k], lanes stride over k, the same order for any tile.
+template <typename T, int C, typename Row>
+__device__ __forceinline__ void contract(const Row &row, const T *gain, float eps, const T *const *w, int n_rows, int K, float (*acc)[RT]) {
+  constexpr int V = Vec<T>::N;
+  const int lane = threadIdx.x & 31;
+  float inv[RT];
+#pragma unroll
+  for (int i = 0; i < RT; ++i) {
+    inv[i] = 0.f;
+#pragma unroll
+    for (int c = 0; c < C; ++c) acc[c][i] = 0.f;
+  }
+  if (gain) {
+    for (int k = lane * V; k < K; k += 32 * V)
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+        if (i < n_rows) {
+          float xv[V];
+          row(i, k, xv);
+#pragma unroll
+          for (int e = 0; e < V; ++e) inv[i] = fmaf(xv[e], xv[e], inv[i]);
+        }
+#pragma unroll
+    for (int i = 0; i < RT; ++i) inv[i] = 1.0f / sqrtf(warp_sum(inv[i]) / (float)K + eps);
+  }
+  for (int k = lane * V; k < K; k += 32 * V) {
+    Vec<T> wv[C], gv;
+#pragma unroll
+    for (int c = 0; c < C; ++c) wv[c].load(w[c] + k);
+    if (gain) gv.load(gain + k);
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+      if (i < n_rows) {
+        float xv[V];
+        row(i, k, xv);
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+          const float a = gain ? to_f<T>(from_f<T>(gv.get(e) * (xv[e] * inv[i]))) : xv[e];
+#pragma unroll
+          for (int c = 0; c < C; ++c) acc[c][i] = fmaf(a, wv[c].get(e), acc[c][i]);
+        }
+      }
+  }
+#pragma unroll
+  for (int c = 0; c < C; ++c)
+#pragma unroll
+    for (int i = 0; i < RT; ++i) acc[c][i] = warp_sum(acc[c][i]);
+}
+
+// Lane i's value of a tile's rows.
+__device__ __forceinline__ float of_row(const float *acc, int lane) {
+  float v = acc[0];
+#pragma unroll
+  for (int i = 1; i < RT; ++i) v = lane == i ? acc[i] : v;
+  return v;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_constant__ SmallParams p) {
+  extern __shared__ float sq[];            // [WARPS][h] the query of each warp's attention unit
+  __shared__ int flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int gw = blockIdx.x * WARPS + warp, nw = gridDim.x * WARPS;
+  const int rows = p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows;
+  const int tiles = (rows + RT - 1) / RT;
+  const int d = p.d, h = p.h, half = h >> 1, dq = p.H * h, dkv = p.Hkv * h;
+  int target = p.base;
+  T *q = (T *)p.q, *att = (T *)p.att, *act = (T *)p.act;
+
+  // a row of the residual stream: in front of the first layer still the token's embedding
+  int r0 = 0;
+  bool embedded = true;
+  auto residual = [&](int i, int k, float *xv) {
+    constexpr int V = Vec<T>::N;
+    if (embedded) {
+      Vec<T> e;
+      e.load((const T *)p.embed + (size_t)p.b.tok[r0 + i] * d + k);
+#pragma unroll
+      for (int j = 0; j < V; ++j) xv[j] = e.get(j);
+    } else {
+#pragma unroll
+      for (int j = 0; j < V; j += 4) {
+        const float4 v = __ldcg(reinterpret_cast<const float4 *>(p.x + (size_t)(r0 + i) * d + k + j));
+        xv[j] = v.x; xv[j + 1] = v.y; xv[j + 2] = v.z; xv[j + 3] = v.w;
+      }
+    }
+  };
+  auto stored = [&](const T *base, int K) {
+    return [=](int i, int k, float *xv) {
+      constexpr int V = Vec<T>::N;
+      Vec<T> e;
+      e.v = __ldcg(reinterpret_cast<const decltype(e.v) *>(base + (size_t)i * K + k));
+#pragma unroll
+      for (int j = 0; j < V; ++j) xv[j] = e.get(j);
+    };
+  };
+
+  for (int l = 0; l < p.n_layers; ++l) {
+    const LayerPtrs &w = p.layer[l];
+    const size_t layer_off = (size_t)l * p.max_seq * dkv;
+    // ---- q, k, v of the normalised rows, rotary positions, cache append.  A unit: dimensions i and i + half of a head
+    const int pairs = (p.H + 2 * p.Hkv) * half;
+    for (int u = gw; u < pairs * tiles; u += nw) {
+      const int head = (u % pairs) / half, i = (u % pairs) % half;
+      r0 = u / pairs * RT;
+      const int n = min(RT, rows - r0);
+      const bool is_q = head < p.H, is_v = head >= p.H + p.Hkv;
+      const int hh = is_q ? head : is_v ? head - p.H - p.Hkv : head - p.H;
+      const T *base = (const T *)(is_q ? w.wq : is_v ? w.wv : w.wk) + ((size_t)hh * h + i) * d;
+      const T *const ws[2] = {base, base + (size_t)half * d};
+      float acc[2][RT];
+      contract<T, 2>(residual, (const T *)w.attn_norm, p.eps, ws, n, d, acc);
+      if (lane < n) {
+        const int r = r0 + lane;
+        const float a = of_row(acc[0], lane), b = of_row(acc[1], lane);
+        float ra = a, rb = b;
+        if (!is_v) {
+          const size_t ti = (size_t)p.b.pos[r] * half + i;
+          const float c = p.cos_t[ti], s = p.sin_t[ti];
+          ra = a * c - b * s;
+          rb = b * c + a * s;
+        }
+        T *dst = is_q ? q + (size_t)r * dq + hh * h
+                      : (T *)(is_v ? p.v_cache : p.k_cache) + layer_off + (size_t)(p.L + r) * dkv + hh * h;
+        dst[i] = from_f<T>(ra);
+        dst[i + half] = from_f<T>(rb);
+      }
+    }
+    if (!p.argmax && l + 1 == p.n_layers) return;
+    if (!grid_barrier(p, target, &flag)) return;
+    // ---- attention, a warp per (row, head): keys by virtual position in groups of 32, online softmax
+    for (int u = gw; u < rows * p.H; u += nw) {
+      const int r = u / p.H, a = u % p.H, kvh = a / (p.H / p.Hkv);
+      float *myq = sq + warp * h;
+      __syncwarp();
+      for (int i = lane; i < h; i += 32) myq[i] = to_f<T>(__ldcg(q + (size_t)r * dq + a * h + i));
+      __syncwarp();
+      const int lin_end = p.b.lin_end[r], seg_start = p.b.seg_start[r], n_vis = lin_end + p.b.seg_len[r];
+      const T *kb = (const T *)p.k_cache + layer_off + kvh * h, *vb = (const T *)p.v_cache + layer_off + kvh * h;
+      float m = -INFINITY, sum = 0.f;
+      float o[4] = {0.f, 0.f, 0.f, 0.f};                 // dims lane, lane + 32, .. (h <= 128)
+      const int nd = h >> 5;
+      for (int p0 = 0; p0 < n_vis; p0 += 32) {
+        const int pos = p0 + lane;
+        const bool valid = pos < n_vis;
+        const int slot = pos < lin_end ? pos : seg_start + (pos - lin_end);
+        float sc = -INFINITY;
+        if (valid) {
+          const T *kr = kb + (size_t)slot * dkv;
+          float acc = 0.f;
+#pragma unroll 4
+          for (int i = 0; i < h; i += Vec<T>::N) {
+            Vec<T> kv;
+            kv.v = __ldcg(reinterpret_cast<const decltype(kv.v) *>(kr + i));
+#pragma unroll
+            for (int e = 0; e < Vec<T>::N; ++e) acc = fmaf(myq[i + e], kv.get(e), acc);
+          }
+          sc = acc * p.scale;
+        }
+        const float m_new = fmaxf(m, warp_max(sc));
+        const float corr = expf(m - m_new);
+        const float pw = valid ? expf(sc - m_new) : 0.f;
+        sum = sum * corr + warp_sum(pw);
+#pragma unroll
+        for (int dd = 0; dd < 4; ++dd) o[dd] *= corr;
+        const int cnt = min(32, n_vis - p0);
+#pragma unroll 8
+        for (int t = 0; t < cnt; ++t) {
+          const float pt = __shfl_sync(FULL, pw, t);
+          const int st = __shfl_sync(FULL, slot, t);
+          const T *vr = vb + (size_t)st * dkv;
+#pragma unroll
+          for (int dd = 0; dd < 4; ++dd)
+            if (dd < nd) o[dd] = fmaf(pt, to_f<T>(__ldcg(vr + lane + 32 * dd)), o[dd]);
+        }
+        m = m_new;
+      }
+      const float inv = 1.0f / sum;
+#pragma unroll
+      for (int dd = 0; dd < 4; ++dd)
+        if (dd < nd) att[(size_t)r * dq + a * h + lane + 32 * dd] = from_f<T>(o[dd] * inv);
+    }
+    if (!grid_barrier(p, target, &flag)) return;
+    // ---- a column of a projection back into the residual stream
+    auto project = [&](const T *src, const void *weight, int K) {
+      for (int u = gw; u < d * tiles; u += nw) {
+        const int n_col = u % d;
+        r0 = u / d * RT;
+        const int n = min(RT, rows - r0);
+        const T *const ws[1] = {(const T *)weight + (size_t)n_col * K};
+        float acc[1][RT];
+        contract<T, 1>(stored(src + (size_t)r0 * K, K), (const T *)nullptr, 0.f, ws, n, K, acc);
+        if (lane < n) {
+          const int r = r0 + lane;
+          float *x = p.x + (size_t)r * d + n_col;
+          const float old = embedded ? to_f<T>(((const T *)p.embed)[(size_t)p.b.tok[r] * d + n_col]) : __ldcg(x);
+          __stcg(x, old + of_row(acc[0], lane));
+        }
+      }
+    };
+    project(att, w.wo, dq);
+    embedded = false;
+    if (!grid_barrier(p, target, &flag)) return;
+    // ---- SiLU(gate) * up
+    for (int u = gw; u < p.F * tiles; u += nw) {
+      const int n_col = u % p.F;
+      r0 = u / p.F * RT;
+      const int n = min(RT, rows - r0);
+      const T *const ws[2] = {(const T *)w.w_gate + (size_t)n_col * d, (const T *)w.w_up + (size_t)n_col * d};
+      float acc[2][RT];
+      contract<T, 2>(residual, (const T *)w.ffn_norm, p.eps, ws, n, d, acc);
+      if (lane < n) {
+        const float g = of_row(acc[0], lane), up = of_row(acc[1], lane);
+        act[(size_t)(r0 + lane) * p.F + n_col] = from_f<T>(g / (1.0f + expf(-g)) * up);
+      }
+    }
+    if (!grid_barrier(p, target, &flag)) return;
+    project(act, w.w_down, p.F);
+    if (!grid_barrier(p, target, &flag)) return;
+  }
+  // ---- LM head
+  for (int u = gw; u < p.V * tiles; u += nw) {
+    const int n_col = u % p.V;
+    r0 = u / p.V * RT;
+    const int n = min(RT, rows - r0);
+    const T *const ws[1] = {(const T *)p.lm_head + (size_t)n_col * d};
+    float acc[1][RT];
+    contract<T, 1>(residual, (const T *)p.final_norm, p.eps, ws, n, d, acc);
+    if (lane < n) __stcg(p.logits + (size_t)(r0 + lane) * p.V + n_col, of_row(acc[0], lane));
+  }
+  if (!grid_barrier(p, target, &flag)) return;
+  // ---- greedy choice, a warp per row; the smallest index among equals
+  for (int r = gw; r < rows; r += nw) {
+    float best = -INFINITY;
+    int idx = INT_MAX;
+#pragma unroll 4
+    for (int i = lane; i < p.V; i += 32) {
+      const float v = __ldcg(p.logits + (size_t)r * p.V + i);
+      if (v > best || (v == best && i < idx)) { best = v; idx = i; }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      const float v2 = __shfl_xor_sync(FULL, best, o);
+      const int i2 = __shfl_xor_sync(FULL, idx, o);
+      if (v2 > best || (v2 == best && i2 < idx)) { best = v2; idx = i2; }
+    }
+    if (lane == 0) p.argmax[r] = idx == INT_MAX ? 0 : idx;
+  }
+}
+
+}  // namespace
+
+// Narrow models only: every warp reads its rows itself (twice where they are normalised), which a wide model's step would
+// pay for, and a wide model's steps are not what its launches cost.
+bool forward_small_supported(const ouro_model_desc &d) { return d.n_layers <= MAX_LAYERS && d.d_model <= 512 && d.d_ffn <= 2048; }
+
+int launch_forward_small(ouro_ctx *c, int which, int rows, const int *rows_dev, int32_t *argmax, float *logits) {
+  ModelRt &M = c->m[which];
+  const ouro_model_desc &d = M.d;
+  SmallParams p{};
+  for (int l = 0; l < d.n_layers; ++l)
+    p.layer[l] = {M.attn_norm[l], M.wq[l], M.wk[l], M.wv[l], M.wo[l], M.ffn_norm[l], M.w_gate[l], M.w_up[l], M.w_down[l]};
+  p.embed = M.embed; p.final_norm = M.final_norm; p.lm_head = M.lm_head;
+  p.k_cache = M.k_cache; p.v_cache = M.v_cache;
+  p.cos_t = M.rope_cos; p.sin_t = M.rope_sin;
+  p.b = M.blk;
+  p.n_layers = d.n_layers; p.d = d.d_model; p.H = d.n_heads; p.Hkv = d.n_kv_heads; p.h = d.head_dim; p.F = d.d_ffn;
+  p.V = d.vocab; p.max_seq = d.max_seq; p.L = M.L;
+  p.eps = d.rms_eps;
+  p.scale = 1.0f / sqrtf((float)d.head_dim);
+  p.rows = rows; p.rows_dev = rows_dev;
+  p.x = c->a.x; p.q = c->a.q; p.att = c->a.att; p.act = c->a.act;
+  p.logits = logits; p.argmax = argmax;
+  p.arrived = c->arrived_dev;
+  p.base = c->arrived_host;
+  p.status = &c->st->status;
+  // as many CTAs as the widest step has units for: a barrier of fewer CTAs is no dearer
+  const long tiles = (rows + RT - 1) / RT;
+  const long units = tiles * std::max<long>(std::max<long>(d.d_ffn, argmax ? d.vocab : 0), (d.n_heads + 2 * d.n_kv_heads) * (d.head_dim / 2));
+  const int grid = (int)std::max<long>(1, std::min<long>(c->sms, (units + WARPS - 1) / WARPS));
+  const int barriers = argmax ? 5 * d.n_layers + 1 : 5 * (d.n_layers - 1);
+  c->arrived_host = (int)((unsigned)c->arrived_host + (unsigned)(barriers * grid));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = THREADS;
+  cfg.dynamicSmemBytes = (size_t)WARPS * d.head_dim * sizeof(float);
+  cfg.stream = c->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  OURO_COUNT_LAUNCH();
+  const cudaError_t e = d.dtype == OURO_BF16 ? cudaLaunchKernelEx(&cfg, forward_small_kernel<__nv_bfloat16>, p)
+                                             : cudaLaunchKernelEx(&cfg, forward_small_kernel<float>, p);
+  if (e != cudaSuccess) {
+    c->err = std::string("one-launch forward: ") + cudaGetErrorString(e);
+    return OURO_ECUDA;
+  }
+  return OURO_OK;
+}

@@ -1152,6 +1152,8 @@ bool ouro_fast_available(ouro_ctx *c, int which) {
   return d.head_dim == 64 || d.head_dim == 128;
 }
 
+bool ouro_fast_layers(ouro_ctx *c, int which) { return c->fast && c->fast->s.m[which].ok; }
+
 // The embedding gather runs in front of the first layer's q,k,v GEMM, inside its launch.
 int ouro_fast_embed(ouro_ctx *c, int which, int rows) {
   if (!c->fast || !c->fast->s.m[which].ok) return OURO_ESTATE;

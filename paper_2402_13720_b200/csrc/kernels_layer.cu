@@ -8,43 +8,7 @@
 // That is what makes Ouroboros output bit-identical to one-token-at-a-time greedy decoding on this
 // library (the paper observes small differences "caused by floating point error", Appendix A).
 #include "ouro_internal.h"
-
-#define FULL 0xffffffffu
-
-template <typename T> __device__ __forceinline__ float to_f(T v);
-template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
-template <typename T> __device__ __forceinline__ T from_f(float v);
-template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
-
-template <typename T> struct Vec;       // 16-byte vector of T
-template <> struct Vec<float> {
-  static constexpr int N = 4;
-  float4 v;
-  __device__ __forceinline__ void load(const float *p) { v = *reinterpret_cast<const float4 *>(p); }
-  __device__ __forceinline__ float get(int i) const { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
-};
-template <> struct Vec<__nv_bfloat16> {
-  static constexpr int N = 8;
-  uint4 v;
-  __device__ __forceinline__ void load(const __nv_bfloat16 *p) { v = *reinterpret_cast<const uint4 *>(p); }
-  __device__ __forceinline__ float get(int i) const {
-    uint32_t w = (i >> 1) == 0 ? v.x : (i >> 1) == 1 ? v.y : (i >> 1) == 2 ? v.z : v.w;
-    return __uint_as_float((i & 1) ? (w & 0xffff0000u) : (w << 16));
-  }
-};
-
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-  return v;
-}
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(FULL, v, o));
-  return v;
-}
+#include "generic.cuh"
 
 // ------------------------------------------------------------------------------ rotary table
 // cos/sin of pos * theta^(-2i/h), evaluated in double once at set-up.

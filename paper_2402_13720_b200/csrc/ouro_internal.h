@@ -129,6 +129,9 @@ struct ouro_ctx {
   // by the kernel itself, payload first, then a sequence number the host polls.
   int32_t *mbox = nullptr, *mbox_dev = nullptr;
   int32_t mseq = 0;
+  int sms = 0;                         // multiprocessors of the context's device
+  int *arrived_dev = nullptr;          // barrier arrivals of the one-launch forwards, never reset but with the context ...
+  int arrived_host = 0;                // ... and what that word holds once everything launched so far is done
   const int *cur_rows_dev = nullptr;   // during a forward: where the kernels read the block's true row count, or NULL
   ouro_drafter_fn drafter = nullptr;
   void *drafter_user = nullptr;
@@ -199,6 +202,10 @@ void launch_rope_append(const ouro_model_desc &d, const float *qkv, const int32_
                         cudaStream_t s);
 void launch_attention_simple(const ouro_model_desc &d, const void *q, const void *k_cache, const void *v_cache,
                              const BlockDev &b, int rows, int layer, void *out, cudaStream_t s);
+
+// ---- forward_small.cu ----------------------------------------------------------------------------
+bool forward_small_supported(const ouro_model_desc &d);
+int launch_forward_small(ouro_ctx *c, int which, int rows, const int *rows_dev, int32_t *argmax, float *logits);
 
 // ---- attn_tc.cu --------------------------------------------------------------------------------
 bool attention_tc_supported(const ouro_model_desc &d);

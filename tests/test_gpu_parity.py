@@ -975,3 +975,39 @@ def test_draft_catches_up_on_a_long_prompt():
         out, st = eng.generate(prompt, 24)
         assert np.array_equal(out, van) and st["full_accepts"] == st["target_calls"]
     eng.close()
+
+
+# ------------------------------------------------------------ the one-launch forward of small generic models
+
+@pytest.mark.parametrize("dtype,d,heads,kv,hd,ffn,vocab", [
+    ("f32", 128, 4, 4, 32, 344, 512), ("f32", 72, 3, 1, 32, 104, 1000), ("f32", 512, 4, 2, 128, 2048, 264),
+    ("bf16", 96, 2, 1, 96, 136, 520), ("bf16", 200, 4, 2, 64, 72, 1032)])
+def test_one_launch_forward_matches_oracle_and_single_kernels(dtype, d, heads, kv, hd, ffn, vocab):
+    """Widths that are no multiple of a warp's stride, one kv head, head dims 32 to 128, the widest model the one-launch
+    forward takes; blocks of 1 to 100 rows.  Against the oracle, against the same block through the single kernels (which
+    run while one kernel class is being timed), and a row's logits do not depend on the block."""
+    desc = synth.ModelDesc(2, d, heads, kv, hd, ffn, vocab, 192, dtype)
+    P = synth.DecodeParams(4, 5, 3, 16, 8)
+    eng, W = make(desc, P, 9)
+    _verify_case(eng, W, desc, P, 9, 40, _fp32_tol if dtype == "f32" else _bf16_tol)
+    rng = np.random.default_rng(9)
+    for n in (1, 3, 4, 5, 37, 100):
+        tokens = rng.integers(0, vocab, n).astype(np.int32)
+        outs = []
+        for timed in (False, True):
+            eng.profile_enable("norm" if timed else "off")
+            eng.set_state(30, 1)                      # on the keys the prefill above left
+            eng.assemble_causal(binding.OURO_TARGET, tokens)
+            am, lg = eng.verify_forward(want_logits=True)
+            outs.append((am[:n].clone(), lg[:n].clone()))
+        eng.profile_enable("off")
+        scale = outs[1][1].abs().amax()
+        # fp32: sums of at most 2048 products in another order; bf16: one rounding of an activation may fall the other way
+        assert float((outs[0][1] - outs[1][1]).abs().amax() / scale) < (1e-5 if dtype == "f32" else BF16_REL)
+        eng.set_state(30, 1)
+        for i in range(min(n, 5)):                    # token by token
+            eng.assemble_causal(binding.OURO_TARGET, tokens[i: i + 1])
+            _, lg = eng.verify_forward(want_logits=True)
+            assert torch.equal(lg[0], outs[0][1][i])
+            eng.advance(binding.OURO_TARGET, 1)
+    eng.close()
