@@ -1,7 +1,6 @@
 // Folding the per-span pieces of the split attention into the block's attention output.
 //
-// Both tensor-core attention kernels cut a row's keys into aligned spans of SPAN_KEYS and leave, per (row, head, span),
-// the span's score maximum (log2 domain), its sum of exponentials and its unnormalised output.  A (row, head) pair is
+// Both tensor-core attention kernels cut a row's keys into spans and leave, per (row, head, span), the span's score maximum (log2 domain), its sum of exponentials and its unnormalised output.  A (row, head) pair is
 // folded by one warp: first the largest span maximum, then one weighted sum over the spans in ascending order.  The
 // arithmetic involves the pair's own spans only, so it does not matter which kernel, CTA or warp runs it; it runs in
 // the kernel that consumes the attention output (the output projection), spread over all its CTAs.
@@ -12,7 +11,25 @@
 
 namespace fold {
 
-constexpr int SPAN_KEYS = 512;
+// The spans, by absolute position.  Head dim 64 (mma.sync kernel): the first 1024 keys in spans of one chunk of 128, since a
+// CTA walks its chunks one after the other (2 to 2.5 us each) and a short context would keep a few CTAs busy; the others in
+// spans of four, so that a long context leaves few pieces to fold (1.1B draft, 389 keys: 3981 -> 3573 us, with a window
+// over 521 keys 6971 -> 6347 us).  Head dim 128 (tcgen05 kernel): spans of four throughout - what a short span saves there
+// (three passes of 1.75 us of one CTA) the set-up of the additional CTAs and the fold cost again (7B step 3526 us, with
+// short spans 3549; prefill 12.4 ms and 13.3).
+constexpr int CHUNK = 128, LONG_CHUNKS = 4, LONG_KEYS = LONG_CHUNKS * CHUNK;
+constexpr int MAX_SPANS = 64;            // two per lane of the folding warp
+constexpr int MAX_KEYS = 32 * LONG_KEYS;
+__host__ __device__ constexpr int short_spans(int head_dim) { return head_dim == 64 ? 8 : 0; }
+__host__ __device__ constexpr int span_count(int head_dim, int keys) {     // spans that hold the keys [0, keys)
+  return keys <= short_spans(head_dim) * CHUNK ? (keys + CHUNK - 1) / CHUNK
+                                               : short_spans(head_dim) + (keys - short_spans(head_dim) * CHUNK + LONG_KEYS - 1) / LONG_KEYS;
+}
+__host__ __device__ constexpr int span_chunks(int head_dim, int s) { return s < short_spans(head_dim) ? 1 : LONG_CHUNKS; }
+__host__ __device__ constexpr int span_start(int head_dim, int s) {
+  return s < short_spans(head_dim) ? s * CHUNK : short_spans(head_dim) * CHUNK + (s - short_spans(head_dim)) * LONG_KEYS;
+}
+static_assert(span_count(64, MAX_KEYS) <= MAX_SPANS, "spans of the longest context");
 
 struct Params {
   const float *part;               // [rows][H][cap][PIECE]; NULL: nothing to fold
@@ -37,8 +54,8 @@ __device__ __forceinline__ void store_bf16(__nv_bfloat16 *dst, const float2 &a, 
   *reinterpret_cast<__nv_bfloat162 *>(dst) = __floats2bfloat162_rn(a.x * s, a.y * s);
 }
 
-// Pairs first, first + step, .. (pair = row * H + head).  Lane c fetches span c's maximum and sum (cap <= 32) while every
-// lane fetches its dims of up to UNR spans: one round trip to L2 up to 16 spans (8192 keys), two beyond.
+// Pairs first, first + step, .. (pair = row * H + head).  Lane c fetches the maxima and sums of spans c and c + 32 while
+// every lane fetches its dims of up to UNR spans: one round trip to L2 up to 16 spans, then one more per 16.
 template <int HD>
 __device__ __forceinline__ void pairs(const Params &p, int rows, int first, int step, int lane) {
   typedef typename Dims<HD>::V V;
@@ -46,11 +63,12 @@ __device__ __forceinline__ void pairs(const Params &p, int rows, int first, int 
   const int n_pairs = rows * p.H;
 #pragma unroll 1
   for (int q = first; q < n_pairs; q += step) {
-    const int r = q / p.H, ns = (p.lin_end[r] + p.seg_len[r] + SPAN_KEYS - 1) / SPAN_KEYS;
+    const int r = q / p.H, ns = span_count(HD, p.lin_end[r] + p.seg_len[r]);
     const float *src = p.part + (size_t)q * p.cap * PW;
-    float2 ml = make_float2(-INFINITY, 0.f);
-    if (lane < ns) ml = __ldcg(reinterpret_cast<const float2 *>(src + (size_t)lane * PW));
-    float mx = -INFINITY, w_l = 0.f, l = 0.f;
+    float2 ml = make_float2(-INFINITY, 0.f), ml2 = ml;
+    if (lane < ns) ml = __ldcg(reinterpret_cast<const float2 *>(src + lane * PW));
+    if (lane + 32 < ns) ml2 = __ldcg(reinterpret_cast<const float2 *>(src + (lane + 32) * PW));
+    float l = 0.f;
     V acc{};
 #pragma unroll 1
     for (int c0 = 0; c0 < ns; c0 += UNR) {
@@ -61,15 +79,18 @@ __device__ __forceinline__ void pairs(const Params &p, int rows, int first, int 
         if (c0 + cc < ns) o[cc] = __ldcg(reinterpret_cast<const V *>(src + (size_t)(c0 + cc) * PW + 4 + DPL * lane));
       }
       if (c0 == 0) {
-        mx = ml.x;
+        float mx = fmaxf(ml.x, ml2.x);
 #pragma unroll
         for (int s = 16; s; s >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
-        w_l = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - mx);          // mx is finite: the first span holds a visible key
+        ml.x = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - mx);         // the spans' weights; mx is finite: the first span holds a
+        ml2.x = (ml2.x == -INFINITY) ? 0.f : exp2f(ml2.x - mx);      // visible key
+      } else if (c0 == 32) {
+        ml = ml2;
       }
 #pragma unroll
       for (int cc = 0; cc < UNR; ++cc) {
         if (c0 + cc >= ns) break;                                    // uniform in the warp
-        const float w = __shfl_sync(0xffffffffu, w_l, c0 + cc);
+        const float w = __shfl_sync(0xffffffffu, ml.x, c0 + cc);     // (lane: modulo 32)
         l += __shfl_sync(0xffffffffu, ml.y, c0 + cc) * w;
         add_scaled(acc, o[cc], w);
       }

@@ -5,7 +5,7 @@
 // described by the number of keys it sees and by where its last keys live (its own candidate's cache slots),
 // and the kernel maps "virtual positions" 0..n_vis-1 to cache slots on the fly.
 //
-// Work split.  Keys are cut by virtual position into aligned spans of 512; one CTA handles one (kv head, span)
+// Work split.  Keys are cut by virtual position into spans of one or four chunks (attn_fold.cuh); one CTA handles one (kv head, span)
 // for up to 64 query rows (rows x query heads of the group; further rows go to further CTAs, which find the same
 // keys in L2), so every cached byte is read from HBM once.  The CTA
 // walks its span in chunks of 128 keys: K and V rows of the next chunk stream into a second shared-memory
@@ -43,8 +43,7 @@ extern "C" int ouro_trace_read_attn_tc(unsigned long long *out_host) {
 namespace {
 
 constexpr int CH = 128;            // keys per chunk
-constexpr int SC = 4;              // chunks per span
-constexpr int SPAN = CH * SC;
+static_assert(CH == fold::CHUNK, "the fold's spans");
 constexpr int WARPS = 8;
 constexpr int KW = CH / WARPS;     // keys per warp in the S phase (two 8-key MMA tiles)
 constexpr int THREADS = WARPS * 32;
@@ -167,8 +166,8 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
   }
   __syncthreads();
   for (int r = 0; r < rows; ++r) nv_max = max(nv_max, s_nvis[r]);
-  const int span0 = sc * SPAN;
-  const int n_chunks = min(SC, (nv_max - span0 + CH - 1) / CH);       // chunks of this span anybody sees
+  const int span0 = fold::span_start(HD, sc);
+  const int n_chunks = min(fold::span_chunks(HD, sc), (nv_max - span0 + CH - 1) / CH);       // chunks of this span anybody sees
 
   // Stages the part of chunk ci every row shares (virtual positions below the cache length) and zeroes the rest.
   auto stage_common = [&](int ci, int buf) {
@@ -436,12 +435,12 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
 }  // namespace
 
 bool attention_tc_supported(const ouro_model_desc &d) {
-  return d.dtype == OURO_BF16 && (d.head_dim == 64 || d.head_dim == 128) && d.max_seq <= 32 * SPAN;   // the fold looks at one span per lane
+  return d.dtype == OURO_BF16 && (d.head_dim == 64 || d.head_dim == 128) && d.max_seq <= fold::MAX_KEYS;   // the fold looks at two spans per lane
 }
 
 size_t attention_tc_scratch_bytes(const ouro_model_desc &d) {
   if (!attention_tc_supported(d)) return 0;
-  size_t cap = (d.max_seq + SPAN - 1) / SPAN;
+  size_t cap = fold::span_count(d.head_dim, d.max_seq);
   return (size_t)OURO_TEXT_ROWS * d.n_heads * cap * (d.head_dim + 4) * sizeof(float);
 }
 
@@ -465,7 +464,7 @@ bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_
   p.v = (const __nv_bfloat16 *)v_cache + off;
   p.lin_end = b.lin_end; p.seg_start = b.seg_start; p.seg_len = b.seg_len; p.group = b.group;
   p.rows = rows; p.H = d.n_heads; p.Hkv = d.n_kv_heads; p.L = L;
-  p.cap = (d.max_seq + SPAN - 1) / SPAN;
+  p.cap = fold::span_count(d.head_dim, d.max_seq);
   p.scale_log2 = 1.4426950408889634f / sqrtf((float)d.head_dim);
   p.part = part;
   p.out = (__nv_bfloat16 *)out;
@@ -475,7 +474,7 @@ bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_
   // rounds of a short block run side by side: 16 rows each while all CTAs are resident at once.  (1.1B draft, 19 rows x 8
   // heads over 540 keys: 27.0 us on 24 CTAs of 64 rows, 11.3 us on 80 CTAs of 16.)  Beyond that, larger rounds read the
   // keys less often.
-  const int n_spans = (n_vis_max + SPAN - 1) / SPAN;
+  const int n_spans = fold::span_count(d.head_dim, n_vis_max);
   const int mt = parts * n_spans * d.n_kv_heads * ((m_all + 15) / 16) <= SHORT_ROUNDS ? 1 : 4, qr = 16 * mt;
   p.rounds = (m_all + qr - 1) / qr;
   dim3 grid(n_spans, d.n_kv_heads, parts * p.rounds);

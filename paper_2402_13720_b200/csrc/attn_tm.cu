@@ -4,7 +4,7 @@
 // forward under a mask in which a phrase suffix sees the prefix, the draft and itself (Eq. 8); a row is described
 // by the number of keys it sees and by where its last keys live, and keys are addressed by "virtual position".
 //
-// Work split.  Keys are cut by virtual position into aligned spans of 512; one CTA handles one (span, kv head)
+// Work split.  Keys are cut by virtual position into spans of four chunks (attn_fold.cuh); one CTA handles one (span, kv head)
 // for a round of up to 128 query rows (block rows x query heads of the group, ordered group by group).  It walks
 // the span in chunks of 128 keys.  Per chunk:
 //     S = Q K^T      one 128 x 128 x 128 tcgen05 contraction into TMEM (Q and K K-major in 128-byte swizzle),
@@ -54,9 +54,7 @@ namespace {
 
 constexpr int HD = 128;
 constexpr int CH = 128;            // keys per chunk
-constexpr int SC = 4;              // chunks per span
-constexpr int SPAN = CH * SC;
-static_assert(SPAN == fold::SPAN_KEYS, "the fold's spans");
+static_assert(CH == fold::CHUNK, "the fold's spans");
 constexpr int QR = 128;            // query rows per round = TMEM lanes
 constexpr int PW = fold::PIECE<HD>;
 constexpr int ROW_THREADS = 256;  // two threads per query row
@@ -70,7 +68,7 @@ constexpr int OFF_K = OFF_Q + TILE;          // two stages
 constexpr int OFF_V = OFF_K + 2 * TILE;      // two stages
 constexpr int OFF_P = OFF_V + 2 * TILE;      // two buffers
 constexpr int OFF_MISC = OFF_P + 2 * TILE;
-constexpr int MAX_ITEMS = SC * 33;
+constexpr int MAX_ITEMS = fold::LONG_CHUNKS * 33;
 constexpr int MAX_GROUPS = 32;
 
 struct Misc {
@@ -222,7 +220,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
   const int zb = blockIdx.z * OURO_MAX_ROWS, L = p.L + zb;
   const int rows = min(OURO_MAX_ROWS, (p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows) - zb);   // written before the forward pass began
   const int32_t *group = p.group + zb, *lin_end = p.lin_end + zb, *seg_start = p.seg_start + zb, *seg_len = p.seg_len + zb;
-  const int g = p.H / p.Hkv, dkv = p.Hkv * HD, M_all = g * rows, span0 = sc * SPAN;
+  const int g = p.H / p.Hkv, dkv = p.Hkv * HD, M_all = g * rows, span0 = fold::span_start(HD, sc);
 
   if (tid == 0) TRACE(0);
   if (tid == 32) {
@@ -316,7 +314,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
     int rmax = 0, n = 0;
     for (int o = 0; o < ng; ++o) rmax = max(rmax, ms->gmax[o]);
     if (rmax > span0) {
-      const int nch = min(SC, (rmax - span0 + CH - 1) / CH);
+      const int nch = min(fold::span_chunks(HD, sc), (rmax - span0 + CH - 1) / CH);
       for (int ci = 0; ci < nch; ++ci) {
         const int c0 = span0 + ci * CH;
         if (c0 + CH <= L) {
@@ -676,7 +674,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
 
 bool attention_tm_supported(const ouro_model_desc &d) {
   return d.dtype == OURO_BF16 && d.head_dim == HD && d.n_heads % d.n_kv_heads == 0 && d.n_heads / d.n_kv_heads <= 255 &&
-         d.max_seq <= 32 * SPAN;              // the fold looks at one span per lane
+         d.max_seq <= fold::MAX_KEYS;         // the fold looks at two spans per lane
 }
 
 int attention_tm_setup() {
@@ -705,16 +703,16 @@ bool launch_attention_tm(const ouro_model_desc &d, const void *q, const void *km
   p.v = (const __nv_bfloat16 *)v_cache + off;
   p.lin_end = b.lin_end; p.seg_start = b.seg_start; p.seg_len = b.seg_len; p.group = b.group;
   p.rows = rows; p.H = d.n_heads; p.Hkv = d.n_kv_heads; p.L = L;
-  p.cap = (d.max_seq + SPAN - 1) / SPAN;
+  p.cap = fold::span_count(HD, d.max_seq);
   p.row0 = layer * d.max_seq;
   p.scale_log2 = 1.4426950408889634f / sqrtf((float)d.head_dim);
   p.part = part;
   p.out = (__nv_bfloat16 *)out;
-  p.direct = n_vis_max <= SPAN;
+  p.direct = fold::span_count(HD, n_vis_max) <= 1;
   p.status = status;
   p.rows_dev = rows_dev;
   const int m_all = (d.n_heads / d.n_kv_heads) * std::min<int>(rows, OURO_MAX_ROWS);
-  p.n_spans = (n_vis_max + SPAN - 1) / SPAN;
+  p.n_spans = fold::span_count(HD, n_vis_max);
   dim3 grid(p.n_spans * d.n_kv_heads, (m_all + QR - 1) / QR, (rows + OURO_MAX_ROWS - 1) / OURO_MAX_ROWS);
   launch_pdl(attn_tm_kernel, grid, THREADS, SMEM_BYTES, s, p);
   return !p.direct;

@@ -1243,7 +1243,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
       f.rows_dev = c->cur_rows_dev;
       f.rows = rows;
       f.H = d.n_heads;
-      f.cap = (d.max_seq + fold::SPAN_KEYS - 1) / fold::SPAN_KEYS;
+      f.cap = fold::span_count(d.head_dim, d.max_seq);
       f.head_dim = d.head_dim;
     }
   }

@@ -1011,3 +1011,39 @@ def test_one_launch_forward_matches_oracle_and_single_kernels(dtype, d, heads, k
             assert torch.equal(lg[0], outs[0][1][i])
             eng.advance(binding.OURO_TARGET, 1)
     eng.close()
+
+
+# ------------------------------------------------------------ spans of the attention
+
+@pytest.mark.parametrize("heads,kv,hd", [(2, 1, 128), (4, 2, 64)])
+@pytest.mark.parametrize("L", [120, 127, 1018, 1023, 1024, 5114, 13306])
+def test_attention_spans_match_oracle(heads, kv, hd, L):
+    """Blocks that straddle the end of a chunk (128), of the short spans (1024), of the first batch of the fold (16 spans:
+    5120 keys) and of a lane's first span (32 spans: 13312): logits against the oracle, and a suffix row's logits equal
+    those of the same token decoded alone, bit for bit."""
+    desc = synth.ModelDesc(1, 256, heads, kv, hd, 256, 520, 13400, "bf16")
+    P = synth.DecodeParams(3, 6, 2, 4, 8, seed_prompt=False)
+    eng, W = make(desc, P, 10)
+    k, v = synth.kv_fill(desc, 3, L, device="cuda:0")
+    eng.tm.k_cache.copy_(k); eng.tm.v_cache.copy_(v)
+    cache = tf.KVCache(desc, k.double().cpu().numpy(), v.double().cpu().numpy(), L)
+    rng = np.random.default_rng(L)
+    d = rng.integers(0, desc.vocab, 3).tolist()
+    eng.phrase_update(np.concatenate([np.full((2, 1), d[-1]), rng.integers(0, desc.vocab, (2, 5))], axis=1))
+    eng.set_state(L, 17)
+    eng.assemble_candidates(draft=d)
+    tok = eng.block_get()[0].tolist()
+    assert len(tok) == 14
+    _, logits = eng.verify_forward(want_logits=True)
+    got = logits[:14].clone()
+    tokens, pos, _, vis = ob.build_block(L, 17, d, [tok[4:9], tok[9:14]])
+    assert tok == tokens
+    _bf16_tol(got.cpu().numpy().astype(np.float64), tf.forward(W, cache, tokens, pos, vis))
+    for rows in ([0, 1, 2, 3, 4, 5, 6, 7, 8], [0, 1, 2, 3, 9, 10, 11, 12, 13]):
+        eng.set_state(L, 17)
+        for r in rows:
+            eng.assemble_causal(binding.OURO_TARGET, [tok[r]])
+            _, lg = eng.verify_forward(want_logits=True)
+            assert torch.equal(lg[0], got[r]), r
+            eng.advance(binding.OURO_TARGET, 1)
+    eng.close()
