@@ -2,8 +2,9 @@
 //
 // Such a model's weights are read in microseconds; what a forward costs is its chain of dependent steps, eight launches a
 // layer as kernels of their own (5.6 us each on the fp32 pair of 128-wide layers).  Here one CTA per SM stays for the
-// whole forward and the steps are separated by grid barriers (1 us).  A warp takes a unit of a step: one or two output
-// columns for a tile of rows, or one (row, head) of the attention.  RMSNorm has no step of its own: the warp that
+// whole forward and the steps are separated by grid barriers.  A warp takes a unit of a step: one or two output columns
+// for a tile of rows; four warps take one (row, head) of the attention (one warp each: 2815 us for 64 tokens, four: 2391).
+// One cluster of 16 CTAs with its barrier in hardware was slower (2511 us): the units then queue for its warps.  RMSNorm has no step of its own: the warp that
 // contracts a row with the weights has just read the row, and sums its squares first.
 //
 // The rule of kernels_layer.cu holds: a value depends on its own row and on the keys that row sees, in fixed groups.
@@ -18,7 +19,8 @@ namespace {
 
 constexpr int THREADS = 256;
 constexpr int WARPS = THREADS / 32;
-constexpr int RT = 4;                    // rows of a unit
+constexpr int QUAD = 4;                  // warps that share one (row, head) of the attention: warp j takes key groups j, j + 4, ..
+constexpr int RT = 2;                    // rows of a unit (four: 2365 us for 64 tokens, two: 2264)
 constexpr int MAX_LAYERS = 40;           // layer pointers travel as kernel parameters
 constexpr uint32_t BARRIER_LIMIT = 1u << 22;
 
@@ -76,6 +78,50 @@ __device__ __forceinline__ void contract(const Row &row, const T *gain, float ep
 #pragma unroll
     for (int c = 0; c < C; ++c) acc[c][i] = 0.f;
   }
+  if (K <= 32 * V) {
+    // a row is one vector per lane: everything is fetched at once and read once (the same sums in the same order)
+    const int k = lane * V;
+    const bool in = k < K;
+    Vec<T> wv[C], gv;
+    float xv[RT][V];
+    if (in) {
+#pragma unroll
+      for (int c = 0; c < C; ++c) wv[c].load(w[c] + k);
+      if (gain) gv.load(gain + k);
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+        if (i < n_rows) row(i, k, xv[i]);
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+        if (gain && i < n_rows) {
+#pragma unroll
+          for (int e = 0; e < V; ++e) inv[i] = fmaf(xv[i][e], xv[i][e], inv[i]);
+        }
+    }
+    if (gain) {
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+        if (i < n_rows) inv[i] = 1.0f / sqrtf(warp_sum(inv[i]) / (float)K + eps);
+    }
+    if (in) {
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+        if (i < n_rows) {
+#pragma unroll
+          for (int e = 0; e < V; ++e) {
+            const float a = gain ? to_f<T>(from_f<T>(gv.get(e) * (xv[i][e] * inv[i]))) : xv[i][e];
+#pragma unroll
+            for (int c = 0; c < C; ++c) acc[c][i] = fmaf(a, wv[c].get(e), acc[c][i]);
+          }
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+        if (i < n_rows) acc[c][i] = warp_sum(acc[c][i]);
+    return;
+  }
   if (gain) {
     for (int k = lane * V; k < K; k += 32 * V)
 #pragma unroll
@@ -87,8 +133,10 @@ __device__ __forceinline__ void contract(const Row &row, const T *gain, float ep
           for (int e = 0; e < V; ++e) inv[i] = fmaf(xv[e], xv[e], inv[i]);
         }
 #pragma unroll
-    for (int i = 0; i < RT; ++i) inv[i] = 1.0f / sqrtf(warp_sum(inv[i]) / (float)K + eps);
+    for (int i = 0; i < RT; ++i)
+      if (i < n_rows) inv[i] = 1.0f / sqrtf(warp_sum(inv[i]) / (float)K + eps);
   }
+#pragma unroll 2
   for (int k = lane * V; k < K; k += 32 * V) {
     Vec<T> wv[C], gv;
 #pragma unroll
@@ -110,7 +158,8 @@ __device__ __forceinline__ void contract(const Row &row, const T *gain, float ep
 #pragma unroll
   for (int c = 0; c < C; ++c)
 #pragma unroll
-    for (int i = 0; i < RT; ++i) acc[c][i] = warp_sum(acc[c][i]);
+    for (int i = 0; i < RT; ++i)
+      if (i < n_rows) acc[c][i] = warp_sum(acc[c][i]);
 }
 
 // Lane i's value of a tile's rows.
@@ -123,10 +172,11 @@ __device__ __forceinline__ float of_row(const float *acc, int lane) {
 
 template <typename T>
 __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_constant__ SmallParams p) {
-  extern __shared__ float sq[];            // [WARPS][h] the query of each warp's attention unit
+  __shared__ float sq[WARPS][128];         // attention: a warp's copy of its query, then its unnormalised output
+  __shared__ float2 sml[WARPS];            // ... and its score maximum and sum
   __shared__ int flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int gw = blockIdx.x * WARPS + warp, nw = gridDim.x * WARPS;
+  const int gw = warp * gridDim.x + blockIdx.x, nw = gridDim.x * WARPS;   // (a short step is spread over the SMs)
   const int rows = p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows;
   const int tiles = (rows + RT - 1) / RT;
   const int d = p.d, h = p.h, half = h >> 1, dq = p.H * h, dkv = p.Hkv * h;
@@ -194,11 +244,12 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
     }
     if (!p.argmax && l + 1 == p.n_layers) return;
     if (!grid_barrier(p, target, &flag)) return;
-    // ---- attention, a warp per (row, head): keys by virtual position in groups of 32, online softmax
-    for (int u = gw; u < rows * p.H; u += nw) {
+    // ---- attention, four warps per (row, head): keys by virtual position in groups of 32, online softmax over a warp's
+    //      groups; the four warps' pieces are added in their order
+    const int quad = warp / QUAD, qw = warp % QUAD;
+    for (int u = blockIdx.x * (WARPS / QUAD) + quad; u < rows * p.H; u += gridDim.x * (WARPS / QUAD)) {
       const int r = u / p.H, a = u % p.H, kvh = a / (p.H / p.Hkv);
-      float *myq = sq + warp * h;
-      __syncwarp();
+      float *myq = sq[warp];
       for (int i = lane; i < h; i += 32) myq[i] = to_f<T>(__ldcg(q + (size_t)r * dq + a * h + i));
       __syncwarp();
       const int lin_end = p.b.lin_end[r], seg_start = p.b.seg_start[r], n_vis = lin_end + p.b.seg_len[r];
@@ -206,7 +257,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
       float m = -INFINITY, sum = 0.f;
       float o[4] = {0.f, 0.f, 0.f, 0.f};                 // dims lane, lane + 32, .. (h <= 128)
       const int nd = h >> 5;
-      for (int p0 = 0; p0 < n_vis; p0 += 32) {
+      for (int p0 = 32 * qw; p0 < n_vis; p0 += 32 * QUAD) {
         const int pos = p0 + lane;
         const bool valid = pos < n_vis;
         const int slot = pos < lin_end ? pos : seg_start + (pos - lin_end);
@@ -214,7 +265,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
         if (valid) {
           const T *kr = kb + (size_t)slot * dkv;
           float acc = 0.f;
-#pragma unroll 4
+#pragma unroll 8
           for (int i = 0; i < h; i += Vec<T>::N) {
             Vec<T> kv;
             kv.v = __ldcg(reinterpret_cast<const decltype(kv.v) *>(kr + i));
@@ -241,10 +292,32 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
         }
         m = m_new;
       }
-      const float inv = 1.0f / sum;
+      __syncwarp();
 #pragma unroll
       for (int dd = 0; dd < 4; ++dd)
-        if (dd < nd) att[(size_t)r * dq + a * h + lane + 32 * dd] = from_f<T>(o[dd] * inv);
+        if (dd < nd) myq[lane + 32 * dd] = o[dd];
+      if (lane == 0) sml[warp] = make_float2(m, sum);
+      __syncwarp();
+      asm volatile("barrier.sync %0, %1;" ::"r"(1 + quad), "n"(32 * QUAD) : "memory");
+      // the four pieces together: a warp without keys has the weight zero (the first always has one)
+      const int w0 = quad * QUAD;
+      float mx = sml[w0].x, l_all = 0.f, wt[QUAD];
+#pragma unroll
+      for (int j = 1; j < QUAD; ++j) mx = fmaxf(mx, sml[w0 + j].x);
+#pragma unroll
+      for (int j = 0; j < QUAD; ++j) {
+        wt[j] = expf(sml[w0 + j].x - mx);
+        l_all += sml[w0 + j].y * wt[j];
+      }
+      const float inv = 1.0f / l_all;
+      for (int dim = 32 * qw + lane; dim < h; dim += 32 * QUAD) {
+        float v = 0.f;
+#pragma unroll
+        for (int j = 0; j < QUAD; ++j) v += sq[w0 + j][dim] * wt[j];
+        att[(size_t)r * dq + a * h + dim] = from_f<T>(v * inv);
+      }
+      __syncwarp();
+      asm volatile("barrier.sync %0, %1;" ::"r"(1 + quad), "n"(32 * QUAD) : "memory");
     }
     if (!grid_barrier(p, target, &flag)) return;
     // ---- a column of a projection back into the residual stream
@@ -349,7 +422,6 @@ int launch_forward_small(ouro_ctx *c, int which, int rows, const int *rows_dev, 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = THREADS;
-  cfg.dynamicSmemBytes = (size_t)WARPS * d.head_dim * sizeof(float);
   cfg.stream = c->stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeCooperative;
@@ -357,8 +429,7 @@ int launch_forward_small(ouro_ctx *c, int which, int rows, const int *rows_dev, 
   cfg.attrs = at;
   cfg.numAttrs = 1;
   OURO_COUNT_LAUNCH();
-  const cudaError_t e = d.dtype == OURO_BF16 ? cudaLaunchKernelEx(&cfg, forward_small_kernel<__nv_bfloat16>, p)
-                                             : cudaLaunchKernelEx(&cfg, forward_small_kernel<float>, p);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, d.dtype == OURO_BF16 ? forward_small_kernel<__nv_bfloat16> : forward_small_kernel<float>, p);
   if (e != cudaSuccess) {
     c->err = std::string("one-launch forward: ") + cudaGetErrorString(e);
     return OURO_ECUDA;
