@@ -801,15 +801,24 @@ static int draft_step(ouro_ctx *c, int32_t *out_dev, int *calls) {
   int last = 0;
   TRY(feed_text(c, OURO_DRAFT, (int)c->seq.size(), &last));
   *calls += 1;
-  if (!ext) launch_pick_token(c->a.argmax, last, out_dev, c->stream);
   for (int i = 1; i < gamma; ++i) {
-    TRY(ouro_assemble_causal(c, OURO_DRAFT, out_dev + i - 1, 1));
+    if (ext) {
+      TRY(ouro_assemble_causal(c, OURO_DRAFT, out_dev + i - 1, 1));
+    } else {                                       // draft token i becomes the next block in the launch that picks it
+      if (D.L + 1 > D.d.max_seq) return fail(c, OURO_ECAPACITY, "cache length + block rows exceeds max_seq");
+      launch_pick_assemble(D.blk, c->a.argmax, last, out_dev + i - 1, D.L, c->stream);
+      last = 0;
+      D.blk_rows = 1;
+      D.blk_rows_dev = false;
+      D.blk_L = D.L;
+      D.blk_is_candidate = false;
+    }
     TRY(forward(c, OURO_DRAFT, c->a.argmax, nullptr));
     D.L += 1;
     D.blk_rows = 0;
     *calls += 1;
-    if (!ext) launch_pick_token(c->a.argmax, 0, out_dev + i, c->stream);
   }
+  if (!ext) launch_pick_token(c->a.argmax, last, out_dev + gamma - 1, c->stream);
   CKL();
   return OURO_OK;
 }

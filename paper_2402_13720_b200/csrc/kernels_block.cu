@@ -644,10 +644,34 @@ void launch_vanilla_accept(DevState *st, const int32_t *o, int32_t *seq_dev, cud
   vanilla_accept_kernel<<<1, 1, 0, s>>>(st, o, seq_dev);
 }
 
-__global__ void pick_token_kernel(const int32_t *src, int index, int32_t *dst) { *dst = src[index]; }
+__global__ void pick_token_kernel(const int32_t *src, int index, int32_t *dst) {
+  pdl_wait();
+  *dst = src[index];
+}
 void launch_pick_token(const int32_t *src, int index, int32_t *dst, cudaStream_t s) {
   OURO_COUNT_LAUNCH();
-  pick_token_kernel<<<1, 1, 0, s>>>(src, index, dst);
+  launch_pdl(pick_token_kernel, 1, 1, 0, s, src, index, dst);
+}
+
+// A drafted token joins the draft and is the whole of the next block: one launch instead of two, in place while the
+// forward before drains.  The kernels after it start when it has finished (it does not trigger them), as they expect of
+// an assembling kernel.
+__global__ void pick_assemble_kernel(BlockDev b, const int32_t *src, int index, int32_t *dst, int L) {
+  pdl_wait();
+  const int32_t token = src[index];
+  *dst = token;
+  b.tok[0] = token;
+  b.pos[0] = L;
+  b.group[0] = 0;
+  b.lin_end[0] = L + 1;
+  b.seg_start[0] = 0;
+  b.seg_len[0] = 0;
+  b.mask[0] = 1;
+  b.mask[1] = 0;
+}
+void launch_pick_assemble(const BlockDev &b, const int32_t *src, int index, int32_t *dst, int L, cudaStream_t s) {
+  OURO_COUNT_LAUNCH();
+  launch_pdl(pick_assemble_kernel, 1, 1, 0, s, b, src, index, dst, L);
 }
 
 // Text of n_seq tokens ending in the pending token; with fill, the earlier positions are recorded as 0.

@@ -181,6 +181,7 @@ void launch_draft_window_harvest(const BlockDev &b, DevState *st, const PoolDev 
                                  int n, int W, int32_t *win, cudaStream_t s);
 void launch_argmax(const float *logits, int rows, int vocab, int32_t *out, cudaStream_t s);
 void launch_pick_token(const int32_t *src, int index, int32_t *dst, cudaStream_t s);
+void launch_pick_assemble(const BlockDev &b, const int32_t *src, int index, int32_t *dst, int L, cudaStream_t s);
 void launch_set_state(DevState *st, int32_t *seq_dev, int n_seq, int pending, int fill, cudaStream_t s);
 
 // ---- kernel launchers (kernels_layer.cu) ---------------------------------------------------------
