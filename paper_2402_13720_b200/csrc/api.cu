@@ -179,8 +179,8 @@ static bool mem_ok(const ouro_model_mem *m) {
 }
 
 int ouro_fast_setup(ouro_ctx *c);  // tensor maps etc. of the tensor-core paths (gemm_tc.cu)
-void ouro_fast_reset(ouro_ctx *c, bool force);   // clears split-K / chain counters (always, or only after a device-side give-up)
-void ouro_fast_mark_dirty(ouro_ctx *c);
+void ouro_fast_reset(ouro_ctx *c);               // forgets a chain of GEMMs under construction
+Leftovers ouro_fast_leftovers(ouro_ctx *c);
 bool ouro_fast_available(ouro_ctx *c, int which);   // model `which` runs on the tensor-core kernels
 bool ouro_fast_layers(ouro_ctx *c, int which);      // its GEMMs do
 
@@ -247,7 +247,7 @@ extern "C" int ouro_create(const ouro_model_desc *t, const ouro_model_mem *tm, c
       (e = cudaMemsetAsync(n->arrived_dev, 0, sizeof(int), n->stream)) != cudaSuccess)
     return bail(OURO_ECUDA, std::string("device set-up: ") + cudaGetErrorString(e));
   launch_pool_clear(n->pool, n->st, n->stream);
-  launch_set_state(n->st, n->seq_dev, 1, 0, 1, n->stream);
+  launch_set_state(n->st, n->seq_dev, 1, 0, 1, Leftovers(), n->stream);
   int rc = ouro_fast_setup(n);
   if (rc != OURO_OK) return bail(rc, n->err);
   if ((e = cudaStreamSynchronize(n->stream)) != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess)
@@ -282,10 +282,10 @@ extern "C" int ouro_reset(ouro_ctx *c, int keep_pool) {
   forget_blocks(c);
   c->seq.assign(1, 0);
   c->step = 0;
-  ouro_fast_reset(c, true);
+  ouro_fast_reset(c);
   CK(cudaMemsetAsync(c->arrived_dev, 0, sizeof(int), c->stream));      // a barrier that gave up leaves the count short
   c->arrived_host = 0;
-  launch_set_state(c->st, c->seq_dev, 1, 0, 1, c->stream);
+  launch_set_state(c->st, c->seq_dev, 1, 0, 1, ouro_fast_leftovers(c), c->stream);
   if (!keep_pool) launch_pool_clear(c->pool, c->st, c->stream);
   CKL();
   return OURO_OK;
@@ -301,8 +301,8 @@ extern "C" int ouro_set_state(ouro_ctx *c, int32_t cache_len, int32_t pending) {
   c->seq.assign((size_t)cache_len + 1, 0);
   c->seq.back() = pending;
   c->step = 0;
-  ouro_fast_reset(c, false);
-  launch_set_state(c->st, c->seq_dev, cache_len + 1, pending, 1, c->stream);
+  ouro_fast_reset(c);
+  launch_set_state(c->st, c->seq_dev, cache_len + 1, pending, 1, ouro_fast_leftovers(c), c->stream);
   CKL();
   return OURO_OK;
 }
@@ -578,7 +578,7 @@ extern "C" int ouro_prefill(ouro_ctx *c, const int32_t *prompt, int32_t n) {
     if (prompt[i] < 0 || prompt[i] >= T.d.vocab) return fail(c, OURO_EINVAL, "prompt token out of range");
   c->seq.assign(prompt, prompt + n);
   CK(cudaMemcpyAsync(c->seq_dev, c->seq.data(), (size_t)n * 4, cudaMemcpyHostToDevice, c->stream));
-  launch_set_state(c->st, c->seq_dev, n, prompt[n - 1], 0, c->stream);
+  launch_set_state(c->st, c->seq_dev, n, prompt[n - 1], 0, ouro_fast_leftovers(c), c->stream);
   if ((c->p.flags & OURO_SEED_PROMPT) && n >= c->p.beta)
     launch_pool_update(c->pool, c->st, c->seq_dev, n - c->p.beta + 1, c->p.beta, 1, c->stream);
   CKL();
@@ -675,10 +675,7 @@ static int accept_step(ouro_ctx *c, const int32_t *argmax_dev, AcceptOut *r) {
     CK(cudaStreamSynchronize(s));
     memcpy(r, c->pin, sizeof(AcceptOut));
   }
-  if (r->status != 0) {
-    ouro_fast_mark_dirty(c);
-    return fail(c, OURO_ETIMEOUT, "device status word " + std::to_string(r->status));
-  }
+  if (r->status != 0) return fail(c, OURO_ETIMEOUT, "device status word " + std::to_string(r->status));
   if (r->n_acc < 1 || r->n_acc > gamma + S + 1) return fail(c, OURO_ECUDA, "acceptance returned an impossible count");
   c->seq.insert(c->seq.end(), r->accepted, r->accepted + r->n_acc);
   T.L = L + r->n_acc;
@@ -913,10 +910,7 @@ extern "C" int ouro_generate_vanilla(ouro_ctx *c, const int32_t *prompt, int32_t
   CK(cudaMemcpyAsync(out, c->seq_dev + base, (size_t)n * 4, cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(c->pin, &c->st->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  if (c->pin[0] != 0) {
-    ouro_fast_mark_dirty(c);
-    return fail(c, OURO_ETIMEOUT, "device status word " + std::to_string(c->pin[0]));
-  }
+  if (c->pin[0] != 0) return fail(c, OURO_ETIMEOUT, "device status word " + std::to_string(c->pin[0]));
   CK(cudaEventElapsedTime(&st.ms_total, c->ev[0], c->ev[5]));
   st.ms_target = st.ms_total;
   c->seq.insert(c->seq.end(), out, out + n);

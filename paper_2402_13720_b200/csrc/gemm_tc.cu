@@ -888,7 +888,6 @@ struct FastState {
   int chain_kind[MAX_CHAIN] = {0, 0, 0, 0};
   bool fuse = true;             // run consecutive GEMMs as one launch
   long pf_ffn_rows = 0;         // rows of gate and of up the attention kernel prefetches into L2 besides the output projection (< 0: nothing)
-  bool dirty = false;           // a bounded wait gave up: counters must be cleared before the next launch
   uint32_t wait_limit = 1u << 22;   // polls of a partial-tile wait (ouro_debug_set_wait_limit)
 };
 constexpr int MAX_TILES = 4096;
@@ -1121,21 +1120,26 @@ static void push_gemm(ouro_ctx *c, Gemm &p, int kind, const CUtensorMap *xmaps, 
   if (last || split || cp.n == MAX_CHAIN) flush_chain(c);
 }
 
-// Clears what an aborted launch may have left behind (partial tiles nobody fetched, chain counters).
-void ouro_fast_reset(ouro_ctx *c, bool force) {
+// Forgets the chain under construction.
+void ouro_fast_reset(ouro_ctx *c) {
   if (!c->fast) return;
-  FastState &s = c->fast->s;
-  s.chain.args.n = 0;
-  s.chain.args.fold.part = nullptr;
-  s.chain.args.embed.table = nullptr;
-  if (!force && !s.dirty) return;
-  cudaMemsetAsync(s.slots, 0xff, slots_bytes(), c->stream);
-  cudaMemsetAsync(s.finished, 0, CHAIN_BYTES, c->stream);
-  for (int &v : s.finished_host) v = 0;
-  s.dirty = false;
+  ChainArgs &cp = c->fast->s.chain.args;
+  cp.n = 0;
+  cp.fold.part = nullptr;
+  cp.embed.table = nullptr;
 }
-void ouro_fast_mark_dirty(ouro_ctx *c) {
-  if (c->fast) c->fast->s.dirty = true;
+// What the launches so far leave behind if one of them has given up.
+Leftovers ouro_fast_leftovers(ouro_ctx *c) {
+  Leftovers l;
+  if (!c->fast) return l;
+  const FastState &s = c->fast->s;
+  l.slots = (uint4 *)s.slots;
+  l.n_slots = slots_bytes() / sizeof(uint4);
+  l.empty = EMPTY;
+  l.counters = s.finished;
+  l.n_counters = MAX_CHAIN + 1;
+  for (int i = 0; i <= MAX_CHAIN; ++i) l.value[i] = s.finished_host[i];
+  return l;
 }
 extern "C" int ouro_debug_set_wait_limit(ouro_ctx *c, int64_t polls) {
   if (!c) return OURO_EINVAL;

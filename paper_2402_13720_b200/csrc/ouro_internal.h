@@ -182,7 +182,16 @@ void launch_draft_window_harvest(const BlockDev &b, DevState *st, const PoolDev 
 void launch_argmax(const float *logits, int rows, int vocab, int32_t *out, cudaStream_t s);
 void launch_pick_token(const int32_t *src, int index, int32_t *dst, cudaStream_t s);
 void launch_pick_assemble(const BlockDev &b, const int32_t *src, int index, int32_t *dst, int L, cudaStream_t s);
-void launch_set_state(DevState *st, int32_t *seq_dev, int n_seq, int pending, int fill, cudaStream_t s);
+// What a launch whose bounded wait gave up leaves in device memory, and what has to stand there before the status word may be
+// cleared: partial sums nobody fetched (the words are empty again) and hand-over counters short of what the host expects.
+struct Leftovers {
+  uint4 *slots = nullptr;
+  size_t n_slots = 0;                  // 16-byte pieces
+  uint32_t empty = 0;
+  int *counters = nullptr;
+  int n_counters = 0, value[8] = {};
+};
+void launch_set_state(DevState *st, int32_t *seq_dev, int n_seq, int pending, int fill, const Leftovers &left, cudaStream_t s);
 
 // ---- kernel launchers (kernels_layer.cu) ---------------------------------------------------------
 struct GemmSegs {  // up to three weight matrices [n_i, K] stacked along the output dimension

@@ -852,6 +852,52 @@ def test_bounded_wait_gives_up_and_the_context_recovers():
     eng.close()
 
 
+@pytest.mark.parametrize("fuse", ["0", "1"])
+def test_give_up_that_nobody_read_ends_with_the_state(monkeypatch, fuse):
+    """Only acceptance and the whole loops read the status word.  A wait that runs out in a forward or while drafting leaves
+    sums nobody fetched in the partial-tile slots; set_state clears the status, so the slots must be empty again with it: the
+    step that follows gives the bits it gave before and no time-out.  One launch per GEMM (no hand-over counter in the way)
+    and chained launches; one row and a candidate block."""
+    monkeypatch.setenv("OURO_FUSE", fuse)
+    P = synth.DecodeParams(4, 9, 4, 16, 8, harvest_matched=False, harvest_candidates=False, harvest_accepted=False)
+    eng, _ = make(MIDB, P, 2, draft=MIDB)          # d 256: every q,k,v tile is split four ways
+    prompt = synth.prompt(2, MIDB.vocab, 40, 0.4, 4, 8)
+    eng.reset(); eng.prefill(prompt)
+    L, d = len(prompt) - 1, [1, 2, 3, int(prompt[5])]
+
+    def step():
+        eng.set_state(L, int(prompt[-1]))
+        eng.assemble_candidates(draft=d)
+        am, lg = eng.verify_forward(want_logits=True)
+        n = len(eng.block_get()[0])
+        return am[:n].clone(), lg[:n].clone(), eng.accept_and_compact()[3].tolist()
+
+    def one_row():
+        eng.assemble_causal(binding.OURO_TARGET, [5])
+        eng.verify_forward()
+
+    def candidates():
+        eng.assemble_candidates(draft=d)
+        eng.verify_forward()
+
+    want = step()
+    for give_up in (one_row, candidates, eng.draft):
+        eng.set_state(L, int(prompt[-1]))
+        eng.set_wait_limit(0)
+        give_up()
+        eng.set_wait_limit(-1)
+        got = step()
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1]) and got[2] == want[2], give_up
+    eng.set_wait_limit(0)
+    one_row()
+    eng.set_wait_limit(-1)
+    eng.reset()
+    eng.prefill(prompt)
+    got = step()
+    assert torch.equal(got[1], want[1])
+    eng.close()
+
+
 def test_tile_counter_generations_wrap_around(monkeypatch):
     """The split-K tile counters carry a generation number that grows with every GEMM; when the numbers are used up
     the words are cleared and counting starts over.  Started a few hundred GEMMs before that point, a generation
