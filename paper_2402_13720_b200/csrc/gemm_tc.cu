@@ -115,17 +115,17 @@ struct GemmParams {
 // gate/up -> down -> next layer's q,k,v or the LM head).  The weight producer runs straight on into the next GEMM's
 // tiles; the activations of GEMM i + 1 are fetched once GEMM i has finished all its tiles, which the CTAs learn from
 // a counter in global memory (one per chain position, counting finished tiles, never reset: the host passes the value
-// it will have reached).  All GEMMs of a chain have the same rows / t_pad / stages.
+// it will have reached, both modulo 2^32).  All GEMMs of a chain have the same rows / t_pad / stages.
 constexpr int MAX_CHAIN = 4;
 struct ChainArgs {
   GemmParams g[MAX_CHAIN];
   int n;
-  int *finished;            // [MAX_CHAIN + 1] tiles finished, per chain position (monotonic); last: CTAs done folding
-  int target[MAX_CHAIN];    // value finished[i] has when GEMM i of this launch is complete
+  uint32_t *finished;         // [MAX_CHAIN + 1] tiles finished, per chain position; last: CTAs done folding
+  uint32_t target[MAX_CHAIN]; // value finished[i] has when GEMM i of this launch is complete
   // The first GEMM's activations may be the attention output, still in per-span pieces: every CTA first folds a share
   // of the (row, head) pairs, and the first activation tile is fetched once all CTAs have.
   fold::Params fold;
-  int fold_target;                // value finished[MAX_CHAIN] has once every CTA has done its share of the work in front
+  uint32_t fold_target;           // value finished[MAX_CHAIN] has once every CTA has done its share of the work in front
   // ... or the embedding rows of the block's tokens (first layer): gathered by all CTAs the same way.
   struct Embed {
     const __nv_bfloat16 *table;   // [vocab][d]; NULL: nothing to gather
@@ -279,12 +279,13 @@ __device__ __forceinline__ void locate(const GemmParams &p, int tile, int &seg, 
   valid = min(TILE_N, p.a_rows[seg] - row0);
 }
 
-// Bounded wait until GEMM `i` of the chain has finished all its tiles (acquire).
-__device__ __forceinline__ bool counter_wait(const int *counter, int target, const int *status, uint32_t limit) {
+// Bounded wait until GEMM `i` of the chain has finished all its tiles (acquire).  The counters pass 2^31 after some hundred
+// thousand forwards, so they are compared by their distance, and unsigned: a signed difference that overflows is no order.
+__device__ __forceinline__ bool counter_wait(const uint32_t *counter, uint32_t target, const int *status, uint32_t limit) {
   for (uint32_t spin = 0; spin < limit; ++spin) {
-    int seen;
+    uint32_t seen;
     asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
-    if (seen - target >= 0) return true;
+    if (seen - target < 0x80000000u) return true;
     if ((spin & 15) == 15 && *(volatile const int *)status != 0) return false;   // some CTA has given up: nobody waits on
   }
   return false;
@@ -513,7 +514,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       }
       __threadfence();
       epi_barrier();
-      if (et == 0) atomicAdd(cp.finished + MAX_CHAIN, 1);
+      if (et == 0) atomicAdd(cp.finished + MAX_CHAIN, 1u);
       if (cp.embed.table) {
         // the first GEMM's per-token factors are sums over what ALL CTAs gathered
         if (et == 0) wait_flag[0] = counter_wait(cp.finished + MAX_CHAIN, cp.fold_target, p0.status, 1u << 22) && !*abort_flag;
@@ -733,7 +734,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
         group_barrier(grp);
         // every contributor counts towards the hand-over itself: the GEMM is finished once all shares of all tiles
         // are (the host passes the total), and nobody has to learn that it was the last of its tile
-        if (gi == 0 && publish && !wait_flag[2]) atomicAdd(cp.finished + ci, 1);
+        if (gi == 0 && publish && !wait_flag[2]) atomicAdd(cp.finished + ci, 1u);
       }
       if (gi == 0 && grp == 0) TRACE(11);
       epi_barrier();
@@ -799,7 +800,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
           finish(std::false_type{}, s.tile, et, EPI_THREADS, 0, 1, 0, stage, c0, min(c1, rows));
           if (publish && c1 == t_pad) __threadfence();
           epi_barrier();
-          if (publish && c1 == t_pad && et == 0) atomicAdd(cp.finished + ci, 1);
+          if (publish && c1 == t_pad && et == 0) atomicAdd(cp.finished + ci, 1u);
         }
       } else {
         // partial tile: parked in this CTA's slot, for its contributors to fetch; added up after the loop
@@ -882,8 +883,8 @@ struct FastState {
   float *tile_max = nullptr;    // LM head: per-tile best logit and index of every token
   int *tile_arg = nullptr;
   float *ss = nullptr;          // per-tile sums of squares of the residual stream (RMSNorm folded into the GEMMs)
-  int *finished = nullptr;      // [MAX_CHAIN] finished-tile counters of the chained GEMMs (device)
-  int finished_host[MAX_CHAIN + 1] = {0, 0, 0, 0, 0};   // the values those counters have once everything launched so far is done
+  uint32_t *finished = nullptr; // [MAX_CHAIN + 1] finished-tile counters of the chained GEMMs (device)
+  uint32_t finished_host[MAX_CHAIN + 1] = {0, 0, 0, 0, 0};   // the values those counters have once everything launched so far is done
   ChainParams chain{};          // GEMMs collected for the next launch
   int chain_kind[MAX_CHAIN] = {0, 0, 0, 0};
   bool fuse = true;             // run consecutive GEMMs as one launch
@@ -945,19 +946,22 @@ int ouro_fast_setup(ouro_ctx *c) {
   f->s.grid = sms < MAX_GRID ? sms : MAX_GRID;
   f->s.smem_max = smem;
   f->s.slots = c->a.scratch;
-  f->s.finished = (int *)((char *)c->a.scratch + slots_bytes());
+  f->s.finished = (uint32_t *)((char *)c->a.scratch + slots_bytes());
   {
     const char *e = getenv("OURO_FUSE");                       // OURO_FUSE=0: every GEMM is a launch of its own
     f->s.fuse = !(e && e[0] == '0');
     const char *pf = getenv("OURO_PF_ROWS");
     if (pf) f->s.pf_ffn_rows = atol(pf);
+    const char *c0 = getenv("OURO_COUNT_START");                // test aid: what the hand-over counters start at
+    if (c0)
+      for (uint32_t &v : f->s.finished_host) v = (uint32_t)strtoul(c0, nullptr, 0);
   }
   f->s.tile_max = (float *)((char *)c->a.scratch + slots_bytes() + CHAIN_BYTES);
   f->s.tile_arg = (int *)((char *)f->s.tile_max + tile_best_bytes());
   f->s.ss = (float *)((char *)f->s.tile_arg + tile_best_bytes());
   f->s.attn_part = (float *)((char *)f->s.ss + ss_bytes());
   if (cudaMemsetAsync(f->s.slots, 0xff, slots_bytes(), c->stream) != cudaSuccess ||
-      cudaMemsetAsync(f->s.finished, 0, CHAIN_BYTES, c->stream) != cudaSuccess ||
+      cudaMemcpyAsync(f->s.finished, f->s.finished_host, sizeof(f->s.finished_host), cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<SOME>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||

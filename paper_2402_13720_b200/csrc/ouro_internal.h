@@ -188,8 +188,9 @@ struct Leftovers {
   uint4 *slots = nullptr;
   size_t n_slots = 0;                  // 16-byte pieces
   uint32_t empty = 0;
-  int *counters = nullptr;
-  int n_counters = 0, value[8] = {};
+  uint32_t *counters = nullptr;
+  int n_counters = 0;
+  uint32_t value[8] = {};
 };
 void launch_set_state(DevState *st, int32_t *seq_dev, int n_seq, int pending, int fill, const Leftovers &left, cudaStream_t s);
 

@@ -898,25 +898,29 @@ def test_give_up_that_nobody_read_ends_with_the_state(monkeypatch, fuse):
     eng.close()
 
 
-def test_tile_counter_generations_wrap_around(monkeypatch):
-    """The split-K tile counters carry a generation number that grows with every GEMM; when the numbers are used up
-    the words are cleared and counting starts over.  Started a few hundred GEMMs before that point, a generation
-    crosses it and must still equal plain decoding token for token (which crosses it at another place)."""
-    monkeypatch.setenv("OURO_GEN_START", str((1 << 22) - 300))
+@pytest.mark.parametrize("start", [(1 << 31) - 1500, (1 << 32) - 1500])
+def test_hand_over_counters_pass_the_ends_of_their_range(monkeypatch, start):
+    """The counters by which the GEMMs of a chain hand over are never reset and are compared by their distance.  Started 1500
+    finished shares below 2^31 and 2^32 (a forward of this model counts 24 to 96 per chain position), the more than 80
+    forwards of this test take every one of them across; the text equals that of a context that starts at zero, and the
+    resets and the set_state in between leave the counters alone."""
     P = synth.DecodeParams(4, 9, 4, 32, 8)
-    eng, _ = make(MIDB, P, 5)
     prompt = synth.prompt(5, MIDB.vocab, 64, 0.3, 8, 32)
-    van, _ = eng.generate_vanilla(prompt, 48)
-    truth = np.concatenate([prompt, van, np.zeros(32, dtype=np.int32)])
+    eng0, _ = make(MIDB, P, 5)
+    want, _ = eng0.generate_vanilla(prompt, 48)
+    eng0.close()
+    monkeypatch.setenv("OURO_COUNT_START", str(start))
+    eng, _ = make(MIDB, P, 5)
+    van, _ = eng.generate_vanilla(prompt, 20)
+    assert np.array_equal(van, want[:20])
+    truth = np.concatenate([prompt, want, np.zeros(32, dtype=np.int32)])
     eng.set_drafter(lambda seq, g, step: synth.corrupt_drafts(1, truth, len(seq), g, MIDB.vocab, 0.1, 0.05, step))
     out, stats = eng.generate(prompt, 48)
     eng.set_drafter(None)
-    assert np.array_equal(out, van) and stats["target_calls"] < 48
+    assert np.array_equal(out, want) and stats["target_calls"] < 48
+    eng.set_state(70, 3)
+    assert np.array_equal(eng.generate_vanilla(prompt, 48)[0], want)
     eng.close()
-    monkeypatch.delenv("OURO_GEN_START")
-    eng2, _ = make(MIDB, P, 5)                       # and the same text from the usual starting point
-    assert np.array_equal(eng2.generate_vanilla(prompt, 48)[0], van)
-    eng2.close()
 
 
 # ------------------------------------------------- phrase generation during the draft forward (Section 3.1)
