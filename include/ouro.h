@@ -233,11 +233,12 @@ enum {
 uint64_t ouro_kernel_launches(void);
 int ouro_profile_enable(ouro_ctx *ctx, int kernel_class);
 /* Test aid for the give-up path of the bounded device-side waits (no counterpart in the paper).  A GEMM tile whose K
- * range is split across CTAs is finished once all contributors have published their partial sums; the waiting thread
- * polls a counter at most `polls` times (default 1 << 22; negative restores the default).  0 makes the wait give up
- * at once: the kernels return normally, the status word is raised, the next call that reads results back
- * (ouro_accept_and_compact, ouro_generate, ouro_generate_vanilla) returns OURO_ETIMEOUT, and ouro_reset makes the
- * context usable again.  OURO_ESTATE when the context does not run the tensor-core kernels. */
+ * range is split across CTAs is finished once all contributors have published their partial sums, and the steps of a
+ * small model's one-launch forward are separated by barriers; the waiting threads poll memory at most `polls` times
+ * (default 1 << 22; negative restores the default).  0 makes these waits give up at once: the kernels return normally,
+ * the status word is raised, the next call that reads results back (ouro_accept_and_compact, ouro_verify_step,
+ * ouro_generate, ouro_generate_vanilla) returns OURO_ETIMEOUT, and ouro_reset or ouro_set_state makes the context usable
+ * again.  OURO_ESTATE when no kernel of the context waits in this way. */
 int ouro_debug_set_wait_limit(ouro_ctx *ctx, int64_t polls);
 int ouro_profile_read(ouro_ctx *ctx, float *ms_total, int32_t *launches);
 

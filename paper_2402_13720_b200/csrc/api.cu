@@ -102,7 +102,7 @@ static size_t carve(ouro_ctx *c, char *base, const ouro_model_desc *t, const our
   int S = p->beta - 1;
   int32_t *cand_suffix = cv.take<int32_t>((size_t)std::max(1, p->K * S));
   int32_t *cand_count = cv.take<int32_t>(1);
-  int *arrived = cv.take<int>(1);
+  uint32_t *met = cv.take<uint32_t>(2);
   int32_t *draft_dev = cv.take<int32_t>(p->gamma);
   int32_t *win_dev = cv.take<int32_t>(OURO_MAX_WINDOW);
   PoolDev pool{};
@@ -135,7 +135,7 @@ static size_t carve(ouro_ctx *c, char *base, const ouro_model_desc *t, const our
     c->seq_dev = seq_dev;
     c->cand_suffix = cand_suffix;
     c->cand_count = cand_count;
-    c->arrived_dev = arrived;
+    c->met_dev = met;
     c->draft_dev = draft_dev;
     c->win_dev = win_dev;
     c->pool = pool;
@@ -180,7 +180,7 @@ static bool mem_ok(const ouro_model_mem *m) {
 
 int ouro_fast_setup(ouro_ctx *c);  // tensor maps etc. of the tensor-core paths (gemm_tc.cu)
 void ouro_fast_reset(ouro_ctx *c);               // forgets a chain of GEMMs under construction
-Leftovers ouro_fast_leftovers(ouro_ctx *c);
+Leftovers ouro_leftovers(ouro_ctx *c);
 bool ouro_fast_available(ouro_ctx *c, int which);   // model `which` runs on the tensor-core kernels
 bool ouro_fast_layers(ouro_ctx *c, int which);      // its GEMMs do
 
@@ -244,7 +244,7 @@ extern "C" int ouro_create(const ouro_model_desc *t, const ouro_model_mem *tm, c
     }
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&n->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-      (e = cudaMemsetAsync(n->arrived_dev, 0, sizeof(int), n->stream)) != cudaSuccess)
+      (e = cudaMemsetAsync(n->met_dev, 0, 2 * sizeof(uint32_t), n->stream)) != cudaSuccess)
     return bail(OURO_ECUDA, std::string("device set-up: ") + cudaGetErrorString(e));
   launch_pool_clear(n->pool, n->st, n->stream);
   launch_set_state(n->st, n->seq_dev, 1, 0, 1, Leftovers(), n->stream);
@@ -283,9 +283,7 @@ extern "C" int ouro_reset(ouro_ctx *c, int keep_pool) {
   c->seq.assign(1, 0);
   c->step = 0;
   ouro_fast_reset(c);
-  CK(cudaMemsetAsync(c->arrived_dev, 0, sizeof(int), c->stream));      // a barrier that gave up leaves the count short
-  c->arrived_host = 0;
-  launch_set_state(c->st, c->seq_dev, 1, 0, 1, ouro_fast_leftovers(c), c->stream);
+  launch_set_state(c->st, c->seq_dev, 1, 0, 1, ouro_leftovers(c), c->stream);
   if (!keep_pool) launch_pool_clear(c->pool, c->st, c->stream);
   CKL();
   return OURO_OK;
@@ -302,7 +300,7 @@ extern "C" int ouro_set_state(ouro_ctx *c, int32_t cache_len, int32_t pending) {
   c->seq.back() = pending;
   c->step = 0;
   ouro_fast_reset(c);
-  launch_set_state(c->st, c->seq_dev, cache_len + 1, pending, 1, ouro_fast_leftovers(c), c->stream);
+  launch_set_state(c->st, c->seq_dev, cache_len + 1, pending, 1, ouro_leftovers(c), c->stream);
   CKL();
   return OURO_OK;
 }
@@ -363,6 +361,15 @@ static int mbox_wait(ouro_ctx *c, int slot, int32_t seq) {
 static bool small_forward(ouro_ctx *c, int which) {
   const bool timed = c->prof_class >= OURO_PROF_EMBED && c->prof_class <= OURO_PROF_ARGMAX;
   return !ouro_fast_available(c, which) && !ouro_fast_layers(c, which) && forward_small_supported(c->m[which].d) && !timed;
+}
+
+extern "C" int ouro_debug_set_wait_limit(ouro_ctx *c, int64_t polls) {
+  if (!c) return OURO_EINVAL;
+  bool waits = false;                              // some launch of this context waits for other CTAs
+  for (int w = 0; w < 2; ++w) waits = waits || (c->m[w].present && (ouro_fast_layers(c, w) || forward_small_supported(c->m[w].d)));
+  if (!waits) return OURO_ESTATE;
+  c->wait_limit = polls < 0 ? (1u << 22) : (uint32_t)std::min<int64_t>(polls, 1u << 22);
+  return OURO_OK;
 }
 
 extern "C" int ouro_assemble_candidates(ouro_ctx *c, const int32_t *draft_dev, const int32_t *suffix_dev,
@@ -578,7 +585,7 @@ extern "C" int ouro_prefill(ouro_ctx *c, const int32_t *prompt, int32_t n) {
     if (prompt[i] < 0 || prompt[i] >= T.d.vocab) return fail(c, OURO_EINVAL, "prompt token out of range");
   c->seq.assign(prompt, prompt + n);
   CK(cudaMemcpyAsync(c->seq_dev, c->seq.data(), (size_t)n * 4, cudaMemcpyHostToDevice, c->stream));
-  launch_set_state(c->st, c->seq_dev, n, prompt[n - 1], 0, ouro_fast_leftovers(c), c->stream);
+  launch_set_state(c->st, c->seq_dev, n, prompt[n - 1], 0, ouro_leftovers(c), c->stream);
   if ((c->p.flags & OURO_SEED_PROMPT) && n >= c->p.beta)
     launch_pool_update(c->pool, c->st, c->seq_dev, n - c->p.beta + 1, c->p.beta, 1, c->stream);
   CKL();

@@ -9,7 +9,9 @@
 //
 // The rule of kernels_layer.cu holds: a value depends on its own row and on the keys that row sees, in fixed groups.
 //
-// The barriers are bounded: on expiry the CTA raises the context's status word and leaves, and so do the others.
+// The barriers are bounded: on expiry the CTA raises the context's status word and leaves, and so do the others.  Their counts
+// begin and end a launch at zero, on the device alone: a launch that was refused, or one replayed from a graph, needs
+// no book-keeping on the host.
 #include <algorithm>
 
 #include "ouro_internal.h"
@@ -22,7 +24,6 @@ constexpr int WARPS = THREADS / 32;
 constexpr int QUAD = 4;                  // warps that share one (row, head) of the attention: warp j takes key groups j, j + 4, ..
 constexpr int RT = 2;                    // rows of a unit (four: 2365 us for 64 tokens, two: 2264)
 constexpr int MAX_LAYERS = 40;           // layer pointers travel as kernel parameters
-constexpr uint32_t BARRIER_LIMIT = 1u << 22;
 
 struct LayerPtrs { const void *attn_norm, *wq, *wk, *wv, *wo, *ffn_norm, *w_gate, *w_up, *w_down; };
 struct SmallParams {
@@ -39,26 +40,31 @@ struct SmallParams {
   void *q, *att, *act;     // [rows][dq], [rows][dq], [rows][F]
   float *logits;           // [rows][V]
   int32_t *argmax;         // [rows]; NULL: the last layer ends with its keys and values
-  int *arrived;            // CTAs arrived at barriers, ever
-  int base;                // what it holds when the launch begins
+  uint32_t *met;           // [2] CTAs arrived: at all barriers but the last, and at the last
+  uint32_t wait_limit;     // polls of a barrier before it gives up
   int *status;
 };
 static_assert(sizeof(SmallParams) <= 4096, "kernel parameters");
 
-// All CTAs of the grid (one per SM, launched cooperatively) meet; writes before are visible after.  False: given up.
-__device__ __forceinline__ bool grid_barrier(const SmallParams &p, int &target, int *flag) {
-  target += gridDim.x;
+// All CTAs of the grid (one per SM, launched cooperatively) meet; writes before are visible after.  False: given up, by this
+// launch or by one before it (gave_up), whose counts then stand where it left them.
+// Nobody arrives at the last barrier before having left those in front of it, so the count of those goes back to zero
+// behind it; the last one's goes back to zero before the next launch's first barrier (see the kernel's beginning).
+__device__ __forceinline__ bool grid_barrier(const SmallParams &p, uint32_t &target, bool last, int gave_up, int *flag) {
+  uint32_t *const count = p.met + (last ? 1 : 0);
+  target = last ? gridDim.x : target + gridDim.x;
   __syncthreads();
   if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.arrived) : "memory");
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
     int ok = 0;
-    for (uint32_t spin = 0; spin < BARRIER_LIMIT; ++spin) {
-      int seen;
-      asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(p.arrived) : "memory");
-      if (seen - target >= 0) { ok = 1; break; }
+    for (uint32_t spin = 0; spin < p.wait_limit && !gave_up; ++spin) {
+      uint32_t seen;
+      asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
+      if (seen >= target) { ok = 1; break; }
       if ((spin & 63) == 63 && *(volatile const int *)p.status != 0) break;
     }
     if (!ok) atomicExch(p.status, 1);
+    else if (last && blockIdx.x == 0) *(volatile uint32_t *)p.met = 0;
     *flag = ok;
   }
   __syncthreads();
@@ -180,7 +186,10 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
   const int rows = p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows;
   const int tiles = (rows + RT - 1) / RT;
   const int d = p.d, h = p.h, half = h >> 1, dq = p.H * h, dkv = p.Hkv * h;
-  int target = p.base;
+  uint32_t target = 0;
+  int gave_up = 0;
+  if (threadIdx.x == 0) gave_up = *(volatile const int *)p.status;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile uint32_t *)(p.met + 1) = 0;    // (made visible by the first barrier's arrival)
   T *q = (T *)p.q, *att = (T *)p.att, *act = (T *)p.act;
 
   // a row of the residual stream: in front of the first layer still the token's embedding
@@ -243,7 +252,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
       }
     }
     if (!p.argmax && l + 1 == p.n_layers) return;
-    if (!grid_barrier(p, target, &flag)) return;
+    if (!grid_barrier(p, target, false, gave_up, &flag)) return;
     // ---- attention, four warps per (row, head): keys by virtual position in groups of 32, online softmax over a warp's
     //      groups; the four warps' pieces are added in their order
     const int quad = warp / QUAD, qw = warp % QUAD;
@@ -319,7 +328,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
       __syncwarp();
       asm volatile("barrier.sync %0, %1;" ::"r"(1 + quad), "n"(32 * QUAD) : "memory");
     }
-    if (!grid_barrier(p, target, &flag)) return;
+    if (!grid_barrier(p, target, false, gave_up, &flag)) return;
     // ---- a column of a projection back into the residual stream
     auto project = [&](const T *src, const void *weight, int K) {
       for (int u = gw; u < d * tiles; u += nw) {
@@ -339,7 +348,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
     };
     project(att, w.wo, dq);
     embedded = false;
-    if (!grid_barrier(p, target, &flag)) return;
+    if (!grid_barrier(p, target, false, gave_up, &flag)) return;
     // ---- SiLU(gate) * up
     for (int u = gw; u < p.F * tiles; u += nw) {
       const int n_col = u % p.F;
@@ -353,9 +362,9 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
         act[(size_t)(r0 + lane) * p.F + n_col] = from_f<T>(g / (1.0f + expf(-g)) * up);
       }
     }
-    if (!grid_barrier(p, target, &flag)) return;
+    if (!grid_barrier(p, target, false, gave_up, &flag)) return;
     project(act, w.w_down, p.F);
-    if (!grid_barrier(p, target, &flag)) return;
+    if (!grid_barrier(p, target, !p.argmax && l + 2 == p.n_layers, gave_up, &flag)) return;
   }
   // ---- LM head
   for (int u = gw; u < p.V * tiles; u += nw) {
@@ -367,7 +376,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
     contract<T, 1>(residual, (const T *)p.final_norm, p.eps, ws, n, d, acc);
     if (lane < n) __stcg(p.logits + (size_t)(r0 + lane) * p.V + n_col, of_row(acc[0], lane));
   }
-  if (!grid_barrier(p, target, &flag)) return;
+  if (!grid_barrier(p, target, true, gave_up, &flag)) return;
   // ---- greedy choice, a warp per row; the smallest index among equals
   for (int r = gw; r < rows; r += nw) {
     float best = -INFINITY;
@@ -410,15 +419,13 @@ int launch_forward_small(ouro_ctx *c, int which, int rows, const int *rows_dev, 
   p.rows = rows; p.rows_dev = rows_dev;
   p.x = c->a.x; p.q = c->a.q; p.att = c->a.att; p.act = c->a.act;
   p.logits = logits; p.argmax = argmax;
-  p.arrived = c->arrived_dev;
-  p.base = c->arrived_host;
+  p.met = c->met_dev;
+  p.wait_limit = c->wait_limit;
   p.status = &c->st->status;
   // as many CTAs as the widest step has units for: a barrier of fewer CTAs is no dearer
   const long tiles = (rows + RT - 1) / RT;
   const long units = tiles * std::max<long>(std::max<long>(d.d_ffn, argmax ? d.vocab : 0), (d.n_heads + 2 * d.n_kv_heads) * (d.head_dim / 2));
   const int grid = (int)std::max<long>(1, std::min<long>(c->sms, (units + WARPS - 1) / WARPS));
-  const int barriers = argmax ? 5 * d.n_layers + 1 : 5 * (d.n_layers - 1);
-  c->arrived_host = (int)((unsigned)c->arrived_host + (unsigned)(barriers * grid));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = THREADS;

@@ -889,7 +889,6 @@ struct FastState {
   int chain_kind[MAX_CHAIN] = {0, 0, 0, 0};
   bool fuse = true;             // run consecutive GEMMs as one launch
   long pf_ffn_rows = 0;         // rows of gate and of up the attention kernel prefetches into L2 besides the output projection (< 0: nothing)
-  uint32_t wait_limit = 1u << 22;   // polls of a partial-tile wait (ouro_debug_set_wait_limit)
 };
 constexpr int MAX_TILES = 4096;
 constexpr int CHAIN_BYTES = 256;           // the chain counters
@@ -1113,7 +1112,7 @@ static void push_gemm(ouro_ctx *c, Gemm &p, int kind, const CUtensorMap *xmaps, 
   p.status = &c->st->status;
   p.rows_dev = c->cur_rows_dev;
   p.trace_id = kind;
-  p.wait_limit = s.wait_limit;
+  p.wait_limit = c->wait_limit;
   ChainArgs &cp = s.chain.args;
   if (cp.n > 0 && cp.g[0].rows != rows) flush_chain(c);             // cannot happen inside one forward
   s.chain_kind[cp.n] = kind;
@@ -1133,8 +1132,9 @@ void ouro_fast_reset(ouro_ctx *c) {
   cp.embed.table = nullptr;
 }
 // What the launches so far leave behind if one of them has given up.
-Leftovers ouro_fast_leftovers(ouro_ctx *c) {
+Leftovers ouro_leftovers(ouro_ctx *c) {
   Leftovers l;
+  l.met = c->met_dev;
   if (!c->fast) return l;
   const FastState &s = c->fast->s;
   l.slots = (uint4 *)s.slots;
@@ -1144,12 +1144,6 @@ Leftovers ouro_fast_leftovers(ouro_ctx *c) {
   l.n_counters = MAX_CHAIN + 1;
   for (int i = 0; i <= MAX_CHAIN; ++i) l.value[i] = s.finished_host[i];
   return l;
-}
-extern "C" int ouro_debug_set_wait_limit(ouro_ctx *c, int64_t polls) {
-  if (!c) return OURO_EINVAL;
-  if (!c->fast) return OURO_ESTATE;
-  c->fast->s.wait_limit = polls < 0 ? (1u << 22) : (uint32_t)std::min<int64_t>(polls, 1u << 22);
-  return OURO_OK;
 }
 
 // The row count of a candidate block may stay on the device when every kernel of the forward reads it from there:

@@ -683,6 +683,7 @@ __global__ void set_state_kernel(DevState *st, int32_t *seq_dev, int n_seq, int 
   if (st->status != 0) {
     for (size_t i = threadIdx.x; i < left.n_slots; i += blockDim.x) left.slots[i] = make_uint4(left.empty, left.empty, left.empty, left.empty);
     if ((int)threadIdx.x < left.n_counters) left.counters[threadIdx.x] = left.value[threadIdx.x];
+    if (left.met && threadIdx.x < 2) left.met[threadIdx.x] = 0;
   }
   __syncthreads();
   if (threadIdx.x == 0) {

@@ -130,8 +130,8 @@ struct ouro_ctx {
   int32_t *mbox = nullptr, *mbox_dev = nullptr;
   int32_t mseq = 0;
   int sms = 0;                         // multiprocessors of the context's device
-  int *arrived_dev = nullptr;          // barrier arrivals of the one-launch forwards, never reset but with the context ...
-  int arrived_host = 0;                // ... and what that word holds once everything launched so far is done
+  uint32_t *met_dev = nullptr;         // [2] barrier arrivals of the one-launch forwards
+  uint32_t wait_limit = 1u << 22;      // polls of a wait for other CTAs (ouro_debug_set_wait_limit)
   const int *cur_rows_dev = nullptr;   // during a forward: where the kernels read the block's true row count, or NULL
   ouro_drafter_fn drafter = nullptr;
   void *drafter_user = nullptr;
@@ -183,7 +183,8 @@ void launch_argmax(const float *logits, int rows, int vocab, int32_t *out, cudaS
 void launch_pick_token(const int32_t *src, int index, int32_t *dst, cudaStream_t s);
 void launch_pick_assemble(const BlockDev &b, const int32_t *src, int index, int32_t *dst, int L, cudaStream_t s);
 // What a launch whose bounded wait gave up leaves in device memory, and what has to stand there before the status word may be
-// cleared: partial sums nobody fetched (the words are empty again) and hand-over counters short of what the host expects.
+// cleared: partial sums nobody fetched (the words are empty again), hand-over counters short of what the host expects, barrier
+// arrivals (none).
 struct Leftovers {
   uint4 *slots = nullptr;
   size_t n_slots = 0;                  // 16-byte pieces
@@ -191,6 +192,7 @@ struct Leftovers {
   uint32_t *counters = nullptr;
   int n_counters = 0;
   uint32_t value[8] = {};
+  uint32_t *met = nullptr;             // [2]
 };
 void launch_set_state(DevState *st, int32_t *seq_dev, int n_seq, int pending, int fill, const Leftovers &left, cudaStream_t s);
 

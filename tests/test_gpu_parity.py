@@ -1063,6 +1063,84 @@ def test_one_launch_forward_matches_oracle_and_single_kernels(dtype, d, heads, k
     eng.close()
 
 
+def test_one_launch_forward_gives_up_and_the_context_recovers():
+    """The barriers of the one-launch forward are bounded.  With no polls allowed they give up at once (every CTA leaves, the
+    status word is raised): acceptance and plain decoding report it, and a reset, or set_state without anybody having read
+    the status, makes the context compute what it did before."""
+    P = synth.DecodeParams(3, 4, 4, 8, 4)
+    eng, W = make(TINY, P, 2, draft=TINY)
+    _verify_case(eng, W, TINY, P, 2, 40, _fp32_tol)
+    eng.accept_and_compact()
+    prompt = synth.prompt(2, TINY.vocab, 40, 0.4, 4, 8)
+    want, _ = eng.generate_vanilla(prompt, 12)
+
+    def logits():
+        eng.set_state(30, 7)                                    # on the keys of the prompt
+        eng.assemble_causal(binding.OURO_TARGET, [4, 9, 2])
+        return eng.verify_forward(want_logits=True)[1][:3].clone()
+
+    ref = logits()
+    for call in (eng.verify_forward, eng.draft):
+        eng.set_state(30, 7)
+        eng.set_wait_limit(0)
+        eng.assemble_causal(binding.OURO_TARGET, [4, 9, 2])
+        call()
+        eng.set_wait_limit(-1)
+        assert torch.equal(logits(), ref)
+    eng.set_wait_limit(0)
+    with pytest.raises(binding.OuroError) as e:
+        eng.generate_vanilla(prompt, 4)
+    assert e.value.status == binding.OURO_ETIMEOUT
+    eng.reset(); eng.prefill(prompt)
+    eng.assemble_candidates(draft=[1, 2, int(prompt[5])])
+    eng.verify_forward()
+    with pytest.raises(binding.OuroError) as e:
+        eng.accept_and_compact()
+    assert e.value.status == binding.OURO_ETIMEOUT
+    eng.set_wait_limit(-1)
+    _verify_case(eng, W, TINY, P, 2, 40, _fp32_tol)
+    eng.accept_and_compact()
+    assert np.array_equal(eng.generate_vanilla(prompt, 12)[0], want)
+    eng.close()
+
+
+@pytest.mark.parametrize("layers", [1, 2])
+def test_one_launch_forward_replays_from_a_graph(layers):
+    """A captured forward (block assembled inside the graph) gives at every replay what the same calls give uncaptured, with
+    other forwards of the context in between: nothing of the barriers is counted on the host."""
+    desc = dataclasses.replace(TINY, n_layers=layers)
+    P = synth.DecodeParams(3, 4, 4, 8, 4)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        eng, _ = make(desc, P, 4)
+        eng.prefill(synth.prompt(4, desc.vocab, 50, 0.4, 4, 8))
+        tokens = torch.zeros(9, dtype=torch.int32, device="cuda:0")
+
+        def block():
+            eng._ck(eng.L.ouro_assemble_causal(eng.ctx, binding.OURO_TARGET, tokens.data_ptr(), 9))
+            return eng.verify_forward(want_logits=True)
+
+        block()
+        side.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            block()
+        rng = np.random.default_rng(4)
+        for _ in range(6):
+            tokens.copy_(torch.as_tensor(rng.integers(0, desc.vocab, 9).astype(np.int32)))
+            am, lg = block()
+            want = am[:9].clone(), lg[:9].clone()
+            eng.argmax.zero_(); eng.logits.zero_()
+            for _ in range(3):
+                graph.replay()
+            assert torch.equal(eng.argmax[:9], want[0]) and torch.equal(eng.logits[:9], want[1])
+            eng.assemble_causal(binding.OURO_TARGET, [1, 2])
+            eng.verify_forward()
+        side.synchronize()
+        del graph
+        eng.close()
+
+
 # ------------------------------------------------------------ spans of the attention
 
 @pytest.mark.parametrize("heads,kv,hd", [(2, 1, 128), (4, 2, 64)])
