@@ -284,8 +284,9 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
           sc = acc * p.scale;
         }
         const float m_new = fmaxf(m, warp_max(sc));
-        const float corr = expf(m - m_new);
-        const float pw = valid ? expf(sc - m_new) : 0.f;
+        const float at = m_new == -INFINITY ? 0.f : m_new;      // all this warp's scores so far overflowed: weights zero, not NaN
+        const float corr = expf(m - at);
+        const float pw = valid ? expf(sc - at) : 0.f;
         sum = sum * corr + warp_sum(pw);
 #pragma unroll
         for (int dd = 0; dd < 4; ++dd) o[dd] *= corr;

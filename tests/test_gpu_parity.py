@@ -1063,6 +1063,35 @@ def test_one_launch_forward_matches_oracle_and_single_kernels(dtype, d, heads, k
     eng.close()
 
 
+def test_one_launch_forward_with_scores_that_overflow():
+    """Keys so large that a whole group's scores are -infinity in fp32 have the weight zero, whichever of the four warps of a row
+    walks the group and whether it comes first, alone or last there.  wk = wq makes the cached key of the row itself its
+    rotated query; the oracle's float64 scores stay finite and give those keys exactly nothing."""
+    desc = synth.ModelDesc(1, 64, 2, 2, 32, 96, 100, 256, "f32")
+    w = synth.model_weights(desc, 6, device="cuda:0")
+    w["layers"][0]["wq"].mul_(40.0)
+    w["layers"][0]["wk"].copy_(w["layers"][0]["wq"])
+    eng = binding.Engine(desc, w, synth.DecodeParams(2, 3, 1, 4, 4))
+    W = tf.Weights(desc, {k: ([{n: t.cpu() for n, t in lw.items()} for lw in v] if k == "layers" else v.cpu()) for k, v in w.items()})
+    L = 210                                                       # seven groups: warps 0 to 2 walk two, warp 3 one
+    k, v = synth.kv_fill(desc, 3, L, device="cuda:0")
+    for groups in ((1,), (2, 6), (3,), (4,), (1, 2, 3, 5), (0, 4, 5)):
+        eng.tm.k_cache.copy_(k); eng.tm.v_cache.copy_(v)
+        eng.set_state(L, 5)
+        eng.assemble_causal(binding.OURO_TARGET, [5])
+        eng.verify_forward()
+        q = eng.tm.k_cache[0, L].clone()
+        assert float(q.abs().sum(1).min()) > 4.0
+        for g in groups:
+            eng.tm.k_cache[0, 32 * g: 32 * g + 32] = -1e38 * q.sign()
+        cache = tf.KVCache(desc, eng.tm.k_cache.double().cpu().numpy(), eng.tm.v_cache.double().cpu().numpy(), L)
+        eng.assemble_causal(binding.OURO_TARGET, [5])
+        _, logits = eng.verify_forward(want_logits=True)
+        want = tf.forward(W, cache, [5], [L], np.ones((1, L + 1), dtype=bool))
+        _fp32_tol(logits[:1].cpu().numpy().astype(np.float64), want)
+    eng.close()
+
+
 def test_one_launch_forward_gives_up_and_the_context_recovers():
     """The barriers of the one-launch forward are bounded.  With no polls allowed they give up at once (every CTA leaves, the
     status word is raised): acceptance and plain decoding report it, and a reset, or set_state without anybody having read
