@@ -65,8 +65,8 @@ def test_static_scratch_head_equals_the_definition_twice(d_model, vocab):
 
 @pytest.mark.parametrize("d_model,vocab", [(64, 18944), (192, 19080), (128, 23048), (128, 23176), (64, 65536)])
 def test_static_scratch_head_over_all_sms(d_model, vocab):
-    """One CTA per SM (148): 148 tiles exactly, 150 (two left over, cut over the CTAs that have slots), 181 (33 left over
-    with a ragged last tile: whole), 182, and the largest vocabulary (512 tiles: 68 left over, whole)."""
+    """More whole tiles than one CTA per SM (148) takes at once, beside 20, 22, 21, 22 and no tiles that the CTAs with slots
+    share: 148 tiles, 150 and 181 with a ragged last one, 182, and the largest vocabulary (512)."""
     build.build()
     head = synth.tensor(41, 3, (vocab, d_model), 0.02, torch.bfloat16, "cuda:0")
     for call, rows in enumerate((1, 37, 128)):
@@ -75,6 +75,21 @@ def test_static_scratch_head_over_all_sms(d_model, vocab):
         _check_against_definition(x, head, arg, logits)
         few, _ = binding.lm_head_static(x[:1].contiguous(), head)
         assert torch.equal(few, arg[:1])                         # a row's choice does not depend on the others
+
+
+def test_static_scratch_head_keeps_the_precision_of_its_cut_tiles():
+    """250 tiles of 4096 columns: 26 are summed along K in pieces (the remainder of a launch over the 32 CTAs that have
+    slots), the others in one chain.  The pieces' sum is nearer to the exact one, so a launch that handled the remainder
+    whole would show it: the error of those columns against float64 would equal that of the others (measured: 0.75 of it)."""
+    build.build()
+    d_model, vocab, rows = 4096, 32000, 37
+    x = synth.tensor(51, 4, (rows, d_model), 1.0, torch.bfloat16, "cuda:0")
+    head = synth.tensor(52, 3, (vocab, d_model), 0.02, torch.bfloat16, "cuda:0")
+    _, logits = binding.lm_head_static(x, head, want_logits=True)
+    err = torch.cat([logits[:, a: a + 4000].double() - x.double() @ head[a: a + 4000].double().T for a in range(0, vocab, 4000)], 1)
+    cut = (vocab // 128 - 26) * 128
+    whole, pieces = (float(e.square().mean().sqrt()) for e in (err[:, :cut], err[:, cut:]))
+    assert pieces < 0.9 * whole, (pieces, whole)
 
 
 def test_static_scratch_head_matches_verify_forward_twice():
