@@ -79,6 +79,7 @@ _SIGNATURES = {
     "ouro_draft": (C.c_int, [C.c_void_p, C.c_void_p]),
     "ouro_kernel_launches": (C.c_uint64, []),
     "ouro_lm_head_static": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int32, C.c_int32, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p]),
+    "ouro_debug_static_scratch": (C.c_int, [C.POINTER(C.c_void_p), C.POINTER(C.c_size_t)]),
     "ouro_profile_enable": (C.c_int, [C.c_void_p, C.c_int]),
     "ouro_debug_set_wait_limit": (C.c_int, [C.c_void_p, C.c_int64]),
     "ouro_profile_read": (C.c_int, [C.c_void_p, _F32P, _I32P]),

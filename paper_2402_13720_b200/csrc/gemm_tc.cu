@@ -1286,10 +1286,21 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
 
 // Final norm, LM head and greedy choice.  The GEMM's epilogue keeps, per 128-entry vocabulary tile, each
 // token's best logit and index; a small kernel then picks the best tile per token.  logits may be NULL.
-__global__ void argmax_tiles_kernel(const float *tile_max, const int *tile_arg, int tiles, int32_t *out) {
+// With `tidy` (the static scratch, which calls share) the scratch is left as the next call expects it, whatever this call or
+// one that overlapped with it has left there: no partial sums, status zero, its value handed on in `reported`.
+struct Tidy {
+  float *slots = nullptr;      // [n_slots][128][128]; a call of `rows` rows has used the first rows x 128 words of each
+  int n_slots = 0, *status = nullptr, *reported = nullptr;
+};
+__global__ void argmax_tiles_kernel(const float *tile_max, const int *tile_arg, int tiles, int32_t *out, const Tidy tidy) {
   pdl_trigger();
   pdl_wait();
   const int t = blockIdx.x;
+  if (tidy.slots) {
+    for (int s = threadIdx.x >> 5; s < tidy.n_slots; s += blockDim.x >> 5)
+      part_empty(tidy.slots + ((size_t)s * OURO_MAX_ROWS + t) * TILE_N + 4 * (threadIdx.x & 31));
+    if (t == 0 && threadIdx.x == 0) *tidy.reported = atomicExch(tidy.status, 0);
+  }
   // compared through the same order-preserving integer image as inside the tiles (-0.0 below +0.0), so that the
   // choice does not depend on where a tile boundary falls
   uint32_t bv = 0;
@@ -1336,7 +1347,7 @@ int ouro_fast_head(ouro_ctx *c, int which, int rows, float *logits, int32_t *arg
     ProfScope ps(c, OURO_PROF_ARGMAX);
     OURO_COUNT_LAUNCH();
     launch_pdl(argmax_tiles_kernel, rows, 128, 0, c->stream, (const float *)c->fast->s.tile_max, (const int *)c->fast->s.tile_arg,
-               (int)((d.vocab + TILE_N - 1) / TILE_N), argmax_dev);
+               (int)((d.vocab + TILE_N - 1) / TILE_N), argmax_dev, Tidy());
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -1377,7 +1388,7 @@ namespace {
 unsigned char *g_na_ptr[NA_MAX_DEVICES] = {};      // device address of g_static_scratch, per device
 int g_na_smem[NA_MAX_DEVICES] = {};
 int g_na_sms[NA_MAX_DEVICES] = {};
-std::atomic<bool> g_na_ready[NA_MAX_DEVICES] = {};  // the slots are empty and the status word is zero
+std::atomic<bool> g_na_ready[NA_MAX_DEVICES] = {};  // the array has been cleared; every call leaves it clear
 
 // Once per device, with that device current: resolve the array's device address and size the kernel's
 // shared memory.  Returns OURO_OK or an error with a text for ouro_last_error(NULL).
@@ -1412,6 +1423,17 @@ int na_setup(int dev) {
 }
 }  // namespace
 
+extern "C" int ouro_debug_static_scratch(void **dev_ptr, size_t *slot_bytes) {
+  int dev = 0;
+  if (!dev_ptr || !slot_bytes) return OURO_EINVAL;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= NA_MAX_DEVICES) return OURO_ECUDA;
+  const int rc = na_setup(dev);
+  if (rc != OURO_OK) return rc;
+  *dev_ptr = g_na_ptr[dev];
+  *slot_bytes = NA_SLOT_BYTES;
+  return OURO_OK;
+}
+
 extern "C" int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, int32_t rows, int32_t d_model, int32_t vocab,
                                    int32_t *argmax_dev, float *logits_dev, void *cuda_stream) {
   if (!x_dev || !lm_head_dev || !argmax_dev) {
@@ -1434,7 +1456,8 @@ extern "C" int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, i
   cudaStream_t s = (cudaStream_t)cuda_stream;
   unsigned char *base = g_na_ptr[dev];
   const int tiles = (vocab + TILE_N - 1) / TILE_N;
-  // the slots are empty (see EMPTY): cleared by the first call on the device, and every call leaves them so
+  // the slots are empty (see EMPTY) and the status word is zero: cleared by the first call on the device, and left so by the
+  // second kernel of every call, so that what calls that overlapped against the rules did to one another ends with them
   cudaError_t e = cudaSuccess;
   if (!g_na_ready[dev].load(std::memory_order_acquire)) {
     e = cudaMemsetAsync(base, 0xff, NA_SLOT_BYTES, s);
@@ -1478,15 +1501,20 @@ extern "C" int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, i
   p.per = cut.per;
   p.whole0 = cut_by % grid;
   gemm_tc_kernel<SOME><<<grid, THREADS, g_na_smem[dev], s>>>(kp);
-  argmax_tiles_kernel<<<rows, 128, 0, s>>>(p.tile_max, p.tile_arg, tiles, argmax_dev);
+  Tidy tidy;
+  tidy.slots = p.scratch;
+  tidy.n_slots = 2 * cut_by;
+  tidy.status = p.status;
+  tidy.reported = p.status + 1;
+  argmax_tiles_kernel<<<rows, 128, 0, s>>>(p.tile_max, p.tile_arg, tiles, argmax_dev, tidy);
   int status = 0;
   if ((e = cudaGetLastError()) != cudaSuccess ||
-      (e = cudaMemcpyAsync(&status, p.status, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+      (e = cudaMemcpyAsync(&status, tidy.reported, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
       (e = cudaStreamSynchronize(s)) != cudaSuccess) {
     ouro_set_global_error(std::string("ouro_lm_head_static: ") + cudaGetErrorString(e));
     return OURO_ECUDA;
   }
-  g_na_ready[dev].store(status == 0, std::memory_order_release);   // after a give-up the next call clears the array
+  g_na_ready[dev].store(true, std::memory_order_release);
   if (status != 0) {
     ouro_set_global_error("ouro_lm_head_static: a bounded device-side wait gave up");
     return OURO_ETIMEOUT;

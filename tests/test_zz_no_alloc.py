@@ -17,6 +17,8 @@ vocabulary of 4000 (32 tiles) takes only whole tiles, 2048 (16 tiles) splits eve
 CTAs.  Every shape is run twice in a row with different rows, so a counter or a slot left over from the
 previous call would show.
 """
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -113,6 +115,38 @@ def test_static_scratch_head_matches_verify_forward_twice():
         top2 = ref_logits.topk(2, dim=1).values
         safe = (top2[:, 0] - top2[:, 1]) > 2 * err + 1e-6
         assert int(safe.sum()) >= 1 and torch.equal(arg[safe], ref_arg[safe])
+
+
+def test_static_scratch_is_left_clear_whatever_a_call_finds_in_it():
+    """Calls that overlap on a device race on the array, which the header forbids; what they leave there must not reach a
+    later call.  Stand-in for such leftovers: the slots and the status word filled by hand.  The call that meets them may be
+    wrong or report it, but it leaves no partial sum and no status behind, and the next one gives the bits of the first."""
+    build.build()
+    head = synth.tensor(61, 3, (2048, 256), 0.02, torch.bfloat16, "cuda:0")
+    x = synth.tensor(62, 4, (37, 256), 1.0, torch.bfloat16, "cuda:0")
+    want = binding.lm_head_static(x, head, want_logits=True)
+    ptr, nbytes = C.c_void_p(), C.c_size_t()
+    assert binding.lib().ouro_debug_static_scratch(C.byref(ptr), C.byref(nbytes)) == binding.OURO_OK
+
+    class Scratch:
+        __cuda_array_interface__ = dict(shape=(nbytes.value // 4 + 2,), typestr="<i4", data=(ptr.value, False), version=2)
+
+    words = torch.as_tensor(Scratch(), device="cuda:0")
+    slots, status = words[:-2].view(-1, 128 * 128), words[-2:]
+    assert bool((slots == -1).all()) and int(status[0]) == 0
+    for garbage in (0, 0x3F800000):
+        slots[:, : 37 * 128] = garbage
+        torch.cuda.synchronize()
+        binding.lm_head_static(x, head)
+        assert bool((slots == -1).all()) and int(status[0]) == 0
+        got = binding.lm_head_static(x, head, want_logits=True)
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    status[0] = 1                                                # a give-up of another call: reported once, then gone
+    torch.cuda.synchronize()
+    with pytest.raises(binding.OuroError):
+        binding.lm_head_static(x, head)
+    got = binding.lm_head_static(x, head, want_logits=True)
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
 
 
 def test_static_scratch_head_breaks_exact_ties_towards_the_smallest_id():
