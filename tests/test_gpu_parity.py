@@ -898,6 +898,68 @@ def test_give_up_that_nobody_read_ends_with_the_state(monkeypatch, fuse):
     eng.close()
 
 
+def _partial_tile_slots(eng):
+    """The words of the workspace that carry partial sums between CTAs, all 0xffffffff in a fresh context: the run of that
+    length that ends in front of the hand-over counters."""
+    n = 160 * 2 * 128 * 256
+    ws = eng.workspace.view(torch.int32)
+    other = torch.cat([(ws != -1).nonzero().flatten(), torch.tensor([ws.numel()], device=ws.device)])
+    ends = other[1:][other.diff() > n].tolist()
+    assert len(ends) == 1
+    return ws[ends[0] - n: ends[0]]
+
+
+@pytest.mark.parametrize("heads,kv,hd", [(8, 2, 64), (4, 2, 128)])
+def test_every_launch_leaves_the_partial_tile_slots_empty(heads, kv, hd):
+    """A scratch word counts as arrived when it is anything but EMPTY, so whoever fetches a sum empties the word again.
+    After forwards of every kernel size (up to 48, 128 and 256 rows, whose slots are laid out differently), with the row count
+    on the device or on the host, and after whole loops, no word may be left full."""
+    desc = synth.ModelDesc(2, 256, heads, kv, hd, 704, 1000, 700, "bf16")
+    P = synth.DecodeParams(4, 9, 4, 16, 8)
+    eng, _ = make(desc, P, 3, draft=desc)
+    slots = _partial_tile_slots(eng)
+    prompt = synth.prompt(3, desc.vocab, 420, 0.4, 4, 8)
+
+    def empty():
+        torch.cuda.synchronize()
+        return bool((slots == -1).all())
+
+    for n in (1, 15, 48, 49, 100, 128):
+        eng.reset()
+        eng.assemble_causal(binding.OURO_TARGET, prompt[:n])
+        eng.verify_forward()
+        assert empty(), n
+    for n in (130, 200, 257, 420):
+        eng.reset()
+        eng.prefill(prompt[:n])
+        assert empty(), n
+    eng.draft()
+    assert empty()
+    eng.assemble_candidates(draft=[1, 2, 3, int(prompt[5])])
+    eng.verify_forward()
+    eng.accept_and_compact()
+    assert empty()
+    eng.generate(prompt[:140], 24)
+    assert empty()
+    eng.close()
+
+
+def test_partial_sums_that_are_nan_arrive():
+    """The word that stands for "not there yet" is a NaN.  Sums that are NaN must arrive all the same: a token whose embedding is
+    NaN gives NaN logits and no time-out, and leaves no word full."""
+    P = synth.DecodeParams(4, 9, 4, 16, 8)
+    w = synth.model_weights(MIDB, 2, device="cuda:0")
+    w["embed"][7] = float("nan")
+    eng = binding.Engine(MIDB, w, P)
+    slots = _partial_tile_slots(eng)
+    eng.prefill(np.arange(20, 40))
+    eng.assemble_candidates(draft=[1, 2, 3, 7])
+    _, logits = eng.verify_forward(want_logits=True)
+    eng.accept_and_compact()                                      # (would raise on a time-out)
+    assert bool(logits[4].isnan().all()) and bool((slots == -1).all())
+    eng.close()
+
+
 @pytest.mark.parametrize("start", [(1 << 31) - 1500, (1 << 32) - 1500])
 def test_hand_over_counters_pass_the_ends_of_their_range(monkeypatch, start):
     """The counters by which the GEMMs of a chain hand over are never reset and are compared by their distance.  Started 1500
