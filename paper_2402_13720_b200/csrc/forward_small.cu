@@ -2,10 +2,11 @@
 //
 // Such a model's weights are read in microseconds; what a forward costs is its chain of dependent steps, eight launches a
 // layer as kernels of their own (5.6 us each on the fp32 pair of 128-wide layers).  Here one CTA per SM stays for the
-// whole forward and the steps are separated by grid barriers.  A warp takes a unit of a step: one or two output columns
-// for a tile of rows; four warps take one (row, head) of the attention (one warp each: 2815 us for 64 tokens, four: 2391).
-// One cluster of 16 CTAs with its barrier in hardware was slower (2511 us): the units then queue for its warps.  RMSNorm has no step of its own: the warp that
-// contracts a row with the weights has just read the row, and sums its squares first.
+// whole forward and the steps are separated by grid barriers.  A warp takes a unit of a step: one, two or four output
+// columns for a tile of rows; four warps take one (row, head) of the attention (one warp each: 2815 us for 64 tokens, four:
+// 2391).  One cluster of 16 CTAs with its barrier in hardware was slower (2511 us): the units then queue for its warps.
+// RMSNorm has no step of its own: the warp that contracts a row with the weights has just read the row, and sums its
+// squares first.
 //
 // The rule of kernels_layer.cu holds: a value depends on its own row and on the keys that row sees, in fixed groups.
 //
@@ -13,6 +14,7 @@
 // begin and end a launch at zero, on the device alone: a launch that was refused, or one replayed from a graph, needs
 // no book-keeping on the host.
 #include <algorithm>
+#include <type_traits>
 
 #include "ouro_internal.h"
 #include "generic.cuh"
@@ -22,7 +24,6 @@ namespace {
 constexpr int THREADS = 256;
 constexpr int WARPS = THREADS / 32;
 constexpr int QUAD = 4;                  // warps that share one (row, head) of the attention: warp j takes key groups j, j + 4, ..
-constexpr int RT = 2;                    // rows of a unit (four: 2365 us for 64 tokens, two: 2264)
 constexpr int MAX_LAYERS = 40;           // layer pointers travel as kernel parameters
 
 struct LayerPtrs { const void *attn_norm, *wq, *wk, *wv, *wo, *ffn_norm, *w_gate, *w_up, *w_down; };
@@ -73,7 +74,7 @@ __device__ __forceinline__ bool grid_barrier(const SmallParams &p, uint32_t &tar
 
 // Contractions of a tile of rows with C weight rows, the rows normalised on the way (gain != NULL):
 //   acc[c][i] = sum_k T(gain[k] * x[i][k] / rms(x[i])) * w[c][k], lanes stride over k, the same order for any tile.
-template <typename T, int C, typename Row>
+template <typename T, int C, int RT, typename Row>
 __device__ __forceinline__ void contract(const Row &row, const T *gain, float eps, const T *const *w, int n_rows, int K, float (*acc)[RT]) {
   constexpr int V = Vec<T>::N;
   const int lane = threadIdx.x & 31;
@@ -84,7 +85,7 @@ __device__ __forceinline__ void contract(const Row &row, const T *gain, float ep
 #pragma unroll
     for (int c = 0; c < C; ++c) acc[c][i] = 0.f;
   }
-  if (K <= 32 * V) {
+  if (RT <= 2 && K <= 32 * V) {
     // a row is one vector per lane: everything is fetched at once and read once (the same sums in the same order)
     const int k = lane * V;
     const bool in = k < K;
@@ -128,55 +129,57 @@ __device__ __forceinline__ void contract(const Row &row, const T *gain, float ep
         if (i < n_rows) acc[c][i] = warp_sum(acc[c][i]);
     return;
   }
+  // Rows beyond the tile's last repeat it (their sums are not used): the rows' loads are then under way together, where a branch
+  // around each would wait for one before the next is requested.
   if (gain) {
-    for (int k = lane * V; k < K; k += 32 * V)
+    for (int k = lane * V; k < K; k += 32 * V) {
+      float xv[RT][V];
+#pragma unroll
+      for (int i = 0; i < RT; ++i) row(min(i, n_rows - 1), k, xv[i]);
 #pragma unroll
       for (int i = 0; i < RT; ++i)
-        if (i < n_rows) {
-          float xv[V];
-          row(i, k, xv);
 #pragma unroll
-          for (int e = 0; e < V; ++e) inv[i] = fmaf(xv[e], xv[e], inv[i]);
-        }
+        for (int e = 0; e < V; ++e) inv[i] = fmaf(xv[i][e], xv[i][e], inv[i]);
+    }
 #pragma unroll
-    for (int i = 0; i < RT; ++i)
-      if (i < n_rows) inv[i] = 1.0f / sqrtf(warp_sum(inv[i]) / (float)K + eps);
+    for (int i = 0; i < RT; ++i) inv[i] = 1.0f / sqrtf(warp_sum(inv[i]) / (float)K + eps);
   }
-#pragma unroll 2
+#pragma unroll (RT <= 2 ? 2 : 1)
   for (int k = lane * V; k < K; k += 32 * V) {
     Vec<T> wv[C], gv;
 #pragma unroll
     for (int c = 0; c < C; ++c) wv[c].load(w[c] + k);
     if (gain) gv.load(gain + k);
+    float xv[RT][V];
+#pragma unroll
+    for (int i = 0; i < RT; ++i) row(min(i, n_rows - 1), k, xv[i]);
 #pragma unroll
     for (int i = 0; i < RT; ++i)
-      if (i < n_rows) {
-        float xv[V];
-        row(i, k, xv);
 #pragma unroll
-        for (int e = 0; e < V; ++e) {
-          const float a = gain ? to_f<T>(from_f<T>(gv.get(e) * (xv[e] * inv[i]))) : xv[e];
+      for (int e = 0; e < V; ++e) {
+        const float a = gain ? to_f<T>(from_f<T>(gv.get(e) * (xv[i][e] * inv[i]))) : xv[i][e];
 #pragma unroll
-          for (int c = 0; c < C; ++c) acc[c][i] = fmaf(a, wv[c].get(e), acc[c][i]);
-        }
+        for (int c = 0; c < C; ++c) acc[c][i] = fmaf(a, wv[c].get(e), acc[c][i]);
       }
   }
 #pragma unroll
   for (int c = 0; c < C; ++c)
 #pragma unroll
-    for (int i = 0; i < RT; ++i)
-      if (i < n_rows) acc[c][i] = warp_sum(acc[c][i]);
+    for (int i = 0; i < RT; ++i) acc[c][i] = warp_sum(acc[c][i]);
 }
 
 // Lane i's value of a tile's rows.
-__device__ __forceinline__ float of_row(const float *acc, int lane) {
+template <int RT>
+__device__ __forceinline__ float of_row(const float (&acc)[RT], int lane) {
   float v = acc[0];
 #pragma unroll
   for (int i = 1; i < RT; ++i) v = lane == i ? acc[i] : v;
   return v;
 }
 
-template <typename T>
+// WIDE: steps with work for many warps may take larger units (by_rows and the head).  A kernel of its own, so that the short
+// blocks of a narrow model, which wait for their instructions as much as for anything else, run the shorter code.
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_constant__ SmallParams p) {
   __shared__ float sq[WARPS][128];         // attention: a warp's copy of its query, then its unnormalised output
   __shared__ float2 sml[WARPS];            // ... and its score maximum and sum
@@ -184,7 +187,6 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gw = warp * gridDim.x + blockIdx.x, nw = gridDim.x * WARPS;   // (a short step is spread over the SMs)
   const int rows = p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows;
-  const int tiles = (rows + RT - 1) / RT;
   const int d = p.d, h = p.h, half = h >> 1, dq = p.H * h, dkv = p.Hkv * h;
   uint32_t target = 0;
   int gave_up = 0;
@@ -192,7 +194,18 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
   if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile uint32_t *)(p.met + 1) = 0;    // (made visible by the first barrier's arrival)
   T *q = (T *)p.q, *att = (T *)p.att, *act = (T *)p.act;
 
-  // a row of the residual stream: in front of the first layer still the token's embedding
+  // Rows of a unit, for a step of n columns (groups of them, pairs): two, so that a short block is spread over many warps (64
+  // tokens of the fp32 pair: 2264 us, four rows 2365); eight where more than half the warps have a unit even so, since a unit
+  // reads its weights once for all its rows (fp32, 512 x 2048, vocabulary 32000, 128 rows: 11.9 ms with two rows and one
+  // column of the head a unit, 1.96 ms with eight and four; a row's sums are the same either way).
+  auto by_rows = [&](int n, auto body) {
+    if constexpr (WIDE)
+      if (rows > 2 && n * ((rows + 7) / 8) > nw / 2) return body(std::integral_constant<int, 8>{});
+    body(std::integral_constant<int, 2>{});
+  };
+
+  // a row of the residual stream: in front of the first layer still the token's embedding.  (Rows come through L1: the units of
+  // a tile read the same ones, and the barrier's acquire makes what other SMs wrote visible.)
   int r0 = 0;
   bool embedded = true;
   auto residual = [&](int i, int k, float *xv) {
@@ -205,7 +218,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
     } else {
 #pragma unroll
       for (int j = 0; j < V; j += 4) {
-        const float4 v = __ldcg(reinterpret_cast<const float4 *>(p.x + (size_t)(r0 + i) * d + k + j));
+        const float4 v = *reinterpret_cast<const float4 *>(p.x + (size_t)(r0 + i) * d + k + j);
         xv[j] = v.x; xv[j + 1] = v.y; xv[j + 2] = v.z; xv[j + 3] = v.w;
       }
     }
@@ -214,7 +227,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
     return [=](int i, int k, float *xv) {
       constexpr int V = Vec<T>::N;
       Vec<T> e;
-      e.v = __ldcg(reinterpret_cast<const decltype(e.v) *>(base + (size_t)i * K + k));
+      e.load(base + (size_t)i * K + k);
 #pragma unroll
       for (int j = 0; j < V; ++j) xv[j] = e.get(j);
     };
@@ -225,6 +238,9 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
     const size_t layer_off = (size_t)l * p.max_seq * dkv;
     // ---- q, k, v of the normalised rows, rotary positions, cache append.  A unit: dimensions i and i + half of a head
     const int pairs = (p.H + 2 * p.Hkv) * half;
+    by_rows(pairs, [&](auto rt) {
+    constexpr int RT = decltype(rt)::value;
+    const int tiles = (rows + RT - 1) / RT;
     for (int u = gw; u < pairs * tiles; u += nw) {
       const int head = (u % pairs) / half, i = (u % pairs) % half;
       r0 = u / pairs * RT;
@@ -234,10 +250,10 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
       const T *base = (const T *)(is_q ? w.wq : is_v ? w.wv : w.wk) + ((size_t)hh * h + i) * d;
       const T *const ws[2] = {base, base + (size_t)half * d};
       float acc[2][RT];
-      contract<T, 2>(residual, (const T *)w.attn_norm, p.eps, ws, n, d, acc);
+      contract<T, 2, RT>(residual, (const T *)w.attn_norm, p.eps, ws, n, d, acc);
       if (lane < n) {
         const int r = r0 + lane;
-        const float a = of_row(acc[0], lane), b = of_row(acc[1], lane);
+        const float a = of_row<RT>(acc[0], lane), b = of_row<RT>(acc[1], lane);
         float ra = a, rb = b;
         if (!is_v) {
           const size_t ti = (size_t)p.b.pos[r] * half + i;
@@ -251,6 +267,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
         dst[i + half] = from_f<T>(rb);
       }
     }
+    });
     if (!p.argmax && l + 1 == p.n_layers) return;
     if (!grid_barrier(p, target, false, gave_up, &flag)) return;
     // ---- attention, four warps per (row, head): keys by virtual position in groups of 32, online softmax over a warp's
@@ -332,51 +349,75 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
     if (!grid_barrier(p, target, false, gave_up, &flag)) return;
     // ---- a column of a projection back into the residual stream
     auto project = [&](const T *src, const void *weight, int K) {
-      for (int u = gw; u < d * tiles; u += nw) {
-        const int n_col = u % d;
-        r0 = u / d * RT;
-        const int n = min(RT, rows - r0);
-        const T *const ws[1] = {(const T *)weight + (size_t)n_col * K};
-        float acc[1][RT];
-        contract<T, 1>(stored(src + (size_t)r0 * K, K), (const T *)nullptr, 0.f, ws, n, K, acc);
-        if (lane < n) {
-          const int r = r0 + lane;
-          float *x = p.x + (size_t)r * d + n_col;
-          const float old = embedded ? to_f<T>(((const T *)p.embed)[(size_t)p.b.tok[r] * d + n_col]) : __ldcg(x);
-          __stcg(x, old + of_row(acc[0], lane));
+      by_rows(d, [&](auto rt) {
+        constexpr int RT = decltype(rt)::value;
+        const int tiles = (rows + RT - 1) / RT;
+        for (int u = gw; u < d * tiles; u += nw) {
+          const int n_col = u % d;
+          r0 = u / d * RT;
+          const int n = min(RT, rows - r0);
+          const T *const ws[1] = {(const T *)weight + (size_t)n_col * K};
+          float acc[1][RT];
+          contract<T, 1, RT>(stored(src + (size_t)r0 * K, K), (const T *)nullptr, 0.f, ws, n, K, acc);
+          if (lane < n) {
+            const int r = r0 + lane;
+            float *x = p.x + (size_t)r * d + n_col;
+            const float old = embedded ? to_f<T>(((const T *)p.embed)[(size_t)p.b.tok[r] * d + n_col]) : __ldcg(x);
+            __stcg(x, old + of_row<RT>(acc[0], lane));
+          }
         }
-      }
+      });
     };
     project(att, w.wo, dq);
     embedded = false;
     if (!grid_barrier(p, target, false, gave_up, &flag)) return;
     // ---- SiLU(gate) * up
-    for (int u = gw; u < p.F * tiles; u += nw) {
-      const int n_col = u % p.F;
-      r0 = u / p.F * RT;
-      const int n = min(RT, rows - r0);
-      const T *const ws[2] = {(const T *)w.w_gate + (size_t)n_col * d, (const T *)w.w_up + (size_t)n_col * d};
-      float acc[2][RT];
-      contract<T, 2>(residual, (const T *)w.ffn_norm, p.eps, ws, n, d, acc);
-      if (lane < n) {
-        const float g = of_row(acc[0], lane), up = of_row(acc[1], lane);
-        act[(size_t)(r0 + lane) * p.F + n_col] = from_f<T>(g / (1.0f + expf(-g)) * up);
+    by_rows(p.F, [&](auto rt) {
+      constexpr int RT = decltype(rt)::value;
+      const int tiles = (rows + RT - 1) / RT;
+      for (int u = gw; u < p.F * tiles; u += nw) {
+        const int n_col = u % p.F;
+        r0 = u / p.F * RT;
+        const int n = min(RT, rows - r0);
+        const T *const ws[2] = {(const T *)w.w_gate + (size_t)n_col * d, (const T *)w.w_up + (size_t)n_col * d};
+        float acc[2][RT];
+        contract<T, 2, RT>(residual, (const T *)w.ffn_norm, p.eps, ws, n, d, acc);
+        if (lane < n) {
+          const float g = of_row<RT>(acc[0], lane), up = of_row<RT>(acc[1], lane);
+          act[(size_t)(r0 + lane) * p.F + n_col] = from_f<T>(g / (1.0f + expf(-g)) * up);
+        }
       }
-    }
+    });
     if (!grid_barrier(p, target, false, gave_up, &flag)) return;
     project(act, w.w_down, p.F);
     if (!grid_barrier(p, target, !p.argmax && l + 2 == p.n_layers, gave_up, &flag)) return;
   }
-  // ---- LM head
-  for (int u = gw; u < p.V * tiles; u += nw) {
-    const int n_col = u % p.V;
-    r0 = u / p.V * RT;
-    const int n = min(RT, rows - r0);
-    const T *const ws[1] = {(const T *)p.lm_head + (size_t)n_col * d};
-    float acc[1][RT];
-    contract<T, 1>(residual, (const T *)p.final_norm, p.eps, ws, n, d, acc);
-    if (lane < n) __stcg(p.logits + (size_t)(r0 + lane) * p.V + n_col, of_row(acc[0], lane));
+  // ---- LM head: four columns of a unit where all warps have one even so
+  auto head = [&](auto cols, auto rt) {
+    constexpr int CN = decltype(cols)::value, RT = decltype(rt)::value;
+    const int tiles = (rows + RT - 1) / RT, groups = (p.V + CN - 1) / CN;
+    for (int u = gw; u < groups * tiles; u += nw) {
+      const int col = u % groups * CN;
+      r0 = u / groups * RT;
+      const int n = min(RT, rows - r0);
+      const T *ws[CN];
+#pragma unroll
+      for (int c = 0; c < CN; ++c) ws[c] = (const T *)p.lm_head + (size_t)min(col + c, p.V - 1) * d;
+      float acc[CN][RT];
+      contract<T, CN, RT>(residual, (const T *)p.final_norm, p.eps, ws, n, d, acc);
+      if (lane < n) {
+#pragma unroll
+        for (int c = 0; c < CN; ++c)
+          if (col + c < p.V) __stcg(p.logits + (size_t)(r0 + lane) * p.V + col + c, of_row<RT>(acc[c], lane));
+      }
+    }
+  };
+  bool fours = false;
+  if constexpr (WIDE) {
+    fours = p.V >= 4 * nw;
+    if (fours) by_rows(p.V / 4, [&](auto rt) { head(std::integral_constant<int, 4>{}, rt); });
   }
+  if (!fours) by_rows(p.V, [&](auto rt) { head(std::integral_constant<int, 1>{}, rt); });
   if (!grid_barrier(p, target, true, gave_up, &flag)) return;
   // ---- greedy choice, a warp per row; the smallest index among equals
   for (int r = gw; r < rows; r += nw) {
@@ -399,8 +440,9 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
 
 }  // namespace
 
-// Narrow models only: every warp reads its rows itself (twice where they are normalised), which a wide model's step would
-// pay for, and a wide model's steps are not what its launches cost.
+// Narrow models, as far as both sides were measured: at the bound (512 x 2048, vocabulary 32000, four layers) one launch
+// takes 272 us for one row and 1.96 ms for 128 behind 64 keys, the single kernels 543 us and 3.40 ms; at 128 x 344 it is 39
+// and 138 us against 87 and 547.  The choice hangs on the model alone: the two sum a row's squares in another order.
 bool forward_small_supported(const ouro_model_desc &d) { return d.n_layers <= MAX_LAYERS && d.d_model <= 512 && d.d_ffn <= 2048; }
 
 int launch_forward_small(ouro_ctx *c, int which, int rows, const int *rows_dev, int32_t *argmax, float *logits) {
@@ -424,7 +466,7 @@ int launch_forward_small(ouro_ctx *c, int which, int rows, const int *rows_dev, 
   p.wait_limit = c->wait_limit;
   p.status = &c->st->status;
   // as many CTAs as the widest step has units for: a barrier of fewer CTAs is no dearer
-  const long tiles = (rows + RT - 1) / RT;
+  const long tiles = (rows + 1) / 2;
   const long units = tiles * std::max<long>(std::max<long>(d.d_ffn, argmax ? d.vocab : 0), (d.n_heads + 2 * d.n_kv_heads) * (d.head_dim / 2));
   const int grid = (int)std::max<long>(1, std::min<long>(c->sms, (units + WARPS - 1) / WARPS));
   cudaLaunchConfig_t cfg = {};
@@ -436,8 +478,13 @@ int launch_forward_small(ouro_ctx *c, int which, int rows, const int *rows_dev, 
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  const long nw = (long)grid * WARPS, pairs = (d.n_heads + 2 * d.n_kv_heads) * (d.head_dim / 2);
+  const long widest = std::max(std::max<long>(d.d_model, pairs), std::max<long>(d.d_ffn, argmax ? d.vocab : 0));
+  const bool wide = (argmax && d.vocab >= 4 * nw) || (rows > 2 && widest * ((rows + 7) / 8) > nw / 2);
   OURO_COUNT_LAUNCH();
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, d.dtype == OURO_BF16 ? forward_small_kernel<__nv_bfloat16> : forward_small_kernel<float>, p);
+  const auto kernel = d.dtype == OURO_BF16 ? (wide ? forward_small_kernel<__nv_bfloat16, true> : forward_small_kernel<__nv_bfloat16, false>)
+                                           : (wide ? forward_small_kernel<float, true> : forward_small_kernel<float, false>);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p);
   if (e != cudaSuccess) {
     c->err = std::string("one-launch forward: ") + cudaGetErrorString(e);
     return OURO_ECUDA;

@@ -1093,10 +1093,12 @@ def test_draft_catches_up_on_a_long_prompt():
 
 @pytest.mark.parametrize("dtype,d,heads,kv,hd,ffn,vocab", [
     ("f32", 128, 4, 4, 32, 344, 512), ("f32", 72, 3, 1, 32, 104, 1000), ("f32", 512, 4, 2, 128, 2048, 264),
-    ("bf16", 96, 2, 1, 96, 136, 520), ("bf16", 200, 4, 2, 64, 72, 1032)])
+    ("bf16", 96, 2, 1, 96, 136, 520), ("bf16", 200, 4, 2, 64, 72, 1032),
+    ("f32", 136, 4, 4, 32, 1208, 4739), ("bf16", 328, 2, 1, 96, 2040, 5001)])
 def test_one_launch_forward_matches_oracle_and_single_kernels(dtype, d, heads, kv, hd, ffn, vocab):
     """Widths that are no multiple of a warp's stride, one kv head, head dims 32 to 128, the widest model the one-launch
-    forward takes; blocks of 1 to 100 rows.  Against the oracle, against the same block through the single kernels (which
+    forward takes, vocabularies whose columns are taken four at a time with a rest; blocks of 1 to 100 rows (units of two and
+    eight rows).  Against the oracle, against the same block through the single kernels (which
     run while one kernel class is being timed), and a row's logits do not depend on the block."""
     desc = synth.ModelDesc(2, d, heads, kv, hd, ffn, vocab, 192, dtype)
     P = synth.DecodeParams(4, 5, 3, 16, 8)
