@@ -677,24 +677,25 @@ void launch_pick_assemble(const BlockDev &b, const int32_t *src, int index, int3
 // Text of n_seq tokens ending in the pending token; with fill, the earlier positions are recorded as 0.  The status word is
 // cleared, and with it what a launch that raised it left behind: nobody need have read the status in between.
 __global__ void set_state_kernel(DevState *st, int32_t *seq_dev, int n_seq, int pending, int fill, const Leftovers left) {
+  const int status = blockIdx.x == 0 ? *(volatile const int32_t *)&st->status : 0;     // (asked for first, needed last)
   if (fill)
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_seq - 1; i += gridDim.x * blockDim.x) seq_dev[i] = 0;
   if (blockIdx.x != 0) return;
-  if (st->status != 0) {
-    for (size_t i = threadIdx.x; i < left.n_slots; i += blockDim.x) left.slots[i] = make_uint4(left.empty, left.empty, left.empty, left.empty);
-    if ((int)threadIdx.x < left.n_counters) left.counters[threadIdx.x] = left.value[threadIdx.x];
-    if (left.met && threadIdx.x < 2) left.met[threadIdx.x] = 0;
-  }
-  __syncthreads();
   if (threadIdx.x == 0) {
     seq_dev[n_seq - 1] = pending;
     st->pending = pending;
     st->n_seq = n_seq;
     st->n_cand = 0;
     st->n_rows = 0;
-    st->status = 0;
     st->win_valid = 0;
   }
+  if (status != 0) {
+    for (size_t i = threadIdx.x; i < left.n_slots; i += blockDim.x) left.slots[i] = make_uint4(left.empty, left.empty, left.empty, left.empty);
+    if ((int)threadIdx.x < left.n_counters) left.counters[threadIdx.x] = left.value[threadIdx.x];
+    if (left.met && threadIdx.x < 2) left.met[threadIdx.x] = 0;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) st->status = 0;
 }
 void launch_set_state(DevState *st, int32_t *seq_dev, int n_seq, int pending, int fill, const Leftovers &left, cudaStream_t s) {
   OURO_COUNT_LAUNCH();
