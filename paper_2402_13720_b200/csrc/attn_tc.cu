@@ -53,8 +53,6 @@ constexpr int THREADS = WARPS * 32;
 // instruction fetches.  A row's arithmetic does not involve its tile's index or the other rows, so both sizes give the
 // same bits.
 
-constexpr int SHORT_ROUNDS = 2 * 148;   // CTAs of 16-row rounds that are resident at once (74 KB of shared memory each)
-
 struct AttnParams {
   const __nv_bfloat16 *q;          // [rows][H*HD] rotated queries
   const __nv_bfloat16 *k, *v;      // this layer's cache: [max_seq][Hkv*HD]
@@ -454,7 +452,7 @@ int attention_tc_setup() {
 
 // n_vis_max: an upper bound of the number of keys any row of the block sees (cache length + rows).
 bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_cache, const void *v_cache, const BlockDev &b,
-                         int rows, int L, int n_vis_max, int layer, float *part, void *out, const int *rows_dev, cudaStream_t s) {
+                         int rows, int L, int n_vis_max, int layer, float *part, void *out, const int *rows_dev, int sms, cudaStream_t s) {
   OURO_COUNT_LAUNCH();
   AttnParams p;
   p.rows_dev = rows_dev;
@@ -470,12 +468,13 @@ bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_
   p.out = (__nv_bfloat16 *)out;
   const int parts = (rows + OURO_MAX_ROWS - 1) / OURO_MAX_ROWS;
   const int m_all = (d.n_heads / d.n_kv_heads) * std::min<int>(rows, OURO_MAX_ROWS);   // query rows per kv head (an upper bound when the count is on the device)
-  // A round of 16 query rows takes 9-11 us (its chain of latencies over four chunks), one of 64 rows 14-27 us, and the
-  // rounds of a short block run side by side: 16 rows each while all CTAs are resident at once.  (1.1B draft, 19 rows x 8
-  // heads over 540 keys: 27.0 us on 24 CTAs of 64 rows, 11.3 us on 80 CTAs of 16.)  Beyond that, larger rounds read the
-  // keys less often.
+  // A round of 16 query rows over a span of four chunks takes 9-11 us (its chain of latencies), one of 64 rows 14-27 us, and
+  // the rounds of a short block run side by side: 16 rows each while all CTAs are resident at once.  (1.1B draft, 19 rows x 8
+  // heads over 540 keys, in spans of four chunks: 27.0 us on 24 CTAs of 64 rows, 11.3 us on 80 CTAs of 16.)  Beyond that,
+  // larger rounds read the keys less often.  An SM holds two such CTAs at head dim 64 (74 KB of shared memory), one at 128.
   const int n_spans = fold::span_count(d.head_dim, n_vis_max);
-  const int mt = parts * n_spans * d.n_kv_heads * ((m_all + 15) / 16) <= SHORT_ROUNDS ? 1 : 4, qr = 16 * mt;
+  const int resident = (d.head_dim == 64 ? 2 : 1) * sms;
+  const int mt = parts * n_spans * d.n_kv_heads * ((m_all + 15) / 16) <= resident ? 1 : 4, qr = 16 * mt;
   p.rounds = (m_all + qr - 1) / qr;
   dim3 grid(n_spans, d.n_kv_heads, parts * p.rounds);
   p.direct = n_spans <= 1;                                  // a single span: nothing to fold

@@ -1234,7 +1234,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
     }
     else if (attention_tc_supported(d))
       pieces = launch_attention_tc(d, a.q, M.k_cache, M.v_cache, M.blk, rows, M.L, M.L + rows, l, c->fast->s.attn_part, a.att,
-                                   c->cur_rows_dev, s);
+                                   c->cur_rows_dev, c->sms, s);
     else
       launch_attention_simple(d, a.q, M.k_cache, M.v_cache, M.blk, rows, l, a.att, s);
     if (pieces) {                    // folded by the output projection's launch, all its CTAs taking part

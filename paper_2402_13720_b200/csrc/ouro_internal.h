@@ -226,7 +226,7 @@ size_t attention_tc_scratch_bytes(const ouro_model_desc &d);
 int attention_tc_setup();
 // Both return true when the spans still have to be folded by the kernel that consumes `out` (attn_fold.cuh).
 bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_cache, const void *v_cache, const BlockDev &b,
-                         int rows, int L, int n_vis_max, int layer, float *part, void *out, const int *rows_dev, cudaStream_t s);
+                         int rows, int L, int n_vis_max, int layer, float *part, void *out, const int *rows_dev, int sms, cudaStream_t s);
 
 // ---- attn_tm.cu (tcgen05 path, head dim 128) ---------------------------------------------------
 bool attention_tm_supported(const ouro_model_desc &d);
