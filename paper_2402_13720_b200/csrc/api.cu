@@ -738,7 +738,7 @@ static int draft_step_phrases(ouro_ctx *c, int32_t *out_dev, int *calls) {
     if (n < 1) return fail(c, OURO_ESTATE, "draft cache ahead of the text");
     launch_draft_lookup_assemble(c->pool, D.blk, c->st, tokens, n, c->cand_suffix, c->cand_count, D.L, S, K, s);
     CKL();
-    CK(cudaMemcpyAsync(c->pin, &c->st->n_rows, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(c->pin, &c->st->d_rows, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     D.blk_rows = c->pin[0];
     D.blk_rows_dev = false;

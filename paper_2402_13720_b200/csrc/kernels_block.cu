@@ -434,8 +434,8 @@ __global__ void draft_lookup_assemble_kernel(PoolDev P, BlockDev b, DevState *st
   __syncthreads();
   const int nc = S > 0 ? min(*count, K) : 0, B = n + nc * S, r = threadIdx.x;
   if (r == 0) {
-    st->n_cand = nc;
-    st->n_rows = B;
+    st->d_cand = nc;
+    st->d_rows = B;
   }
   if (r >= B) return;
   u64 m0 = 0, m1 = 0;
@@ -472,7 +472,7 @@ __global__ void draft_accept_compact_kernel(BlockDev b, DevState *st, const int3
   __shared__ int s_chosen, s_m;
   __shared__ int32_t s_bonus;
   if (threadIdx.x == 0) {
-    const int nc = st->n_cand;
+    const int nc = st->d_cand;
     int chosen = -1, best = -1;
     int32_t bonus = o[n - 1];
     for (int j = 0; j < nc; ++j) {
@@ -533,11 +533,7 @@ __global__ void draft_window_assemble_kernel(BlockDev b, DevState *st, const int
     }
   }
   __syncthreads();
-  if (r == 0) {
-    st->win_valid = 1;
-    st->n_cand = W > 0 ? 1 : 0;
-    st->n_rows = n + W;
-  }
+  if (r == 0) st->win_valid = 1;
   if (r >= n + W) return;
   u64 m0 = 0, m1 = 0;
   if (r < n) {

@@ -61,6 +61,8 @@ struct DevState {
   int32_t d_keep;    // draft tokens the round added (at most what was still missing of gamma)
   int32_t d_cached;  // how many of them have their K/V in the draft cache (matched suffix tokens kept)
   int32_t win_valid; // the lookahead window holds guesses (0 after a reset: the next draft forward fills it from the text)
+  int32_t d_rows;    // rows of the draft model's last assembled block, and its candidates: a target block that is assembled
+  int32_t d_cand;    // already keeps n_rows and n_cand
 };
 
 // Per-row description of a query block.  Row r attends, in this order, cache slots [0, lin_end[r])

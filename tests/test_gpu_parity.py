@@ -627,6 +627,33 @@ def test_phrase_level_drafting_bf16_self_draft():
     assert res[1]["draft_calls"] < res[0]["draft_calls"] == 4 * res[0]["target_calls"]     # c of Eq. 6 above 1
 
 
+@pytest.mark.parametrize("kind", ["phrases", "window"])
+@pytest.mark.parametrize("desc", [TINY, MIDB], ids=["f32", "bf16"])
+def test_drafting_leaves_an_assembled_target_block_alone(desc, kind):
+    """A candidate block's row and candidate counts stay on the device until the forward and the acceptance read them.
+    Drafting in between (its blocks have counts of their own) must not change them: block, logits and acceptance are those
+    of the same calls without it."""
+    P = synth.DecodeParams(3, 4, 3, 16, 8, harvest_matched=False, harvest_candidates=False, harvest_accepted=False,
+                           draft_phrases=kind == "phrases", window=6 if kind == "window" else 0)
+    eng, _ = make(desc, P, 2, draft=desc)
+    prompt = synth.prompt(2, desc.vocab, 40, 0.5, 4, 8)
+    L, d = len(prompt) - 1, torch.tensor([1, 2, int(prompt[5])], dtype=torch.int32, device="cuda:0")
+    eng.prefill(prompt)
+    res = []
+    for between in (False, True):
+        eng.set_state(L, int(prompt[-1]))
+        eng._ck(eng.L.ouro_assemble_candidates(eng.ctx, d.data_ptr(), None, None))
+        if between:
+            eng.draft()
+        am, lg = eng.verify_forward(want_logits=True)
+        logits = lg.clone()
+        tok = eng.block_get()[0].tolist()
+        assert len(tok) > 1 + P.gamma                             # some phrase was found, and not all rows of K candidates
+        res.append((tok, logits[: len(tok)], eng.accept_and_compact()[3].tolist()))
+    assert res[0][0] == res[1][0] and torch.equal(res[0][1], res[1][1]) and res[0][2] == res[1][2]
+    eng.close()
+
+
 def test_phrase_level_drafting_edge_cases():
     """Long catch-up (the uncached text does not fit one block beside the candidates), K = 0 (every round is a plain
     single-token forward) and beta = 1 (phrases have no suffix): the drafts stay those of token-level drafting."""
