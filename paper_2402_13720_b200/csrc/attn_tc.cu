@@ -471,10 +471,11 @@ bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_
   // A round of 16 query rows over a span of four chunks takes 9-11 us (its chain of latencies), one of 64 rows 14-27 us, and
   // the rounds of a short block run side by side: 16 rows each while all CTAs are resident at once.  (1.1B draft, 19 rows x 8
   // heads over 540 keys, in spans of four chunks: 27.0 us on 24 CTAs of 64 rows, 11.3 us on 80 CTAs of 16.)  Beyond that,
-  // larger rounds read the keys less often.  An SM holds two such CTAs at head dim 64 (74 KB of shared memory), one at 128.
+  // larger rounds read the keys less often, unless a single round of 16 takes all rows.  An SM holds two such CTAs at head dim
+  // 64 (74 KB of shared memory), one at 128.
   const int n_spans = fold::span_count(d.head_dim, n_vis_max);
   const int resident = (d.head_dim == 64 ? 2 : 1) * sms;
-  const int mt = parts * n_spans * d.n_kv_heads * ((m_all + 15) / 16) <= resident ? 1 : 4, qr = 16 * mt;
+  const int mt = m_all <= 16 || parts * n_spans * d.n_kv_heads * ((m_all + 15) / 16) <= resident ? 1 : 4, qr = 16 * mt;
   p.rounds = (m_all + qr - 1) / qr;
   dim3 grid(n_spans, d.n_kv_heads, parts * p.rounds);
   p.direct = n_spans <= 1;                                  // a single span: nothing to fold
