@@ -59,6 +59,7 @@ struct AttnParams {
   const int32_t *lin_end, *seg_start, *seg_len, *group;
   int rows, H, Hkv, L, cap;        // L: cache length before the block; cap: span slots per (row, head)
   int rounds;                      // rounds of query rows per 128 block rows
+  int in_waves;                    // the grid's order, see launch_attention_tc
   float scale_log2;
   float *part;                     // [rows][H][cap][PIECE]: max (log2 domain), sum, -, -, unnormalised output
   __nv_bfloat16 *out;              // [rows][H*HD]
@@ -148,11 +149,12 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
   // (written by the assembling kernel, which is not launched programmatically and so has finished) and cache rows
   // below the cache length.  The queries and the block's own K/V rows come from the kernel just before this one.
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int sc = blockIdx.x, kvh = blockIdx.y;
+  const int sc = p.in_waves ? gridDim.z - 1 - blockIdx.z : blockIdx.x, kvh = p.in_waves ? blockIdx.x : blockIdx.y;
+  const int rnd = p.in_waves ? blockIdx.y : blockIdx.z;
   const int g = p.H / p.Hkv, dkv = p.Hkv * HD;
   // a block of more than 128 rows (known text: one group, rows in order) is handled 128 rows at a time, the cache in front
   // of a part being the cache in front of the block and the rows before the part
-  const int zb = (int)blockIdx.z / p.rounds * OURO_MAX_ROWS, L = p.L + zb;
+  const int zb = rnd / p.rounds * OURO_MAX_ROWS, L = p.L + zb;
   const int rows = min(OURO_MAX_ROWS, (p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows) - zb);   // written before the forward pass began
   const int32_t *group = p.group + zb, *lin_end = p.lin_end + zb, *seg_start = p.seg_start + zb, *seg_len = p.seg_len + zb;
   const int M_all = g * rows;
@@ -187,7 +189,7 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
 
   {
     // ---------------------------------------------------------------- this CTA's round of up to 64 query rows
-    const int m0 = (int)blockIdx.z % p.rounds * QR;
+    const int m0 = rnd % p.rounds * QR;
     // Query rows are ordered group by group (a group's rows for head 0, then for head 1, ..), so that the 64 rows
     // of a round belong to few groups and the chunk that holds block keys needs few passes.  Rows of this thread
     // in row tile mt: lane/4 and +8.
@@ -477,7 +479,13 @@ bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_
   const int resident = (d.head_dim == 64 ? 2 : 1) * sms;
   const int mt = m_all <= 16 || parts * n_spans * d.n_kv_heads * ((m_all + 15) / 16) <= resident ? 1 : 4, qr = 16 * mt;
   p.rounds = (m_all + qr - 1) / qr;
-  dim3 grid(n_spans, d.n_kv_heads, parts * p.rounds);
+  // A grid of several waves begins with the last span and has every (kv head, round) of a span before the next one: the long
+  // spans, and the one with the block's own keys and a pass per group, then do not end it, and the rounds of a span find its
+  // keys in L2 (1.1B shape, four layers, 128 rows behind 1200 keys: 559 -> 486 us, behind 12200: 1134 -> 1082 us).  One wave
+  // has its spans side by side (one row behind 2000 keys: 206 us, with the long spans' CTAs next to one another 216 us).
+  const int per_sm = d.head_dim == 64 ? (mt == 1 ? 3 : 2) : 1;
+  p.in_waves = parts * p.rounds * n_spans * d.n_kv_heads > per_sm * sms;
+  const dim3 grid = p.in_waves ? dim3(d.n_kv_heads, parts * p.rounds, n_spans) : dim3(n_spans, d.n_kv_heads, parts * p.rounds);
   p.direct = n_spans <= 1;                                  // a single span: nothing to fold
   if (d.head_dim == 128) {
     if (mt == 1) launch_pdl(attn_span_kernel<128, 1>, grid, THREADS, Smem<128, 1>::BYTES, s, p);
