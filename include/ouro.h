@@ -138,7 +138,8 @@ int ouro_prefill(ouro_ctx *ctx, const int32_t *prompt_host, int32_t n);
 
 /* Declares both caches to already hold cache_len tokens (contents supplied by the caller) with the given
  * pending token: entry state for stepping from a synthetic cache.  Text positions < cache_len are
- * recorded as token 0. */
+ * recorded as token 0.  Like ouro_reset and ouro_prefill it clears the status of an earlier time-out, read or not, and what
+ * the kernels that gave up left behind. */
 int ouro_set_state(ouro_ctx *ctx, int32_t cache_len, int32_t pending_token);
 int ouro_get_state(ouro_ctx *ctx, int32_t *target_len, int32_t *draft_len, int32_t *pending_token);
 
@@ -160,9 +161,9 @@ int ouro_pool_import(ouro_ctx *ctx, const int32_t *ngrams_host, int32_t n);
  * position ids (trunk row b: L+b; suffix row (j,i): L+gamma+i) and the Eq. 8 visibility.  draft_dev
  * [gamma].  suffix_dev / count_dev as written by ouro_phrase_lookup; pass NULL for both to have the
  * pool looked up with key d_gamma here.  Asynchronous when the target runs on the tensor-core kernels (bf16,
- * supported shapes): the block's row count 1 + gamma + K' (beta-1) then stays on the device, the forward is
- * launched for the largest block the parameters allow and ouro_block_get reports the true count.  Otherwise the
- * call synchronises to read the count. */
+ * supported shapes) or as a one-launch forward (other models up to 512 x 2048): the block's row count
+ * 1 + gamma + K' (beta-1) then stays on the device, the forward is launched for the largest block the parameters allow
+ * and ouro_block_get reports the true count.  Otherwise the call synchronises to read the count. */
 int ouro_assemble_candidates(ouro_ctx *ctx, const int32_t *draft_dev, const int32_t *suffix_dev,
                              const int32_t *count_dev);
 /* Plain causal block of n tokens (tokens_dev [n]) for model `which`: prefill, catch-up, vanilla decoding. */
@@ -251,14 +252,15 @@ int ouro_profile_read(ouro_ctx *ctx, float *ms_total, int32_t *launches);
  *   argmax_dev   [rows] int32 out: greedy token per row (ties -> smallest id)
  *   logits_dev   [rows, vocab] fp32 out, or NULL
  * Limits: 1 <= rows <= 128, d_model a multiple of 64, vocab a multiple of 8 and <= 65536; anything else returns
- * OURO_EINVAL with a text in ouro_last_error(NULL).  The split-K scratch, counters and per-tile maxima live in a
+ * OURO_EINVAL with a text in ouro_last_error(NULL).  The split-K scratch and the per-tile maxima live in a
  * 5 MiB array inside the library image; every GPU that loads the library holds it until the process exits.
  * The first call on each device resolves that array's device address and sizes the kernel's shared memory;
  * make that first call outside any stream capture, with the device current.  All calls on a device share the
  * array: two calls whose GPU work overlaps (different streams or threads) race on it - serialise them.
  * The call enqueues on cuda_stream (a cudaStream_t, NULL = default), then synchronises that stream and returns
- * OURO_ETIMEOUT if a bounded device-side wait gave up.  It runs on 32 SMs only (the scratch is sized per CTA), so
- * it is slower than ouro_verify_forward's head pass; results agree with it to rounding (another split of K). */
+ * OURO_ETIMEOUT if a bounded device-side wait gave up.  All SMs stream the weights, but only 32 CTAs share tiles along K
+ * (the scratch is sized per CTA), so it is slower than ouro_verify_forward's head pass; results agree with it to rounding
+ * (another split of K). */
 int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, int32_t rows, int32_t d_model, int32_t vocab,
                         int32_t *argmax_dev, float *logits_dev, void *cuda_stream);
 /* Test aid: device address of that array on the current device, and the bytes at its beginning that hold partial sums (all

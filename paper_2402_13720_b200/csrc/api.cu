@@ -384,8 +384,8 @@ extern "C" int ouro_assemble_candidates(ouro_ctx *c, const int32_t *draft_dev, c
     launch_assemble_candidates(M.blk, c->st, draft_dev, suffix_dev, count_dev, M.L, gamma, S, K, c->stream);
   CKL();
   if (ouro_fast_available(c, OURO_TARGET) || small_forward(c, OURO_TARGET)) {
-    // The tensor-core kernels and the one-launch forward read the block's row count from device memory: the forward is launched for the largest
-    // block these parameters allow and the host never waits for the lookup.
+    // The tensor-core kernels and the one-launch forward read the block's row count from device memory: the forward is
+    // launched for the largest block these parameters allow and the host never waits for the lookup.
     M.blk_rows = 1 + gamma + K * S;
     M.blk_rows_dev = true;
   } else {
@@ -562,7 +562,7 @@ extern "C" int ouro_advance(ouro_ctx *c, int which, int32_t n) {
 // for 128.
 static int feed_text(ouro_ctx *c, int which, int upto, int *last_row) {
   ModelRt &M = c->m[which];
-  const int widest = ouro_fast_available(c, which) ? OURO_TEXT_ROWS : OURO_MAX_ROWS;
+  const int widest = ouro_fast_available(c, which) ? (int)OURO_TEXT_ROWS : (int)OURO_MAX_ROWS;
   while (M.L < upto) {
     const int left = upto - M.L;
     const bool outputs = last_row && left <= OURO_MAX_ROWS;

@@ -1,9 +1,10 @@
 // Folding the per-span pieces of the split attention into the block's attention output.
 //
-// Both tensor-core attention kernels cut a row's keys into spans and leave, per (row, head, span), the span's score maximum (log2 domain), its sum of exponentials and its unnormalised output.  A (row, head) pair is
-// folded by one warp: first the largest span maximum, then one weighted sum over the spans in ascending order.  The
-// arithmetic involves the pair's own spans only, so it does not matter which kernel, CTA or warp runs it; it runs in
-// the kernel that consumes the attention output (the output projection), spread over all its CTAs.
+// Both tensor-core attention kernels cut a row's keys into spans and leave, per (row, head, span), the span's score maximum
+// (log2 domain), its sum of exponentials and its unnormalised output.  A (row, head) pair is folded by one warp: first the
+// largest span maximum, then one weighted sum over the spans in ascending order.  The arithmetic involves the pair's own
+// spans only, so it does not matter which kernel, CTA or warp runs it; it runs in the kernel that consumes the attention
+// output (the output projection), spread over all its CTAs.
 #pragma once
 
 #include <cuda_bf16.h>

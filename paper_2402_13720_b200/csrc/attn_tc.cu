@@ -5,14 +5,14 @@
 // described by the number of keys it sees and by where its last keys live (its own candidate's cache slots),
 // and the kernel maps "virtual positions" 0..n_vis-1 to cache slots on the fly.
 //
-// Work split.  Keys are cut by virtual position into spans of one or four chunks (attn_fold.cuh); one CTA handles one (kv head, span)
-// for up to 64 query rows (rows x query heads of the group; further rows go to further CTAs, which find the same
-// keys in L2), so every cached byte is read from HBM once.  The CTA
+// Work split.  Keys are cut by virtual position into spans of one or four chunks (attn_fold.cuh); one CTA handles one
+// (kv head, span) for 16 or up to 64 query rows (rows x query heads of the group; further rows go to further CTAs, which
+// find the same keys in L2), so every cached byte is read from HBM once.  The CTA
 // walks its span in chunks of 128 keys: K and V rows of the next chunk stream into a second shared-memory
 // buffer (cp.async) while the current one is used.  Per chunk: the 8 warps split the keys for S = Q K^T
 // (mma.sync), agree on each row's chunk maximum through shared memory, write P = exp2(S - max) as bf16 to shared
 // memory, then split the head dimension for O += P V.  Running (max, sum, O) are kept per row across the chunks
-// of the span; a second kernel folds the spans of a row in ascending order and normalises.
+// of the span; the kernel that consumes the output folds the spans of a row in ascending order and normalises.
 //
 // Chunks below the cache length are the same for all rows.  A chunk holding the block's own keys differs
 // between the trunk and each candidate: it is processed once per group, with that group's keys swapped into the
@@ -146,7 +146,8 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
   pdl_trigger();
   TRACE(0);
   // Everything up to pdl_wait() reads only what was complete before the forward pass began: the block description
-  // (written by the assembling kernel, which is not launched programmatically and so has finished) and cache rows
+  // (the kernel that assembles it waits for what came before and lets nobody start early: it does not trigger its
+  // dependents, launched programmatically or not, and so has finished when the forward's first kernel begins) and cache rows
   // below the cache length.  The queries and the block's own K/V rows come from the kernel just before this one.
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sc = p.in_waves ? gridDim.z - 1 - blockIdx.z : blockIdx.x, kvh = p.in_waves ? blockIdx.x : blockIdx.y;
@@ -410,7 +411,7 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
     for (int i = 0; i < 2 * MT; ++i) {
       if (nv[i] <= span0) continue;
       if (p.direct) {
-        // what the merge kernel would compute from this single span: weight exp2(0) = 1, then o * (1 / l)
+        // what the fold would compute from this single span: weight exp2(0) = 1, then o * (1 / l)
         const float inv = 1.0f / l_run[i];
 #pragma unroll
         for (int nt = 0; nt < NT2; ++nt) {

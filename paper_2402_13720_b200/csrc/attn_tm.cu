@@ -4,8 +4,8 @@
 // forward under a mask in which a phrase suffix sees the prefix, the draft and itself (Eq. 8); a row is described
 // by the number of keys it sees and by where its last keys live, and keys are addressed by "virtual position".
 //
-// Work split.  Keys are cut by virtual position into spans of four chunks (attn_fold.cuh); one CTA handles one (span, kv head)
-// for a round of up to 128 query rows (block rows x query heads of the group, ordered group by group).  It walks
+// Work split.  Keys are cut by virtual position into spans of four chunks (attn_fold.cuh); one CTA handles one (span,
+// kv head) for a round of up to 128 query rows (block rows x query heads of the group, ordered group by group).  It walks
 // the span in chunks of 128 keys.  Per chunk:
 //     S = Q K^T      one 128 x 128 x 128 tcgen05 contraction into TMEM (Q and K K-major in 128-byte swizzle),
 //     softmax        the threads of query row t read its 128 scores from TMEM, mask by virtual position, keep a
@@ -259,7 +259,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
   }
   pdl_trigger();
   // Everything up to pdl_wait() reads only what was complete before the forward pass began: the block description
-  // (written by the assembling kernel, which is not launched programmatically and so has finished) and cache rows
+  // (the kernel that assembles it waits for what came before and lets nobody start early: it does not trigger its
+  // dependents, launched programmatically or not, and so has finished when the forward's first kernel begins) and cache rows
   // below the cache length.  The queries and the block's own K/V rows come from the kernel just before this one.
 
   // ---- groups are contiguous row ranges: find their first rows (warps 0-3, one block row per thread)
@@ -642,7 +643,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
       lsum[h * QR + t] = l_run;
       asm volatile("bar.sync 1, %0;" ::"n"(ROW_THREADS) : "memory");
       if (has && nv > span0 && p.direct) {
-        // what the merge kernel would compute from this single span: weight exp2(0) = 1, then o * (1 / l)
+        // what the fold would compute from this single span: weight exp2(0) = 1, then o * (1 / l)
         const float inv = 1.0f / (lsum[t] + lsum[QR + t]);
         __nv_bfloat16 *dst = p.out + ((size_t)(zb + r) * p.H + kvh * g + hq) * HD + h * 64;
 #pragma unroll

@@ -1363,8 +1363,8 @@ int ouro_fast_head(ouro_ctx *c, int which, int rows, float *logits, int32_t *arg
 // Some users of this library cannot give it a workspace: a serving process that handed all device memory to
 // its own arena at start-up (a later cudaMalloc simply fails), or a latency-critical loop that must not run
 // into the implicit device synchronisation an allocation can cause.  For them this one call keeps everything
-// the GEMM needs besides its inputs and outputs - the partial-tile slots of the split-K schedule, the tile
-// counters, the per-tile maxima and a status word - in a fixed array that is part of the library image.
+// the GEMM needs besides its inputs and outputs - the partial-tile slots of the split-K schedule, the per-tile
+// maxima and a status word - in a fixed array that is part of the library image.
 // Every GPU that loads the library carries these 5 MiB until the process exits.
 //
 // The array's name is only meaningful in device code.  Host code must ask the runtime for its device address

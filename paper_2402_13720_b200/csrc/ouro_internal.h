@@ -93,10 +93,10 @@ struct ModelRt {
   int32_t blk_rows = 0; // rows of the current block (0 = none assembled)
   int32_t blk_L = -1;   // cache length the block was assembled for
   bool blk_is_candidate = false;
-  bool blk_rows_dev = false;  // blk_rows is an upper bound; the true count is DevState::n_rows (tensor-core path only)
+  bool blk_rows_dev = false;  // blk_rows is an upper bound; the true count is DevState::n_rows (tensor-core and one-launch forwards)
 };
 
-struct Activations {  // sized for OURO_MAX_ROWS rows of the larger model
+struct Activations {  // sized for OURO_MAX_ROWS rows of the larger model, 16-bit ones and x for OURO_TEXT_ROWS
   float *x;        // residual stream [rows, d_model]
   void *xn;        // normed activations [rows, d_model], model dtype
   float *qkv;      // [rows, d_q + 2 d_kv]
