@@ -264,7 +264,7 @@ int ouro_profile_read(ouro_ctx *ctx, float *ms_total, int32_t *launches);
 int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, int32_t rows, int32_t d_model, int32_t vocab,
                         int32_t *argmax_dev, float *logits_dev, void *cuda_stream);
 /* Test aid: device address of that array on the current device, and the bytes at its beginning that hold partial sums (all
- * 0xff between calls; a status word and a copy of it follow, zero between calls). */
+ * 0xff between calls; the status word follows, zero unless the last call gave up). */
 int ouro_debug_static_scratch(void **dev_ptr, size_t *slot_bytes);
 
 #ifdef __cplusplus

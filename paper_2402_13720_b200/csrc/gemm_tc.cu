@@ -1286,21 +1286,18 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
 
 // Final norm, LM head and greedy choice.  The GEMM's epilogue keeps, per 128-entry vocabulary tile, each
 // token's best logit and index; a small kernel then picks the best tile per token.  logits may be NULL.
-// With `tidy` (the static scratch, which calls share) the scratch is left as the next call expects it, whatever this call or
-// one that overlapped with it has left there: no partial sums, status zero, its value handed on in `reported`.
+// With `tidy` (the static scratch, which calls share) no partial sums are left for the next call, whatever this call or one that
+// overlapped with it has left there.
 struct Tidy {
   float *slots = nullptr;      // [n_slots][128][128]; a call of `rows` rows has used the first rows x 128 words of each
-  int n_slots = 0, *status = nullptr, *reported = nullptr;
+  int n_slots = 0;
 };
 __global__ void argmax_tiles_kernel(const float *tile_max, const int *tile_arg, int tiles, int32_t *out, const Tidy tidy) {
   pdl_trigger();
   pdl_wait();
   const int t = blockIdx.x;
-  if (tidy.slots) {
-    for (int s = threadIdx.x >> 5; s < tidy.n_slots; s += blockDim.x >> 5)
-      part_empty(tidy.slots + ((size_t)s * OURO_MAX_ROWS + t) * TILE_N + 4 * (threadIdx.x & 31));
-    if (t == 0 && threadIdx.x == 0) *tidy.reported = atomicExch(tidy.status, 0);
-  }
+  for (int s = threadIdx.x >> 5; s < tidy.n_slots; s += blockDim.x >> 5)
+    part_empty(tidy.slots + ((size_t)s * OURO_MAX_ROWS + t) * TILE_N + 4 * (threadIdx.x & 31));
   // compared through the same order-preserving integer image as inside the tiles (-0.0 below +0.0), so that the
   // choice does not depend on where a tile boundary falls
   uint32_t bv = 0;
@@ -1388,7 +1385,7 @@ namespace {
 unsigned char *g_na_ptr[NA_MAX_DEVICES] = {};      // device address of g_static_scratch, per device
 int g_na_smem[NA_MAX_DEVICES] = {};
 int g_na_sms[NA_MAX_DEVICES] = {};
-std::atomic<bool> g_na_ready[NA_MAX_DEVICES] = {};  // the array has been cleared; every call leaves it clear
+std::atomic<bool> g_na_ready[NA_MAX_DEVICES] = {};  // the slots are empty and the status word is zero, and every call leaves them so
 
 // Once per device, with that device current: resolve the array's device address and size the kernel's
 // shared memory.  Returns OURO_OK or an error with a text for ouro_last_error(NULL).
@@ -1456,10 +1453,12 @@ extern "C" int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, i
   cudaStream_t s = (cudaStream_t)cuda_stream;
   unsigned char *base = g_na_ptr[dev];
   const int tiles = (vocab + TILE_N - 1) / TILE_N;
-  // the slots are empty (see EMPTY) and the status word is zero: cleared by the first call on the device, and left so by the
-  // second kernel of every call, so that what calls that overlapped against the rules did to one another ends with them
+  // The slots are empty (see EMPTY) and the status word is zero: cleared by the first call on the device and by the one after
+  // a give-up.  The second kernel of every call empties the slots that the call has used, so that what calls that overlapped
+  // against the rules did to one another ends with them.
   cudaError_t e = cudaSuccess;
-  if (!g_na_ready[dev].load(std::memory_order_acquire)) {
+  const bool clear = !g_na_ready[dev].load(std::memory_order_acquire);
+  if (clear) {
     e = cudaMemsetAsync(base, 0xff, NA_SLOT_BYTES, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(base + NA_OFF_STATUS, 0, NA_OFF_TMAX - NA_OFF_STATUS, s);
   }
@@ -1504,20 +1503,19 @@ extern "C" int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, i
   Tidy tidy;
   tidy.slots = p.scratch;
   tidy.n_slots = 2 * cut_by;
-  tidy.status = p.status;
-  tidy.reported = p.status + 1;
   argmax_tiles_kernel<<<rows, 128, 0, s>>>(p.tile_max, p.tile_arg, tiles, argmax_dev, tidy);
   int status = 0;
   if ((e = cudaGetLastError()) != cudaSuccess ||
-      (e = cudaMemcpyAsync(&status, tidy.reported, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+      (e = cudaMemcpyAsync(&status, p.status, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
       (e = cudaStreamSynchronize(s)) != cudaSuccess) {
     ouro_set_global_error(std::string("ouro_lm_head_static: ") + cudaGetErrorString(e));
     return OURO_ECUDA;
   }
-  g_na_ready[dev].store(true, std::memory_order_release);
-  if (status != 0) {
+  if (status != 0) {                             // (only the call that has cleared the array may call it clear)
+    g_na_ready[dev].store(false, std::memory_order_release);
     ouro_set_global_error("ouro_lm_head_static: a bounded device-side wait gave up");
     return OURO_ETIMEOUT;
   }
+  if (clear) g_na_ready[dev].store(true, std::memory_order_release);
   return OURO_OK;
 }

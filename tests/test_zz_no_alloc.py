@@ -119,8 +119,8 @@ def test_static_scratch_head_matches_verify_forward_twice():
 
 def test_static_scratch_is_left_clear_whatever_a_call_finds_in_it():
     """Calls that overlap on a device race on the array, which the header forbids; what they leave there must not reach a
-    later call.  Stand-in for such leftovers: the slots and the status word filled by hand.  The call that meets them may be
-    wrong or report it, but it leaves no partial sum and no status behind, and the next one gives the bits of the first."""
+    later call.  Stand-in for such leftovers: the slots filled by hand.  The call that meets them may be wrong, but it leaves
+    no partial sum behind, and the next one gives the bits of the first.  A raised status word is reported once."""
     build.build()
     head = synth.tensor(61, 3, (2048, 256), 0.02, torch.bfloat16, "cuda:0")
     x = synth.tensor(62, 4, (37, 256), 1.0, torch.bfloat16, "cuda:0")
@@ -129,10 +129,10 @@ def test_static_scratch_is_left_clear_whatever_a_call_finds_in_it():
     assert binding.lib().ouro_debug_static_scratch(C.byref(ptr), C.byref(nbytes)) == binding.OURO_OK
 
     class Scratch:
-        __cuda_array_interface__ = dict(shape=(nbytes.value // 4 + 2,), typestr="<i4", data=(ptr.value, False), version=2)
+        __cuda_array_interface__ = dict(shape=(nbytes.value // 4 + 1,), typestr="<i4", data=(ptr.value, False), version=2)
 
     words = torch.as_tensor(Scratch(), device="cuda:0")
-    slots, status = words[:-2].view(-1, 128 * 128), words[-2:]
+    slots, status = words[:-1].view(-1, 128 * 128), words[-1:]
     assert bool((slots == -1).all()) and int(status[0]) == 0
     for garbage in (0, 0x3F800000):
         slots[:, : 37 * 128] = garbage
