@@ -16,13 +16,14 @@ struct Span {  // one piece of a CTA's work: k-blocks [kb0, kb1) of `tile`
 
 // Work of one CTA.  The last R = tiles mod grid tiles are cut stream-K fashion into equal contiguous spans of
 // the (tile, k-block) space and come first, so that their partial sums are added up while the whole tiles
-// (tile c, c + grid, ...) that follow are still streaming.  Where only some CTAs share the cut tiles, the whole tiles are
-// dealt out from the first CTA behind them.  Depends on (tiles, kb, grid, splitters) only.
+// (tile c, c + grid, ...) that follow are still streaming.  Where only the first `sharers` CTAs share the cut tiles, the
+// whole tiles are dealt out from the first CTA behind them, round by round; `sit_out` leaves the sharers out of the first
+// round.  Depends on (tiles, kb, grid, splitters) only.
 // The host works the cut out (GemmParams::t0, ::per): a walker is built by four warps of every CTA for every GEMM, and
 // each integer division by a run-time number there is 0.1 us in front of the first load.
 struct SpanWalker {
-  int kb, per, t0, it, end, whole, grid, cta;
-  __device__ SpanWalker(int tiles, int kb_, int t0_, int per_, int whole0, int grid_, int cta_) {
+  int kb, per, t0, it, end, whole, step, grid, cta;
+  __device__ SpanWalker(int tiles, int kb_, int t0_, int per_, int sharers, bool sit_out, int grid_, int cta_) {
     kb = kb_;
     grid = grid_;
     cta = cta_;
@@ -31,7 +32,9 @@ struct SpanWalker {
     const int total = (tiles - t0) * kb;
     it = min(total, cta * per);
     end = min(total, it + per);
-    whole = cta >= whole0 ? cta - whole0 : cta - whole0 + grid;
+    const int first = sit_out ? grid - sharers : grid;       // whole tiles of the first round
+    whole = cta >= sharers ? cta - sharers : first + cta + (sit_out ? grid : 0) - sharers;
+    step = cta >= sharers ? first : grid;
   }
   __device__ int owner_slot(int tile, int owner) const { return ((tile - t0) * kb <= owner * per) ? 0 : 1; }
   __device__ bool next(Span &s) {
@@ -53,7 +56,8 @@ struct SpanWalker {
       s.n_contrib = 1;
       s.slot = 0;
       s.first_owner = cta;
-      whole += grid;
+      whole += step;
+      step = grid;
       return true;
     }
     return false;
