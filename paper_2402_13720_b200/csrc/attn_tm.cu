@@ -95,6 +95,7 @@ struct TmParams {
   const int32_t *lin_end, *seg_start, *seg_len, *group;
   int rows, H, Hkv, L, cap, row0;  // row0: first row of this layer in the tensor maps
   int n_spans;
+  int own_spans, slices;           // spans that hold keys of the block itself (the last ones), and CTAs that share their groups
   float scale_log2;
   float *part;                     // [rows][H][cap][PIECE]: max (log2 domain), sum, -, -, unnormalised output
   __nv_bfloat16 *out;              // [rows][H*HD], written here only when `direct`
@@ -213,8 +214,11 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
   Misc *ms = reinterpret_cast<Misc *>(smem + OFF_MISC);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // blockIdx.x walks (span, kv head) with the last span of every head first: it holds the block's own keys and
-  // takes one pass per group, so it should not be what the grid ends on
-  const int sc = p.n_spans - 1 - blockIdx.x / p.Hkv, kvh = blockIdx.x % p.Hkv, m0 = blockIdx.y * QR;
+  // takes one pass per group, so it should not be what the grid ends on.  Where SMs would be idle otherwise, `slices` CTAs
+  // share the groups of such a span, group o going to slice o mod slices (see launch_attention_tm).
+  const int kvh = blockIdx.x % p.Hkv, m0 = blockIdx.y * QR, part = blockIdx.x / p.Hkv - p.own_spans * p.slices;
+  const int sc = part < 0 ? p.n_spans - 1 - (part + p.own_spans * p.slices) / p.slices : p.n_spans - 1 - p.own_spans - part;
+  const int slices = part < 0 ? p.slices : 1, slice = part < 0 ? (part + p.own_spans * p.slices) % p.slices : 0;
   // a block of more than 128 rows (known text: one group, rows in order) is handled 128 rows at a time, the cache in front
   // of a part being the cache in front of the block and the rows before the part
   const int zb = blockIdx.z * OURO_MAX_ROWS, L = p.L + zb;
@@ -303,8 +307,10 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
       while (o + 1 < ng && m >= g * ms->gs[o + 1]) ++o;
       const int a = ms->gs[o], n = ms->gs[o + 1] - a, e = m - g * a;
       const int r = a + e % n, hq = e / n;
-      info = r | (hq << 8) | (o << 16);
-      atomicMax(&ms->gmax[o], ms->lin[r] + ms->len[r]);
+      if (slices == 1 || o % slices == slice) {
+        info = r | (hq << 8) | (o << 16);
+        atomicMax(&ms->gmax[o], ms->lin[r] + ms->len[r]);
+      }
     }
     ms->map[tid] = info;
   }
@@ -687,8 +693,8 @@ int attention_tm_setup() {
 // 64 x 128 box in 128-byte swizzle.  Returns true when the spans still have to be folded (attn_fold.cuh: by the kernel
 // that consumes the attention output); with a single span the kernel has written `out` itself.
 bool launch_attention_tm(const ouro_model_desc &d, const void *q, const void *kmap, const void *vmap, const void *k_cache,
-                         const void *v_cache, const BlockDev &b, int rows, int L, int n_vis_max, int layer, float *part,
-                         void *out, int *status, const int *rows_dev, const L2Prefetch &pf, cudaStream_t s) {
+                         const void *v_cache, const BlockDev &b, int rows, int groups, int L, int n_vis_max, int layer, float *part,
+                         void *out, int *status, const int *rows_dev, const L2Prefetch &pf, int sms, cudaStream_t s) {
   OURO_COUNT_LAUNCH();
   TmParams p;
   for (int r = 0; r < 3; ++r) {
@@ -714,7 +720,15 @@ bool launch_attention_tm(const ouro_model_desc &d, const void *q, const void *km
   p.rows_dev = rows_dev;
   const int m_all = (d.n_heads / d.n_kv_heads) * std::min<int>(rows, OURO_MAX_ROWS);
   p.n_spans = fold::span_count(HD, n_vis_max);
-  dim3 grid(p.n_spans * d.n_kv_heads, (m_all + QR - 1) / QR, (rows + OURO_MAX_ROWS - 1) / OURO_MAX_ROWS);
+  // The chunk with the block's own keys takes one pass of 1.75 us per group (trunk, each candidate), one after the other in
+  // one CTA: with 32 heads behind 411 keys 8 passes on 32 SMs.  As far as all CTAs are resident at once (one per SM), the
+  // groups of such a span are spread over several CTAs, each of which walks the span's common chunks for its own rows: the
+  // same work for a row, and its keys come from L2.  (7B step behind 411 keys, 37 rows: 3535 -> 3337 us; 34B shape, 8 layers, 69
+  // rows: 2192 -> 2155; two small layers: 103 -> 94.)  With more CTAs than SMs the second wave would cost what the passes save.
+  const int rounds = (m_all + QR - 1) / QR, parts = (rows + OURO_MAX_ROWS - 1) / OURO_MAX_ROWS, per_span = d.n_kv_heads * rounds * parts;
+  p.own_spans = p.n_spans - L / fold::LONG_KEYS;
+  p.slices = std::max(1, std::min(groups, (sms / per_span - (p.n_spans - p.own_spans)) / p.own_spans));
+  dim3 grid((p.n_spans - p.own_spans + p.own_spans * p.slices) * d.n_kv_heads, rounds, parts);
   launch_pdl(attn_tm_kernel, grid, THREADS, SMEM_BYTES, s, p);
   return !p.direct;
 }

@@ -1230,7 +1230,8 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
         pf.ptr[2] = M.w_up[l]; pf.bytes[2] = head;
       }
       pieces = launch_attention_tm(d, a.q, &c->fast->s.m[which].kmap, &c->fast->s.m[which].vmap, M.k_cache, M.v_cache, M.blk, rows,
-                                   M.L, M.L + rows, l, c->fast->s.attn_part, a.att, &c->st->status, c->cur_rows_dev, pf, s);
+                                   M.blk_is_candidate ? 1 + std::max(1, c->p.K) : 1, M.L, M.L + rows, l, c->fast->s.attn_part, a.att,
+                                   &c->st->status, c->cur_rows_dev, pf, c->sms, s);
     }
     else if (attention_tc_supported(d))
       pieces = launch_attention_tc(d, a.q, M.k_cache, M.v_cache, M.blk, rows, M.L, M.L + rows, l, c->fast->s.attn_part, a.att,

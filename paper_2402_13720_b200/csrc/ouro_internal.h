@@ -241,5 +241,5 @@ struct L2Prefetch {
   size_t bytes[3] = {0, 0, 0};
 };
 bool launch_attention_tm(const ouro_model_desc &d, const void *q, const void *kmap, const void *vmap, const void *k_cache,
-                         const void *v_cache, const BlockDev &b, int rows, int L, int n_vis_max, int layer, float *part,
-                         void *out, int *status, const int *rows_dev, const L2Prefetch &pf, cudaStream_t s);
+                         const void *v_cache, const BlockDev &b, int rows, int groups, int L, int n_vis_max, int layer, float *part,
+                         void *out, int *status, const int *rows_dev, const L2Prefetch &pf, int sms, cudaStream_t s);

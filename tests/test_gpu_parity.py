@@ -1295,3 +1295,31 @@ def test_attention_spans_match_oracle(heads, kv, hd, L):
             assert torch.equal(lg[0], got[r]), r
             eng.advance(binding.OURO_TARGET, 1)
     eng.close()
+
+
+@pytest.mark.parametrize("kv,K,L", [(1, 16, 300), (16, 4, 411), (37, 4, 127), (74, 3, 500), (30, 4, 505), (100, 2, 411)])
+def test_groups_shared_by_several_ctas_are_bit_identical_to_plain_decoding(kv, K, L):
+    """Head dim 128: trunk and candidates of one span are shared by as many CTAs as SMs are left (here all groups alone, five
+    groups on four CTAs, four on two, two spans with block keys, one CTA).  A suffix row's logits equal, bit for bit, those of the
+    same token decoded as plain text."""
+    desc = synth.ModelDesc(1, 256, kv, kv, 128, 320, 512, L + 80, "bf16")
+    P = synth.DecodeParams(3, 4, K, 4, 32, seed_prompt=False)
+    eng, _ = make(desc, P, 5)
+    k, v = synth.kv_fill(desc, 3, L, device="cuda:0")
+    eng.tm.k_cache.copy_(k); eng.tm.v_cache.copy_(v)
+    rng = np.random.default_rng(L)
+    d = rng.integers(0, desc.vocab, 3).tolist()
+    eng.set_state(L, 9)
+    eng.phrase_update(np.concatenate([np.full((K, 1), d[-1]), rng.integers(0, desc.vocab, (K, 3))], axis=1).astype(np.int32))
+    eng.assemble_candidates(draft=d)
+    tok = eng.block_get()[0]
+    assert len(tok) == 4 + 3 * K
+    packed = eng.verify_forward(want_logits=True)[1][: len(tok)].clone()
+    for j in (0, K // 2, K - 1):
+        eng.set_state(L, 9)
+        own = list(range(4)) + list(range(4 + 3 * j, 7 + 3 * j))
+        for r in own:
+            eng.assemble_causal(binding.OURO_TARGET, [int(tok[r])])
+            assert torch.equal(eng.verify_forward(want_logits=True)[1][0], packed[r]), (j, r)
+            eng.advance(binding.OURO_TARGET, 1)
+    eng.close()
