@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
   if (warp == 0) {
     const int n = ms->n_items;
     while (early < 2 && early < n && ((ms->items[early] >> 3) & 63) == 63 && span0 + (ms->items[early] & 7) * CH + CH <= p.L) {
-      if (lane == 0) request_tile(early, ms->items[early] & 7);
+      if (elect_one()) request_tile(early, ms->items[early] & 7);
       ++early;
     }
   }
@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
         const int it = ms->items[i], ci = it & 7, go = (it >> 3) & 63, st = i & 1;
         if (i >= early) {
           if (i >= 2) mbar_wait(&ms->empty[st], ((i >> 1) - 1) & 1, ms, p.status);
-          if (lane == 0) {
+          if (elect_one()) {
             if (it & IT_REUSE) mbar_arrive(&ms->full[st]);   // nothing to fetch: the phase completes at once
             else request_tile(i, ci);
           }
@@ -423,11 +423,11 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
           }
           fence_async_smem();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&ms->patched[st]);
+          if (elect_one()) mbar_arrive(&ms->patched[st]);
         }
       }
       // nothing of this CTA may still be in flight when it leaves: wait (bounded) for the last tile of each stage
-      if (lane == 0) {
+      if (elect_one()) {
         for (int st = 0; st < 2; ++st) {
           const int n_st = (n_items + 1 - st) >> 1;        // tiles requested into this stage
           if (n_st == 0) continue;
@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
       }
     } else if (warp == 1) {
       // ================================================================ contraction issue
-      if (lane == 0) {
+      if (elect_one()) {
         bool issued = false;
         uint32_t patch_par = 0;                        // bit st: parity of the next patched tile of stage st
         auto issue_s = [&](int i) {

@@ -59,7 +59,6 @@ constexpr int EPI_WARPS = 8;      // two per TMEM lane quarter
 constexpr int EPI_THREADS = 32 * EPI_WARPS;
 constexpr int ACT_WARP = 2 + EPI_WARPS;
 constexpr int THREADS = 32 * (ACT_WARP + 1);   // warp 0 weight TMA, warp 1 MMA, warps 2..9 epilogue, warp 10 activation TMA
-constexpr int W_PRODUCERS = 2;    // lanes of warp 0 that issue the weight copies, stage by stage in turn (a power of two, smaller than the ring)
 constexpr int MAX_GRID = 160;
 constexpr uint32_t SPIN_LIMIT = 1u << 24;
 constexpr unsigned long long HINT_EVICT_FIRST = 0x12F0000000000000ull;
@@ -353,7 +352,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
-    if (lane < W_PRODUCERS) {
+    if (elect_one()) {
       // The weights do not depend on the previous kernel, so this warp never waits for it: the ring fills with
       // weight tiles while the predecessor drains.  The activation tiles come from another warp, after its wait.
       // One thread runs this loop once per 16 KB stage; at 40 GB/s per SM that is every 0.4 us, so the loop carries
@@ -372,18 +371,16 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
         const CUtensorMap *m0 = &kp.maps[ci].a[seg];
         uint8_t *sa = ring + (size_t)st * stage_bytes;
         for (int kb = s.kb0; kb < s.kb1; ++kb, ++n) {
-          if ((n & (W_PRODUCERS - 1)) == (uint32_t)lane) {           // the lanes take the stages in turn
-            if (round > 0) {
-              ok = mbar_wait(&empty[st], (round - 1) & 1, abort_flag) && !*abort_flag;
-              if (!ok) break;
-            }
-            mbar_expect_tx(&full[st], A_BYTES);
-            if (swiglu) {
-              tma_load_2d(sa, &kp.maps[ci].a[0], &full[st], kb * BLOCK_K, row0, HINT_EVICT_FIRST);
-              tma_load_2d(sa + A_BYTES / 2, &kp.maps[ci].a[1], &full[st], kb * BLOCK_K, row0, HINT_EVICT_FIRST);
-            } else {
-              tma_load_2d(sa, m0, &full[st], kb * BLOCK_K, row0, HINT_EVICT_FIRST);
-            }
+          if (round > 0) {
+            ok = mbar_wait(&empty[st], (round - 1) & 1, abort_flag) && !*abort_flag;
+            if (!ok) break;
+          }
+          mbar_expect_tx(&full[st], A_BYTES);
+          if (swiglu) {
+            tma_load_2d(sa, &kp.maps[ci].a[0], &full[st], kb * BLOCK_K, row0, HINT_EVICT_FIRST);
+            tma_load_2d(sa + A_BYTES / 2, &kp.maps[ci].a[1], &full[st], kb * BLOCK_K, row0, HINT_EVICT_FIRST);
+          } else {
+            tma_load_2d(sa, m0, &full[st], kb * BLOCK_K, row0, HINT_EVICT_FIRST);
           }
           sa += stage_bytes;
           if (++st == n_stages) { st = 0; ++round; sa = ring; }
@@ -396,7 +393,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
     }
   } else if (warp == ACT_WARP) {
     // ---------------------------------------------------------------- activation producer
-    if (lane == 0) {
+    if (elect_one()) {
       pdl_wait();                                  // the first GEMM's activations are the previous kernel's output
       uint32_t n = 0, round = 0;
       int st = 0;
@@ -436,7 +433,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p0.t_pad >> 3) << 17) | ((uint32_t)(TILE_N >> 4) << 24);
       uint32_t n = 0, item = 0, round = 0;
       int st = 0;
@@ -827,7 +824,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
   // ------------------------------------------------------------------ teardown
   fence_before_sync();
   __syncthreads();
-  if (*abort_flag && ((warp == 0 && lane < W_PRODUCERS) || (warp == ACT_WARP && lane == 0))) {
+  if (*abort_flag && n_issued > 0) {               // (the two producer threads)
     // Somebody gave up: copies this lane issued may still be landing in this CTA's shared memory.  Wait (bounded) for
     // the last one of every stage before the CTA leaves; a stage whose other half was never requested cannot
     // complete its phase, which the limit covers (the bytes themselves arrive within microseconds).
@@ -837,7 +834,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       mbar_wait(&full[st], (last / n_stages) & 1, nullptr, 1u << 14);
     }
   }
-  if (*abort_flag && warp == 1 && lane == 0) {     // ... and no contraction may still be running when TMEM is given back
+  if (*abort_flag && warp == 1 && elect_one()) {   // ... and no contraction may still be running when TMEM is given back
     mma_commit(drain_bar);
     mbar_wait(drain_bar, 0, nullptr, 1u << 16);
   }
