@@ -9,9 +9,8 @@
 //   * one persistent CTA per SM; the (tile, k-block) iteration space is cut into equal contiguous spans
 //     (stream-K), so every SM streams the same number of bytes whatever N and K are;
 //   * a span that covers only part of a tile's K range leaves a partial tile in scratch memory.  After its last
-//     MMA every contributor of a tile adds up a share of the tile's tokens (token t belongs to contributor
-//     t mod n) in ascending K order and runs the epilogue on them.  The partial sums carry their own arrival (see
-//     EMPTY).  A CTA waits for the others' partials only
+//     MMA every CTA adds up a share of the tokens of all such tiles, in ascending K order, and runs the epilogue on them.
+//     The partial sums carry their own arrival (see EMPTY).  A CTA waits for the others' partials only
 //     after it has published all of its own, so the waits cannot form a cycle (and they are bounded); the
 //     result does not depend on arrival order;
 //   * warp 0 issues TMA loads into a ring of shared-memory stages (128-byte swizzle), warp 1 issues
@@ -80,6 +79,7 @@ struct GemmParams {
   int kb;             // k-blocks per tile (K / 64)
   int t0, per;        // tiles below t0 are handled whole; the others are cut into spans of `per` k-blocks (ws::cut)
   int sharers, sit_out;   // CTAs that share the cut tiles where not all do (else 0), and whether the first round of whole tiles leaves them out
+  int finishers;      // CTAs (the first ones) that add up and finish the cut tiles' tokens, each a share of all of them
   int t_pad;          // tokens padded to a multiple of 16 (MMA N)
   int rows;           // valid tokens (an upper bound when rows_dev is set)
   const int *rows_dev;  // NULL, or where the block's true row count sits in device memory: the host then sizes the
@@ -143,7 +143,7 @@ struct ChainParams {
   ChainArgs args;
 };
 static_assert(sizeof(ChainParams) <= 4096, "kernel parameters");
-constexpr int MISC_BYTES = 512 + 2 * OURO_TEXT_ROWS * 4;   // barriers, flags, per-token factors and positions
+constexpr int MISC_BYTES = 512 + 2 * OURO_TEXT_ROWS * 4 + MAX_GRID * 4;   // barriers, flags, per-token factors and positions, cut tiles
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -222,8 +222,6 @@ __device__ __forceinline__ float ordered_f32(uint32_t u) {
 // x * sigmoid(x) with the fast exponential and reciprocal (the result is rounded to bf16 right after)
 __device__ __forceinline__ float silu(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
 __device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory"); }
-// one half of the epilogue warps; grp = 0 or 1
-__device__ __forceinline__ void group_barrier(int grp) { asm volatile("bar.sync %0, %1;" ::"r"(2 + grp), "n"(EPI_THREADS / 2) : "memory"); }
 // Partial sums travel between CTAs without flags: a scratch word is EMPTY until its contributor has stored the sum, and
 // whoever fetches it (exactly one thread of one CTA) empties it again.  The fetching thread polls the words themselves, so
 // a partial tile costs one store and one load latency; with a fence, an arrival counter and a poll of that in between it
@@ -296,8 +294,8 @@ __device__ __forceinline__ bool chain_wait(const ChainArgs &cp, int i) {
 
 // The kernel by the block's size.  What a GEMM executes once per CTA it mostly waits for as instructions, so that the
 // short blocks' kernel is kept short (and free of spills: a hundred bytes of them cost 4 % of a decoding step).
-enum { FEW = 0, SOME = 1, MANY = 2 };      // up to FEW_ROWS, up to 128, up to 256 rows (known text)
-constexpr int FEW_ROWS = 48;
+enum { ONE = 0, FEW = 1, SOME = 2, MANY = 3 };      // up to ONE_ROWS, FEW_ROWS, 128 and 256 rows (known text)
+constexpr int ONE_ROWS = 32, FEW_ROWS = 48;
 template <int SIZE>
 __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_constant__ ChainParams kp) {
   extern __shared__ uint8_t smem_raw[];
@@ -316,10 +314,10 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
   uint32_t *tmem_base_p = (uint32_t *)(bars + 36);
   volatile int *abort_flag = (volatile int *)(bars + 37);
   volatile int *wait_flag = (volatile int *)(bars + 39);   // [0..1]: outcome of an accumulator wait; [2]: a fix-up gave up
-  volatile int *pend = (volatile int *)(bars + 50);         // [2][4]: tile, contributors, first contributor
   uint64_t *drain_bar = bars + 44;                          // give-up path: "every contraction issued so far has completed"
   float *rs = (float *)(bars + 56);                         // [256] per-token factor 1/rms of the consumed activations
   int *spos = (int *)(rs + OURO_TEXT_ROWS);                 // [256] token positions (rotary table rows), QKV epilogue
+  uint32_t *cuts = (uint32_t *)(spos + OURO_TEXT_ROWS);     // [160] of every cut tile: first contributor | contributors << 16
 
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -528,28 +526,28 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
     const int rows = p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows;
     SpanWalker w(p);
     Span s;
-    int n_pend = 0;                                              // partial tiles this CTA contributed to (<= 2), see pend
+    // this CTA's share of the cut tiles is still to be finished  (spans as long as a tile: each is one tile, and whole)
+    bool due = p.per > 0 && p.per < p.kb && (int)blockIdx.x < p.finishers;
     float *stage = xchg;                                         // [stage_tok tokens][STAGE_PITCH] fp32, 128 tile rows each
 
     // Finishing tokens of a tile.  Whatever produced the accumulator values - this CTA's own whole tile, parked
     // in shared memory token-major, or the partial tiles of all contributors in scratch - the last step is the
-    // same: a group of G threads walks over "its" tokens, a warp's 32 lanes holding the tile's 128 rows (= output
+    // same: a warp walks over tokens, its 32 lanes holding the tile's 128 rows (= output
     // columns) four apiece, so every global access is a 16-byte piece of a contiguous 512-byte row.
-    //   whole tile:  tokens t_base + tg + TG i below t_lim (one staged chunk of tokens)
-    //   split tile:  contributor `my` of n takes the tokens t = my (mod n), that is my + n (tg + TG i), and adds the
-    //                partials up in ascending K order as they arrive
+    //   whole tile:  tokens t_base + (epilogue warp) + 8 i below t_lim (one staged chunk of tokens)
+    //   cut tile:    tb tokens from t_base on, as far as they are below t_lim; the partials are added up in ascending K order as
+    //                they arrive
     // Returns false (warp-uniform) when the wait for a partial gave up.
-    auto finish = [&](auto split_c, int tile, int gi, int G, int my, int n, int first, float *stg, int t_base, int t_lim) -> bool {
+    auto finish = [&](auto split_c, int tile, float *stg, int tbn, int t_base, int t_lim) -> bool {
       constexpr bool SPLIT = decltype(split_c)::value;
       const bool swiglu = p.mode == MODE_SWIGLU;                     // tile rows 0..63: gate of 64 features, 64..127: up
       int seg = 0, row0 = 0, col0 = 0, valid = TILE_N;
       if (!swiglu) locate(p, tile, seg, row0, col0, valid);
-      const int ng = gi & 31, tg = gi >> 5, TG = G >> 5;
+      const int ng = lane;
       const int col = col0 + 4 * ng;
       // Every matrix has a multiple of 8 output features (the shape checks see to it), so a thread's four columns are
       // inside the matrix together or not at all.
       const bool full4 = 4 * ng < valid;
-      const int js = n * TG;                                         // step between this warp's tokens
       const int cm = row0 + 4 * ng;                                  // first of this thread's 4 columns inside q, k or v
       const int half = p.head_dim >> 1;
       const bool res_norm = p.mode == MODE_RESIDUAL && p.gain != nullptr;
@@ -636,7 +634,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
 
       if constexpr (!SPLIT) {
 #pragma unroll 1
-        for (int t = t_base + tg; t < t_lim; t += TG)                // tokens are uniform inside a warp
+        for (int t = t_base + warp - 2; t < t_lim; t += EPI_WARPS)   // tokens are uniform inside a warp
           finish_token(t, *reinterpret_cast<const float4 *>(stg + (size_t)(t - t_base) * STAGE_PITCH + 4 * ng));
         return true;
       } else {
@@ -645,7 +643,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
         // up to 48 rows the shorter code is as fast or faster: 1.1B draft 4.07 -> 3.98 ms, 37 rows of 7B 3.49 ms either way).
         // With sixteen pieces the registers spill.  They are fetched without asking first whether they are there: a probe in
         // front is one more round trip to L2 between two GEMMs.
-        const int tbn = SIZE != FEW && (n <= 4 || (n <= 8 && t_lim > js)) ? 4 : 1;
+        const uint32_t of = cuts[tile - p.t0];
+        const int first = of & 0xffff, n = of >> 16;
         float *slot = stg + (size_t)(warp - 2) * 4 * TILE_N + 4 * lane;       // this thread's 16 bytes of four parked tokens
         auto gather = [&](auto tb_c, int tb) -> bool {
           constexpr int TB = decltype(tb_c)::value, CB = 12 / TB;
@@ -663,7 +662,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
                 const float *src = p.scratch + ((owner * 2 + w.owner_slot(tile, owner)) * slot_floats + tb * TILE_N + 4 * ng);
 #pragma unroll
                 for (int j = 0; j < TB; ++j)
-                  tmp[cc][j] = part_load(src + j * js * TILE_N, c0 + cc < n && tb + j * js < t_lim);
+                  tmp[cc][j] = part_load(src + j * TILE_N, c0 + cc < n && tb + j < t_lim);
               }
 #pragma unroll
               for (int cc = 0; cc < CB; ++cc)
@@ -680,7 +679,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
               float *src = p.scratch + ((owner * 2 + w.owner_slot(tile, owner)) * slot_floats + tb * TILE_N + 4 * ng);
 #pragma unroll
               for (int j = 0; j < TB; ++j) {
-                if (c0 + cc < n && tb + j * js < t_lim) part_empty(src + j * js * TILE_N);
+                if (c0 + cc < n && tb + j < t_lim) part_empty(src + j * TILE_N);
                 acc[j].x += __uint_as_float(tmp[cc][j].x); acc[j].y += __uint_as_float(tmp[cc][j].y);
                 acc[j].z += __uint_as_float(tmp[cc][j].z); acc[j].w += __uint_as_float(tmp[cc][j].w);
               }
@@ -698,46 +697,47 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
           for (int j = 0; j < TB; ++j) *reinterpret_cast<float4 *>(slot + j * TILE_N) = acc[j];
           return true;
         };
-        for (int tb = my + n * tg; tb < t_lim; tb += tbn * js) {
-          if (res_norm && full4) {
-            for (int j = 0; j < tbn && tb + j * js < t_lim; ++j)
-              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(slot + j * TILE_N)),
-                           "l"(p.out_f32 + (size_t)(tb + j * js) * p.ldo + col) : "memory");
-          }
-          if (!(SIZE != FEW && tbn == 4 ? gather(std::integral_constant<int, SIZE == FEW ? 1 : 4>{}, tb)
-                                        : gather(std::integral_constant<int, 1>{}, tb)))
-            return false;
-          if (gi == 0) TRACE(12);
-#pragma unroll 1
-          for (int j = 0; j < tbn; ++j) {
-            const int t = tb + j * js;
-            if (t < t_lim) finish_token(t, *reinterpret_cast<const float4 *>(slot + j * TILE_N));
-          }
+        if (res_norm && full4) {
+          for (int j = 0; j < tbn && t_base + j < t_lim; ++j)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(slot + j * TILE_N)),
+                         "l"(p.out_f32 + (size_t)(t_base + j) * p.ldo + col) : "memory");
         }
+        if (!(SIZE != ONE && tbn == 4 ? gather(std::integral_constant<int, SIZE == ONE ? 1 : 4>{}, t_base)
+                                      : gather(std::integral_constant<int, 1>{}, t_base)))
+          return false;
+        if (et == 0) TRACE(12);
+#pragma unroll 1
+        for (int j = 0; j < tbn && t_base + j < t_lim; ++j)
+          finish_token(t_base + j, *reinterpret_cast<const float4 *>(slot + j * TILE_N));
         return true;
       }
     };
 
-    // Partial tiles.  Called once this CTA has published all its own partials, so waiting for the others cannot
-    // form a cycle.  The (at most two) tiles are finished side by side, each by one half of the epilogue threads.
+    // Cut tiles.  Called once this CTA has published all its own partials, so waiting for the others cannot form a cycle.  The
+    // (tile, tokens) pairs of all cut tiles are dealt out to all warps of the launch: with the contributors of a tile sharing its
+    // tokens, the two tiles of a CTA whose span crosses a boundary decided how long it took (7B q,k,v, 37 rows: 7.5 us behind the
+    // last contraction, now 5.6; output projection 5.8, now 3.9; 7B step 3221 -> 3154 us, 34B shape, 8 layers, 69 rows, 2121 ->
+    // 2065 us).
     auto run_fixups = [&]() {
-      const int grp = et / (EPI_THREADS / 2), gi = et % (EPI_THREADS / 2);
-      epi_barrier();
-      if (grp < n_pend) {
-        const int tile = pend[4 * grp], n = pend[4 * grp + 1], first = pend[4 * grp + 2];
-        if (!finish(std::true_type{}, tile, gi, EPI_THREADS / 2, (int)blockIdx.x - first, n, first, stage, 0, rows))
+      const int n_cut = p.tiles - p.t0, warps = p.finishers * EPI_WARPS;
+      // one token at a time, or four where there are more tokens than warps (7B step with 37 rows 3172 -> 3152 us; the longer code
+      // costs a block that never needs it more: 19 rows of the 1.1B shape 5800 -> 5827 us, so up to ONE_ROWS there is none)
+      const int tbn = SIZE != ONE && n_cut * rows > warps ? 4 : 1, items = n_cut * ((rows + tbn - 1) / tbn);
+#pragma unroll 1
+      for (int it = (warp - 2) * p.finishers + (int)blockIdx.x; it < items; it += warps) {
+        const int group = it < n_cut ? 0 : it / n_cut;             // (one token: no division on the way to the next GEMM)
+        if (!finish(std::true_type{}, p.t0 + it - group * n_cut, stage, tbn, group * tbn, rows)) {
           wait_flag[2] = 1;
-        if (gi == 0 && grp == 0) TRACE(10);
-        if (publish) __threadfence();                                // this thread's outputs, before the tile counts as finished
-        group_barrier(grp);
-        // every contributor counts towards the hand-over itself: the GEMM is finished once all shares of all tiles
-        // are (the host passes the total), and nobody has to learn that it was the last of its tile
-        if (gi == 0 && publish && !wait_flag[2]) atomicAdd(cp.finished + ci, 1u);
+          break;
+        }
       }
-      if (gi == 0 && grp == 0) TRACE(11);
+      if (et == 0) TRACE(10);
+      if (publish) __threadfence();                                // this thread's outputs, before the CTA's share counts as finished
       epi_barrier();
+      if (et == 0 && publish && !wait_flag[2]) atomicAdd(cp.finished + ci, 1u);
+      if (et == 0) TRACE(11);
       if (wait_flag[2]) ok = false;
-      n_pend = 0;
+      due = false;
     };
 
     if (ci > 0) {
@@ -761,15 +761,19 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       spos[et] = (p.mode == MODE_QKV && et < rows) ? p.pos[et] : 0;
     }
     if (et == 0) wait_flag[2] = 0;
+    if (p.per > 0 && et < p.tiles - p.t0) {                          // (fewer cut tiles than CTAs)
+      const int first = et * p.kb / p.per;
+      cuts[et] = (uint32_t)first | (uint32_t)((et * p.kb + p.kb - 1) / p.per - first + 1) << 16;
+    }
     epi_barrier();
 
     for (;;) {
       const bool more = w.next(s);
       const int a = item & 1;
       // the stream-K spans come first: once the whole tiles start, this CTA has published all its partials and
-      // can add up its shares while the tensor cores work on the whole tile  (one call site: the routine is inlined)
+      // can add up its share while the tensor cores work on the whole tile  (one call site: the routine is inlined)
       if (!more && et == 0) TRACE(5);
-      if (n_pend > 0 && (!more || s.n_contrib == 1)) run_fixups();
+      if (due && (!more || s.n_contrib == 1)) run_fixups();
       if (!ok || !more) break;
       // one thread waits (bounded) and tells the others, so that all leave the loop together
       if (et == 0) wait_flag[a] = mbar_wait(&acc_full[a], (item >> 1) & 1, abort_flag) && !*abort_flag;
@@ -795,7 +799,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
             if (lane == 0) mbar_arrive(&acc_empty[a]);
           }
           epi_barrier();
-          finish(std::false_type{}, s.tile, et, EPI_THREADS, 0, 1, 0, stage, c0, min(c1, rows));
+          finish(std::false_type{}, s.tile, stage, 0, c0, min(c1, rows));
           if (publish && c1 == t_pad) __threadfence();
           epi_barrier();
           if (publish && c1 == t_pad && et == 0) atomicAdd(cp.finished + ci, 1u);
@@ -812,8 +816,6 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
         fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[a]);
-        if (et == 0) { pend[4 * n_pend] = s.tile; pend[4 * n_pend + 1] = s.n_contrib; pend[4 * n_pend + 2] = s.first_owner; }
-        ++n_pend;
       }
       ++item;
     }
@@ -959,6 +961,7 @@ int ouro_fast_setup(ouro_ctx *c) {
   f->s.attn_part = (float *)((char *)f->s.ss + ss_bytes());
   if (cudaMemsetAsync(f->s.slots, 0xff, slots_bytes(), c->stream) != cudaSuccess ||
       cudaMemcpyAsync(f->s.finished, f->s.finished_host, sizeof(f->s.finished_host), cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
+      cudaFuncSetAttribute(gemm_tc_kernel<ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<SOME>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
@@ -1063,13 +1066,9 @@ static int grid_for(const FastState &s, int tiles, int kb) {
   const long total = (long)tiles * kb;
   return total < s.grid ? (int)total : s.grid;
 }
-// What the hand-over counter of a GEMM reaches: one count per whole tile and one per contributor of a split tile
-// (the schedule of weight_stream.cuh, worked out on the host).
-static int finish_units(const GemmParams &g) {
-  int units = g.t0;
-  for (int rel = 0; rel < g.tiles - g.t0; ++rel) units += (rel * g.kb + g.kb - 1) / g.per - (rel * g.kb) / g.per + 1;
-  return units;
-}
+// What the hand-over counter of a GEMM advances by: one count per whole tile and one per CTA that has finished its share of the
+// cut tiles.
+static int finish_units(const GemmParams &g) { return g.per == g.kb ? g.tiles : g.t0 + (g.per > 0 ? g.finishers : 0); }
 // Launches the GEMMs collected so far as one chain.
 static void flush_chain(ouro_ctx *c) {
   FastState &s = c->fast->s;
@@ -1083,6 +1082,7 @@ static void flush_chain(ouro_ctx *c) {
     const ws::Cut cut = ws::cut(cp.g[i].tiles, cp.g[i].kb, grid, grid);
     cp.g[i].t0 = cut.t0;
     cp.g[i].per = cut.per;
+    cp.g[i].finishers = grid;
   }
   for (int i = 0; i + 1 < cp.n; ++i) cp.target[i] = (s.finished_host[i] += finish_units(cp.g[i]));
   if (cp.fold.part || cp.embed.table) cp.fold_target = (s.finished_host[MAX_CHAIN] += grid);
@@ -1091,7 +1091,9 @@ static void flush_chain(ouro_ctx *c) {
   {
     ProfScope ps(c, per_kind ? kind_class[s.chain_kind[0]] : OURO_PROF_GEMM);
     const int t_pad = cp.g[0].t_pad;
-    launch_pdl(t_pad > OURO_MAX_ROWS ? gemm_tc_kernel<MANY> : t_pad > FEW_ROWS ? gemm_tc_kernel<SOME> : gemm_tc_kernel<FEW>, grid, THREADS, (size_t)s.smem_max, c->stream, s.chain);
+    launch_pdl(t_pad > OURO_MAX_ROWS ? gemm_tc_kernel<MANY> : t_pad > FEW_ROWS ? gemm_tc_kernel<SOME>
+               : t_pad > ONE_ROWS ? gemm_tc_kernel<FEW> : gemm_tc_kernel<ONE>,
+               grid, THREADS, (size_t)s.smem_max, c->stream, s.chain);
   }
   cp.n = 0;
   cp.fold.part = nullptr;
@@ -1497,6 +1499,7 @@ extern "C" int ouro_lm_head_static(const void *x_dev, const void *lm_head_dev, i
   p.t0 = cut.t0;
   p.per = cut.per;
   p.sharers = cut_by % grid;
+  p.finishers = cut_by;
   // A sharer's pieces cost it up to a tile and the round trip of their sum: where the whole tiles need no further round
   // without it, it sits the first one out (32000 x 1024, 128 rows: 66 -> 56 us; 50000 x 8192, 37 rows: 178 -> 171 us).
   const int others = grid - p.sharers, rounds = (cut.t0 + grid - 1) / grid;

@@ -1012,6 +1012,30 @@ def test_hand_over_counters_pass_the_ends_of_their_range(monkeypatch, start):
     eng.close()
 
 
+@pytest.mark.parametrize("ffn", [9408, 9472, 9536, 1600])
+def test_cut_tiles_at_the_edges_of_their_number(ffn):
+    """Gate / up tiles of 64 features, eight k-blocks each, on 148 CTAs: 147 of them (a CTA's share of the k-blocks is a whole tile,
+    so nothing is cut), 148 (all whole), 149 (one cut into eight pieces), 25 (every CTA has a piece of two k-blocks).  One, 40 and 100 rows,
+    whose tokens are finished one or four at a time: logits against the oracle, and a row's bits do not show its block."""
+    desc = synth.ModelDesc(1, 512, 4, 2, 128, ffn, 1000, 192, "bf16")
+    P = synth.DecodeParams(4, 5, 3, 16, 8)
+    eng, W = make(desc, P, 7)
+    _verify_case(eng, W, desc, P, 7, 40, _bf16_tol)
+    tokens = np.random.default_rng(ffn).integers(0, desc.vocab, 100).astype(np.int32)
+    rows = []
+    for n in (40, 100):
+        eng.set_state(30, 1)
+        eng.assemble_causal(binding.OURO_TARGET, tokens[:n])
+        rows.append(eng.verify_forward(want_logits=True)[1][:40].clone())
+    assert torch.equal(rows[0], rows[1])
+    eng.set_state(30, 1)
+    for i in range(4):
+        eng.assemble_causal(binding.OURO_TARGET, tokens[i: i + 1])
+        assert torch.equal(eng.verify_forward(want_logits=True)[1][0], rows[0][i])
+        eng.advance(binding.OURO_TARGET, 1)
+    eng.close()
+
+
 # ------------------------------------------------- phrase generation during the draft forward (Section 3.1)
 
 def test_lookahead_window_matches_oracle_c1():
