@@ -85,14 +85,14 @@ static size_t carve(ouro_ctx *c, char *base, const ouro_model_desc *t, const our
   size_t F = mx([](const ouro_model_desc *m) { return (size_t)m->d_ffn; });
   size_t V = mx([](const ouro_model_desc *m) { return (size_t)m->vocab; });
   Activations a{};
-  // rows of a block: R, and OURO_TEXT_ROWS = 2 R where blocks of known text run on the tensor cores (16-bit activations then
-  // fill the same space)
+  // rows of a block: R of up to 32 bits, and OURO_TEXT_ROWS of 16 bits where blocks of known text run on the tensor cores
+  static_assert(OURO_TEXT_ROWS * 2 >= OURO_MAX_ROWS * 4, "32-bit activations of a candidate block fit beside");
   a.x = cv.take<float>(OURO_TEXT_ROWS * dm);
-  a.xn = cv.take<float>(R * dm);
+  a.xn = cv.take<__nv_bfloat16>(OURO_TEXT_ROWS * dm);
   a.qkv = cv.take<float>(R * dqkv);
-  a.q = cv.take<float>(R * dq);
-  a.att = cv.take<float>(R * dq);
-  a.act = cv.take<float>(R * F);
+  a.q = cv.take<__nv_bfloat16>(OURO_TEXT_ROWS * dq);
+  a.att = cv.take<__nv_bfloat16>(OURO_TEXT_ROWS * dq);
+  a.act = cv.take<__nv_bfloat16>(OURO_TEXT_ROWS * F);
   a.logits = cv.take<float>(R * V);
   a.argmax = cv.take<int32_t>(R);
   a.scratch_bytes = ouro_scratch_bytes(t, d);
@@ -558,8 +558,7 @@ extern "C" int ouro_advance(ouro_ctx *c, int which, int32_t n) {
 
 // Runs model `which` over text positions [M.L, upto) taken from seq_dev, in blocks.  With last_row the outputs of the
 // last block stay in a.argmax (row index of the last position returned through last_row); the others only leave their
-// keys and values, and are as wide as the kernels take: streaming the weights once for 256 rows costs a third more than
-// for 128.
+// keys and values, and are as wide as the kernels take.
 static int feed_text(ouro_ctx *c, int which, int upto, int *last_row) {
   ModelRt &M = c->m[which];
   const int widest = ouro_fast_available(c, which) ? (int)OURO_TEXT_ROWS : (int)OURO_MAX_ROWS;

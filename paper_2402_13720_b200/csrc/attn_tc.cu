@@ -442,7 +442,7 @@ bool attention_tc_supported(const ouro_model_desc &d) {
 size_t attention_tc_scratch_bytes(const ouro_model_desc &d) {
   if (!attention_tc_supported(d)) return 0;
   size_t cap = fold::span_count(d.head_dim, d.max_seq);
-  return (size_t)OURO_TEXT_ROWS * d.n_heads * cap * (d.head_dim + 4) * sizeof(float);
+  return (size_t)OURO_PART_ROWS * d.n_heads * cap * (d.head_dim + 4) * sizeof(float);
 }
 
 template <int HD, int MT>

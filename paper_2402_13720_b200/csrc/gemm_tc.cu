@@ -27,6 +27,8 @@
 #include "ouro_internal.h"
 #include "weight_stream.cuh"
 #include "attn_fold.cuh"
+#include "gemm_text.cuh"
+#include "row_ops.cuh"
 
 void ouro_set_global_error(const std::string &msg);   // api.cu
 
@@ -101,7 +103,7 @@ struct GemmParams {
   int head_dim, dq, dkv, L;
   const __nv_bfloat16 *gain;  // MODE_RESIDUAL: gain of the norm that follows (NULL: plain residual add)
   __nv_bfloat16 *xb;          // MODE_RESIDUAL: bf16(gain * x_new), [rows, ldo]
-  float *ss_out;              // MODE_RESIDUAL: [tiles][256] per-tile sums of squares of x_new
+  float *ss_out;              // MODE_RESIDUAL: [tiles][OURO_TEXT_ROWS] per-tile sums of squares of x_new
   const float *ss_in;         // other modes: sums of squares of the activation rows (NULL: no scaling)
   int ss_tiles;
   float ss_inv_d, eps;
@@ -127,23 +129,15 @@ struct ChainArgs {
   fold::Params fold;
   uint32_t fold_target;           // value finished[MAX_CHAIN] has once every CTA has done its share of the work in front
   // ... or the embedding rows of the block's tokens (first layer): gathered by all CTAs the same way.
-  struct Embed {
-    const __nv_bfloat16 *table;   // [vocab][d]; NULL: nothing to gather
-    const int32_t *tok;           // [rows]
-    const __nv_bfloat16 *gain;    // first norm's gain [d]
-    float *x;                     // residual stream [rows][d]
-    __nv_bfloat16 *xb;            // bf16(gain * x) [rows][d]
-    float *ss;                    // [d / 128][256] sums of squares per 128-column tile
-    const int *rows_dev;
-    int rows, d;
-  } embed;
+  rowops::Embed embed;
 };
 struct ChainParams {
   GemmMaps maps[MAX_CHAIN];
   ChainArgs args;
 };
 static_assert(sizeof(ChainParams) <= 4096, "kernel parameters");
-constexpr int MISC_BYTES = 512 + 2 * OURO_TEXT_ROWS * 4 + MAX_GRID * 4;   // barriers, flags, per-token factors and positions, cut tiles
+constexpr int MAX_CHAIN_ROWS = OURO_PART_ROWS;   // rows of a launch, the widest tcgen05 tile; more than OURO_MAX_ROWS are known text
+constexpr int MISC_BYTES = 512 + 2 * MAX_CHAIN_ROWS * 4 + MAX_GRID * 4;   // barriers, flags, per-token factors and positions, cut tiles
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -219,8 +213,6 @@ __device__ __forceinline__ uint32_t ordered_u32(float f) {
 __device__ __forceinline__ float ordered_f32(uint32_t u) {
   return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
-// x * sigmoid(x) with the fast exponential and reciprocal (the result is rounded to bf16 right after)
-__device__ __forceinline__ float silu(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
 __device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory"); }
 // Partial sums travel between CTAs without flags: a scratch word is EMPTY until its contributor has stored the sum, and
 // whoever fetches it (exactly one thread of one CTA) empties it again.  The fetching thread polls the words themselves, so
@@ -304,7 +296,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
   const GemmParams &p0 = cp.g[0];                 // rows, t_pad and stages are common to the chain
   const int n_stages = p0.stages, t_pad = p0.t_pad;
   const int b_bytes = t_pad * BLOCK_K * 2;
-  constexpr int MAX_ROWS = SIZE == MANY ? OURO_TEXT_ROWS : OURO_MAX_ROWS, stage_tok = stage_tokens(MAX_ROWS);
+  constexpr int MAX_ROWS = SIZE == MANY ? MAX_CHAIN_ROWS : OURO_MAX_ROWS, stage_tok = stage_tokens(MAX_ROWS);
   constexpr int slot_floats = MAX_ROWS * TILE_N;  // (all slots together stay below 2^31 bytes)
   const int stage_bytes = A_BYTES + b_bytes;
   uint8_t *ring = smem;
@@ -316,8 +308,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
   volatile int *wait_flag = (volatile int *)(bars + 39);   // [0..1]: outcome of an accumulator wait; [2]: a fix-up gave up
   uint64_t *drain_bar = bars + 44;                          // give-up path: "every contraction issued so far has completed"
   float *rs = (float *)(bars + 56);                         // [256] per-token factor 1/rms of the consumed activations
-  int *spos = (int *)(rs + OURO_TEXT_ROWS);                 // [256] token positions (rotary table rows), QKV epilogue
-  uint32_t *cuts = (uint32_t *)(spos + OURO_TEXT_ROWS);     // [160] of every cut tile: first contributor | contributors << 16
+  int *spos = (int *)(rs + MAX_CHAIN_ROWS);                 // [256] token positions (rotary table rows), QKV epilogue
+  uint32_t *cuts = (uint32_t *)(spos + MAX_CHAIN_ROWS);     // [160] of every cut tile: first contributor | contributors << 16
 
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -484,29 +476,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       if (cp.fold.part) {
         fold::run(cp.fold, gw, nw, lane);
       } else {
-        // Embedding rows into the residual stream, plus what the first norm's consumer needs: bf16(gain * x) and the
-        // sums of squares per 128-column tile.  One warp per (row, tile): four columns per lane.
-        const ChainArgs::Embed &e = cp.embed;
-        const int rows = e.rows_dev ? min(e.rows, __ldg(e.rows_dev)) : e.rows, tiles = (e.d + TILE_N - 1) / TILE_N;
-        for (int it = gw; it < rows * tiles; it += nw) {
-          const int r = it / tiles, col = (it - r * tiles) * TILE_N + 4 * lane;
-          float sq = 0.f;
-          if (col < e.d) {                                            // d is a multiple of 64: four columns are in or out together
-            const uint2 raw = __ldg(reinterpret_cast<const uint2 *>(e.table + (size_t)__ldg(e.tok + r) * e.d + col));
-            const uint2 graw = __ldg(reinterpret_cast<const uint2 *>(e.gain + col));
-            const __nv_bfloat162 a01 = *reinterpret_cast<const __nv_bfloat162 *>(&raw.x), a23 = *reinterpret_cast<const __nv_bfloat162 *>(&raw.y);
-            const __nv_bfloat162 g01 = *reinterpret_cast<const __nv_bfloat162 *>(&graw.x), g23 = *reinterpret_cast<const __nv_bfloat162 *>(&graw.y);
-            const float v[4] = {__low2float(a01), __high2float(a01), __low2float(a23), __high2float(a23)};
-            const float gv[4] = {__low2float(g01), __high2float(g01), __low2float(g23), __high2float(g23)};
-            *reinterpret_cast<float4 *>(e.x + (size_t)r * e.d + col) = make_float4(v[0], v[1], v[2], v[3]);
-            __nv_bfloat162 lo = __floats2bfloat162_rn(gv[0] * v[0], gv[1] * v[1]), hi = __floats2bfloat162_rn(gv[2] * v[2], gv[3] * v[3]);
-            *reinterpret_cast<uint2 *>(e.xb + (size_t)r * e.d + col) = make_uint2(*(uint32_t *)&lo, *(uint32_t *)&hi);
-            sq = (v[0] * v[0] + v[1] * v[1]) + (v[2] * v[2] + v[3] * v[3]);
-          }
-#pragma unroll
-          for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-          if (lane == 0) e.ss[(size_t)(it - r * tiles) * OURO_TEXT_ROWS + r] = sq;
-        }
+        rowops::embed(cp.embed, gw, nw, lane);
       }
       __threadfence();
       epi_barrier();
@@ -569,8 +539,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
             __nv_bfloat162 hi = __floats2bfloat162_rn(__low2float(g23) * y.z, __high2float(g23) * y.w);
             *reinterpret_cast<uint2 *>(p.xb + (size_t)t * p.ldo + col) = make_uint2(*(uint32_t *)&lo, *(uint32_t *)&hi);
           }
-          float sq = 0.f;
-          sq += y.x * y.x; sq += y.y * y.y; sq += y.z * y.z; sq += y.w * y.w;
+          float sq = rowops::squares(y.x, y.y, y.z, y.w);
 #pragma unroll
           for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
           if (lane == 0) p.ss_out[(size_t)tile * OURO_TEXT_ROWS + t] = sq;
@@ -588,7 +557,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
                                           __shfl_xor_sync(0xffffffffu, v4.z, x), __shfl_xor_sync(0xffffffffu, v4.w, x));
             if (swiglu) {
               const int feat = tile * 64 + 4 * ng;
-              v4 = make_float4(silu(v4.x) * o4.x, silu(v4.y) * o4.y, silu(v4.z) * o4.z, silu(v4.w) * o4.w);
+              v4 = make_float4(rowops::silu(v4.x) * o4.x, rowops::silu(v4.y) * o4.y, rowops::silu(v4.z) * o4.z, rowops::silu(v4.w) * o4.w);
               dst = p.out_bf16 + (size_t)t * p.a_rows[0] + feat;
               store = ng < 16 && feat < p.a_rows[0];
             } else {
@@ -596,7 +565,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
               const float4 cs = *reinterpret_cast<const float4 *>(p.cos_t + ti);
               float4 sn = *reinterpret_cast<const float4 *>(p.sin_t + ti);
               if ((cm & half) == 0) sn = make_float4(-sn.x, -sn.y, -sn.z, -sn.w);     // lower half: a cos - b sin
-              v4 = make_float4(v4.x * cs.x + o4.x * sn.x, v4.y * cs.y + o4.y * sn.y, v4.z * cs.z + o4.z * sn.z, v4.w * cs.w + o4.w * sn.w);
+              v4 = make_float4(rowops::rotate(v4.x, o4.x, cs.x, sn.x), rowops::rotate(v4.y, o4.y, cs.y, sn.y),
+                               rowops::rotate(v4.z, o4.z, cs.z, sn.z), rowops::rotate(v4.w, o4.w, cs.w, sn.w));
               dst = seg == 0 ? p.q_out + (size_t)t * p.dq + cm : p.k_out + (size_t)(p.L + t) * p.dkv + cm;
             }
           } else {
@@ -638,9 +608,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
           finish_token(t, *reinterpret_cast<const float4 *>(stg + (size_t)(t - t_base) * STAGE_PITCH + 4 * ng));
         return true;
       } else {
-        // Twelve pieces are under way together: one token of twelve contributors, or, where there are more tokens than warps
-        // and few contributors, four tokens of three (7B prefill 13.2 -> 11.9 ms, 69 rows of the 34B shape 2.155 -> 2.130 ms;
-        // up to 48 rows the shorter code is as fast or faster: 1.1B draft 4.07 -> 3.98 ms, 37 rows of 7B 3.49 ms either way).
+        // Twelve pieces are under way together: one token of twelve contributors, or, where there are more tokens than warps, four
+        // tokens of three (7B prefill 13.2 -> 11.9 ms, 69 rows of the 34B shape 2.155 -> 2.130 ms).
         // With sixteen pieces the registers spill.  They are fetched without asking first whether they are there: a probe in
         // front is one more round trip to L2 between two GEMMs.
         const uint32_t of = cuts[tile - p.t0];
@@ -749,13 +718,13 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       if (!ok) break;
       __threadfence();
     }
-    static_assert(EPI_THREADS >= OURO_TEXT_ROWS, "one thread per token");
-    if (et < OURO_TEXT_ROWS) {
+    static_assert(EPI_THREADS >= MAX_CHAIN_ROWS, "one thread per token");
+    if (et < MAX_CHAIN_ROWS) {
       float r = 1.0f;
       if (p.ss_in && et < rows) {
         float sum = 0.f;
         for (int i = 0; i < p.ss_tiles; ++i) sum += p.ss_in[(size_t)i * OURO_TEXT_ROWS + et];
-        r = 1.0f / sqrtf(sum * p.ss_inv_d + p.eps);
+        r = rowops::inv_rms(sum, p.ss_inv_d, p.eps);
       }
       rs[et] = r;
       spos[et] = (p.mode == MODE_QKV && et < rows) ? p.pos[et] : 0;
@@ -805,7 +774,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
           if (publish && c1 == t_pad && et == 0) atomicAdd(cp.finished + ci, 1u);
         }
       } else {
-        // partial tile: parked in this CTA's slot, for its contributors to fetch; added up after the loop
+        // partial tile: parked in this CTA's slot, for whoever finishes its tokens to fetch
         float *mine = p.scratch + ((int)blockIdx.x * 2 + s.slot) * slot_floats;
         for (int t0 = 16 * wh; t0 < rows; t0 += 32) {
           tmem_ld16(taddr + t0, v);
@@ -865,6 +834,7 @@ bool make_map(CUtensorMap *m, const void *base, int rows, int K, int box_rows) {
 
 struct LayerMaps {
   CUtensorMap wq, wk, wv, wo, wg, wu, wd;
+  CUtensorMap hq, hk, hv, ho, hd;       // half tiles: boxes of 64 rows, as wg and wu have them
 };
 struct FastModel {
   bool ok = false;
@@ -872,7 +842,7 @@ struct FastModel {
   CUtensorMap head;
   CUtensorMap kmap, vmap;               // K and V caches as [layers * max_seq][kv width], box 64 x 128 (tcgen05 attention)
   bool kv_maps = false;
-  CUtensorMap x_d[16], x_q[16], x_f[16];   // activations normed [256, d], attention out [256, dq], SwiGLU out [256, F]; box rows 16, 32, .., 256
+  CUtensorMap x_d[16], x_q[16], x_f[16];   // activations normed [512, d], attention out [512, dq], SwiGLU out [512, F]; box rows 16, 32, .., 256
 };
 struct FastState {
   FastModel m[2];
@@ -893,7 +863,7 @@ struct FastState {
 constexpr int MAX_TILES = 4096;
 constexpr int CHAIN_BYTES = 256;           // the chain counters
 
-size_t slots_bytes() { return (size_t)MAX_GRID * 2 * TILE_N * OURO_TEXT_ROWS * sizeof(float); }
+size_t slots_bytes() { return (size_t)MAX_GRID * 2 * TILE_N * MAX_CHAIN_ROWS * sizeof(float); }
 size_t tile_best_bytes() { return (size_t)MAX_TILES * OURO_MAX_ROWS * 4; }
 constexpr int MAX_SS_TILES = 64;           // d_model <= 8192
 size_t ss_bytes() { return (size_t)MAX_SS_TILES * OURO_TEXT_ROWS * sizeof(float); }
@@ -965,7 +935,7 @@ int ouro_fast_setup(ouro_ctx *c) {
       cudaFuncSetAttribute(gemm_tc_kernel<FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<SOME>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      attention_tc_setup() != OURO_OK || attention_tm_setup() != OURO_OK) {
+      text_gemm_setup() != OURO_OK || attention_tc_setup() != OURO_OK || attention_tm_setup() != OURO_OK) {
     delete f;
     c->err = "tensor-core GEMM set-up failed";
     return OURO_ECUDA;
@@ -983,7 +953,9 @@ int ouro_fast_setup(ouro_ctx *c) {
       ok = make_map(&lm.wq, M.wq[l], dq, d.d_model, TILE_N) && make_map(&lm.wk, M.wk[l], dkv, d.d_model, TILE_N) &&
            make_map(&lm.wv, M.wv[l], dkv, d.d_model, TILE_N) && make_map(&lm.wo, M.wo[l], d.d_model, dq, TILE_N) &&
            make_map(&lm.wg, M.w_gate[l], d.d_ffn, d.d_model, 64) && make_map(&lm.wu, M.w_up[l], d.d_ffn, d.d_model, 64) &&
-           make_map(&lm.wd, M.w_down[l], d.d_model, d.d_ffn, TILE_N);
+           make_map(&lm.wd, M.w_down[l], d.d_model, d.d_ffn, TILE_N) && make_map(&lm.hq, M.wq[l], dq, d.d_model, 64) &&
+           make_map(&lm.hk, M.wk[l], dkv, d.d_model, 64) && make_map(&lm.hv, M.wv[l], dkv, d.d_model, 64) &&
+           make_map(&lm.ho, M.wo[l], d.d_model, dq, 64) && make_map(&lm.hd, M.w_down[l], d.d_model, d.d_ffn, 64);
     }
     ok = ok && make_map(&fm.head, M.lm_head, d.vocab, d.d_model, TILE_N);
     if (ok && attention_tm_supported(d)) {
@@ -1156,6 +1128,10 @@ bool ouro_fast_available(ouro_ctx *c, int which) {
 
 bool ouro_fast_layers(ouro_ctx *c, int which) { return c->fast && c->fast->s.m[which].ok; }
 
+// Blocks that run on the kernels of gemm_text.cu: those longer than a chained launch takes.  (Up to there the chain is faster: 7B
+// shape, four layers, 129 rows 429 us and 660, 192 rows 514 and 666; 34B shape, two layers, 192 rows 369 and 418.)
+static bool text_rows(int rows) { return rows > MAX_CHAIN_ROWS; }
+
 // The embedding gather runs in front of the first layer's q,k,v GEMM, inside its launch.
 int ouro_fast_embed(ouro_ctx *c, int which, int rows) {
   if (!c->fast || !c->fast->s.m[which].ok) return OURO_ESTATE;
@@ -1163,7 +1139,7 @@ int ouro_fast_embed(ouro_ctx *c, int which, int rows) {
   ChainArgs &cp = c->fast->s.chain.args;
   cp.n = 0;
   cp.fold.part = nullptr;
-  ChainArgs::Embed &e = cp.embed;
+  rowops::Embed own, &e = text_rows(rows) ? own : cp.embed;
   e.table = (const __nv_bfloat16 *)M.embed;
   e.tok = M.blk.tok;
   e.gain = (const __nv_bfloat16 *)M.attn_norm[0];
@@ -1173,6 +1149,125 @@ int ouro_fast_embed(ouro_ctx *c, int which, int rows) {
   e.rows_dev = c->cur_rows_dev;
   e.rows = rows;
   e.d = M.d.d_model;
+  e.ss_pitch = OURO_TEXT_ROWS;
+  if (text_rows(rows)) launch_text_embed(own, c->sms, c->stream);
+  return OURO_OK;
+}
+
+// One layer of a block of known text (text_rows) on the kernels of gemm_text.cu: the same values as in
+// the decoding launches, which is why it asks where those cut a GEMM's tiles along K.
+static int text_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
+  FastState &fs = c->fast->s;
+  ModelRt &M = c->m[which];
+  FastModel &fm = fs.m[which];
+  const ouro_model_desc &d = M.d;
+  const int dq = d.n_heads * d.head_dim, dkv = d.n_kv_heads * d.head_dim;
+  Activations &a = c->a;
+  cudaStream_t s = c->stream;
+  const LayerMaps &lm = fm.layers[l];
+  static const int kind_class[4] = {OURO_PROF_QKV, OURO_PROF_WO, OURO_PROF_GATEUP, OURO_PROF_DOWN};
+  const bool per_kind = c->prof_class >= OURO_PROF_QKV && c->prof_class <= OURO_PROF_HEAD;
+  // the grid of the launch that has this GEMM while decoding: alone (the first q,k,v), or with the others of its chain
+  auto grid_of = [&](int layer, int kind) {
+    const WeightSide w = weight_side(d, fm, layer, kind);
+    return grid_for(fs, w.tiles, w.K / BLOCK_K);
+  };
+  auto chain_grid = [&](int kind) {
+    if (!fs.fuse || (kind == G_QKV && l == 0)) return grid_of(l, kind);
+    const int first = kind == G_QKV ? l - 1 : l;                  // the chain begins with this layer's output projection
+    return std::max(std::max(grid_of(first, G_WO), grid_of(first, G_GATEUP)),
+                    std::max(grid_of(first, G_DOWN), first + 1 < d.n_layers ? grid_of(first + 1, G_QKV) : grid_of(0, G_HEAD)));
+  };
+  auto gemm = [&](TextGemm &g, int kind, const CUtensorMap *xmaps) {
+    const WeightSide w = weight_side(d, fm, l, kind);
+    for (int i = 0; i < 3; ++i) { g.w_tiles[i] = w.a_tiles[i]; g.w_rows[i] = w.a_rows[i]; }
+    g.w_count = w.a_count;
+    g.tiles = w.tiles;
+    g.kb = w.K / BLOCK_K;
+    const int grid = chain_grid(kind);
+    const ws::Cut cut = ws::cut(g.tiles, g.kb, grid, grid);
+    g.t0 = cut.t0;
+    g.per = cut.per;
+    g.a = xmaps[OURO_MAX_ROWS / 16 - 1];
+    g.rows = rows;
+    g.status = &c->st->status;
+    ProfScope ps(c, per_kind ? kind_class[kind] : OURO_PROF_GEMM);
+    launch_text_gemm(g, c->sms, s);
+  };
+  auto consume = [&](TextGemm &g) { g.ss_in = fs.ss; g.ss_tiles = (d.d_model + TILE_N - 1) / TILE_N; g.ss_inv_d = 1.0f / (float)d.d_model; g.eps = d.rms_eps; };
+  auto produce = [&](TextGemm &g, const void *gain) {
+    g.mode = TEXT_RESIDUAL;
+    g.x = a.x; g.ldx = d.d_model;
+    g.gain = (const __nv_bfloat16 *)gain; g.xb = (__nv_bfloat16 *)a.xn; g.ss_out = fs.ss;
+  };
+  {
+    TextGemm g{};
+    const size_t off = (size_t)l * d.max_seq * dkv;
+    g.mode = TEXT_QKV;
+    g.w[0] = lm.hq; g.w[1] = lm.hk; g.w[2] = lm.hv;
+    consume(g);
+    g.pos = M.blk.pos; g.cos_t = M.rope_cos; g.sin_t = M.rope_sin;
+    g.q_out = (__nv_bfloat16 *)a.q;
+    g.k_out = (__nv_bfloat16 *)M.k_cache + off;
+    g.v_out = (__nv_bfloat16 *)M.v_cache + off;
+    g.head_dim = d.head_dim; g.dq = dq; g.dkv = dkv; g.L = M.L;
+    gemm(g, G_QKV, fm.x_d);
+  }
+  if (kv_only) return OURO_OK;
+  {
+    ProfScope ps(c, OURO_PROF_ATTENTION);
+    // in one launch where every row's keys lie in one span, else in parts whose pieces are folded one after the other
+    const bool direct = fold::span_count(d.head_dim, M.L + rows) <= 1;
+    for (int r0 = 0; r0 < rows; r0 += OURO_PART_ROWS) {
+      const int n = direct ? rows : std::min<int>(OURO_PART_ROWS, rows - r0);
+      BlockDev b = M.blk;
+      b.tok += r0; b.pos += r0; b.group += r0; b.lin_end += r0; b.seg_start += r0; b.seg_len += r0; b.mask += 2 * r0;
+      const __nv_bfloat16 *q = (const __nv_bfloat16 *)a.q + (size_t)r0 * dq;
+      __nv_bfloat16 *out = (__nv_bfloat16 *)a.att + (size_t)r0 * dq;
+      bool pieces;
+      if (fm.kv_maps) {
+        L2Prefetch pf;
+        if (r0 + n >= rows) { pf.ptr[0] = M.wo[l]; pf.bytes[0] = (size_t)d.d_model * dq * 2; }
+        pieces = launch_attention_tm(d, q, &fm.kmap, &fm.vmap, M.k_cache, M.v_cache, b, n, 1, M.L + r0, M.L + r0 + n, l, fs.attn_part, out,
+                                     &c->st->status, nullptr, pf, c->sms, s);
+      } else {
+        pieces = launch_attention_tc(d, q, M.k_cache, M.v_cache, b, n, M.L + r0, M.L + r0 + n, l, fs.attn_part, out, nullptr, c->sms, s);
+      }
+      if (pieces) {
+        fold::Params f{};
+        f.part = fs.attn_part;
+        f.out = out;
+        f.lin_end = b.lin_end;
+        f.seg_len = b.seg_len;
+        f.rows = n;
+        f.H = d.n_heads;
+        f.cap = fold::span_count(d.head_dim, d.max_seq);
+        f.head_dim = d.head_dim;
+        launch_text_fold(f, c->sms, s);
+      }
+      if (direct) break;
+    }
+  }
+  {
+    TextGemm g{};
+    g.w[0] = lm.ho;
+    produce(g, M.ffn_norm[l]);
+    gemm(g, G_WO, fm.x_q);
+  }
+  {
+    TextGemm g{};
+    g.mode = TEXT_SWIGLU;
+    g.w[0] = lm.wg; g.w[1] = lm.wu;
+    consume(g);
+    g.act = (__nv_bfloat16 *)a.act;
+    gemm(g, G_GATEUP, fm.x_d);
+  }
+  {
+    TextGemm g{};
+    g.w[0] = lm.hd;
+    produce(g, l + 1 < d.n_layers ? M.attn_norm[l + 1] : M.final_norm);
+    gemm(g, G_DOWN, fm.x_f);
+  }
   return OURO_OK;
 }
 
@@ -1180,6 +1275,15 @@ int ouro_fast_embed(ouro_ctx *c, int which, int rows) {
 // qualify.
 int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
   if (!c->fast || !c->fast->s.m[which].ok) return OURO_ESTATE;
+  if (text_rows(rows)) {
+    const int rc = text_layer(c, which, l, rows, kv_only);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) {
+      c->err = std::string("text layer launch: ") + cudaGetErrorString(e);
+      return OURO_ECUDA;
+    }
+    return rc;
+  }
   ModelRt &M = c->m[which];
   FastModel &fm = c->fast->s.m[which];
   const ouro_model_desc &d = M.d;

@@ -48,9 +48,13 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 #endif
 
-// Rows of a block whose outputs nobody reads: long stretches of known text on the tensor-core path.  The weights are
-// streamed once for all of them, and 256 is the widest tcgen05 tile.
-enum { OURO_TEXT_ROWS = 2 * OURO_MAX_ROWS };
+// Rows of a block whose outputs nobody reads: long stretches of known text on the tensor-core path, two units of gemm_text.cu.
+// With 256 rows its pairs of SMs had half as much to do for the output and down projections, and the weights were streamed
+// twice as often.
+enum { OURO_TEXT_ROWS = 4 * OURO_MAX_ROWS };
+
+// Rows whose attention is in per-span pieces at a time: a longer block of known text is attended to in parts of this many.
+enum { OURO_PART_ROWS = 2 * OURO_MAX_ROWS };
 
 // Device-resident scalars of one decoding stream.
 struct DevState {

@@ -1125,6 +1125,36 @@ def test_prefill_in_wide_blocks_is_bit_identical_to_short_blocks(heads, kv, hd):
     eng.close()
 
 
+@pytest.mark.parametrize("d,heads,kv,hd,ffn", [(4928, 2, 2, 64, 9536), (256, 91, 91, 64, 640), (512, 75, 25, 128, 4800)])
+def test_long_text_blocks_with_two_tiles_per_pair(d, heads, kv, hd, ffn):
+    """Prompts beyond 256 rows, widths for which a pair of SMs takes two weight tiles at a time: an odd number of tiles (the last
+    one is contracted twice), matrices whose last tile is half empty, rows up to and around the edges of a pair's 256 tokens and of its
+    two halves.  Keys and values equal, bit for bit, those left by blocks of up to 100 rows."""
+    desc = synth.ModelDesc(2, d, heads, kv, hd, ffn, 520, 560, "bf16")
+    P = synth.DecodeParams(3, 4, 2, 16, 8, seed_prompt=False)
+    eng = binding.Engine(desc, synth.model_weights(desc, 6, device="cuda:0"), P)
+    text = np.random.default_rng(6).integers(0, desc.vocab, 530).astype(np.int32)
+    eng.reset()
+    at = 0
+    while at < 520:
+        n = min(100, 520 - at)
+        eng.assemble_causal(binding.OURO_TARGET, text[at: at + n])
+        eng.verify_forward()
+        eng.advance(binding.OURO_TARGET, n)
+        at += n
+    torch.cuda.synchronize()
+    want = [c[:, :at].clone() for c in (eng.tm.k_cache, eng.tm.v_cache)]
+    assert bool(torch.isfinite(want[0].float()).all()) and float(want[1].float().abs().max()) > 0
+    for n in (258, 300, 385, 386, 513, 520):
+        eng.reset()
+        eng.tm.k_cache.zero_(); eng.tm.v_cache.zero_()
+        eng.prefill(text[:n])
+        for got, ref in zip((eng.tm.k_cache, eng.tm.v_cache), want):
+            assert torch.equal(got[:, : n - 1], ref[:, : n - 1]), n
+            assert not bool(got[:, n - 1:].any()), n
+    eng.close()
+
+
 def test_draft_catches_up_on_a_long_prompt():
     """The draft model's first block is the whole prompt, the last 128 rows of it or fewer with outputs: its drafts equal
     those of the same model as the target (self-draft), which accepts every one of them."""
