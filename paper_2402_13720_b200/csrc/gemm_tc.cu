@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
     }
   } else {
     // ---------------------------------------------------------------- epilogue warps
-    pdl_wait();
+    if (!cp.fold.part) pdl_wait();               // (the fold waits itself)
     const int q = warp & 3;                      // TMEM lane quarter this warp may read
     const int nl = q * 32 + lane;                // row of the tile held by this thread
     const int et = threadIdx.x - 64;             // 0..255 among the epilogue threads

@@ -517,7 +517,6 @@ __global__ void __launch_bounds__(256) text_embed_kernel(const rowops::Embed e) 
 // (Lets nobody start early: the attention of a second part reads, ahead of its dependency wait, cache rows that this block's
 // q,k,v GEMM has written, and that GEMM has completed once this kernel has.)
 __global__ void __launch_bounds__(256) text_fold_kernel(const fold::Params f) {
-  pdl_wait();
   fold::run(f, blockIdx.x * 8 + (threadIdx.x >> 5), gridDim.x * 8, threadIdx.x & 31);
 }
 
