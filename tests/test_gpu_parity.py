@@ -84,6 +84,25 @@ def test_pool_matches_oracle(sets, ways, beta):
     eng.close()
 
 
+@pytest.mark.parametrize("sets,ways,beta,tokens", [(1, 40, 3, 9), (64, 4, 2, 90), (256, 8, 16, 12), (32, 33, 6, 40)])
+def test_pool_takes_long_lists_in_order(sets, ways, beta, tokens):
+    """A list of phrases is shared by the warps of a block, a set's phrases staying in one warp: lists of 1 to 700 sliding windows
+    with few tokens (the same set and phrase again and again, sets that overflow), one set and more sets than warps.  Entries,
+    stamps and the counter for what follows as in the oracle, which inserts one after the other."""
+    P = synth.DecodeParams(2, beta, 3, sets, ways)
+    eng, _ = make(TINY, P)
+    ref = oracle_pool(P)
+    rng = np.random.default_rng(tokens)
+    for n in (1, 31, 32, 33, 700, 5):
+        text = rng.integers(0, tokens, n + beta - 1)
+        grams = np.stack([text[i: i + beta] for i in range(n)])
+        eng.phrase_update(grams)
+        for g in grams:
+            ref.insert(g)
+        assert gpu_pool_rows(eng) == pool_rows(ref), n
+    eng.close()
+
+
 # ------------------------------------------------------------------------- candidate packing
 
 @pytest.mark.parametrize("gamma,beta,K,n_fill", [(4, 4, 4, 60), (3, 9, 4, 80), (2, 3, 0, 10), (5, 6, 3, 0), (1, 2, 16, 50)])
