@@ -5,7 +5,8 @@
 // by the number of keys it sees and by where its last keys live, and keys are addressed by "virtual position".
 //
 // Work split.  Keys are cut by virtual position into spans of four chunks (attn_fold.cuh); one CTA handles one (span,
-// kv head) for a round of up to 128 query rows (block rows x query heads of the group, ordered group by group).  It walks
+// kv head) for a round of up to 128 query rows (block rows x query heads of the group, ordered group by group); of a span that
+// holds keys of the block itself, several CTAs may each take some of the groups.  It walks
 // the span in chunks of 128 keys.  Per chunk:
 //     S = Q K^T      one 128 x 128 x 128 tcgen05 contraction into TMEM (Q and K K-major in 128-byte swizzle),
 //     softmax        the threads of query row t read its 128 scores from TMEM, mask by virtual position, keep a
