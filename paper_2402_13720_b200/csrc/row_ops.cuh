@@ -49,7 +49,8 @@ __device__ __forceinline__ void embed(const Embed &e, int first, int step, int l
       const float2 a = unpack(raw.x), b = unpack(raw.y), ga = unpack(graw.x), gb = unpack(graw.y);
       *reinterpret_cast<float4 *>(e.x + (size_t)r * e.d + col) = make_float4(a.x, a.y, b.x, b.y);
       *reinterpret_cast<uint2 *>(e.xb + (size_t)r * e.d + col) = make_uint2(pack(ga.x * a.x, ga.y * a.y), pack(gb.x * b.x, gb.y * b.y));
-      sq = squares(a.x, a.y, b.x, b.y);
+      // (bf16 values: each square is exact in 32 bits, and this is their sum two by two, however it is contracted)
+      sq = __fadd_rn(__fmaf_rn(a.x, a.x, __fmul_rn(a.y, a.y)), __fmaf_rn(b.x, b.x, __fmul_rn(b.y, b.y)));
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);

@@ -1174,6 +1174,70 @@ def test_long_text_blocks_with_two_tiles_per_pair(d, heads, kv, hd, ffn):
     eng.close()
 
 
+def _round_bf16(x):
+    u = np.asarray(x, dtype=np.float32).view(np.uint32)
+    return ((u + 0x7fff + ((u >> 16) & 1)) & 0xffff0000).astype(np.uint32).view(np.float32)
+
+
+@pytest.mark.parametrize("rows", [16, 200, 300, 512])
+def test_norm_factor_of_an_embedding_row_to_the_last_bit(rows):
+    """The first norm divides by the root of a sum of squares over 128-column tiles, added up two by two in 32 bits: the columns of a
+    group of four, then the 32 groups in halves, then the tiles in order.  Embeddings for which this sum and one along the columns of a
+    group give neighbouring factors; values in front of the norm (single weights on columns that are one, so no sum can round) that
+    land on different sides of a bf16 rounding with the two.  Gathered by the chained launch (16 and 200 rows) and by the kernel of
+    long blocks."""
+    d, kv, n_tok, per_tok = 512, 4, 16, 16
+    rng = np.random.default_rng(1)
+    x = _round_bf16(rng.standard_normal((20000, d)).astype(np.float32))
+    x[:, :3] = 1
+    sq = (x * x).reshape(-1, d // 128, 32, 4)
+
+    def factor(groups):
+        i = np.arange(32)
+        for o in (16, 8, 4, 2, 1):
+            groups = groups + groups[..., i ^ o]
+        total = np.zeros(len(groups), dtype=np.float32)
+        for tile in range(groups.shape[1]):
+            total = total + groups[:, tile, 0]
+        return np.float32(1) / np.sqrt((total.astype(np.float64) / d + np.float64(np.float32(1e-5))).astype(np.float32))
+
+    by_twos = factor((sq[..., 0] + sq[..., 1]) + (sq[..., 2] + sq[..., 3]))
+    in_a_row = factor(((sq[..., 0] + sq[..., 1]) + sq[..., 2]) + sq[..., 3])
+    pick = np.flatnonzero(by_twos != in_a_row)[:n_tok]
+    assert len(pick) == n_tok
+    values = []
+    for t in pick:
+        found = 0
+        while found < per_tok:
+            middle = np.float32(1 + (2 * int(rng.integers(0, 128)) + 1) / 256)         # between two bf16 values
+            near = (middle / by_twos[t]).view(np.int32) + np.arange(-6, 7, dtype=np.int32)
+            near = near.view(np.float32)
+            split = _round_bf16(near * by_twos[t]) != _round_bf16(near * in_a_row[t])
+            if split.any():
+                values.append(near[split][0])
+                found += 1
+    values = np.array(values, dtype=np.float32)                                       # one per feature of the values: 16 per token
+    desc = synth.ModelDesc(1, d, kv, kv, 64, 64, 64, 600, "bf16")
+    w = synth.model_weights(desc, 1, device="cuda:0")
+    w["embed"].zero_()
+    w["embed"][:n_tok] = torch.as_tensor(x[pick], device="cuda:0").bfloat16()
+    lw = w["layers"][0]
+    lw["attn_norm"].fill_(1)
+    lw["wv"].zero_()
+    rest = values.copy()
+    for column in range(3):                                                           # 24 bits in three bf16 weights
+        part = _round_bf16(rest)
+        lw["wv"][:, column] = torch.as_tensor(part, device="cuda:0").bfloat16()
+        rest = rest - part
+    assert not rest.any()
+    eng = binding.Engine(desc, w, synth.DecodeParams(3, 4, 2, 16, 8, seed_prompt=False))
+    text = np.resize(np.arange(n_tok, dtype=np.int32), rows + 1)
+    eng.prefill(text)
+    got = eng.tm.v_cache[0, :rows].reshape(rows, -1).float().cpu().numpy()
+    assert np.array_equal(got, _round_bf16(values[None, :] * by_twos[pick][text[:rows], None]))
+    eng.close()
+
+
 def test_draft_catches_up_on_a_long_prompt():
     """The draft model's first block is the whole prompt, the last 128 rows of it or fewer with outputs: its drafts equal
     those of the same model as the target (self-draft), which accepts every one of them."""
