@@ -18,6 +18,7 @@
 
 #include "ouro_internal.h"
 #include "generic.cuh"
+#include "row_ops.cuh"
 
 namespace {
 
@@ -265,8 +266,8 @@ __global__ void __launch_bounds__(THREADS, 1) forward_small_kernel(const __grid_
         const float a = of_row<RT>(acc[0], lane), b = of_row<RT>(acc[1], lane);
         float ra = a, rb = b;
         if (!is_v) {
-          ra = a * c - b * s;
-          rb = b * c + a * s;
+          ra = rowops::rotate(a, b, c, -s);
+          rb = rowops::rotate(b, a, c, s);
         }
         T *dst = is_q ? q + (size_t)r * dq + hh * h
                       : (T *)(is_v ? p.v_cache : p.k_cache) + layer_off + (size_t)(p.L + r) * dkv + hh * h;

@@ -1291,6 +1291,33 @@ def test_one_launch_forward_matches_oracle_and_single_kernels(dtype, d, heads, k
     eng.close()
 
 
+@pytest.mark.parametrize("heads,kv,hd", [(4, 2, 32), (3, 1, 128)])
+def test_one_launch_forward_rotates_as_spelled_out(heads, kv, hd):
+    """A rotated pair (a, b) of a key is (a c - b s, b c + a s) with the second product of each rounded first and the first one fused into
+    the sum.  With the key weights equal to the value weights the value cache holds the pair in front of the rotation: keys to the
+    last bit, one row per unit, two and eight."""
+    desc = synth.ModelDesc(2, 72, heads, kv, hd, 104, 1000, 400, "f32")
+    w = synth.model_weights(desc, 3, device="cuda:0")
+    for lw in w["layers"]:
+        lw["wk"].copy_(lw["wv"])
+    eng = binding.Engine(desc, w, synth.DecodeParams(3, 4, 2, 16, 8, seed_prompt=False))
+    text = np.random.default_rng(3).integers(0, desc.vocab, 139).astype(np.int32)
+    at = 0
+    for n in (1, 10, 128):
+        eng.assemble_causal(binding.OURO_TARGET, text[at: at + n])
+        eng.verify_forward()
+        eng.advance(binding.OURO_TARGET, n)
+        at += n
+    half = hd // 2
+    v = eng.tm.v_cache[:, :at].cpu().numpy()
+    angle = np.arange(at)[:, None] * np.power(desc.rope_theta, -np.arange(half) / half)
+    c, s = (f(angle).astype(np.float32)[None, :, None, :] for f in (np.cos, np.sin))
+    a, b = v[..., :half], v[..., half:]
+    want = np.concatenate([(a.astype(np.float64) * c - (b * s)).astype(np.float32), (b.astype(np.float64) * c + (a * s)).astype(np.float32)], -1)
+    assert np.array_equal(eng.tm.k_cache[:, :at].cpu().numpy(), want)
+    eng.close()
+
+
 def test_one_launch_forward_with_scores_that_overflow():
     """Keys so large that a whole group's scores are -infinity in fp32 have the weight zero, whichever of the four warps of a row
     walks the group and whether it comes first, alone or last there.  wk = wq makes the cached key of the row itself its
