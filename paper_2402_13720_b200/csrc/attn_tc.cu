@@ -58,6 +58,7 @@ struct AttnParams {
   const __nv_bfloat16 *k, *v;      // this layer's cache: [max_seq][Hkv*HD]
   const int32_t *lin_end, *seg_start, *seg_len, *group;
   int rows, H, Hkv, L, cap;        // L: cache length before the block; cap: span slots per (row, head)
+  int ready;                       // cache rows that were complete before the forward began (all an early fetch may touch); <= L
   int rounds;                      // rounds of query rows per 128 block rows
   int in_waves;                    // the grid's order, see launch_attention_tc
   float scale_log2;
@@ -148,7 +149,8 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
   // Everything up to pdl_wait() reads only what was complete before the forward pass began: the block description
   // (the kernel that assembles it waits for what came before and lets nobody start early: it does not trigger its
   // dependents, launched programmatically or not, and so has finished when the forward's first kernel begins) and cache rows
-  // below the cache length.  The queries and the block's own K/V rows come from the kernel just before this one.
+  // below p.ready, the cache length in front of the whole block.  The queries and the block's own K/V rows come from the q,k,v
+  // GEMM, the kernel just before this one or, for a later part of a long block, before the parts in front of it.
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sc = p.in_waves ? gridDim.z - 1 - blockIdx.z : blockIdx.x, kvh = p.in_waves ? blockIdx.x : blockIdx.y;
   const int rnd = p.in_waves ? blockIdx.y : blockIdx.z;
@@ -217,10 +219,11 @@ __global__ void __launch_bounds__(THREADS) attn_span_kernel(const AttnParams p) 
     if (!__syncthreads_or(any_row)) return;            // nobody in this round reaches the span
     const int n_mt = (min(QR, M_all - m0) + 15) >> 4;  // row tiles that hold query rows; the others are skipped
 
-    if (zb == 0) stage_common(0, 0);                    // chunk 0 (its rows below the cache length) is on its way ...
+    const bool early = min(L, span0 + CH) <= p.ready;   // (uniform: one span and one part per CTA)
+    if (early) stage_common(0, 0);                      // chunk 0 (its rows below the cache length) is on its way ...
     TRACE(1);
     pdl_wait();                                         // ... while the previous kernel finishes
-    if (zb != 0) stage_common(0, 0);
+    if (!early) stage_common(0, 0);
     TRACE(2);
     for (int idx = threadIdx.x; idx < QR * CPR; idx += THREADS) {
       int row = idx / CPR, ch = idx % CPR, m = m0 + row;
@@ -455,7 +458,7 @@ int attention_tc_setup() {
 
 // n_vis_max: an upper bound of the number of keys any row of the block sees (cache length + rows).
 bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_cache, const void *v_cache, const BlockDev &b,
-                         int rows, int L, int n_vis_max, int layer, float *part, void *out, const int *rows_dev, int sms, cudaStream_t s) {
+                         int rows, int L, int ready, int n_vis_max, int layer, float *part, void *out, const int *rows_dev, int sms, cudaStream_t s) {
   OURO_COUNT_LAUNCH();
   AttnParams p;
   p.rows_dev = rows_dev;
@@ -464,7 +467,7 @@ bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_
   p.k = (const __nv_bfloat16 *)k_cache + off;
   p.v = (const __nv_bfloat16 *)v_cache + off;
   p.lin_end = b.lin_end; p.seg_start = b.seg_start; p.seg_len = b.seg_len; p.group = b.group;
-  p.rows = rows; p.H = d.n_heads; p.Hkv = d.n_kv_heads; p.L = L;
+  p.rows = rows; p.H = d.n_heads; p.Hkv = d.n_kv_heads; p.L = L; p.ready = ready;
   p.cap = fold::span_count(d.head_dim, d.max_seq);
   p.scale_log2 = 1.4426950408889634f / sqrtf((float)d.head_dim);
   p.part = part;

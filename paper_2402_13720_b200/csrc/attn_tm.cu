@@ -95,6 +95,7 @@ struct TmParams {
   const __nv_bfloat16 *k, *v;      // this layer's cache: [max_seq][Hkv*HD]
   const int32_t *lin_end, *seg_start, *seg_len, *group;
   int rows, H, Hkv, L, cap, row0;  // row0: first row of this layer in the tensor maps
+  int ready;                       // cache rows that were complete before the forward began (all an early fetch may touch); <= L
   int n_spans;
   int own_spans, slices;           // spans that hold keys of the block itself (the last ones), and CTAs that share their groups
   float scale_log2;
@@ -266,7 +267,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
   // Everything up to pdl_wait() reads only what was complete before the forward pass began: the block description
   // (the kernel that assembles it waits for what came before and lets nobody start early: it does not trigger its
   // dependents, launched programmatically or not, and so has finished when the forward's first kernel begins) and cache rows
-  // below the cache length.  The queries and the block's own K/V rows come from the kernel just before this one.
+  // below p.ready, the cache length in front of the whole block.  The queries and the block's own K/V rows come from the q,k,v
+  // GEMM, the kernel just before this one or, for a later part of a long block, before the parts in front of it.
 
   // ---- groups are contiguous row ranges: find their first rows (warps 0-3, one block row per thread)
   bool start = false;
@@ -343,8 +345,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
     ms->n_items = n;
   }
   __syncthreads();
-  // ---- every pass gets a K/V stage of its own (pass i: stage i % 2); tiles of chunks wholly below the cache
-  //      length can start streaming in before the previous kernel has finished
+  // ---- every pass gets a K/V stage of its own (pass i: stage i % 2); tiles of chunks wholly in front of the block can
+  //      start streaming in before the previous kernel has finished
   auto request_tile = [&](int i, int ci) {
     const int st = i & 1;
     mbar_expect_tx(&ms->full[st], 2 * TILE);
@@ -357,7 +359,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
   int early = 0;                                       // passes whose tile was requested before the wait
   if (warp == 0) {
     const int n = ms->n_items;
-    while (early < 2 && early < n && ((ms->items[early] >> 3) & 63) == 63 && span0 + (ms->items[early] & 7) * CH + CH <= p.L) {
+    while (early < 2 && early < n && ((ms->items[early] >> 3) & 63) == 63 && span0 + (ms->items[early] & 7) * CH + CH <= p.ready) {
       if (elect_one()) request_tile(early, ms->items[early] & 7);
       ++early;
     }
@@ -694,7 +696,7 @@ int attention_tm_setup() {
 // 64 x 128 box in 128-byte swizzle.  Returns true when the spans still have to be folded (attn_fold.cuh: by the kernel
 // that consumes the attention output); with a single span the kernel has written `out` itself.
 bool launch_attention_tm(const ouro_model_desc &d, const void *q, const void *kmap, const void *vmap, const void *k_cache,
-                         const void *v_cache, const BlockDev &b, int rows, int groups, int L, int n_vis_max, int layer, float *part,
+                         const void *v_cache, const BlockDev &b, int rows, int groups, int L, int ready, int n_vis_max, int layer, float *part,
                          void *out, int *status, const int *rows_dev, const L2Prefetch &pf, int sms, cudaStream_t s) {
   OURO_COUNT_LAUNCH();
   TmParams p;
@@ -710,7 +712,7 @@ bool launch_attention_tm(const ouro_model_desc &d, const void *q, const void *km
   p.k = (const __nv_bfloat16 *)k_cache + off;
   p.v = (const __nv_bfloat16 *)v_cache + off;
   p.lin_end = b.lin_end; p.seg_start = b.seg_start; p.seg_len = b.seg_len; p.group = b.group;
-  p.rows = rows; p.H = d.n_heads; p.Hkv = d.n_kv_heads; p.L = L;
+  p.rows = rows; p.H = d.n_heads; p.Hkv = d.n_kv_heads; p.L = L; p.ready = ready;
   p.cap = fold::span_count(HD, d.max_seq);
   p.row0 = layer * d.max_seq;
   p.scale_log2 = 1.4426950408889634f / sqrtf((float)d.head_dim);

@@ -1228,10 +1228,10 @@ static int text_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
       if (fm.kv_maps) {
         L2Prefetch pf;
         if (r0 + n >= rows) { pf.ptr[0] = M.wo[l]; pf.bytes[0] = (size_t)d.d_model * dq * 2; }
-        pieces = launch_attention_tm(d, q, &fm.kmap, &fm.vmap, M.k_cache, M.v_cache, b, n, 1, M.L + r0, M.L + r0 + n, l, fs.attn_part, out,
+        pieces = launch_attention_tm(d, q, &fm.kmap, &fm.vmap, M.k_cache, M.v_cache, b, n, 1, M.L + r0, M.L, M.L + r0 + n, l, fs.attn_part, out,
                                      &c->st->status, nullptr, pf, c->sms, s);
       } else {
-        pieces = launch_attention_tc(d, q, M.k_cache, M.v_cache, b, n, M.L + r0, M.L + r0 + n, l, fs.attn_part, out, nullptr, c->sms, s);
+        pieces = launch_attention_tc(d, q, M.k_cache, M.v_cache, b, n, M.L + r0, M.L, M.L + r0 + n, l, fs.attn_part, out, nullptr, c->sms, s);
       }
       if (pieces) {
         fold::Params f{};
@@ -1333,11 +1333,11 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
         pf.ptr[2] = M.w_up[l]; pf.bytes[2] = head;
       }
       pieces = launch_attention_tm(d, a.q, &c->fast->s.m[which].kmap, &c->fast->s.m[which].vmap, M.k_cache, M.v_cache, M.blk, rows,
-                                   M.blk_is_candidate ? 1 + std::max(1, c->p.K) : 1, M.L, M.L + rows, l, c->fast->s.attn_part, a.att,
+                                   M.blk_is_candidate ? 1 + std::max(1, c->p.K) : 1, M.L, M.L, M.L + rows, l, c->fast->s.attn_part, a.att,
                                    &c->st->status, c->cur_rows_dev, pf, c->sms, s);
     }
     else if (attention_tc_supported(d))
-      pieces = launch_attention_tc(d, a.q, M.k_cache, M.v_cache, M.blk, rows, M.L, M.L + rows, l, c->fast->s.attn_part, a.att,
+      pieces = launch_attention_tc(d, a.q, M.k_cache, M.v_cache, M.blk, rows, M.L, M.L, M.L + rows, l, c->fast->s.attn_part, a.att,
                                    c->cur_rows_dev, c->sms, s);
     else
       launch_attention_simple(d, a.q, M.k_cache, M.v_cache, M.blk, rows, l, a.att, s);

@@ -514,8 +514,6 @@ __global__ void __launch_bounds__(256) text_embed_kernel(const rowops::Embed e) 
   pdl_wait();
   rowops::embed(e, blockIdx.x * 8 + (threadIdx.x >> 5), gridDim.x * 8, threadIdx.x & 31);
 }
-// (Lets nobody start early: the attention of a second part reads, ahead of its dependency wait, cache rows that this block's
-// q,k,v GEMM has written, and that GEMM has completed once this kernel has.)
 __global__ void __launch_bounds__(256) text_fold_kernel(const fold::Params f) {
   fold::run(f, blockIdx.x * 8 + (threadIdx.x >> 5), gridDim.x * 8, threadIdx.x & 31);
 }

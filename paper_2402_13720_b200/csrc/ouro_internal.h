@@ -239,9 +239,11 @@ int launch_forward_small(ouro_ctx *c, int which, int rows, const int *rows_dev, 
 bool attention_tc_supported(const ouro_model_desc &d);
 size_t attention_tc_scratch_bytes(const ouro_model_desc &d);
 int attention_tc_setup();
-// Both return true when the spans still have to be folded by the kernel that consumes `out` (attn_fold.cuh).
+// Both return true when the spans still have to be folded by the kernel that consumes `out` (attn_fold.cuh).  L: cache length in
+// front of the given rows.  ready: cache rows that were complete before the forward began, which are read ahead of the dependency
+// wait (less than L where the rows are a later part of a block: those between come from the block's own q,k,v GEMM).
 bool launch_attention_tc(const ouro_model_desc &d, const void *q, const void *k_cache, const void *v_cache, const BlockDev &b,
-                         int rows, int L, int n_vis_max, int layer, float *part, void *out, const int *rows_dev, int sms, cudaStream_t s);
+                         int rows, int L, int ready, int n_vis_max, int layer, float *part, void *out, const int *rows_dev, int sms, cudaStream_t s);
 
 // ---- attn_tm.cu (tcgen05 path, head dim 128) ---------------------------------------------------
 bool attention_tm_supported(const ouro_model_desc &d);
@@ -254,5 +256,5 @@ struct L2Prefetch {
   size_t bytes[3] = {0, 0, 0};
 };
 bool launch_attention_tm(const ouro_model_desc &d, const void *q, const void *kmap, const void *vmap, const void *k_cache,
-                         const void *v_cache, const BlockDev &b, int rows, int groups, int L, int n_vis_max, int layer, float *part,
+                         const void *v_cache, const BlockDev &b, int rows, int groups, int L, int ready, int n_vis_max, int layer, float *part,
                          void *out, int *status, const int *rows_dev, const L2Prefetch &pf, int sms, cudaStream_t s);

@@ -1238,6 +1238,46 @@ def test_norm_factor_of_an_embedding_row_to_the_last_bit(rows):
     eng.close()
 
 
+@pytest.mark.parametrize("heads,kv,hd,ffn", [(2, 1, 128, 704), (32, 32, 128, 704), (6, 3, 128, 4800), (256, 1, 128, 64), (8, 2, 64, 704)])
+def test_long_text_block_behind_a_short_cache(heads, kv, hd, ffn):
+    """A draft model that has cached 1 to 300 tokens catches up on a text that ends beyond 512: one block of more than 256 rows, whose
+    attention runs in two parts, the first of which sees one span of keys (nothing to fold) up to a cache of 256.  Keys and values equal,
+    bit for bit, those left by blocks of up to 100 rows, and no read comes ahead of the block's own keys: what stands in the cache
+    before is large and finite."""
+    desc = synth.ModelDesc(3, 256, heads, kv, hd, ffn, 520, 830, "bf16")
+    P = synth.DecodeParams(3, 4, 2, 16, 8, seed_prompt=False)
+    w = synth.model_weights(desc, 6, device="cuda:0")
+    eng = binding.Engine(dataclasses.replace(desc, n_layers=1), w, P, desc, w)
+    text = np.random.default_rng(6).integers(0, desc.vocab, 780).astype(np.int32)
+
+    def cache(begin, end, most=100):
+        while begin < end:
+            n = min(most, end - begin)
+            eng.assemble_causal(binding.OURO_DRAFT, text[begin: begin + n])
+            eng.verify_forward(binding.OURO_DRAFT)
+            eng.advance(binding.OURO_DRAFT, n)
+            begin += n
+
+    eng.reset()
+    cache(0, 767)
+    torch.cuda.synchronize()
+    want = [c[:, :767].clone() for c in (eng.dm.k_cache, eng.dm.v_cache)]
+    assert bool(torch.isfinite(want[0].float()).all()) and float(want[1].float().abs().max()) > 0
+    for L in (1, 100, 200, 255, 256, 257, 300):
+        for n in (513, 600, 767):
+            if n - L <= 257:
+                continue
+            for turn in range(20 if heads < 256 else 2):
+                eng.reset()
+                cache(0, L)
+                eng.dm.k_cache[:, L:].fill_(30 + turn); eng.dm.v_cache[:, L:].fill_(-30 - turn)
+                eng.prefill(text[:n])
+                eng.draft()
+                for got, ref in zip((eng.dm.k_cache, eng.dm.v_cache), want):
+                    assert torch.equal(got[:, :n], ref[:, :n]), (L, n, turn)
+    eng.close()
+
+
 def test_draft_catches_up_on_a_long_prompt():
     """The draft model's first block is the whole prompt, the last 128 rows of it or fewer with outputs: its drafts equal
     those of the same model as the target (self-draft), which accepts every one of them."""
