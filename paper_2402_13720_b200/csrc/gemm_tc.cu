@@ -1216,16 +1216,19 @@ static int text_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
   if (kv_only) return OURO_OK;
   {
     ProfScope ps(c, OURO_PROF_ATTENTION);
-    // in one launch where every row's keys lie in one span, else in parts whose pieces are folded one after the other
-    const bool direct = fold::span_count(d.head_dim, M.L + rows) <= 1;
+    // in one launch where every row's keys lie in one span, else in parts whose pieces are folded one after the other.  A cache
+    // longer than the fold can take has no room for pieces in the workspace: the generic kernel, as in the decoding launches.
+    const bool spans = attention_tc_supported(d), direct = !spans || fold::span_count(d.head_dim, M.L + rows) <= 1;
     for (int r0 = 0; r0 < rows; r0 += OURO_PART_ROWS) {
       const int n = direct ? rows : std::min<int>(OURO_PART_ROWS, rows - r0);
       BlockDev b = M.blk;
       b.tok += r0; b.pos += r0; b.group += r0; b.lin_end += r0; b.seg_start += r0; b.seg_len += r0; b.mask += 2 * r0;
       const __nv_bfloat16 *q = (const __nv_bfloat16 *)a.q + (size_t)r0 * dq;
       __nv_bfloat16 *out = (__nv_bfloat16 *)a.att + (size_t)r0 * dq;
-      bool pieces;
-      if (fm.kv_maps) {
+      bool pieces = false;
+      if (!spans) {
+        launch_attention_simple(d, q, M.k_cache, M.v_cache, b, n, l, out, s);
+      } else if (fm.kv_maps) {
         L2Prefetch pf;
         if (r0 + n >= rows) { pf.ptr[0] = M.wo[l]; pf.bytes[0] = (size_t)d.d_model * dq * 2; }
         pieces = launch_attention_tm(d, q, &fm.kmap, &fm.vmap, M.k_cache, M.v_cache, b, n, 1, M.L + r0, M.L, M.L + r0 + n, l, fs.attn_part, out,

@@ -1278,6 +1278,32 @@ def test_long_text_block_behind_a_short_cache(heads, kv, hd, ffn):
     eng.close()
 
 
+@pytest.mark.parametrize("heads,kv,hd", [(4, 2, 64), (2, 1, 128)])
+def test_long_text_blocks_in_a_cache_beyond_the_span_kernels(heads, kv, hd):
+    """A cache of more than 16384 positions is attended to by the generic kernel, which leaves no pieces (and has no room for them):
+    blocks of 257 to 512 rows of a prompt too.  Keys and values equal, bit for bit, those left by blocks of up to 100 rows."""
+    desc = synth.ModelDesc(2, 256, heads, kv, hd, 704, 520, 16500, "bf16")
+    P = synth.DecodeParams(3, 4, 2, 16, 8, seed_prompt=False)
+    eng, _ = make(desc, P, 6)
+    text = np.random.default_rng(6).integers(0, desc.vocab, 900).astype(np.int32)
+    eng.reset()
+    for at in range(0, 900, 100):
+        eng.assemble_causal(binding.OURO_TARGET, text[at: at + 100])
+        eng.verify_forward()
+        eng.advance(binding.OURO_TARGET, 100)
+    torch.cuda.synchronize()
+    want = [c[:, :900].clone() for c in (eng.tm.k_cache, eng.tm.v_cache)]
+    assert bool(torch.isfinite(want[0].float()).all()) and float(want[1].float().abs().max()) > 0
+    for n in (258, 513, 600, 900):
+        eng.reset()
+        eng.tm.k_cache.zero_(); eng.tm.v_cache.zero_()
+        eng.prefill(text[:n])
+        for got, ref in zip((eng.tm.k_cache, eng.tm.v_cache), want):
+            assert torch.equal(got[:, : n - 1], ref[:, : n - 1]), n
+            assert not bool(got[:, n - 1:].any()), n
+    eng.close()
+
+
 def test_draft_catches_up_on_a_long_prompt():
     """The draft model's first block is the whole prompt, the last 128 rows of it or fewer with outputs: its drafts equal
     those of the same model as the target (self-draft), which accepts every one of them."""
