@@ -506,7 +506,7 @@ static int forward(ouro_ctx *c, int which, int32_t *argmax_dev, float *logits_de
     }
     { ProfScope ps(c, OURO_PROF_ROPE); launch_rope_append(d, a.qkv, M.blk.pos, M.rope_cos, M.rope_sin, rows, L, l, a.q, M.k_cache, M.v_cache, s); }
     if (kv_only) break;
-    { ProfScope ps(c, OURO_PROF_ATTENTION); launch_attention_simple(d, a.q, M.k_cache, M.v_cache, M.blk, rows, l, a.att, s); }
+    { ProfScope ps(c, OURO_PROF_ATTENTION); launch_attention_simple(d, a.q, M.k_cache, M.v_cache, M.blk, rows, c->cur_rows_dev, l, a.att, s); }
     {
       ProfScope ps(c, OURO_PROF_WO);
       GemmSegs wo{{M.wo[l], nullptr, nullptr}, {d.d_model, 0, 0}, 1};

@@ -1227,7 +1227,7 @@ static int text_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
       __nv_bfloat16 *out = (__nv_bfloat16 *)a.att + (size_t)r0 * dq;
       bool pieces = false;
       if (!spans) {
-        launch_attention_simple(d, q, M.k_cache, M.v_cache, b, n, l, out, s);
+        launch_attention_simple(d, q, M.k_cache, M.v_cache, b, n, nullptr, l, out, s);
       } else if (fm.kv_maps) {
         L2Prefetch pf;
         if (r0 + n >= rows) { pf.ptr[0] = M.wo[l]; pf.bytes[0] = (size_t)d.d_model * dq * 2; }
@@ -1343,7 +1343,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
       pieces = launch_attention_tc(d, a.q, M.k_cache, M.v_cache, M.blk, rows, M.L, M.L, M.L + rows, l, c->fast->s.attn_part, a.att,
                                    c->cur_rows_dev, c->sms, s);
     else
-      launch_attention_simple(d, a.q, M.k_cache, M.v_cache, M.blk, rows, l, a.att, s);
+      launch_attention_simple(d, a.q, M.k_cache, M.v_cache, M.blk, rows, c->cur_rows_dev, l, a.att, s);
     if (pieces) {                    // folded by the output projection's launch, all its CTAs taking part
       fold::Params &f = c->fast->s.chain.args.fold;
       f.part = c->fast->s.attn_part;

@@ -195,12 +195,12 @@ void launch_rope_append(const ouro_model_desc &d, const float *qkv, const int32_
 // = p mod 32), mapped to cache slots by the row's two ranges, so a suffix token sees the same key order
 // it would see in plain decoding.  Online softmax across groups in ascending order.
 template <typename T>
-__global__ void attention_simple_kernel(const T *q, const T *k_cache, const T *v_cache, BlockDev b, int H, int Hkv,
+__global__ void attention_simple_kernel(const T *q, const T *k_cache, const T *v_cache, BlockDev b, const int *rows_dev, int H, int Hkv,
                                         int h, size_t layer_off, float scale, T *out) {
   extern __shared__ float sq[];  // [warps][h]
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int r = blockIdx.x, a = blockIdx.y * (blockDim.x >> 5) + warp;
-  if (a >= H) return;
+  if (a >= H || (rows_dev && r >= *rows_dev)) return;      // nobody has described the rows beyond the block's true count
   int kvh = a / (H / Hkv), dkv = Hkv * h;
   float *myq = sq + warp * h;
   for (int i = lane; i < h; i += 32) myq[i] = to_f<T>(q[(size_t)r * H * h + a * h + i]);
@@ -249,7 +249,7 @@ __global__ void attention_simple_kernel(const T *q, const T *k_cache, const T *v
     if (dd < nd) out[(size_t)r * H * h + a * h + lane + 32 * dd] = from_f<T>(o[dd] * inv);
 }
 void launch_attention_simple(const ouro_model_desc &d, const void *q, const void *k_cache, const void *v_cache,
-                             const BlockDev &b, int rows, int layer, void *out, cudaStream_t s) {
+                             const BlockDev &b, int rows, const int *rows_dev, int layer, void *out, cudaStream_t s) {
   OURO_COUNT_LAUNCH();
   size_t off = (size_t)layer * d.max_seq * d.n_kv_heads * d.head_dim;
   int warps = 4;
@@ -258,9 +258,9 @@ void launch_attention_simple(const ouro_model_desc &d, const void *q, const void
   float scale = 1.0f / sqrtf((float)d.head_dim);
   if (d.dtype == OURO_BF16)
     attention_simple_kernel<__nv_bfloat16><<<grid, warps * 32, smem, s>>>((const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k_cache,
-                                                                          (const __nv_bfloat16 *)v_cache, b, d.n_heads, d.n_kv_heads,
+                                                                          (const __nv_bfloat16 *)v_cache, b, rows_dev, d.n_heads, d.n_kv_heads,
                                                                           d.head_dim, off, scale, (__nv_bfloat16 *)out);
   else
-    attention_simple_kernel<float><<<grid, warps * 32, smem, s>>>((const float *)q, (const float *)k_cache, (const float *)v_cache, b,
+    attention_simple_kernel<float><<<grid, warps * 32, smem, s>>>((const float *)q, (const float *)k_cache, (const float *)v_cache, b, rows_dev,
                                                                   d.n_heads, d.n_kv_heads, d.head_dim, off, scale, (float *)out);
 }

@@ -229,7 +229,7 @@ void launch_rope_append(const ouro_model_desc &d, const float *qkv, const int32_
                         const float *sin_t, int rows, int L, int layer, void *q, void *k_cache, void *v_cache,
                         cudaStream_t s);
 void launch_attention_simple(const ouro_model_desc &d, const void *q, const void *k_cache, const void *v_cache,
-                             const BlockDev &b, int rows, int layer, void *out, cudaStream_t s);
+                             const BlockDev &b, int rows, const int *rows_dev, int layer, void *out, cudaStream_t s);
 
 // ---- forward_small.cu ----------------------------------------------------------------------------
 bool forward_small_supported(const ouro_model_desc &d);

@@ -1304,6 +1304,31 @@ def test_long_text_blocks_in_a_cache_beyond_the_span_kernels(heads, kv, hd):
     eng.close()
 
 
+@pytest.mark.parametrize("heads,kv,hd", [(4, 2, 64), (2, 1, 128)])
+def test_candidates_fewer_than_the_launch_is_sized_for_in_a_cache_beyond_the_span_kernels(heads, kv, hd):
+    """The forward of a candidate block is launched for the largest block; a fresh context's first block finds one phrase of eight, and
+    nobody has described the other rows.  The generic attention kernel, which serves caches of more than 16384 positions, leaves them
+    out.  The rows that are there equal, bit for bit, the same tokens decoded one by one."""
+    desc = synth.ModelDesc(2, 256, heads, kv, hd, 704, 520, 16500, "bf16")
+    P = synth.DecodeParams(4, 9, 8, 4, 8)
+    eng, _ = make(desc, P, 6)
+    rng = np.random.default_rng(6)
+    d = [3, 1, 4, 15]
+    eng.set_state(0, 9)
+    eng.phrase_update(np.concatenate([[15], rng.integers(0, desc.vocab, 8)]))
+    eng.assemble_candidates(draft=d)
+    packed = eng.verify_forward(want_logits=True)[1][:13].clone()
+    assert bool(torch.isfinite(packed).all())
+    tok = eng.block_get()[0]
+    assert len(tok) == 13
+    eng.set_state(0, 9)
+    for r in range(13):
+        eng.assemble_causal(binding.OURO_TARGET, [int(tok[r])])
+        assert torch.equal(eng.verify_forward(want_logits=True)[1][0], packed[r]), r
+        eng.advance(binding.OURO_TARGET, 1)
+    eng.close()
+
+
 def test_draft_catches_up_on_a_long_prompt():
     """The draft model's first block is the whole prompt, the last 128 rows of it or fewer with outputs: its drafts equal
     those of the same model as the target (self-draft), which accepts every one of them."""
