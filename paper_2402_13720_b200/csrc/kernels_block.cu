@@ -393,10 +393,7 @@ __global__ void __launch_bounds__(ACCEPT_THREADS) accept_compact_harvest_kernel(
       const int32_t token = i < A ? v.tok[1 + max(i, 0)] : i < A + m ? v.tok[suffix + i - A] : bonus;
       const int32_t value = t == 0 ? A : t == 1 ? v.chosen : t == 2 ? m : t == 3 ? n : t < 4 + ACC ? token : t == 4 + ACC ? status : v.n_cand;
       const bool live = t < 4 + n || t >= 4 + ACC;
-      if (mbox && live) {
-        mbox[MBOX_ACCEPT + 1 + t] = value;
-        __threadfence_system();
-      }
+      if (mbox && live) mbox[MBOX_ACCEPT + 1 + t] = value;
       if (live && t != 4 + ACC) (&st->A)[t] = value;
       if (t >= 4 && t < 4 + n) {
         seq_dev[n_seq + i] = token;
@@ -405,7 +402,11 @@ __global__ void __launch_bounds__(ACCEPT_THREADS) accept_compact_harvest_kernel(
     }
     __syncthreads();
     if (t == 0) {
-      if (mbox) *(volatile int32_t *)(mbox + MBOX_ACCEPT) = seq;     // what the host is polling for: behind the payload
+      if (mbox) {
+        // what the host is polling for: behind the words of all threads, which the barrier has put in front of this fence
+        __threadfence_system();
+        *(volatile int32_t *)(mbox + MBOX_ACCEPT) = seq;
+      }
       st->pending = bonus;
       st->n_seq = n_seq + n;
       int k = 0;
