@@ -742,7 +742,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       // the stream-K spans come first: once the whole tiles start, this CTA has published all its partials and
       // can add up its share while the tensor cores work on the whole tile  (one call site: the routine is inlined)
       if (!more && et == 0) TRACE(5);
-      if (due && (!more || s.n_contrib == 1)) run_fixups();
+      if (due && (!more || s.whole)) run_fixups();
       if (!ok || !more) break;
       // one thread waits (bounded) and tells the others, so that all leave the loop together
       if (et == 0) wait_flag[a] = mbar_wait(&acc_full[a], (item >> 1) & 1, abort_flag) && !*abort_flag;
@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
       if (et == 0) TRACE(4);                       // overwritten per item: the last accumulator's arrival remains
       fence_after_sync();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + a * acc_cols;
-      if (s.n_contrib == 1) {
+      if (s.whole) {
         // whole tile: the accumulators go to shared memory token-major, stage_tok tokens at a time, and are finished
         // from there; the TMEM buffer is handed back as soon as it has been read
         for (int c0 = 0; c0 < t_pad; c0 += stage_tok) {

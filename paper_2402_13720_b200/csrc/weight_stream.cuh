@@ -11,7 +11,8 @@ constexpr int TILE_N = 128;       // weight rows per tile (MMA M)
 constexpr int BLOCK_K = 64;       // bf16 elements per k-block: one 128-byte swizzle row
 
 struct Span {  // one piece of a CTA's work: k-blocks [kb0, kb1) of `tile`
-  int tile, kb0, kb1, n_contrib, slot, first_owner;
+  int tile, kb0, kb1, slot;
+  bool whole;                     // all of the tile's k-blocks: no partial sum
 };
 
 // Work of one CTA.  The last R = tiles mod grid tiles are cut stream-K fashion into equal contiguous spans of
@@ -43,8 +44,7 @@ struct SpanWalker {
       s.tile = t0 + rel;
       s.kb0 = it - rel * kb;
       s.kb1 = min(kb, s.kb0 + (end - it));
-      s.first_owner = (rel * kb) / per;
-      s.n_contrib = (rel * kb + kb - 1) / per - s.first_owner + 1;
+      s.whole = s.kb0 == 0 && s.kb1 == kb;
       s.slot = owner_slot(s.tile, cta);                      // first or last piece of this CTA
       it += s.kb1 - s.kb0;
       return true;
@@ -53,9 +53,8 @@ struct SpanWalker {
       s.tile = whole;
       s.kb0 = 0;
       s.kb1 = kb;
-      s.n_contrib = 1;
+      s.whole = true;
       s.slot = 0;
-      s.first_owner = cta;
       whole += step;
       step = grid;
       return true;
