@@ -107,10 +107,10 @@ __device__ __forceinline__ void mma_pair(uint32_t tmem_d, uint64_t da, uint64_t 
       "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// Arrives on the barrier at this place in both CTAs once every contraction issued so far has completed.
-__device__ __forceinline__ void mma_commit_pair(uint64_t *bar) {
+// Arrives on the barrier at this place in both CTAs (or those of the mask) once every contraction issued so far has completed.
+__device__ __forceinline__ void mma_commit_pair(uint64_t *bar, uint16_t ctas = 3) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
-               "h"((uint16_t)3)
+               "h"(ctas)
                : "memory");
 }
 // 16 columns of this warp's lane quarter
@@ -498,8 +498,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS<WT>, 1) gemm
   fence_before_sync();
   __syncthreads();
   if (*abort_flag && warp == 1 && rank == 0 && elect_one()) {          // ... and no contraction may still be running
-    mma_commit_pair(&drain_bar);
+    mma_commit_pair(&drain_bar, 1);                // (this CTA's barrier alone: the other one may be about to leave)
     mbar_wait(&drain_bar, 0, nullptr, 1u << 16);
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);                    // the last arrivals in the other CTA land within microseconds
   }
   __syncwarp();
   cluster_sync();
