@@ -16,7 +16,8 @@
 // (ws::cut): the contraction goes on into another accumulator at each cut, and the thread that owns (token, tile) adds the pieces
 // up in its registers in ascending order, while the next piece is being contracted.
 // Two threads share a token's 128 columns of a tile, 16 columns each in turn: dimensions 32 or 64 apart - rotary pairs, gate and
-// up - are in one thread, and each holds 64 sums (with all 128 in one thread 1.2 KB of them were spilled).
+// up - are in one thread, and each holds 64 sums (with all 128 in one thread 1.2 KB of them were spilled).  The kernel with two tiles
+// per pair has 576 threads of 96 registers and still spills (300 bytes stored, 432 loaded); the one with a single tile does not.
 //
 // Warp 0 fetches (TMA; weights before, activations after the dependency wait), warp 1 of the pair's first CTA contracts, the
 // others drain and finish: eight warps per weight tile.  Every mbarrier wait is bounded; on expiry the CTA raises the status word and

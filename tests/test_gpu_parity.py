@@ -958,7 +958,7 @@ def _partial_tile_slots(eng):
 @pytest.mark.parametrize("heads,kv,hd", [(8, 2, 64), (4, 2, 128)])
 def test_every_launch_leaves_the_partial_tile_slots_empty(heads, kv, hd):
     """A scratch word counts as arrived when it is anything but EMPTY, so whoever fetches a sum empties the word again.
-    After forwards of every kernel size (up to 48, 128 and 256 rows, whose slots are laid out differently), with the row count
+    After forwards of every kernel size (up to 32, 48, 128 and 256 rows, whose slots are laid out differently), with the row count
     on the device or on the host, and after whole loops, no word may be left full."""
     desc = synth.ModelDesc(2, 256, heads, kv, hd, 704, 1000, 700, "bf16")
     P = synth.DecodeParams(4, 9, 4, 16, 8)
@@ -1116,7 +1116,7 @@ def test_lookahead_window_bf16_self_draft():
 
 @pytest.mark.parametrize("heads,kv,hd", [(4, 2, 128), (8, 2, 64)])
 def test_prefill_in_wide_blocks_is_bit_identical_to_short_blocks(heads, kv, hd):
-    """Prompts beyond 128 tokens are prefilled up to 256 rows at a time, without the LM head and the last layer's second
+    """Prompts beyond 128 tokens are prefilled up to 512 rows at a time, without the LM head and the last layer's second
     half.  A token's keys and values must not show it: they equal, bit for bit, those left by blocks of 1 to 100 rows.
     Lengths around the block edges, one that ends a span of 512 keys, and one with a one-row rest."""
     desc = synth.ModelDesc(3, 512, heads, kv, hd, 704, 1024, 900, "bf16")
