@@ -1129,10 +1129,10 @@ bool ouro_fast_available(ouro_ctx *c, int which) {
 bool ouro_fast_layers(ouro_ctx *c, int which) { return c->fast && c->fast->s.m[which].ok; }
 
 // Blocks that run on the kernels of gemm_text.cu: those longer than a chained launch takes.  Up to there the chain is faster, beyond
-// it would take two.  A prompt's prefill in us with the
-// chain and with gemm_text.cu: 7B shape, four layers, 193 rows 501 and 656, 256 rows 569 and 665, 257
-// rows 862 and 800, 300 rows 927 and 829, 512 rows 1228 and 912; 34B shape, two layers, 256 rows 430 and 454, 257 rows 683 and 610; 1.1B
-// shape, four layers, 256 rows 375 and 410, 257 rows 493 and 480.
+// it would take two.  A prompt's prefill in us with the chain and with gemm_text.cu: 7B shape, four layers, 193 rows 501 and 656, 256
+// rows 569 and 665, 257 rows 862 and 800, 300 rows 927 and 829, 512 rows 1228 and 912; 34B shape, two layers, 256 rows 430 and 454, 257
+// rows 683 and 610; 1.1B shape, four layers, 256 rows 375 and 410, 257 rows 493 and 480; two layers of 512 x 512, 256 rows 106 and 108,
+// 257 rows 136 and 99.  The widest shapes gain last: 70B, two layers, 257 rows 932 and 963, 384 rows 1035 and 1061, 512 rows 1238 and 1118.
 static bool text_rows(int rows) { return rows > MAX_CHAIN_ROWS; }
 
 // The embedding gather runs in front of the first layer's q,k,v GEMM, inside its launch.
