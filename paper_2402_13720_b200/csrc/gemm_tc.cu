@@ -935,7 +935,7 @@ int ouro_fast_setup(ouro_ctx *c) {
       cudaFuncSetAttribute(gemm_tc_kernel<FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<SOME>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      text_gemm_setup() != OURO_OK || attention_tc_setup() != OURO_OK || attention_tm_setup() != OURO_OK) {
+      text_gemm_setup() != OURO_OK || attention_tc_setup() != OURO_OK || attention_tm_setup() != OURO_OK || attention_few_setup() != OURO_OK) {
     delete f;
     c->err = "tensor-core GEMM set-up failed";
     return OURO_ECUDA;
@@ -1338,7 +1338,14 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
         pf.ptr[1] = M.w_gate[l]; pf.bytes[1] = head;
         pf.ptr[2] = M.w_up[l]; pf.bytes[2] = head;
       }
-      pieces = launch_attention_tm(d, a.q, &c->fast->s.m[which].kmap, &c->fast->s.m[which].vmap, M.k_cache, M.v_cache, M.blk, rows,
+      // Rows in order that fill one small tile: in one span its chunks side by side are faster than attn_tm_kernel's one behind
+      // the other (one row behind 150 keys, three 7B layers 289 -> 285 us, two of 512 62.7 -> 59.2; behind 400 keys 300 and 300,
+      // 69.0 -> 62.6).  With more spans they are not (three 7B layers behind 1800 keys 310 -> 322: the CTAs of several spans are the
+      // ones that share the HBM with the weights on their way to the next kernel).
+      if (!M.blk_is_candidate && attention_few_supported(d, rows) && fold::span_count(d.head_dim, M.L + rows) <= 1)
+        pieces = launch_attention_few(d, a.q, M.k_cache, M.v_cache, M.blk, rows, M.L, M.L + rows, l, c->fast->s.attn_part, a.att, c->cur_rows_dev, pf, s);
+      else
+        pieces = launch_attention_tm(d, a.q, &c->fast->s.m[which].kmap, &c->fast->s.m[which].vmap, M.k_cache, M.v_cache, M.blk, rows,
                                    M.blk_is_candidate ? 1 + std::max(1, c->p.K) : 1, M.L, M.L, M.L + rows, l, c->fast->s.attn_part, a.att,
                                    &c->st->status, c->cur_rows_dev, pf, c->sms, s);
     }

@@ -258,3 +258,9 @@ struct L2Prefetch {
 bool launch_attention_tm(const ouro_model_desc &d, const void *q, const void *kmap, const void *vmap, const void *k_cache,
                          const void *v_cache, const BlockDev &b, int rows, int groups, int L, int ready, int n_vis_max, int layer, float *part,
                          void *out, int *status, const int *rows_dev, const L2Prefetch &pf, int sms, cudaStream_t s);
+
+// ---- attn_few.cu (mma.sync, head dim 128, rows in order without candidates) ---------------------
+bool attention_few_supported(const ouro_model_desc &d, int rows);
+int attention_few_setup();
+bool launch_attention_few(const ouro_model_desc &d, const void *q, const void *k_cache, const void *v_cache, const BlockDev &b, int rows, int ready,
+                          int n_vis_max, int layer, float *part, void *out, const int *rows_dev, const L2Prefetch &pf, cudaStream_t s);

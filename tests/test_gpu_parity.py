@@ -1578,3 +1578,46 @@ def test_groups_shared_by_several_ctas_are_bit_identical_to_plain_decoding(kv, K
             assert torch.equal(eng.verify_forward(want_logits=True)[1][0], packed[r]), (j, r)
             eng.advance(binding.OURO_TARGET, 1)
     eng.close()
+
+
+# ------------------------------------------------------------------ a handful of rows
+
+@pytest.mark.parametrize("d,heads,kv,hd,ffn,vocab", [
+    (512, 4, 2, 128, 512, 1000),          # one unit per CTA, every GEMM in pieces of one k-block; half a unit of the vocabulary
+    (320, 5, 5, 64, 9536, 520),           # heads that leave half a tile of every matrix empty; nine units per CTA, one tile cut beside whole ones
+    (2048, 32, 4, 64, 5632, 64000),       # pieces taken in turn, more of them than warps share (q,k,v) and fewer; three passes of the head
+    (2048, 32, 32, 64, 512, 4104),        # three units per CTA that no tile holds together
+    (1024, 8, 8, 128, 24576, 1000),       # activations of 48 KB, three passes of seven units, twenty pieces
+    (7168, 8, 8, 128, 512, 1000),         # four units per CTA, two warps each
+    (4096, 32, 32, 128, 11008, 1000),     # a layer beyond the single row's kernels
+])
+def test_few_rows_are_bit_identical_to_wider_blocks(d, heads, kv, hd, ffn, vocab):
+    """Up to 16 query rows of a kv head without candidates have attention kernels of their own (head dim 128, one span).  A
+    token's logits, choice, keys and values must not show which: blocks of 1, 2, 5, 8, 9 and 16 rows against one block of 40,
+    behind 490 keys, so that the rows pass the end of a span."""
+    desc = synth.ModelDesc(1 if d > 2048 else 2, d, heads, kv, hd, ffn, vocab, 640, "bf16")
+    w = synth.model_weights(desc, 5, device="cuda:0")
+    eng = binding.Engine(desc, w, synth.DecodeParams(4, 5, 3, 16, 8))
+    k, v = synth.kv_fill(desc, 1, 490, device="cuda:0")
+    eng.tm.k_cache.copy_(k)
+    eng.tm.v_cache.copy_(v)
+    tokens = np.random.default_rng(d).integers(0, vocab, 40).astype(np.int32)
+
+    def run(n):
+        eng.set_state(490, 1)
+        argmax, logits = [], []
+        for at in range(0, 40, n):
+            part = tokens[at: at + n]
+            eng.assemble_causal(binding.OURO_TARGET, part)
+            am, lg = eng.verify_forward(want_logits=True)
+            argmax.append(am[: len(part)].clone())
+            logits.append(lg[: len(part)].clone())
+            eng.advance(binding.OURO_TARGET, len(part))
+        return torch.cat(argmax), torch.cat(logits), eng.tm.k_cache[:, :530].clone(), eng.tm.v_cache[:, :530].clone()
+
+    want = run(40)
+    assert bool(want[1].isfinite().all()) and float(want[1].std()) > 0
+    for n in (1, 2, 5, 8, 9, 16):
+        for got, ref in zip(run(n), want):
+            assert torch.equal(got, ref), n
+    eng.close()
