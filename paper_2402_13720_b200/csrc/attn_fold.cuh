@@ -10,6 +10,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "row_ops.cuh"
+
 namespace fold {
 
 // The spans, by absolute position.  Head dim 64 (mma.sync kernel): the first 1024 keys in spans of one chunk of 128, since a
@@ -54,11 +56,21 @@ __device__ __forceinline__ void store_bf16(__nv_bfloat16 *dst, const float4 &a, 
 __device__ __forceinline__ void store_bf16(__nv_bfloat16 *dst, const float2 &a, float s) {
   *reinterpret_cast<__nv_bfloat162 *>(dst) = __floats2bfloat162_rn(a.x * s, a.y * s);
 }
+// One row's output as packets (row_ops.cuh) instead of `out`: this lane's dims, from dim `at` on (a pair of lanes fills a packet
+// where a lane has two).
+struct Packets { uint4 *dst; uint32_t mark; };
+__device__ __forceinline__ void put(const Packets &k, size_t at, const float4 &a, float s) {
+  rowops::put_packet(k.dst + at / 4, rowops::pack(a.x * s, a.y * s), rowops::pack(a.z * s, a.w * s), 0u, k.mark);
+}
+__device__ __forceinline__ void put(const Packets &k, size_t at, const float2 &a, float s) {
+  const uint32_t lo = rowops::pack(a.x * s, a.y * s), hi = __shfl_down_sync(0xffffffffu, lo, 1);
+  if (at % 4 == 0) rowops::put_packet(k.dst + at / 4, lo, hi, 0u, k.mark);
+}
 
 // Pairs first, first + step, .. (pair = row * H + head).  Lane c fetches the maxima and sums of spans c and c + 32 while
 // every lane fetches its dims of up to UNR spans: one round trip to L2 up to 16 spans, then one more per 16.
-template <int HD>
-__device__ __forceinline__ void pairs(const Params &p, int rows, int first, int step, int lane, int keys) {
+template <int HD, bool PACKETS>
+__device__ __forceinline__ void pairs(const Params &p, int rows, int first, int step, int lane, int keys, const Packets &k) {
   typedef typename Dims<HD>::V V;
   constexpr int PW = PIECE<HD>, DPL = HD / 32, UNR = 16;
   const int n_pairs = rows * p.H;
@@ -97,18 +109,20 @@ __device__ __forceinline__ void pairs(const Params &p, int rows, int first, int 
         add_scaled(acc, o[cc], w);
       }
     }
-    store_bf16(p.out + (size_t)q * HD + DPL * lane, acc, 1.0f / l);
+    if constexpr (PACKETS) put(k, (size_t)q * HD + DPL * lane, acc, 1.0f / l);
+    else store_bf16(p.out + (size_t)q * HD + DPL * lane, acc, 1.0f / l);
   }
 }
 
 // The dependency wait is in here: what a warp needs to know of the block (its rows, the keys its first pair sees) was written
 // before the forward pass began and is fetched ahead of it (1.1B draft 3235 -> 3212 us).
-__device__ __forceinline__ void run(const Params &p, int first, int step, int lane) {
+template <bool PACKETS = false>
+__device__ __forceinline__ void run(const Params &p, int first, int step, int lane, const Packets &k = Packets()) {
   const int r = min(first / p.H, p.rows - 1);
   const int rows = p.rows_dev ? min(p.rows, __ldg(p.rows_dev)) : p.rows, keys = p.lin_end[r] + p.seg_len[r];
   pdl_wait();
-  if (p.head_dim == 128) pairs<128>(p, rows, first, step, lane, keys);
-  else pairs<64>(p, rows, first, step, lane, keys);
+  if (p.head_dim == 128) pairs<128, PACKETS>(p, rows, first, step, lane, keys, k);
+  else pairs<64, PACKETS>(p, rows, first, step, lane, keys, k);
 }
 
 }  // namespace fold

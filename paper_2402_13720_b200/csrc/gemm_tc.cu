@@ -817,6 +817,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc_kernel(const __grid_consta
 }
 
 // ------------------------------------------------------------------------------- host side
+#include "gemm_rows.cuh"
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
                                   const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -832,12 +834,44 @@ bool make_map(CUtensorMap *m, const void *base, int rows, int K, int box_rows) {
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// A matrix for the boxes of gemm_rows.cuh: rows of K values as [K / 64][rows][64], or, where a unit holds rotary pairs, as
+// [K / 64][halves of heads][rows of a half][64].
+bool make_map_rows(CUtensorMap *m, const void *base, int rows, int K, int box_rows, int nkb) {
+  cuuint64_t dims[3] = {BLOCK_K, (cuuint64_t)rows, (cuuint64_t)(K / BLOCK_K)};
+  cuuint64_t strides[2] = {(cuuint64_t)K * 2, BLOCK_K * 2};
+  cuuint32_t box[3] = {BLOCK_K, (cuuint32_t)box_rows, (cuuint32_t)nkb};
+  cuuint32_t es[3] = {1, 1, 1};
+  return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+bool make_map_pairs(CUtensorMap *m, const void *base, int rows, int K, int half, int nkb) {
+  cuuint64_t dims[4] = {BLOCK_K, (cuuint64_t)half, (cuuint64_t)(rows / half), (cuuint64_t)(K / BLOCK_K)};
+  cuuint64_t strides[3] = {(cuuint64_t)K * 2, (cuuint64_t)half * K * 2, BLOCK_K * 2};
+  cuuint32_t box[4] = {BLOCK_K, 8, 2, (cuuint32_t)nkb};
+  cuuint32_t es[4] = {1, 1, 1, 1};
+  return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 struct LayerMaps {
   CUtensorMap wq, wk, wv, wo, wg, wu, wd;
   CUtensorMap hq, hk, hv, ho, hd;       // half tiles: boxes of 64 rows, as wg and wu have them
 };
+// What launches of gemm_rows.cuh need of a model: per kind of GEMM how it is dealt out, and its boxes.
+enum { G_QKV = 0, G_WO = 1, G_GATEUP = 2, G_DOWN = 3, G_HEAD = 4 };
+struct RowsModel {
+  int x_bytes = 0;                    // (0: none)
+  int slot = 0;                       // bytes of a ring slot
+  rows_gemm::Plan plan[5];
+  CUtensorMap head;
+  struct Layer { CUtensorMap q, k, v, o, g, u, d; };
+  std::vector<Layer> layers;
+};
 struct FastModel {
   bool ok = false;
+  RowsModel rm;
   std::vector<LayerMaps> layers;
   CUtensorMap head;
   CUtensorMap kmap, vmap;               // K and V caches as [layers * max_seq][kv width], box 64 x 128 (tcgen05 attention)
@@ -856,6 +890,10 @@ struct FastState {
   uint32_t *finished = nullptr; // [MAX_CHAIN + 1] finished-tile counters of the chained GEMMs (device)
   uint32_t finished_host[MAX_CHAIN + 1] = {0, 0, 0, 0, 0};   // the values those counters have once everything launched so far is done
   ChainParams chain{};          // GEMMs collected for the next launch
+  int chain_layer[MAX_CHAIN] = {0, 0, 0, 0}, chain_model = 0;
+  uint4 *packets = nullptr;     // activations on their way: normed, attention out, SwiGLU out  (gemm_rows.cuh)
+  uint32_t mark = 1;            // of the next launch's first packets
+  float *squares = nullptr;     // squares of four columns each of the residual stream, as gemm_rows.cuh leaves them
   int chain_kind[MAX_CHAIN] = {0, 0, 0, 0};
   bool fuse = true;             // run consecutive GEMMs as one launch
   long pf_ffn_rows = 0;         // rows of gate and of up the attention kernel prefetches into L2 besides the output projection (< 0: nothing)
@@ -866,6 +904,21 @@ constexpr int CHAIN_BYTES = 256;           // the chain counters
 size_t slots_bytes() { return (size_t)MAX_GRID * 2 * TILE_N * MAX_CHAIN_ROWS * sizeof(float); }
 size_t tile_best_bytes() { return (size_t)MAX_TILES * OURO_MAX_ROWS * 4; }
 constexpr int MAX_SS_TILES = 64;           // d_model <= 8192
+// A token's activations, the widest of them, in the shared memory of a CTA of gemm_rows.cuh; 0: the model's single rows do not run
+// there.  What those kernels save is the latency between a layer's GEMMs, what they cost is a chain of steps per weight row, and the
+// wider a layer, the more the stream of its weights hides of either.  One row behind 150 / 400 / 1800 keys, us a forward, gemm_tc.cu
+// and here: two layers of 512 (4 MB a layer) 59, 63, 65 and 45, 48, 48; eight of the 1.1B shape (88 MB) 304, 305, 342 and 259, 259,
+// 298; six of 2048 x 8192 (121 MB) 260, 261, 290 and 240, 240, 268; six of 2560 x 6912 (137 MB) 279, 280, 308 and 250, 251, 278;
+// four of 3072 x 8192 (201 MB) 239, 255, 269 and 241, 247, 248; three of the 7B shape (405 MB) 285, 300, 322 and 290, 304, 325.
+int rows_x_bytes(const ouro_model_desc &d) {
+  const int dq = d.n_heads * d.head_dim, dkv = d.n_kv_heads * d.head_dim, x = 2 * std::max(std::max(d.d_model, dq), d.d_ffn);
+  const size_t layer = 2 * (size_t)d.d_model * (2 * (size_t)(dq + dkv) + 3 * (size_t)d.d_ffn);
+  return (d.head_dim == 64 || d.head_dim == 128) && layer <= (size_t)160 << 20 && x <= rows_gemm::MAX_X ? x : 0;
+}
+size_t squares_bytes() { return (size_t)MAX_SS_TILES * (TILE_N / 4) * sizeof(float); }
+size_t packets_bytes(const ouro_model_desc &d) {
+  return (size_t)(d.d_model + d.n_heads * d.head_dim + d.d_ffn) / 4 * sizeof(uint4);
+}
 size_t ss_bytes() { return (size_t)MAX_SS_TILES * OURO_TEXT_ROWS * sizeof(float); }
 
 int stages_for(int t_pad, int smem_max) {
@@ -882,13 +935,62 @@ struct ouro_fast { FastState s; };
 size_t ouro_scratch_bytes(const ouro_model_desc *t, const ouro_model_desc *d) {
   size_t attn = attention_tc_scratch_bytes(*t);
   if (d && attention_tc_scratch_bytes(*d) > attn) attn = attention_tc_scratch_bytes(*d);
-  return slots_bytes() + CHAIN_BYTES + 2 * tile_best_bytes() + ss_bytes() + attn;
+  const size_t packets = std::max(packets_bytes(*t), d ? packets_bytes(*d) : 0);
+  return slots_bytes() + CHAIN_BYTES + 2 * tile_best_bytes() + ss_bytes() + squares_bytes() + packets + attn;
 }
 
 static bool shape_ok(const ouro_model_desc &d) {
   int dq = d.n_heads * d.head_dim;
   return d.dtype == OURO_BF16 && d.d_model % 64 == 0 && d.d_model <= MAX_SS_TILES * TILE_N && dq % 64 == 0 && d.d_ffn % 64 == 0 && d.vocab % 8 == 0 &&
          (d.vocab + TILE_N - 1) / TILE_N <= MAX_TILES && (2 * d.d_ffn + TILE_N - 1) / TILE_N <= MAX_TILES;
+}
+
+// How a GEMM is dealt out to the CTAs, and how many k-blocks a ring slot holds.
+static rows_gemm::Plan rows_plan(int kind, int units, int kb, int tiles, int grid, int slot) {
+  rows_gemm::Plan pl{};
+  const int chunk = (units + grid - 1) / grid;
+  pl.units = units;
+  pl.passes = (chunk + rows_gemm::MAX_UP - 1) / rows_gemm::MAX_UP;
+  pl.up = (chunk + pl.passes - 1) / pl.passes;
+  const ws::Cut cut = ws::cut(tiles, kb, std::min(grid, tiles * kb), std::min(grid, tiles * kb));
+  const bool in_turn = cut.t0 == 0 && cut.per < kb && (pl.up <= 2 || pl.up == 4);      // (as launch_rows will have it, if the grid is what it is alone)
+  const int len = in_turn ? cut.per : kb, fit = std::min(len, slot / (pl.up * rows_gemm::UNIT * 128)), steps = (len + fit - 1) / fit;
+  pl.nkb = (len + steps - 1) / steps;
+  if (kind == G_QKV) { pl.su = rows_gemm::UNIT * pl.nkb; pl.sj = rows_gemm::UNIT; pl.sh = 8; }
+  else if (kind == G_GATEUP) { pl.su = 8; pl.sj = 8 * pl.up; pl.sh = 8 * pl.up * pl.nkb; }
+  else { pl.su = rows_gemm::UNIT; pl.sj = rows_gemm::UNIT * pl.up; pl.sh = 8; }
+  return pl;
+}
+static bool rows_setup(int grid, const ModelRt &M, RowsModel &rm) {
+  const ouro_model_desc &d = M.d;
+  const int dq = d.n_heads * d.head_dim, dkv = d.n_kv_heads * d.head_dim, half = d.head_dim / 2, U = rows_gemm::UNIT;
+  auto tiles = [](int n) { return (n + TILE_N - 1) / TILE_N; };
+  const int n_units[5] = {(dq + 2 * dkv) / U, d.d_model / U, d.d_ffn / 8, d.d_model / U, (d.vocab + U - 1) / U};
+  const int n_tiles[5] = {tiles(dq) + 2 * tiles(dkv), tiles(d.d_model), tiles(2 * d.d_ffn), tiles(d.d_model), tiles(d.vocab)};
+  const int K[5] = {d.d_model, dq, d.d_model, d.d_ffn, d.d_model};
+  // A slot takes two k-blocks of gate and up, more than half of a layer's weights: with room for less or with some left over the ring is
+  // shorter than it could be (one row behind 400 keys, us a forward with slots of 20 / 24 / 30 / 36 KB: eight layers of the 1.1B shape,
+  // five units of gate and up a CTA, 248 / 259 / 270 / 279; six of 2560 x 6912, six units, 267 / 251 / 263 / 257; six of 2048 x 8192,
+  // seven units, 242 / 240 / 237 / 243).
+  rm.slot = rows_gemm::MIN_SLOT;
+  const int gu = rows_plan(G_GATEUP, n_units[G_GATEUP], K[G_GATEUP] / BLOCK_K, n_tiles[G_GATEUP], grid, rm.slot).up;
+  if (gu <= 8) rm.slot = std::max(rm.slot, 2 * gu * U * 128);
+  for (int k = 0; k < 5; ++k) rm.plan[k] = rows_plan(k, n_units[k], K[k] / BLOCK_K, n_tiles[k], grid, rm.slot);
+  auto plain = [&](CUtensorMap *m, const void *w, int rows, int kind) {
+    return make_map_rows(m, w, rows, K[kind], rm.plan[kind].up * (kind == G_GATEUP ? 8 : U), rm.plan[kind].nkb);
+  };
+  bool ok = plain(&rm.head, M.lm_head, d.vocab, G_HEAD);
+  rm.layers.resize(d.n_layers);
+  for (int l = 0; l < d.n_layers && ok; ++l) {
+    RowsModel::Layer &lm = rm.layers[l];
+    ok = make_map_pairs(&lm.q, M.wq[l], dq, d.d_model, half, rm.plan[G_QKV].nkb) &&
+         make_map_pairs(&lm.k, M.wk[l], dkv, d.d_model, half, rm.plan[G_QKV].nkb) &&
+         make_map_pairs(&lm.v, M.wv[l], dkv, d.d_model, half, rm.plan[G_QKV].nkb) &&
+         plain(&lm.o, M.wo[l], d.d_model, G_WO) && plain(&lm.g, M.w_gate[l], d.d_ffn, G_GATEUP) &&
+         plain(&lm.u, M.w_up[l], d.d_ffn, G_GATEUP) && plain(&lm.d, M.w_down[l], d.d_model, G_DOWN);
+  }
+  rm.x_bytes = rows_x_bytes(d);
+  return ok;
 }
 
 int ouro_fast_setup(ouro_ctx *c) {
@@ -929,12 +1031,22 @@ int ouro_fast_setup(ouro_ctx *c) {
   f->s.tile_arg = (int *)((char *)f->s.tile_max + tile_best_bytes());
   f->s.ss = (float *)((char *)f->s.tile_arg + tile_best_bytes());
   f->s.attn_part = (float *)((char *)f->s.ss + ss_bytes());
+  size_t attn = 0, packets = 0;                                 // (one model computes at a time)
+  for (auto &M : c->m)
+    if (M.present) {
+      attn = std::max(attn, attention_tc_scratch_bytes(M.d));
+      packets = std::max(packets, packets_bytes(M.d));
+    }
+  f->s.squares = (float *)((char *)f->s.attn_part + attn);
+  f->s.packets = (uint4 *)((char *)f->s.squares + squares_bytes());
   if (cudaMemsetAsync(f->s.slots, 0xff, slots_bytes(), c->stream) != cudaSuccess ||
+      cudaMemsetAsync(f->s.packets, 0, packets, c->stream) != cudaSuccess ||
       cudaMemcpyAsync(f->s.finished, f->s.finished_host, sizeof(f->s.finished_host), cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<SOME>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      cudaFuncSetAttribute(rows_gemm::gemm_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       text_gemm_setup() != OURO_OK || attention_tc_setup() != OURO_OK || attention_tm_setup() != OURO_OK || attention_few_setup() != OURO_OK) {
     delete f;
     c->err = "tensor-core GEMM set-up failed";
@@ -966,6 +1078,7 @@ int ouro_fast_setup(ouro_ctx *c) {
       ok = make_map(&fm.x_d[i], c->a.xn, OURO_TEXT_ROWS, d.d_model, 16 * (i + 1)) &&
            make_map(&fm.x_q[i], c->a.att, OURO_TEXT_ROWS, dq, 16 * (i + 1)) &&
            make_map(&fm.x_f[i], c->a.act, OURO_TEXT_ROWS, d.d_ffn, 16 * (i + 1));
+    if (ok && rows_x_bytes(d) > 0) ok = rows_setup(f->s.grid, M, fm.rm);
     if (!ok) {
       delete f;
       c->err = "cuTensorMapEncodeTiled failed";
@@ -983,7 +1096,6 @@ void ouro_fast_teardown(ouro_ctx *c) {
 }
 
 // The weight side of one GEMM of the forward: which matrices, how they are tiled, how long K is.
-enum { G_QKV = 0, G_WO = 1, G_GATEUP = 2, G_DOWN = 3, G_HEAD = 4 };
 struct WeightSide {
   CUtensorMap a[3];
   int a_tiles[3] = {0, 0, 0}, a_rows[3] = {0, 0, 0}, a_count = 1, tiles = 0, K = 0;
@@ -1041,6 +1153,50 @@ static int grid_for(const FastState &s, int tiles, int kb) {
 // What the hand-over counter of a GEMM advances by: one count per whole tile and one per CTA that has finished its share of the
 // cut tiles.
 static int finish_units(const GemmParams &g) { return g.per == g.kb ? g.tiles : g.t0 + (g.per > 0 ? g.finishers : 0); }
+static bool rows_launch(const FastModel &fm, int rows) { return rows == 1 && fm.rm.x_bytes > 0; }
+static void launch_rows(ouro_ctx *c) {
+  FastState &s = c->fast->s;
+  ChainArgs &cp = s.chain.args;
+  const RowsModel &rm = s.m[s.chain_model].rm;
+  const ouro_model_desc &d = c->m[s.chain_model].d;
+  const int dq = d.n_heads * d.head_dim;
+  rows_gemm::Params kp;
+  kp.squares_bytes = d.d_model;
+  kp.slot = rm.slot;
+  kp.slots = rows_gemm::slots_for(rm.slot, d.d_model + rm.x_bytes, s.smem_max);
+  kp.mark = s.mark;
+  s.mark += MAX_CHAIN + 1;
+  uint4 *px = s.packets, *patt = px + d.d_model / 4, *pact = patt + dq / 4;
+  const bool front = cp.fold.part || cp.embed.table;
+  int grid = front ? s.grid : 1;
+  for (int i = 0; i < cp.n; ++i) {
+    const int kind = s.chain_kind[i];
+    const GemmParams &g = cp.g[i];
+    rows_gemm::Plan &pl = kp.told.plan[i];
+    pl = rm.plan[kind];
+    grid = std::max(grid, (pl.units + pl.up * pl.passes - 1) / (pl.up * pl.passes));
+    pl.max_pieces = g.per > 0 && g.per < g.kb ? std::min(g.kb, (g.kb - 1) / g.per + 2) : 1;
+    // All units of a pass lie in one tile, and are cut alike, where their number divides a tile's (a matrix begins at a multiple of four).
+    pl.share = pl.up <= 2 || pl.up == 4 ? std::min(std::min(rows_gemm::CW / pl.up, pl.max_pieces), kp.slots - 1) : 1;
+    if (pl.up * pl.max_pieces > rows_gemm::PARKED) pl.share = 1;
+    pl.q_in = pl.q_out = s.squares;
+    pl.x_in = (const __nv_bfloat16 *)(kind == G_WO ? c->a.att : kind == G_DOWN ? c->a.act : c->a.xn);
+    if (i > 0 || front) pl.packets_in = kind == G_WO ? patt : kind == G_DOWN ? pact : px;
+    if (i + 1 < cp.n) pl.packets_out = kind == G_GATEUP ? pact : px;
+    const RowsModel::Layer *l = kind == G_HEAD ? nullptr : &rm.layers[s.chain_layer[i]];
+    CUtensorMap *w = kp.w[i];
+    switch (kind) {
+      case G_QKV: w[0] = l->q; w[1] = l->k; w[2] = l->v; break;
+      case G_WO: w[0] = l->o; break;
+      case G_GATEUP: w[0] = l->g; w[1] = l->u; break;
+      case G_DOWN: w[0] = l->d; break;
+      default: w[0] = rm.head; break;
+    }
+  }
+  kp.front = cp.fold.part ? patt : px;
+  kp.told.args = cp;
+  launch_pdl(rows_gemm::gemm_rows_kernel, grid, rows_gemm::THREADS, (size_t)s.smem_max, c->stream, kp);
+}
 // Launches the GEMMs collected so far as one chain.
 static void flush_chain(ouro_ctx *c) {
   FastState &s = c->fast->s;
@@ -1056,14 +1212,16 @@ static void flush_chain(ouro_ctx *c) {
     cp.g[i].per = cut.per;
     cp.g[i].finishers = grid;
   }
-  for (int i = 0; i + 1 < cp.n; ++i) cp.target[i] = (s.finished_host[i] += finish_units(cp.g[i]));
-  if (cp.fold.part || cp.embed.table) cp.fold_target = (s.finished_host[MAX_CHAIN] += grid);
+  const bool few = rows_launch(s.m[s.chain_model], cp.g[0].rows);
+  for (int i = 0; i + 1 < cp.n && !few; ++i) cp.target[i] = (s.finished_host[i] += finish_units(cp.g[i]));
+  if (!few && (cp.fold.part || cp.embed.table)) cp.fold_target = (s.finished_host[MAX_CHAIN] += grid);
   const bool per_kind = cp.n == 1 && c->prof_class >= OURO_PROF_QKV && c->prof_class <= OURO_PROF_HEAD;
   static const int kind_class[5] = {OURO_PROF_QKV, OURO_PROF_WO, OURO_PROF_GATEUP, OURO_PROF_DOWN, OURO_PROF_HEAD};
   {
     ProfScope ps(c, per_kind ? kind_class[s.chain_kind[0]] : OURO_PROF_GEMM);
     const int t_pad = cp.g[0].t_pad;
-    launch_pdl(t_pad > OURO_MAX_ROWS ? gemm_tc_kernel<MANY> : t_pad > FEW_ROWS ? gemm_tc_kernel<SOME>
+    if (few) launch_rows(c);
+    else launch_pdl(t_pad > OURO_MAX_ROWS ? gemm_tc_kernel<MANY> : t_pad > FEW_ROWS ? gemm_tc_kernel<SOME>
                : t_pad > ONE_ROWS ? gemm_tc_kernel<FEW> : gemm_tc_kernel<ONE>,
                grid, THREADS, (size_t)s.smem_max, c->stream, s.chain);
   }
@@ -1073,7 +1231,7 @@ static void flush_chain(ouro_ctx *c) {
 }
 
 // Adds a GEMM to the chain under construction; `last` launches the chain (something other than a GEMM follows).
-static void push_gemm(ouro_ctx *c, Gemm &p, int kind, const CUtensorMap *xmaps, int K, int rows, bool last) {
+static void push_gemm(ouro_ctx *c, int which, int layer, Gemm &p, int kind, const CUtensorMap *xmaps, int K, int rows, bool last) {
   FastState &s = c->fast->s;
   p.kb = K / BLOCK_K;
   p.rows = rows;
@@ -1088,6 +1246,8 @@ static void push_gemm(ouro_ctx *c, Gemm &p, int kind, const CUtensorMap *xmaps, 
   ChainArgs &cp = s.chain.args;
   if (cp.n > 0 && cp.g[0].rows != rows) flush_chain(c);             // cannot happen inside one forward
   s.chain_kind[cp.n] = kind;
+  s.chain_layer[cp.n] = layer;
+  s.chain_model = which;
   s.chain.maps[cp.n] = p.m;
   cp.g[cp.n++] = p;
   // one launch per GEMM when asked for, and while a single kind of GEMM is being timed
@@ -1320,7 +1480,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
       p.out_f32 = a.qkv;
       p.ldo = dq + 2 * dkv;
     }
-    push_gemm(c, p, G_QKV, fm.x_d, d.d_model, rows, true);       // closes the chain the previous layer began
+    push_gemm(c, which, l, p, G_QKV, fm.x_d, d.d_model, rows, true);       // closes the chain the previous layer began
     if (!fused_rope) {
       ProfScope pr(c, OURO_PROF_ROPE);
       launch_rope_append(d, a.qkv, M.blk.pos, M.rope_cos, M.rope_sin, rows, M.L, l, a.q, M.k_cache, M.v_cache, s);
@@ -1340,9 +1500,10 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
       }
       // Rows in order that fill one small tile: in one span its chunks side by side are faster than attn_tm_kernel's one behind
       // the other (one row behind 150 keys, three 7B layers 289 -> 285 us, two of 512 62.7 -> 59.2; behind 400 keys 300 and 300,
-      // 69.0 -> 62.6).  With more spans they are not (three 7B layers behind 1800 keys 310 -> 322: the CTAs of several spans are the
-      // ones that share the HBM with the weights on their way to the next kernel).
-      if (!M.blk_is_candidate && attention_few_supported(d, rows) && fold::span_count(d.head_dim, M.L + rows) <= 1)
+      // 69.0 -> 62.6).  With more spans they gain in front of gemm_rows.cuh only (two layers of 512 behind 1800 keys 56.6 -> 48.4 us;
+      // three 7B layers, in front of gemm_tc_kernel, 310 -> 322: the CTAs of several spans are the ones that share the HBM with
+      // the weights on their way to the next kernel).
+      if (!M.blk_is_candidate && attention_few_supported(d, rows) && (fold::span_count(d.head_dim, M.L + rows) <= 1 || rows_launch(fm, rows)))
         pieces = launch_attention_few(d, a.q, M.k_cache, M.v_cache, M.blk, rows, M.L, M.L + rows, l, c->fast->s.attn_part, a.att, c->cur_rows_dev, pf, s);
       else
         pieces = launch_attention_tm(d, a.q, &c->fast->s.m[which].kmap, &c->fast->s.m[which].vmap, M.k_cache, M.v_cache, M.blk, rows,
@@ -1374,7 +1535,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
     p.out_f32 = a.x;
     p.ldo = d.d_model;
     produce(p, M.ffn_norm[l]);
-    push_gemm(c, p, G_WO, fm.x_q, dq, rows, false);
+    push_gemm(c, which, l, p, G_WO, fm.x_q, dq, rows, false);
   }
   if (!kv_only) {
     Gemm p{};
@@ -1382,7 +1543,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
     p.mode = MODE_SWIGLU;
     p.out_bf16 = (__nv_bfloat16 *)a.act;
     consume(p);
-    push_gemm(c, p, G_GATEUP, fm.x_d, d.d_model, rows, false);
+    push_gemm(c, which, l, p, G_GATEUP, fm.x_d, d.d_model, rows, false);
   }
   if (!kv_only) {
     Gemm p{};
@@ -1391,7 +1552,7 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
     p.out_f32 = a.x;
     p.ldo = d.d_model;
     produce(p, l + 1 < d.n_layers ? M.attn_norm[l + 1] : M.final_norm);
-    push_gemm(c, p, G_DOWN, fm.x_f, d.d_ffn, rows, false);     // the next layer's q,k,v or the LM head completes the chain
+    push_gemm(c, which, l, p, G_DOWN, fm.x_f, d.d_ffn, rows, false);     // the next layer's q,k,v or the LM head completes the chain
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -1455,13 +1616,15 @@ int ouro_fast_head(ouro_ctx *c, int which, int rows, float *logits, int32_t *arg
     p.tile_max = c->fast->s.tile_max;
     p.tile_arg = c->fast->s.tile_arg;
     p.ss_in = c->fast->s.ss; p.ss_tiles = (d.d_model + TILE_N - 1) / TILE_N; p.ss_inv_d = 1.0f / (float)d.d_model; p.eps = d.rms_eps;
-    push_gemm(c, p, G_HEAD, fm.x_d, d.d_model, rows, true);
+    push_gemm(c, which, 0, p, G_HEAD, fm.x_d, d.d_model, rows, true);
   }
   {
     ProfScope ps(c, OURO_PROF_ARGMAX);
     OURO_COUNT_LAUNCH();
+    const rows_gemm::Plan &pl = fm.rm.plan[G_HEAD];
+    const int entries = rows_launch(fm, rows) ? (pl.units + pl.up - 1) / pl.up : (d.vocab + TILE_N - 1) / TILE_N;
     launch_pdl(argmax_tiles_kernel, rows, 128, 0, c->stream, (const float *)c->fast->s.tile_max, (const int *)c->fast->s.tile_arg,
-               (int)((d.vocab + TILE_N - 1) / TILE_N), argmax_dev, Tidy());
+               entries, argmax_dev, Tidy());
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

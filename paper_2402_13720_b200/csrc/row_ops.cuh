@@ -25,6 +25,26 @@ __device__ __forceinline__ float2 unpack(uint32_t v) {
   return make_float2(__low2float(t), __high2float(t));
 }
 
+// Four bf16 values on their way from the CTA that computed them to all that need them, in one 128-bit word: a poll that finds
+// the mark has the values as well, so that a hand-over costs one store and one load (no fence, no counter, no second load).
+// A mark is used once: nothing is reset, and what a launch that gave up left behind is not taken for anything.
+struct Packet { uint32_t lo, hi, extra, mark; };
+__device__ __forceinline__ void put_packet(uint4 *dst, uint32_t lo, uint32_t hi, uint32_t extra, uint32_t mark) {
+  asm volatile(
+      "{\n\t.reg .b128 v;\n\t.reg .b64 a, b;\n\t"
+      "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\tmov.b128 v, {a, b};\n\t"
+      "st.relaxed.gpu.global.b128 [%0], v;\n\t}" ::"l"(dst), "r"(lo), "r"(hi), "r"(extra), "r"(mark) : "memory");
+}
+__device__ __forceinline__ Packet get_packet(const uint4 *src) {
+  Packet p;
+  asm volatile(
+      "{\n\t.reg .b128 v;\n\t.reg .b64 a, b;\n\t"
+      "ld.relaxed.gpu.global.b128 v, [%4];\n\t"
+      "mov.b128 {a, b}, v;\n\tmov.b64 {%0, %1}, a;\n\tmov.b64 {%2, %3}, b;\n\t}"
+      : "=r"(p.lo), "=r"(p.hi), "=r"(p.extra), "=r"(p.mark) : "l"(src) : "memory");
+  return p;
+}
+
 // Embedding rows of a block's tokens into the residual stream, plus what the first norm's consumer needs: bf16(gain * x) and
 // the sums of squares per 128-column tile.
 struct Embed {
@@ -55,6 +75,20 @@ __device__ __forceinline__ void embed(const Embed &e, int first, int step, int l
 #pragma unroll
     for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
     if (lane == 0) e.ss[(size_t)(it - r * tiles) * e.ss_pitch + r] = sq;
+  }
+}
+
+// The same for one row, as packets: its values and each four columns' squares, instead of xb and ss.
+__device__ __forceinline__ void embed_packets(const Embed &e, int first, int step, int lane, uint4 *packets, uint32_t mark) {
+  for (int it = first; it < (e.d + 127) / 128; it += step) {
+    const int col = it * 128 + 4 * lane;
+    if (col >= e.d) continue;
+    const uint2 raw = __ldg(reinterpret_cast<const uint2 *>(e.table + (size_t)__ldg(e.tok) * e.d + col));
+    const uint2 graw = __ldg(reinterpret_cast<const uint2 *>(e.gain + col));
+    const float2 a = unpack(raw.x), b = unpack(raw.y), ga = unpack(graw.x), gb = unpack(graw.y);
+    *reinterpret_cast<float4 *>(e.x + col) = make_float4(a.x, a.y, b.x, b.y);
+    const float sq = __fadd_rn(__fmaf_rn(a.x, a.x, __fmul_rn(a.y, a.y)), __fmaf_rn(b.x, b.x, __fmul_rn(b.y, b.y)));
+    put_packet(packets + col / 4, pack(ga.x * a.x, ga.y * a.y), pack(gb.x * b.x, gb.y * b.y), __float_as_uint(sq), mark);
   }
 }
 

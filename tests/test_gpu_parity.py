@@ -1592,9 +1592,10 @@ def test_groups_shared_by_several_ctas_are_bit_identical_to_plain_decoding(kv, K
     (4096, 32, 32, 128, 11008, 1000),     # a layer beyond the single row's kernels
 ])
 def test_few_rows_are_bit_identical_to_wider_blocks(d, heads, kv, hd, ffn, vocab):
-    """Up to 16 query rows of a kv head without candidates have attention kernels of their own (head dim 128, one span).  A
-    token's logits, choice, keys and values must not show which: blocks of 1, 2, 5, 8, 9 and 16 rows against one block of 40,
-    behind 490 keys, so that the rows pass the end of a span."""
+    """A single row of a model of small layers runs on GEMM kernels of its own, and up to 16 query rows of a kv head without
+    candidates on attention of their own (head dim 128, in one span or in front of those kernels).  A token's logits,
+    choice, keys and values must not show which: blocks of 1, 2, 5, 8, 9 and 16 rows against one block of 40, behind 490 keys, so
+    that the rows pass the end of a span."""
     desc = synth.ModelDesc(1 if d > 2048 else 2, d, heads, kv, hd, ffn, vocab, 640, "bf16")
     w = synth.model_weights(desc, 5, device="cuda:0")
     eng = binding.Engine(desc, w, synth.DecodeParams(4, 5, 3, 16, 8))
@@ -1620,4 +1621,22 @@ def test_few_rows_are_bit_identical_to_wider_blocks(d, heads, kv, hd, ffn, vocab
     for n in (1, 2, 5, 8, 9, 16):
         for got, ref in zip(run(n), want):
             assert torch.equal(got, ref), n
+    eng.close()
+
+
+@pytest.mark.parametrize("fuse", ["0", "1"])
+def test_single_rows_with_every_gemm_a_launch_of_its_own(monkeypatch, fuse):
+    """The kernels of a single row hand activations over inside a launch and through memory between launches: plain decoding gives
+    the same logits whether GEMMs are chained or not, and those of the wider kernels."""
+    monkeypatch.setenv("OURO_FUSE", fuse)
+    eng, _ = make(MIDB, synth.DecodeParams(4, 9, 4, 16, 8), 2)
+    tokens = np.arange(20, 44, dtype=np.int32)
+    eng.set_state(30, 1)
+    eng.assemble_causal(binding.OURO_TARGET, tokens)
+    want = eng.verify_forward(want_logits=True)[1][:24].clone()
+    eng.set_state(30, 1)
+    for i in range(24):
+        eng.assemble_causal(binding.OURO_TARGET, tokens[i: i + 1])
+        assert torch.equal(eng.verify_forward(want_logits=True)[1][0], want[i]), i
+        eng.advance(binding.OURO_TARGET, 1)
     eng.close()
