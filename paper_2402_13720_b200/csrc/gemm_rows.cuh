@@ -6,8 +6,8 @@
 // the outputs cross it again behind a fence and a counter (2 us).  Here a CTA owns its weight rows for the whole of K: groups of 16
 // (a unit), as many per CTA as an equal split over the SMs gives, so that only finished activations leave it.  They travel
 // in packets that say themselves that they are there (row_ops.cuh), and every CTA gathers all of them into its shared memory.
-// 1.1B draft, four forwards behind 389 keys: 3178 -> 2622 us; a layer 36 -> 29 us, of which 13.5 are its 88 MB at the copy peak and
-// the rest five hand-overs and two launches.
+// 1.1B draft, four forwards behind 389 keys: 3156 -> 2510 us; a layer 36 -> 28 us, of which 13.5 are its 88 MB at the copy peak and
+// the rest four hand-overs, the attention and two launches.
 //
 // The tensor cores are used through mma.sync (16 weight rows x 8 tokens x 16 values of K, operands by ldmatrix): its fragments
 // are as small as a unit, where a tcgen05 tile has 128 rows of which 16 to 80 would be the CTA's, and the sums are in
@@ -18,12 +18,12 @@
 //
 // Warp 0 streams weights into the ring (boxes of [k-blocks][rows][64]), warp 1 works out the token's factor of the norm, CW warps
 // contract.  What they execute is latency as well: a step of a chain waits 47 cycles for the one before, and a warp spends about 4
-// cycles on every other instruction.  So a stage is as large as a slot of the ring (12 KB slots: draft 5061 us) and a slot two k-blocks of the largest GEMM (see
-// rows_setup), it is looked at by
-// the warps that contract it only (one per unit), where all units of a CTA are cut alike the ring takes the k-blocks of several
-// pieces in turn, each for other warps, and the two warps that finish a GEMM's sums leave the next one's activations to the others
-// (2953 -> 2622 us).  Two groups of eight tokens, or the activations of several tokens beside the weights in the ring, were slower
-// than gemm_tc_kernel (two small layers, 13 rows: step 91 -> 129 us; five rows of the 1.1B shape 867 -> 1288).
+// cycles on every other instruction.  So a stage is as large as a slot of the ring (12 KB slots: draft 5061 us) and a slot two k-blocks of the
+// largest GEMM (see rows_setup), a stage is looked at by the warps that contract it only (one per unit), where all units of a CTA
+// are cut alike the ring takes the k-blocks of several pieces in turn, each for other warps, and the two warps that finish a GEMM's
+// sums leave the next one's activations to the others (2953 -> 2622 us).  Two groups of eight tokens, or the activations of several
+// tokens beside the weights in the ring, were slower than gemm_tc_kernel (two small layers, 13 rows: step 91 -> 129 us; five rows
+// of the 1.1B shape 867 -> 1288).
 
 namespace rows_gemm {
 

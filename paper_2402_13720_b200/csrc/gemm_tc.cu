@@ -907,8 +907,8 @@ constexpr int MAX_SS_TILES = 64;           // d_model <= 8192
 // A token's activations, the widest of them, in the shared memory of a CTA of gemm_rows.cuh; 0: the model's single rows do not run
 // there.  What those kernels save is the latency between a layer's GEMMs, what they cost is a chain of steps per weight row, and the
 // wider a layer, the more the stream of its weights hides of either.  One row behind 150 / 400 / 1800 keys, us a forward, gemm_tc.cu
-// and here: two layers of 512 (4 MB a layer) 59, 63, 65 and 45, 48, 48; eight of the 1.1B shape (88 MB) 304, 305, 342 and 259, 259,
-// 298; six of 2048 x 8192 (121 MB) 260, 261, 290 and 240, 240, 268; six of 2560 x 6912 (137 MB) 279, 280, 308 and 250, 251, 278;
+// and here: two layers of 512 (4 MB a layer) 59, 63, 65 and 44, 48, 48; eight of the 1.1B shape (88 MB) 304, 305, 342 and 250, 250,
+// 288; six of 2048 x 8192 (121 MB) 260, 261, 290 and 233, 234, 262; six of 2560 x 6912 (137 MB) 279, 280, 308 and 250, 252, 278;
 // four of 3072 x 8192 (201 MB) 239, 255, 269 and 241, 247, 248; three of the 7B shape (405 MB) 285, 300, 322 and 290, 304, 325.
 int rows_x_bytes(const ouro_model_desc &d) {
   const int dq = d.n_heads * d.head_dim, dkv = d.n_kv_heads * d.head_dim, x = 2 * std::max(std::max(d.d_model, dq), d.d_ffn);
