@@ -892,7 +892,8 @@ struct FastState {
   ChainParams chain{};          // GEMMs collected for the next launch
   int chain_layer[MAX_CHAIN] = {0, 0, 0, 0}, chain_model = 0;
   uint4 *packets = nullptr;     // activations on their way: normed, attention out, SwiGLU out  (gemm_rows.cuh)
-  uint32_t mark = 1;            // of the next launch's first packets
+  size_t packets_size = 0;      // bytes
+  uint32_t mark = 1;            // of the next launch's first packets; never zero, which an empty packet has
   float *squares = nullptr;     // squares of four columns each of the residual stream, as gemm_rows.cuh leaves them
   int chain_kind[MAX_CHAIN] = {0, 0, 0, 0};
   bool fuse = true;             // run consecutive GEMMs as one launch
@@ -1024,8 +1025,10 @@ int ouro_fast_setup(ouro_ctx *c) {
     const char *pf = getenv("OURO_PF_ROWS");
     if (pf) f->s.pf_ffn_rows = atol(pf);
     const char *c0 = getenv("OURO_COUNT_START");                // test aid: what the hand-over counters start at
-    if (c0)
+    if (c0) {
       for (uint32_t &v : f->s.finished_host) v = (uint32_t)strtoul(c0, nullptr, 0);
+      f->s.mark = std::max(1u, (uint32_t)strtoul(c0, nullptr, 0));                   // (and the packets' marks)
+    }
   }
   f->s.tile_max = (float *)((char *)c->a.scratch + slots_bytes() + CHAIN_BYTES);
   f->s.tile_arg = (int *)((char *)f->s.tile_max + tile_best_bytes());
@@ -1039,6 +1042,7 @@ int ouro_fast_setup(ouro_ctx *c) {
     }
   f->s.squares = (float *)((char *)f->s.attn_part + attn);
   f->s.packets = (uint4 *)((char *)f->s.squares + squares_bytes());
+  f->s.packets_size = packets;
   if (cudaMemsetAsync(f->s.slots, 0xff, slots_bytes(), c->stream) != cudaSuccess ||
       cudaMemsetAsync(f->s.packets, 0, packets, c->stream) != cudaSuccess ||
       cudaMemcpyAsync(f->s.finished, f->s.finished_host, sizeof(f->s.finished_host), cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
@@ -1164,6 +1168,10 @@ static void launch_rows(ouro_ctx *c) {
   kp.squares_bytes = d.d_model;
   kp.slot = rm.slot;
   kp.slots = rows_gemm::slots_for(rm.slot, d.d_model + rm.x_bytes, s.smem_max);
+  if (s.mark > UINT32_MAX - (MAX_CHAIN + 1)) {                    // some hours of decoding: the marks begin anew, on empty packets
+    cudaMemsetAsync(s.packets, 0, s.packets_size, c->stream);
+    s.mark = 1;
+  }
   kp.mark = s.mark;
   s.mark += MAX_CHAIN + 1;
   uint4 *px = s.packets, *patt = px + d.d_model / 4, *pact = patt + dq / 4;
