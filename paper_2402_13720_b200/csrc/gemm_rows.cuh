@@ -63,6 +63,7 @@ struct Params {
   int squares_bytes;          // the squares of the activations; those are behind them
   uint4 *front;               // where the work in front leaves its packets
   uint32_t mark;              // of those; GEMM i leaves those with mark + 1 + i
+  uint32_t late;              // test aid: ns that the warp of the factors sleeps before it looks at a GEMM (0)
 };
 static_assert(sizeof(Params) <= 4096, "kernel parameters");
 
@@ -224,7 +225,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_rows_kernel(const __grid_cons
       mbar_init(&empty[s], TAKERS);
     }
     mbar_init(factors_full, 1);
-    mbar_init(x_full, GATHERERS);
+    mbar_init(x_full, GATHERERS + 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -309,12 +310,20 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_rows_kernel(const __grid_cons
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- the factor 1/rms of the activations
+    // This warp looks at every phase of x_full, but nobody waits for its answer where a GEMM has no norm.  So it is one of those
+    // whose arrival completes the next phase: were it late by a GEMM and a hand-over, it would find the parity it waits for
+    // as it was a phase ago, and wait until its limit.
     bool ok = true;
     uint32_t gathered = 0;
     for (int ci = 0; ci < cp.n && ok; ++ci) {
       const GemmParams &p = cp.g[ci];
       const Plan &pl = plans[ci];
       if ((int)blockIdx.x * pl.passes * pl.up >= pl.units) continue;
+      if (lane == 0) {
+        if (kp.late) __nanosleep(kp.late);
+        mbar_arrive(x_full);                                       // has seen the phase before
+      }
+      __syncwarp();
       ok = warp_wait(x_full, gathered++ & 1, abort_flag);
       if (!ok || !p.ss_in) continue;
       float sum = 0.f;

@@ -894,6 +894,7 @@ struct FastState {
   uint4 *packets = nullptr;     // activations on their way: normed, attention out, SwiGLU out  (gemm_rows.cuh)
   size_t packets_size = 0;      // bytes
   uint32_t mark = 1;            // of the next launch's first packets; never zero, which an empty packet has
+  uint32_t late = 0;            // test aid, see rows_gemm::Params
   float *squares = nullptr;     // squares of four columns each of the residual stream, as gemm_rows.cuh leaves them
   int chain_kind[MAX_CHAIN] = {0, 0, 0, 0};
   bool fuse = true;             // run consecutive GEMMs as one launch
@@ -1029,6 +1030,8 @@ int ouro_fast_setup(ouro_ctx *c) {
       for (uint32_t &v : f->s.finished_host) v = (uint32_t)strtoul(c0, nullptr, 0);
       f->s.mark = std::max(1u, (uint32_t)strtoul(c0, nullptr, 0));                   // (and the packets' marks)
     }
+    const char *late = getenv("OURO_LATE_NS");                  // test aid: a late warp in gemm_rows.cuh, at most 0.1 ms a GEMM
+    if (late) f->s.late = (uint32_t)std::min(strtoul(late, nullptr, 0), 100000ul);
   }
   f->s.tile_max = (float *)((char *)c->a.scratch + slots_bytes() + CHAIN_BYTES);
   f->s.tile_arg = (int *)((char *)f->s.tile_max + tile_best_bytes());
@@ -1174,6 +1177,7 @@ static void launch_rows(ouro_ctx *c) {
   }
   kp.mark = s.mark;
   s.mark += MAX_CHAIN + 1;
+  kp.late = s.late;
   uint4 *px = s.packets, *patt = px + d.d_model / 4, *pact = patt + dq / 4;
   const bool front = cp.fold.part || cp.embed.table;
   int grid = front ? s.grid : 1;

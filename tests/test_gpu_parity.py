@@ -1640,3 +1640,25 @@ def test_single_rows_with_every_gemm_a_launch_of_its_own(monkeypatch, fuse):
         assert torch.equal(eng.verify_forward(want_logits=True)[1][0], want[i]), i
         eng.advance(binding.OURO_TARGET, 1)
     eng.close()
+
+
+@pytest.mark.parametrize("fuse", ["0", "1"])
+def test_single_rows_with_a_late_warp(monkeypatch, fuse):
+    """One warp of a single row's kernel works out the norm's factor and has nothing to hand back for the GEMMs without one.  It
+    may be late by more than such a GEMM and the hand-over behind it (here 30 us a GEMM; they take 1 to 5): no time-out, and the same
+    logits.  All GEMMs of this model are a few k-blocks long, so that nothing else holds the others back."""
+    desc = synth.ModelDesc(3, 128, 1, 1, 128, 128, 512, 64, "bf16")
+    w = synth.model_weights(desc, 4, device="cuda:0")
+    prompt = np.arange(3, 20, dtype=np.int32)
+    want = None
+    for late in ("0", "30000"):
+        monkeypatch.setenv("OURO_LATE_NS", late)
+        monkeypatch.setenv("OURO_FUSE", fuse)
+        eng = binding.Engine(desc, w, synth.DecodeParams(4, 5, 3, 16, 8))
+        got = eng.generate_vanilla(prompt, 24)[0].tolist()             # (would raise on a time-out)
+        eng.assemble_causal(binding.OURO_TARGET, [5])
+        got = got, eng.verify_forward(want_logits=True)[1][0].clone()
+        eng.close()
+        if want is None:
+            want = got
+    assert got[0] == want[0] and torch.equal(got[1], want[1])
