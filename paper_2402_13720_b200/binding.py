@@ -82,6 +82,7 @@ _SIGNATURES = {
     "ouro_debug_static_scratch": (C.c_int, [C.POINTER(C.c_void_p), C.POINTER(C.c_size_t)]),
     "ouro_profile_enable": (C.c_int, [C.c_void_p, C.c_int]),
     "ouro_debug_set_wait_limit": (C.c_int, [C.c_void_p, C.c_int64]),
+    "ouro_debug_counts": (C.c_int, [C.c_void_p, C.POINTER(C.c_uint32), C.c_int32]),
     "ouro_profile_read": (C.c_int, [C.c_void_p, _F32P, _I32P]),
     "ouro_generate": (C.c_int, [C.c_void_p, _I32P, C.c_int32, C.c_int32, C.c_int32, _I32P, _I32P, C.POINTER(StatsC)]),
     "ouro_generate_vanilla": (C.c_int, [C.c_void_p, _I32P, C.c_int32, C.c_int32, _I32P, _I32P, C.POINTER(StatsC)]),
@@ -350,6 +351,11 @@ class Engine:
 
     def set_wait_limit(self, polls):
         self._ck(self.L.ouro_debug_set_wait_limit(self.ctx, int(polls)))
+
+    def debug_counts(self):
+        v = (C.c_uint32 * 8)()
+        self._ck(self.L.ouro_debug_counts(self.ctx, v, 8))
+        return dict(status=v[0], rows_launches=v[1], mark=v[2], counters=list(v[3:]))
 
     # ---- loops -------------------------------------------------------------------------------
     def generate(self, prompt, max_new, keep_pool=False):

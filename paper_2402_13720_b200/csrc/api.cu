@@ -372,6 +372,17 @@ extern "C" int ouro_debug_set_wait_limit(ouro_ctx *c, int64_t polls) {
   return OURO_OK;
 }
 
+void ouro_fast_counts(const ouro_ctx *c, uint32_t *values);   // gemm_tc.cu
+extern "C" int ouro_debug_counts(ouro_ctx *c, uint32_t *values, int32_t n) {
+  if (!c || !values || n < 1 || n > OURO_DEBUG_COUNTS) return OURO_EINVAL;
+  uint32_t all[OURO_DEBUG_COUNTS] = {0};
+  CK(cudaStreamSynchronize(c->stream));
+  CK(cudaMemcpy(all, &c->st->status, sizeof(int32_t), cudaMemcpyDeviceToHost));
+  ouro_fast_counts(c, all);
+  memcpy(values, all, (size_t)n * sizeof(uint32_t));
+  return OURO_OK;
+}
+
 extern "C" int ouro_assemble_candidates(ouro_ctx *c, const int32_t *draft_dev, const int32_t *suffix_dev,
                                         const int32_t *count_dev) {
   if (!c || !draft_dev || ((suffix_dev == nullptr) != (count_dev == nullptr))) return OURO_EINVAL;

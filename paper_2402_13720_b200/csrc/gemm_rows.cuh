@@ -43,6 +43,7 @@ static_assert(4 * MAX_UP <= CTHREADS - GTHREADS, "one thread per four columns");
 struct Plan {
   int units, up, passes;      // units of the GEMM; a CTA takes up x passes consecutive ones, `up` at a time
   int nkb;                    // k-blocks per ring slot
+  int cut_per;                // k-blocks of a piece along K if this GEMM is a launch of its own (host)
   int su, sj, sh;             // 128-byte lines from a unit to the next, from a k-block to the next, to the unit's upper eight rows
   int share, max_pieces;      // warps that share a unit's pieces (more than one: the ring takes k-blocks of as many in turn); most pieces a unit has
   const float *q_in;          // squares of four columns each [d / 4] of activations in memory

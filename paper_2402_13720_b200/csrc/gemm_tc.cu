@@ -895,6 +895,7 @@ struct FastState {
   size_t packets_size = 0;      // bytes
   uint32_t mark = 1;            // of the next launch's first packets; never zero, which an empty packet has
   uint32_t late = 0;            // test aid, see rows_gemm::Params
+  uint32_t rows_launches = 0;   // of gemm_rows.cuh so far
   float *squares = nullptr;     // squares of four columns each of the residual stream, as gemm_rows.cuh leaves them
   int chain_kind[MAX_CHAIN] = {0, 0, 0, 0};
   bool fuse = true;             // run consecutive GEMMs as one launch
@@ -907,7 +908,7 @@ size_t slots_bytes() { return (size_t)MAX_GRID * 2 * TILE_N * MAX_CHAIN_ROWS * s
 size_t tile_best_bytes() { return (size_t)MAX_TILES * OURO_MAX_ROWS * 4; }
 constexpr int MAX_SS_TILES = 64;           // d_model <= 8192
 // A token's activations, the widest of them, in the shared memory of a CTA of gemm_rows.cuh; 0: the model's single rows do not run
-// there.  What those kernels save is the latency between a layer's GEMMs, what they cost is a chain of steps per weight row, and the
+// there (nor do they where rows_pay says so).  What those kernels save is the latency between a layer's GEMMs, what they cost is a chain of steps per weight row, and the
 // wider a layer, the more the stream of its weights hides of either.  One row behind 150 / 400 / 1800 keys, us a forward, gemm_tc.cu
 // and here: two layers of 512 (4 MB a layer) 59, 63, 65 and 44, 48, 48; eight of the 1.1B shape (88 MB) 304, 305, 342 and 250, 250,
 // 288; six of 2048 x 8192 (121 MB) 260, 261, 290 and 233, 234, 262; six of 2560 x 6912 (137 MB) 279, 280, 308 and 250, 252, 278;
@@ -947,6 +948,13 @@ static bool shape_ok(const ouro_model_desc &d) {
          (d.vocab + TILE_N - 1) / TILE_N <= MAX_TILES && (2 * d.d_ffn + TILE_N - 1) / TILE_N <= MAX_TILES;
 }
 
+// All units of a pass lie in one tile, and are cut alike, where their number divides a tile's (a matrix begins at a multiple of four): the
+// ring then takes the k-blocks of several pieces in turn.
+static void rows_share(rows_gemm::Plan &pl, int kb, int per, int slots) {
+  pl.max_pieces = per > 0 && per < kb ? std::min(kb, (kb - 1) / per + 2) : 1;
+  pl.share = pl.up <= 2 || pl.up == 4 ? std::min(std::min(rows_gemm::CW / pl.up, pl.max_pieces), slots - 1) : 1;
+  if (pl.up * pl.max_pieces > rows_gemm::PARKED) pl.share = 1;
+}
 // How a GEMM is dealt out to the CTAs, and how many k-blocks a ring slot holds.
 static rows_gemm::Plan rows_plan(int kind, int units, int kb, int tiles, int grid, int slot) {
   rows_gemm::Plan pl{};
@@ -958,12 +966,36 @@ static rows_gemm::Plan rows_plan(int kind, int units, int kb, int tiles, int gri
   const bool in_turn = cut.t0 == 0 && cut.per < kb && (pl.up <= 2 || pl.up == 4);      // (as launch_rows will have it, if the grid is what it is alone)
   const int len = in_turn ? cut.per : kb, fit = std::min(len, slot / (pl.up * rows_gemm::UNIT * 128)), steps = (len + fit - 1) / fit;
   pl.nkb = (len + steps - 1) / steps;
+  pl.cut_per = cut.per;
   if (kind == G_QKV) { pl.su = rows_gemm::UNIT * pl.nkb; pl.sj = rows_gemm::UNIT; pl.sh = 8; }
   else if (kind == G_GATEUP) { pl.su = 8; pl.sj = 8 * pl.up; pl.sh = 8 * pl.up * pl.nkb; }
   else { pl.su = rows_gemm::UNIT; pl.sj = rows_gemm::UNIT * pl.up; pl.sh = 8; }
   return pl;
 }
-static bool rows_setup(int grid, const ModelRt &M, RowsModel &rm) {
+// Whether owned weight rows are faster than gemm_tc_kernel's cut tiles.  They save the tails and the hand-overs' round trips, 5 to 8 us a
+// small layer.  They cost a chain: the k-blocks that the busiest warp of a GEMM takes one behind another, 0.1 us each, where
+// gemm_tc_kernel deals a long K out to all SMs; as far as it is not hidden by the stream, of which 0.4 was found to count.  `late` is the
+// sum of that over a layer, in us, and the line at 2.25, in layers below 11 MB rising to 4 (the stream of a wide layer hides more of
+// the tails there).  One row behind 150 keys, three layers, gemm_tc.cu and here, us a forward, of d_model x d_ffn (late): 512 x 1024 87 and 69 (0.3),
+// 512 x 2048 87 and 85 (3.2), 512 x 4096 91 and 94 (6.5), 512 x 28672 126 and 238 (43); 256 x 2048 88 and 83 (3.3), 256 x 2816 91 and 94 (4.7);
+// 384 x 1024 with 3072 query columns 101 and 108 (4.8); 1024 x 4096 95 and 88 (0.9), 1024 x 11264 114 and 102 (1.9), 1024 x 16384 125 and 128
+// (4.0); 768 x 8448 99 and 104 (2.6); 1536 x 6144 107 and 101 (0.8), 1536 x 9216 115 and 118 (2.3), 1536 x 16896 149 and 160 (6.6); 2048 x 5632
+// 113 and 105 (1.4); 2560 x 7040 136 and 126 (2.0), 2560 x 10240, beyond 160 MB, 151 and 155.  The head costs 1 us more in each of its passes
+// than it does there (one layer of 512 in front of 65536 / 262144 logits 44 / 79 us and 42 / 86), which each layer's saving makes up
+// for a few of.
+static bool rows_pay(const rows_gemm::Plan *plan, const int *kb, int n_layers) {
+  double late = 0, stream = 0;
+  for (int k = 0; k < 4; ++k) {
+    const rows_gemm::Plan &pl = plan[k];
+    const int step = (pl.cut_per + pl.nkb - 1) / pl.nkb * pl.nkb;
+    const int walk = pl.passes * (pl.share == 1 ? kb[k] : (pl.max_pieces + pl.share - 1) / pl.share * step);
+    const double us = (double)pl.units * rows_gemm::UNIT * kb[k] * BLOCK_K * 2 / 6.5e6;
+    late += std::max(0.0, 0.1 * walk - 0.4 * us);
+    stream += us;
+  }
+  return late <= std::max(2.25, 4.0 - 0.25 * stream) && plan[G_HEAD].passes <= 3 * n_layers;
+}
+static bool rows_setup(int grid, int smem_max, const ModelRt &M, RowsModel &rm) {
   const ouro_model_desc &d = M.d;
   const int dq = d.n_heads * d.head_dim, dkv = d.n_kv_heads * d.head_dim, half = d.head_dim / 2, U = rows_gemm::UNIT;
   auto tiles = [](int n) { return (n + TILE_N - 1) / TILE_N; };
@@ -977,7 +1009,13 @@ static bool rows_setup(int grid, const ModelRt &M, RowsModel &rm) {
   rm.slot = rows_gemm::MIN_SLOT;
   const int gu = rows_plan(G_GATEUP, n_units[G_GATEUP], K[G_GATEUP] / BLOCK_K, n_tiles[G_GATEUP], grid, rm.slot).up;
   if (gu <= 8) rm.slot = std::max(rm.slot, 2 * gu * U * 128);
-  for (int k = 0; k < 5; ++k) rm.plan[k] = rows_plan(k, n_units[k], K[k] / BLOCK_K, n_tiles[k], grid, rm.slot);
+  int kb[5];
+  for (int k = 0; k < 5; ++k) {
+    kb[k] = K[k] / BLOCK_K;
+    rm.plan[k] = rows_plan(k, n_units[k], kb[k], n_tiles[k], grid, rm.slot);
+    rows_share(rm.plan[k], kb[k], rm.plan[k].cut_per, rows_gemm::slots_for(rm.slot, d.d_model + rows_x_bytes(d), smem_max));
+  }
+  if (!rows_pay(rm.plan, kb, d.n_layers)) return true;
   auto plain = [&](CUtensorMap *m, const void *w, int rows, int kind) {
     return make_map_rows(m, w, rows, K[kind], rm.plan[kind].up * (kind == G_GATEUP ? 8 : U), rm.plan[kind].nkb);
   };
@@ -1085,7 +1123,7 @@ int ouro_fast_setup(ouro_ctx *c) {
       ok = make_map(&fm.x_d[i], c->a.xn, OURO_TEXT_ROWS, d.d_model, 16 * (i + 1)) &&
            make_map(&fm.x_q[i], c->a.att, OURO_TEXT_ROWS, dq, 16 * (i + 1)) &&
            make_map(&fm.x_f[i], c->a.act, OURO_TEXT_ROWS, d.d_ffn, 16 * (i + 1));
-    if (ok && rows_x_bytes(d) > 0) ok = rows_setup(f->s.grid, M, fm.rm);
+    if (ok && rows_x_bytes(d) > 0) ok = rows_setup(f->s.grid, smem, M, fm.rm);
     if (!ok) {
       delete f;
       c->err = "cuTensorMapEncodeTiled failed";
@@ -1187,10 +1225,7 @@ static void launch_rows(ouro_ctx *c) {
     rows_gemm::Plan &pl = kp.told.plan[i];
     pl = rm.plan[kind];
     grid = std::max(grid, (pl.units + pl.up * pl.passes - 1) / (pl.up * pl.passes));
-    pl.max_pieces = g.per > 0 && g.per < g.kb ? std::min(g.kb, (g.kb - 1) / g.per + 2) : 1;
-    // All units of a pass lie in one tile, and are cut alike, where their number divides a tile's (a matrix begins at a multiple of four).
-    pl.share = pl.up <= 2 || pl.up == 4 ? std::min(std::min(rows_gemm::CW / pl.up, pl.max_pieces), kp.slots - 1) : 1;
-    if (pl.up * pl.max_pieces > rows_gemm::PARKED) pl.share = 1;
+    rows_share(pl, g.kb, g.per, kp.slots);                        // (the cut is the chain's)
     pl.q_in = pl.q_out = s.squares;
     pl.x_in = (const __nv_bfloat16 *)(kind == G_WO ? c->a.att : kind == G_DOWN ? c->a.act : c->a.xn);
     if (i > 0 || front) pl.packets_in = kind == G_WO ? patt : kind == G_DOWN ? pact : px;
@@ -1207,6 +1242,7 @@ static void launch_rows(ouro_ctx *c) {
   }
   kp.front = cp.fold.part ? patt : px;
   kp.told.args = cp;
+  ++s.rows_launches;
   launch_pdl(rows_gemm::gemm_rows_kernel, grid, rows_gemm::THREADS, (size_t)s.smem_max, c->stream, kp);
 }
 // Launches the GEMMs collected so far as one chain.
@@ -1274,6 +1310,15 @@ void ouro_fast_reset(ouro_ctx *c) {
   cp.n = 0;
   cp.fold.part = nullptr;
   cp.embed.table = nullptr;
+}
+// values[1..7] of ouro_debug_counts.
+void ouro_fast_counts(const ouro_ctx *c, uint32_t *values) {
+  if (!c->fast) return;
+  const FastState &s = c->fast->s;
+  static_assert(OURO_DEBUG_COUNTS == 3 + MAX_CHAIN + 1, "one value each");
+  values[1] = s.rows_launches;
+  values[2] = s.mark;
+  for (int i = 0; i <= MAX_CHAIN; ++i) values[3 + i] = s.finished_host[i];
 }
 // What the launches so far leave behind if one of them has given up.
 Leftovers ouro_leftovers(ouro_ctx *c) {

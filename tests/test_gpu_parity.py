@@ -1584,12 +1584,19 @@ def test_groups_shared_by_several_ctas_are_bit_identical_to_plain_decoding(kv, K
 
 @pytest.mark.parametrize("d,heads,kv,hd,ffn,vocab", [
     (512, 4, 2, 128, 512, 1000),          # one unit per CTA, every GEMM in pieces of one k-block; half a unit of the vocabulary
-    (320, 5, 5, 64, 9536, 520),           # heads that leave half a tile of every matrix empty; nine units per CTA, one tile cut beside whole ones
+    (320, 5, 5, 64, 9536, 520),           # heads that leave half a tile of every matrix empty, one tile cut beside whole ones
+    (320, 5, 5, 64, 1280, 520),           # the same on a single row's kernel
     (2048, 32, 4, 64, 5632, 64000),       # pieces taken in turn, more of them than warps share (q,k,v) and fewer; three passes of the head
     (2048, 32, 32, 64, 512, 4104),        # three units per CTA that no tile holds together
-    (1024, 8, 8, 128, 24576, 1000),       # activations of 48 KB, three passes of seven units, twenty pieces
-    (7168, 8, 8, 128, 512, 1000),         # four units per CTA, two warps each
+    (1024, 8, 8, 128, 24576, 1000),       # a down projection that is too long for a single row's kernel
+    (1536, 12, 3, 128, 12288, 1000),      # activations of 24 KB, two passes of six units
+    (1024, 8, 2, 128, 11264, 1000),       # ten units per CTA, one tile cut beside whole ones; nineteen pieces
+    (1024, 8, 2, 128, 4096, 1000),        # four units per CTA, two warps each
+    (256, 2, 1, 128, 1536, 1000),         # as many pieces as are parked at a time
+    (7168, 8, 8, 128, 512, 1000),         # q, k and v too long for a single row's kernel
     (4096, 32, 32, 128, 11008, 1000),     # a layer beyond the single row's kernels
+    (1792, 14, 2, 128, 4864, 1000),       # seven query heads per kv head: two rows fill the attention's tile but for two
+    (1024, 16, 2, 128, 2816, 1000),       # eight: two rows fill it
 ])
 def test_few_rows_are_bit_identical_to_wider_blocks(d, heads, kv, hd, ffn, vocab):
     """A single row of a model of small layers runs on GEMM kernels of its own, and up to 16 query rows of a kv head without
@@ -1662,3 +1669,31 @@ def test_single_rows_with_a_late_warp(monkeypatch, fuse):
         if want is None:
             want = got
     assert got[0] == want[0] and torch.equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("layers,d,heads,kv,hd,ffn,vocab,owned", [
+    (1, 512, 4, 2, 128, 512, 1000, True),
+    (1, 256, 2, 1, 128, 2048, 1000, True),         # 32 k-blocks walked by one warp a unit, in a layer of 3 MB
+    (1, 256, 2, 1, 128, 2816, 1000, False),        # 44
+    (1, 512, 4, 1, 128, 28672, 1000, False),       # 448
+    (1, 384, 48, 6, 64, 1024, 1000, False),        # an output projection of 48
+    (1, 1024, 8, 2, 128, 11264, 1000, True),       # 72 MB
+    (1, 1536, 12, 3, 128, 9216, 1000, False),      # 92 MB, 36 k-blocks of the down projection on 96 CTAs
+    (1, 2048, 32, 4, 64, 5632, 32000, True),
+    (1, 2560, 20, 5, 128, 10240, 1000, False),     # beyond 160 MB
+    (3, 256, 2, 1, 128, 256, 262144, False),       # twelve passes of the head behind three layers
+    (4, 256, 2, 1, 128, 256, 262144, True),        # ... and four
+    (1, 512, 4, 4, 96, 512, 1000, False),          # another head dim
+])
+def test_single_rows_take_the_kernel_that_is_faster(layers, d, heads, kv, hd, ffn, vocab, owned):
+    """Shapes on either side of the lines behind which a single row's own GEMM kernel was measured slower than the
+    kernel of wider blocks (narrow layers with a long K: up to twice as slow)."""
+    desc = synth.ModelDesc(layers, d, heads, kv, hd, ffn, vocab, 64, "bf16")
+    eng = binding.Engine(desc, synth.model_weights(desc, 3, device="cuda:0"), synth.DecodeParams(4, 5, 3, 16, 8))
+    for n in (1, 2):
+        eng.set_state(20, 1)
+        eng.assemble_causal(binding.OURO_TARGET, np.arange(n, dtype=np.int32))
+        eng.verify_forward()
+        counts = eng.debug_counts()
+        assert counts["status"] == 0 and counts["rows_launches"] == (layers + 1 if owned else 0), n     # (layers + 1 launches a row)
+    eng.close()
