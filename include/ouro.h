@@ -241,10 +241,10 @@ int ouro_profile_enable(ouro_ctx *ctx, int kernel_class);
  * ouro_generate, ouro_generate_vanilla) returns OURO_ETIMEOUT, and ouro_reset or ouro_set_state makes the context usable
  * again.  OURO_ESTATE when no kernel of the context waits in this way. */
 int ouro_debug_set_wait_limit(ouro_ctx *ctx, int64_t polls);
-/* Test aid: the first n (at most OURO_DEBUG_COUNTS) of these values, once everything launched so far is done.  [0] the status word; [1]
- * launches so far of the single rows' GEMM kernel; [2] the mark of its next launch; [3..7] the counters by which the GEMMs of a launch of
- * the other kernel hand over, [7] that of the work in front of the first (both modulo 2^32). */
-enum { OURO_DEBUG_COUNTS = 8 };
+/* Test aid: the first n (at most OURO_DEBUG_COUNTS) of these values, once everything launched so far is done.  [0] the status word; [1] and [2]
+ * launches so far of the single rows' GEMM kernel and of the few rows' attention kernel; [3] the mark of the former's next launch; [4..8] the
+ * counters by which the GEMMs of a launch of the other GEMM kernel hand over, [8] that of the work in front of the first (modulo 2^32). */
+enum { OURO_DEBUG_COUNTS = 9 };
 int ouro_debug_counts(ouro_ctx *ctx, uint32_t *values, int32_t n);
 int ouro_profile_read(ouro_ctx *ctx, float *ms_total, int32_t *launches);
 

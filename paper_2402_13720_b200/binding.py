@@ -353,9 +353,9 @@ class Engine:
         self._ck(self.L.ouro_debug_set_wait_limit(self.ctx, int(polls)))
 
     def debug_counts(self):
-        v = (C.c_uint32 * 8)()
-        self._ck(self.L.ouro_debug_counts(self.ctx, v, 8))
-        return dict(status=v[0], rows_launches=v[1], mark=v[2], counters=list(v[3:]))
+        v = (C.c_uint32 * 9)()
+        self._ck(self.L.ouro_debug_counts(self.ctx, v, 9))
+        return dict(status=v[0], rows_launches=v[1], few_launches=v[2], mark=v[3], counters=list(v[4:]))
 
     # ---- loops -------------------------------------------------------------------------------
     def generate(self, prompt, max_new, keep_pool=False):

@@ -3,8 +3,8 @@
 // attn_tm_kernel walks a span of keys chunk by chunk: scores into TMEM, softmax, P to shared memory, P V into TMEM, each
 // behind the one before, and a tile of 128 query rows of which a single token fills one.  That chain, 1.75 us a chunk behind
 // 2 us of set-up, is what plain decoding spends on attention whatever the keys are.  (One row, us a forward, attn_tm_kernel and this
-// one: two layers of 512 behind 150 keys 62.7 and 59.2, behind 400 69.0 and 62.6; three layers of the 7B shape behind 150 keys 289 and
-// 285; of 4096 with 4 kv heads 261 and 257.)  Here up to 16 query rows of a kv head (rows x query heads) are one mma.sync tile, and the four chunks of a
+// one: two layers of 512 behind 150 keys 62.7 and 59.2, behind 400 69.0 and 62.6; three layers of the 7B shape behind 100 keys 289 and
+// 283; where it is used and where it would be slower: attention_few_pays in gemm_tc.cu.)  Here up to 16 query rows of a kv head (rows x query heads) are one mma.sync tile, and the four chunks of a
 // span are worked on at the same time, each by four warps:
 //     S = Q K^T     a warp has 32 of the chunk's keys, their K straight in registers (one 8-byte piece per step and key),
 //     maxima        of all four chunks through shared memory: every chunk then knows the running maximum it would have met,

@@ -896,6 +896,7 @@ struct FastState {
   uint32_t mark = 1;            // of the next launch's first packets; never zero, which an empty packet has
   uint32_t late = 0;            // test aid, see rows_gemm::Params
   uint32_t rows_launches = 0;   // of gemm_rows.cuh so far
+  uint32_t few_launches = 0;    // of attn_few.cu
   float *squares = nullptr;     // squares of four columns each of the residual stream, as gemm_rows.cuh leaves them
   int chain_kind[MAX_CHAIN] = {0, 0, 0, 0};
   bool fuse = true;             // run consecutive GEMMs as one launch
@@ -1311,14 +1312,15 @@ void ouro_fast_reset(ouro_ctx *c) {
   cp.fold.part = nullptr;
   cp.embed.table = nullptr;
 }
-// values[1..7] of ouro_debug_counts.
+// values[1..8] of ouro_debug_counts.
 void ouro_fast_counts(const ouro_ctx *c, uint32_t *values) {
   if (!c->fast) return;
   const FastState &s = c->fast->s;
-  static_assert(OURO_DEBUG_COUNTS == 3 + MAX_CHAIN + 1, "one value each");
+  static_assert(OURO_DEBUG_COUNTS == 4 + MAX_CHAIN + 1, "one value each");
   values[1] = s.rows_launches;
-  values[2] = s.mark;
-  for (int i = 0; i <= MAX_CHAIN; ++i) values[3 + i] = s.finished_host[i];
+  values[2] = s.few_launches;
+  values[3] = s.mark;
+  for (int i = 0; i <= MAX_CHAIN; ++i) values[4 + i] = s.finished_host[i];
 }
 // What the launches so far leave behind if one of them has given up.
 Leftovers ouro_leftovers(ouro_ctx *c) {
@@ -1494,6 +1496,27 @@ static int text_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
   return OURO_OK;
 }
 
+// Whether a block of `rows` rows that sees up to `keys` keys is attended to by attn_few_kernel: rows in order that fill one
+// small tile, whose chunks it takes side by side.  What it saves is attn_tm_kernel's chain; what it costs is that its CTAs, four chunks
+// of K and V in flight each, share the HBM with the weights on their way to the next kernel, more of them the more kv heads and spans, and
+// that P and O of all query rows go through shared memory.  Time of a forward of three layers with attn_tm_kernel over that with this one, both in
+// one process (which differ by half a percent; where in memory a build's kernels lie makes one and the same kernel up to 2 % slower):
+//   one chunk (behind 60 or 110 keys): 1.00 to 1.13 in all of 100 cases (7B shape, one row, 1.04; 16 rows 1.02)
+//   one span, up to 8 query rows, behind 150 to 480 keys: 7B shape (32 kv heads) 1.02 to 1.00, 4096 wide with 16 / 8 / 4 kv heads of 1, 4 and 8
+//   query heads 1.04 to 1.01 / 1.03 to 1.01 / 1.03 to 1.02, 34B shape 1.01 to 1.00, two layers of 512 1.04 to 1.15; the worst 0.99 (32 x 2 heads, 460 keys)
+//   one span, 9 to 16 query rows: up to 2 kv heads 1.02 to 1.13; 4096 wide, 4 x 1 heads, 16 rows 0.98 to 0.96, 8 x 4, four rows 1.00 to 0.98; 34B shape, two
+//   rows 1.00 to 0.98
+//   several spans in front of gemm_tc_kernel: 4096 wide, 32 kv heads, 900 / 1800 keys 0.98 / 0.96
+//   in front of gemm_rows.cuh, kv heads x spans up to 32: 1.03 to 1.18 (2048 wide, 4 x 8 heads behind 4000 keys 1.09); 64: 1024 wide, 8 x 4 behind 4000
+//   keys 0.97, 16 x 1 behind 1800 1.02; 128: 8 x 4 behind 8000 keys 0.94; 512: 32 x 1 behind 8000 keys 0.83
+static bool attention_few_pays(const FastModel &fm, const ouro_model_desc &d, int rows, int keys, bool candidates) {
+  if (candidates || !attention_few_supported(d, rows)) return false;
+  const int spans = fold::span_count(d.head_dim, keys);
+  if (keys <= fold::CHUNK) return true;
+  if (rows_launch(fm, rows)) return spans * d.n_kv_heads <= 32;
+  return spans <= 1 && (d.n_heads / d.n_kv_heads * rows <= 8 || d.n_kv_heads <= 2);
+}
+
 // One decoder layer with the tensor-core GEMMs (kv_only: up to its keys and values); OURO_ESTATE when the model does not
 // qualify.
 int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
@@ -1555,17 +1578,14 @@ int ouro_fast_layer(ouro_ctx *c, int which, int l, int rows, bool kv_only) {
         pf.ptr[1] = M.w_gate[l]; pf.bytes[1] = head;
         pf.ptr[2] = M.w_up[l]; pf.bytes[2] = head;
       }
-      // Rows in order that fill one small tile: in one span its chunks side by side are faster than attn_tm_kernel's one behind
-      // the other (one row behind 150 keys, three 7B layers 289 -> 285 us, two of 512 62.7 -> 59.2; behind 400 keys 300 and 300,
-      // 69.0 -> 62.6).  With more spans they gain in front of gemm_rows.cuh only (two layers of 512 behind 1800 keys 56.6 -> 48.4 us;
-      // three 7B layers, in front of gemm_tc_kernel, 310 -> 322: the CTAs of several spans are the ones that share the HBM with
-      // the weights on their way to the next kernel).
-      if (!M.blk_is_candidate && attention_few_supported(d, rows) && (fold::span_count(d.head_dim, M.L + rows) <= 1 || rows_launch(fm, rows)))
+      if (attention_few_pays(fm, d, rows, M.L + rows, M.blk_is_candidate)) {
+        ++c->fast->s.few_launches;
         pieces = launch_attention_few(d, a.q, M.k_cache, M.v_cache, M.blk, rows, M.L, M.L + rows, l, c->fast->s.attn_part, a.att, c->cur_rows_dev, pf, s);
-      else
+      } else {
         pieces = launch_attention_tm(d, a.q, &c->fast->s.m[which].kmap, &c->fast->s.m[which].vmap, M.k_cache, M.v_cache, M.blk, rows,
                                    M.blk_is_candidate ? 1 + std::max(1, c->p.K) : 1, M.L, M.L, M.L + rows, l, c->fast->s.attn_part, a.att,
                                    &c->st->status, c->cur_rows_dev, pf, c->sms, s);
+      }
     }
     else if (attention_tc_supported(d))
       pieces = launch_attention_tc(d, a.q, M.k_cache, M.v_cache, M.blk, rows, M.L, M.L, M.L + rows, l, c->fast->s.attn_part, a.att,

@@ -1697,3 +1697,24 @@ def test_single_rows_take_the_kernel_that_is_faster(layers, d, heads, kv, hd, ff
         counts = eng.debug_counts()
         assert counts["status"] == 0 and counts["rows_launches"] == (layers + 1 if owned else 0), n     # (layers + 1 launches a row)
     eng.close()
+
+
+@pytest.mark.parametrize("d,heads,kv,ffn,rows,keys,few", [
+    (4096, 32, 32, 11008, 16, 128, True), (4096, 32, 32, 11008, 8, 512, True), (4096, 32, 32, 11008, 9, 129, False),
+    (4096, 32, 32, 11008, 1, 513, False), (4096, 32, 8, 11008, 2, 512, True), (4096, 32, 8, 11008, 2, 513, False), (4096, 32, 8, 11008, 3, 129, False),
+    (4096, 64, 8, 4096, 2, 128, True), (4096, 64, 8, 4096, 2, 200, False), (512, 4, 2, 512, 8, 512, True), (512, 4, 2, 512, 9, 60, False),
+    (512, 4, 2, 512, 2, 513, False), (512, 4, 2, 512, 1, 8192, True), (512, 4, 4, 512, 1, 4096, True), (512, 4, 4, 512, 1, 4097, False),
+    (1024, 32, 32, 2816, 1, 512, True), (1024, 32, 32, 2816, 1, 513, False),
+])
+def test_few_rows_take_the_attention_that_is_faster(d, heads, kv, ffn, rows, keys, few):
+    """Blocks on either side of the lines behind which attention with a span's chunks side by side was measured slower: one chunk or
+    more, one span or more, query rows, kv heads, kv heads times spans in front of the single rows' GEMMs.  `keys`: those the last row
+    sees."""
+    desc = synth.ModelDesc(1, d, heads, kv, 128, ffn, 1000, 8448, "bf16")
+    eng = binding.Engine(desc, synth.model_weights(desc, 3, device="cuda:0"), synth.DecodeParams(4, 5, 3, 16, 8))
+    eng.set_state(keys - rows, 1)
+    eng.assemble_causal(binding.OURO_TARGET, np.arange(rows, dtype=np.int32))
+    eng.verify_forward()
+    counts = eng.debug_counts()
+    assert counts["status"] == 0 and counts["few_launches"] == few
+    eng.close()
