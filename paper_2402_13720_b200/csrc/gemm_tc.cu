@@ -973,28 +973,32 @@ static rows_gemm::Plan rows_plan(int kind, int units, int kb, int tiles, int gri
   else { pl.su = rows_gemm::UNIT; pl.sj = rows_gemm::UNIT * pl.up; pl.sh = 8; }
   return pl;
 }
-// Whether owned weight rows are faster than gemm_tc_kernel's cut tiles.  They save the tails and the hand-overs' round trips, 5 to 8 us a
-// small layer.  They cost a chain: the k-blocks that the busiest warp of a GEMM takes one behind another, 0.1 us each, where
-// gemm_tc_kernel deals a long K out to all SMs; as far as it is not hidden by the stream, of which 0.4 was found to count.  `late` is the
-// sum of that over a layer, in us, and the line at 2.25, in layers below 11 MB rising to 4 (the stream of a wide layer hides more of
-// the tails there).  One row behind 150 keys, three layers, gemm_tc.cu and here, us a forward, of d_model x d_ffn (late): 512 x 1024 87 and 69 (0.3),
-// 512 x 2048 87 and 85 (3.2), 512 x 4096 91 and 94 (6.5), 512 x 28672 126 and 238 (43); 256 x 2048 88 and 83 (3.3), 256 x 2816 91 and 94 (4.7);
-// 384 x 1024 with 3072 query columns 101 and 108 (4.8); 1024 x 4096 95 and 88 (0.9), 1024 x 11264 114 and 102 (1.9), 1024 x 16384 125 and 128
-// (4.0); 768 x 8448 99 and 104 (2.6); 1536 x 6144 107 and 101 (0.8), 1536 x 9216 115 and 118 (2.3), 1536 x 16896 149 and 160 (6.6); 2048 x 5632
-// 113 and 105 (1.4); 2560 x 7040 136 and 126 (2.0), 2560 x 10240, beyond 160 MB, 151 and 155.  The head costs 1 us more in each of its passes
-// than it does there (one layer of 512 in front of 65536 / 262144 logits 44 / 79 us and 42 / 86), which each layer's saving makes up
-// for a few of.
-static bool rows_pay(const rows_gemm::Plan *plan, const int *kb, int n_layers) {
-  double late = 0, stream = 0;
+// Whether owned weight rows are faster than gemm_tc_kernel's cut tiles.  They save the tails and the hand-overs' round trips, 2 to 8 us a
+// layer, and with head dim 128 in several spans of keys the attention in front as well (attention_few_pays).  They cost a chain: the k-blocks
+// that the busiest warp of a GEMM takes one behind another, 0.1 us each, where gemm_tc_kernel deals a long K out to all SMs.  `beyond` is what
+// a layer's chains take longer than the streams of their weights, in us; `late` the same against 0.4 of the streams, of which a long
+// one on few warps does not hide all.  One row, three layers, gemm_tc.cu over here behind 150 / 1800 keys, of d_model x d_ffn (beyond, late),
+// measured on 157 shapes:
+//   head dim 128: 512 x 2048 1.05 / 1.22 (2.9, 3.2), 512 x 3072 1.05 / 1.22 (4.3, 5.1), 768 x 3072 0.96 / 1.13 (4.1, 5.4), 384 x 3072 0.94 / 1.10 (4.5,
+//   5.1), 768 x 4608 0.92 / 1.09 (6.1, 7.3), 256 x 1792 with 2048 query columns 0.90 / 1.04 (5.7, 5.9), 512 x 28672 0.53 / 0.58 (40, 43); 2176 x 3968
+//   1.04 / 1.20 (0, 3.1), 2560 x 7040 1.08 / 1.17 (0, 2.0), 1024 x 11264 1.14 / 1.28 (0, 1.9), 1536 x 9216 0.96 / 0.99 (0, 2.3), 1536 x 16896 0.93 / 0.93
+//   (0.9, 6.6), 4096 x 2048 0.97 / 1.11 (0, 6.3)
+//   head dim 64: 2048 x 5632 1.2 / 1.2 (0, 1.3), 256 x 1600 1.13 / 1.09 (2.5, 2.7), 2240 x 768 1.00 / 1.01 (3.1, 3.6), 384 x 3200 1.06 / 1.07 (4.7, 5.4), 384
+//   x 1024 with 3072 query columns 0.95 / 0.96 (4.5, 4.8), 320 x 1600 0.97 / 0.96 (5.0, 5.2), 1984 x 256 0.88 / 0.90 (5.6, 6.0); 4096 x 4096 with 512
+//   query columns 0.96 / 0.97 (0, 2.9): the worst that is let in
+// The head costs 1 us more in each of its passes than it does there (one layer of 512 in front of 65536 / 262144 logits 44 / 79 us
+// and 42 / 86), which each layer's saving makes up for a few of.
+static bool rows_pay(const rows_gemm::Plan *plan, const int *kb, int head_dim, int n_layers) {
+  double beyond = 0, late = 0;
   for (int k = 0; k < 4; ++k) {
     const rows_gemm::Plan &pl = plan[k];
     const int step = (pl.cut_per + pl.nkb - 1) / pl.nkb * pl.nkb;
-    const int walk = pl.passes * (pl.share == 1 ? kb[k] : (pl.max_pieces + pl.share - 1) / pl.share * step);
-    const double us = (double)pl.units * rows_gemm::UNIT * kb[k] * BLOCK_K * 2 / 6.5e6;
-    late += std::max(0.0, 0.1 * walk - 0.4 * us);
-    stream += us;
+    const double walk = 0.1 * pl.passes * (pl.share == 1 ? kb[k] : (pl.max_pieces + pl.share - 1) / pl.share * step);
+    const double stream = (double)pl.units * rows_gemm::UNIT * kb[k] * BLOCK_K * 2 / 6.5e6;
+    beyond += std::max(0.0, walk - stream);
+    late += std::max(0.0, walk - 0.4 * stream);
   }
-  return late <= std::max(2.25, 4.0 - 0.25 * stream) && plan[G_HEAD].passes <= 3 * n_layers;
+  return beyond <= (head_dim == 128 ? 4.4 : 3.3) && late <= 6.0 && plan[G_HEAD].passes <= 3 * n_layers;
 }
 static bool rows_setup(int grid, int smem_max, const ModelRt &M, RowsModel &rm) {
   const ouro_model_desc &d = M.d;
@@ -1016,7 +1020,7 @@ static bool rows_setup(int grid, int smem_max, const ModelRt &M, RowsModel &rm) 
     rm.plan[k] = rows_plan(k, n_units[k], kb[k], n_tiles[k], grid, rm.slot);
     rows_share(rm.plan[k], kb[k], rm.plan[k].cut_per, rows_gemm::slots_for(rm.slot, d.d_model + rows_x_bytes(d), smem_max));
   }
-  if (!rows_pay(rm.plan, kb, d.n_layers)) return true;
+  if (!rows_pay(rm.plan, kb, d.head_dim, d.n_layers)) return true;
   auto plain = [&](CUtensorMap *m, const void *w, int rows, int kind) {
     return make_map_rows(m, w, rows, K[kind], rm.plan[kind].up * (kind == G_GATEUP ? 8 : U), rm.plan[kind].nkb);
   };

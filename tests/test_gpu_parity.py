@@ -1588,12 +1588,12 @@ def test_groups_shared_by_several_ctas_are_bit_identical_to_plain_decoding(kv, K
     (320, 5, 5, 64, 1280, 520),           # the same on a single row's kernel
     (2048, 32, 4, 64, 5632, 64000),       # pieces taken in turn, more of them than warps share (q,k,v) and fewer; three passes of the head
     (2048, 32, 32, 64, 512, 4104),        # three units per CTA that no tile holds together
-    (1024, 8, 8, 128, 24576, 1000),       # a down projection that is too long for a single row's kernel
+    (1024, 8, 8, 128, 24576, 1000),       # activations of 48 KB, three passes of seven units, twenty pieces: too long for a single row's kernel
     (1536, 12, 3, 128, 12288, 1000),      # activations of 24 KB, two passes of six units
     (1024, 8, 2, 128, 11264, 1000),       # ten units per CTA, one tile cut beside whole ones; nineteen pieces
     (1024, 8, 2, 128, 4096, 1000),        # four units per CTA, two warps each
     (256, 2, 1, 128, 1536, 1000),         # as many pieces as are parked at a time
-    (7168, 8, 8, 128, 512, 1000),         # q, k and v too long for a single row's kernel
+    (7168, 8, 8, 128, 512, 1000),         # four units per CTA, two warps each, k-blocks by the hundred
     (4096, 32, 32, 128, 11008, 1000),     # a layer beyond the single row's kernels
     (1792, 14, 2, 128, 4864, 1000),       # seven query heads per kv head: two rows fill the attention's tile but for two
     (1024, 16, 2, 128, 2816, 1000),       # eight: two rows fill it
@@ -1674,11 +1674,13 @@ def test_single_rows_with_a_late_warp(monkeypatch, fuse):
 @pytest.mark.parametrize("layers,d,heads,kv,hd,ffn,vocab,owned", [
     (1, 512, 4, 2, 128, 512, 1000, True),
     (1, 256, 2, 1, 128, 2048, 1000, True),         # 32 k-blocks walked by one warp a unit, in a layer of 3 MB
-    (1, 256, 2, 1, 128, 2816, 1000, False),        # 44
+    (1, 512, 4, 1, 128, 3072, 1000, True),         # 48
+    (1, 384, 3, 1, 128, 3072, 1000, False),        # ... in a smaller layer
     (1, 512, 4, 1, 128, 28672, 1000, False),       # 448
-    (1, 384, 48, 6, 64, 1024, 1000, False),        # an output projection of 48
+    (1, 256, 15, 5, 64, 1600, 1000, True),         # head dim 64: 25
+    (1, 384, 48, 6, 64, 1024, 1000, False),        # ... an output projection of 48
     (1, 1024, 8, 2, 128, 11264, 1000, True),       # 72 MB
-    (1, 1536, 12, 3, 128, 9216, 1000, False),      # 92 MB, 36 k-blocks of the down projection on 96 CTAs
+    (1, 1536, 12, 3, 128, 16896, 1000, False),     # 88 k-blocks of the down projection, 48 of gate and up, in 152 MB
     (1, 2048, 32, 4, 64, 5632, 32000, True),
     (1, 2560, 20, 5, 128, 10240, 1000, False),     # beyond 160 MB
     (3, 256, 2, 1, 128, 256, 262144, False),       # twelve passes of the head behind three layers
