@@ -234,7 +234,8 @@ enum {
 uint64_t ouro_kernel_launches(void);
 int ouro_profile_enable(ouro_ctx *ctx, int kernel_class);
 /* Test aid for the give-up path of the bounded device-side waits (no counterpart in the paper).  A GEMM tile whose K
- * range is split across CTAs is finished once all contributors have published their partial sums, and the steps of a
+ * range is split across CTAs is finished once all contributors have published their partial sums, the activations of a
+ * single row reach its GEMMs in packets, and the steps of a
  * small model's one-launch forward are separated by barriers; the waiting threads poll memory at most `polls` times
  * (default 1 << 22; negative restores the default).  0 makes these waits give up at once: the kernels return normally,
  * the status word is raised, the next call that reads results back (ouro_accept_and_compact, ouro_verify_step,

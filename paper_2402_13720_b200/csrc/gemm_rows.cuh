@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_rows_kernel(const __grid_cons
         if (pass == 0) {
           if (ct == 0) TRACE(1);
           if (w >= CW - GATHERERS) {
-            good = __all_sync(0xffffffffu, gather(p, pl, kp.mark + ci, ci > 0 ? p.wait_limit : 1u << 22, squares, xs, ct - (CTHREADS - GTHREADS)));
+            good = __all_sync(0xffffffffu, gather(p, pl, kp.mark + ci, p.wait_limit, squares, xs, ct - (CTHREADS - GTHREADS)));
             if (lane == 0) mbar_arrive(x_full);
           }
           if (good) good = warp_wait(x_full, n_gathered & 1, abort_flag);

@@ -110,7 +110,7 @@ struct GemmParams {
   float *scratch;     // [grid][2][128, or 256 in a wide launch][128] partial tiles; a word that holds no partial sum holds EMPTY
   int *status;        // context status word
   int trace_id;           // which GEMM of the layer this is (timeline builds only)
-  uint32_t wait_limit;    // polls of a partial-tile wait before it gives up (1 << 22 unless a test shortens it)
+  uint32_t wait_limit;    // polls of a partial tile, or of packets, before the wait gives up (1 << 22 unless a test shortens it)
 };
 
 // A chain of GEMMs run by one persistent launch, each consuming what the one before produced (output projection ->

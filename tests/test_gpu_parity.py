@@ -899,14 +899,17 @@ def test_bounded_wait_gives_up_and_the_context_recovers():
 
 
 @pytest.mark.parametrize("fuse", ["0", "1"])
-def test_give_up_that_nobody_read_ends_with_the_state(monkeypatch, fuse):
+@pytest.mark.parametrize("ffn", [512, 7168])
+def test_give_up_that_nobody_read_ends_with_the_state(monkeypatch, ffn, fuse):
     """Only acceptance and the whole loops read the status word.  A wait that runs out in a forward or while drafting leaves
     sums nobody fetched in the partial-tile slots; set_state clears the status, so the slots must be empty again with it: the
     step that follows gives the bits it gave before and no time-out.  One launch per GEMM (no hand-over counter in the way)
-    and chained launches; one row and a candidate block."""
+    and chained launches; one row (on the single rows' kernel, which waits for packets, and, with the long FFN, on the kernel of all blocks),
+    a few and a candidate block.  Each time a wait must really have run out."""
     monkeypatch.setenv("OURO_FUSE", fuse)
     P = synth.DecodeParams(4, 9, 4, 16, 8, harvest_matched=False, harvest_candidates=False, harvest_accepted=False)
-    eng, _ = make(MIDB, P, 2, draft=MIDB)          # d 256: every q,k,v tile is split four ways
+    desc = dataclasses.replace(MIDB, d_ffn=ffn)
+    eng, _ = make(desc, P, 2, draft=desc)          # d 256: every q,k,v tile is split four ways
     prompt = synth.prompt(2, MIDB.vocab, 40, 0.4, 4, 8)
     eng.reset(); eng.prefill(prompt)
     L, d = len(prompt) - 1, [1, 2, 3, int(prompt[5])]
@@ -922,25 +925,36 @@ def test_give_up_that_nobody_read_ends_with_the_state(monkeypatch, fuse):
         eng.assemble_causal(binding.OURO_TARGET, [5])
         eng.verify_forward()
 
+    def few_rows():
+        eng.assemble_causal(binding.OURO_TARGET, [5, 6, 7, 8, 9])
+        eng.verify_forward()
+
     def candidates():
         eng.assemble_candidates(draft=d)
         eng.verify_forward()
 
     want = step()
-    for give_up in (one_row, candidates, eng.draft):
+    for give_up in (one_row, few_rows, candidates, eng.draft):
         eng.set_state(L, int(prompt[-1]))
         eng.set_wait_limit(0)
+        before = eng.debug_counts()
         give_up()
+        after = eng.debug_counts()
         eng.set_wait_limit(-1)
+        assert before["status"] == 0 and after["status"] != 0, give_up
+        if give_up is one_row:
+            assert (after["rows_launches"] > before["rows_launches"]) == (ffn == 512)
         got = step()
         assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1]) and got[2] == want[2], give_up
-    eng.set_wait_limit(0)
-    one_row()
-    eng.set_wait_limit(-1)
-    eng.reset()
-    eng.prefill(prompt)
-    got = step()
-    assert torch.equal(got[1], want[1])
+    for give_up in (one_row, few_rows):
+        eng.set_wait_limit(0)
+        give_up()
+        assert eng.debug_counts()["status"] != 0
+        eng.set_wait_limit(-1)
+        eng.reset()
+        eng.prefill(prompt)
+        got = step()
+        assert torch.equal(got[1], want[1]), give_up
     eng.close()
 
 
@@ -955,12 +969,12 @@ def _partial_tile_slots(eng):
     return ws[ends[0] - n: ends[0]]
 
 
-@pytest.mark.parametrize("heads,kv,hd", [(8, 2, 64), (4, 2, 128)])
-def test_every_launch_leaves_the_partial_tile_slots_empty(heads, kv, hd):
+@pytest.mark.parametrize("heads,kv,hd,ffn", [(8, 2, 64, 704), (4, 2, 128, 704), (4, 2, 128, 7168)])
+def test_every_launch_leaves_the_partial_tile_slots_empty(heads, kv, hd, ffn):
     """A scratch word counts as arrived when it is anything but EMPTY, so whoever fetches a sum empties the word again.
     After forwards of every kernel size (up to 32, 48, 128 and 256 rows, whose slots are laid out differently), with the row count
-    on the device or on the host, and after whole loops, no word may be left full."""
-    desc = synth.ModelDesc(2, 256, heads, kv, hd, 704, 1000, 700, "bf16")
+    on the device or on the host, and after whole loops, no word may be left full.  (Single rows use slots with the long FFN only.)"""
+    desc = synth.ModelDesc(2, 256, heads, kv, hd, ffn, 1000, 700, "bf16")
     P = synth.DecodeParams(4, 9, 4, 16, 8)
     eng, _ = make(desc, P, 3, draft=desc)
     slots = _partial_tile_slots(eng)
@@ -970,11 +984,13 @@ def test_every_launch_leaves_the_partial_tile_slots_empty(heads, kv, hd):
         torch.cuda.synchronize()
         return bool((slots == -1).all())
 
-    for n in (1, 15, 48, 49, 100, 128):
+    for n in (1, 2, 15, 48, 49, 100, 128):
         eng.reset()
         eng.assemble_causal(binding.OURO_TARGET, prompt[:n])
         eng.verify_forward()
         assert empty(), n
+        if n == 1:
+            assert (eng.debug_counts()["rows_launches"] > 0) == (ffn == 704)
     for n in (130, 200, 257, 420):
         eng.reset()
         eng.prefill(prompt[:n])
