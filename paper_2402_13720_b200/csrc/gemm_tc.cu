@@ -1215,7 +1215,7 @@ static void launch_rows(ouro_ctx *c) {
   kp.slot = rm.slot;
   kp.slots = rows_gemm::slots_for(rm.slot, d.d_model + rm.x_bytes, s.smem_max);
   if (s.mark > UINT32_MAX - (MAX_CHAIN + 1)) {                    // some hours of decoding: the marks begin anew, on empty packets
-    cudaMemsetAsync(s.packets, 0, s.packets_size, c->stream);
+    if (cudaMemsetAsync(s.packets, 0, s.packets_size, c->stream) != cudaSuccess) return;   // (the layer finds the error; nothing begins anew)
     s.mark = 1;
   }
   kp.mark = s.mark;

@@ -27,7 +27,8 @@ __device__ __forceinline__ float2 unpack(uint32_t v) {
 
 // Four bf16 values on their way from the CTA that computed them to all that need them, in one 128-bit word: a poll that finds
 // the mark has the values as well, so that a hand-over costs one store and one load (no fence, no counter, no second load).
-// A mark is used once: nothing is reset, and what a launch that gave up left behind is not taken for anything.
+// A mark is used once until the host clears all packets and begins anew, before the 32 bits run out: nothing is reset between launches,
+// and what a launch that gave up left behind is not taken for anything.
 struct Packet { uint32_t lo, hi, extra, mark; };
 __device__ __forceinline__ void put_packet(uint4 *dst, uint32_t lo, uint32_t hi, uint32_t extra, uint32_t mark) {
   asm volatile(

@@ -1022,12 +1022,12 @@ def test_partial_sums_that_are_nan_arrive():
     eng.close()
 
 
-@pytest.mark.parametrize("start", [(1 << 31) - 1500, (1 << 32) - 1500])
+@pytest.mark.parametrize("start", [(1 << 31) - 300, (1 << 32) - 300])
 def test_hand_over_counters_pass_the_ends_of_their_range(monkeypatch, start):
-    """The counters by which the GEMMs of a chain hand over are never reset and are compared by their distance.  Started 1500
-    finished shares below 2^31 and 2^32 (a forward of this model counts 24 to 96 per chain position), the more than 80
-    forwards of this test take every one of them across; the text equals that of a context that starts at zero, and the
-    resets and the set_state in between leave the counters alone."""
+    """The counters by which the GEMMs of a chain hand over are never reset and are compared by their distance; the marks of single
+    rows' packets begin anew, on cleared packets, before they run out.  Started 300 below 2^31 and 2^32 (a forward of
+    a block counts 8 to 100 per chain position, one of a single row 20 marks), every one of them goes across; the text equals that of a
+    context that starts at zero, and the resets and the set_state in between leave the counters alone."""
     P = synth.DecodeParams(4, 9, 4, 32, 8)
     prompt = synth.prompt(5, MIDB.vocab, 64, 0.3, 8, 32)
     eng0, _ = make(MIDB, P, 5)
@@ -1044,6 +1044,14 @@ def test_hand_over_counters_pass_the_ends_of_their_range(monkeypatch, start):
     assert np.array_equal(out, want) and stats["target_calls"] < 48
     eng.set_state(70, 3)
     assert np.array_equal(eng.generate_vanilla(prompt, 48)[0], want)
+    counts = eng.debug_counts()
+    gone = [(v - start) % (1 << 32) for i, v in enumerate(counts["counters"]) if i != 3]     # (nobody waits for the last of four GEMMs)
+    assert all(300 < g < 1 << 30 for g in gone), gone
+    assert counts["rows_launches"] > 100
+    if start > 1 << 31:                                            # all launches but the 59 until the marks ran out
+        assert counts["mark"] == 1 + 5 * (counts["rows_launches"] - 59), counts
+    else:
+        assert counts["mark"] == start + 5 * counts["rows_launches"], counts
     eng.close()
 
 
