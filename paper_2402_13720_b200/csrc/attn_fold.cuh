@@ -47,8 +47,10 @@ struct Params {
 template <int HD> constexpr int PIECE = HD + 4;
 template <int HD> struct Dims { typedef float4 V; };
 template <> struct Dims<64> { typedef float2 V; };
-__device__ __forceinline__ void add_scaled(float4 &a, const float4 &o, float w) { a.x += o.x * w; a.y += o.y * w; a.z += o.z * w; a.w += o.w * w; }
-__device__ __forceinline__ void add_scaled(float2 &a, const float2 &o, float w) { a.x += o.x * w; a.y += o.y * w; }
+__device__ __forceinline__ void add_scaled(float4 &a, const float4 &o, float w) {
+  a = make_float4(__fmaf_rn(o.x, w, a.x), __fmaf_rn(o.y, w, a.y), __fmaf_rn(o.z, w, a.z), __fmaf_rn(o.w, w, a.w));
+}
+__device__ __forceinline__ void add_scaled(float2 &a, const float2 &o, float w) { a = make_float2(__fmaf_rn(o.x, w, a.x), __fmaf_rn(o.y, w, a.y)); }
 __device__ __forceinline__ void store_bf16(__nv_bfloat16 *dst, const float4 &a, float s) {
   __nv_bfloat162 lo = __floats2bfloat162_rn(a.x * s, a.y * s), hi = __floats2bfloat162_rn(a.z * s, a.w * s);
   *reinterpret_cast<uint2 *>(dst) = make_uint2(*(uint32_t *)&lo, *(uint32_t *)&hi);
@@ -105,7 +107,7 @@ __device__ __forceinline__ void pairs(const Params &p, int rows, int first, int 
       for (int cc = 0; cc < UNR; ++cc) {
         if (c0 + cc >= ns) break;                                    // uniform in the warp
         const float w = __shfl_sync(0xffffffffu, ml.x, c0 + cc);     // (lane: modulo 32)
-        l += __shfl_sync(0xffffffffu, ml.y, c0 + cc) * w;
+        l = __fmaf_rn(__shfl_sync(0xffffffffu, ml.y, c0 + cc), w, l);
         add_scaled(acc, o[cc], w);
       }
     }

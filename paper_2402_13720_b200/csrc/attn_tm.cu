@@ -535,7 +535,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
           tmem_ld_wait32(v + 32);
           if (act_prev) {
 #pragma unroll
-            for (int j = 0; j < 64; ++j) o_reg[j] = o_reg[j] * alpha_prev + v[j];
+            for (int j = 0; j < 64; ++j) o_reg[j] = __fmaf_rn(o_reg[j], alpha_prev, v[j]);
           }
         }
         pending = false;
@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
             uint32_t w[32];
 #pragma unroll
             for (int j = 0; j < 64; j += 2) {
-              const float p0 = ex2(v[j] * p.scale_log2 - mn), p1 = ex2(v[j + 1] * p.scale_log2 - mn);
+              const float p0 = ex2(__fmaf_rn(v[j], p.scale_log2, -mn)), p1 = ex2(__fmaf_rn(v[j + 1], p.scale_log2, -mn));
               sum4[j & 3] += p0;
               sum4[(j & 3) + 1] += p1;
               w[j >> 1] = pack_bf16(p0, p1);
@@ -617,8 +617,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
               if (active) {
 #pragma unroll
                 for (int j = 0; j < 16; j += 2) {
-                  const float p0 = (pc * 16 + j < nk) ? ex2(v[j] * p.scale_log2 - mn) : 0.f;
-                  const float p1 = (pc * 16 + j + 1 < nk) ? ex2(v[j + 1] * p.scale_log2 - mn) : 0.f;
+                  const float p0 = (pc * 16 + j < nk) ? ex2(__fmaf_rn(v[j], p.scale_log2, -mn)) : 0.f;
+                  const float p1 = (pc * 16 + j + 1 < nk) ? ex2(__fmaf_rn(v[j + 1], p.scale_log2, -mn)) : 0.f;
                   sum4[j & 3] += p0;
                   sum4[(j & 3) + 1] += p1;
                   w[j >> 1] = pack_bf16(p0, p1);
@@ -634,7 +634,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tm_kernel(const __grid_consta
         }
         if (active) {
           alpha = (m_run == -INFINITY) ? 0.f : ex2(m_run - mn);
-          l_run = l_run * alpha + sum;
+          l_run = __fmaf_rn(l_run, alpha, sum);               // (spelled out, as in attn_few_kernel, whose bits are the same)
           m_run = mn;
         }
         fence_async_smem();
