@@ -17,6 +17,22 @@
 #include "row_ops.cuh"
 #include "attn_fold.cuh"
 
+// Optional timeline (compile with -DOURO_TRACE): the points of attn_tm_kernel's, see trace.py.
+#ifdef OURO_TRACE
+__device__ unsigned long long g_attn_few_trace[512][8];
+__device__ __forceinline__ unsigned long long attn_few_trace_now() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)::"memory");
+  return t;
+}
+#define TRACE(slot) do { const int cta_ = blockIdx.y * gridDim.x + blockIdx.x; if (threadIdx.x == 0 && cta_ < 512) g_attn_few_trace[cta_][slot] = attn_few_trace_now(); } while (0)
+extern "C" int ouro_trace_read_attn_few(unsigned long long *out_host) {
+  return (int)cudaMemcpyFromSymbol(out_host, g_attn_few_trace, sizeof(g_attn_few_trace));
+}
+#else
+#define TRACE(slot) do { } while (0)
+#endif
+
 namespace {
 
 constexpr int HD = 128, CH = fold::CHUNK, CHUNKS = fold::LONG_CHUNKS;
@@ -77,6 +93,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_few_kernel(const FewParams p)
   const uint32_t sm_u = smem_u32(smem);
   float *s_max = (float *)(smem + OFF_MAX), *s_sum = (float *)(smem + OFF_SUM);
   pdl_trigger();
+  TRACE(0);
   const int tid = threadIdx.x, lane = tid & 31, team = tid / (32 * TEAM), tw = (tid >> 5) & (TEAM - 1);
   const int sc = blockIdx.x, kvh = blockIdx.y, dkv = p.Hkv * HD, g = p.H / p.Hkv;
   if (tid == 0) {
@@ -134,7 +151,9 @@ __global__ void __launch_bounds__(THREADS, 1) attn_few_kernel(const FewParams p)
     for (int i = tw * 32 + lane; i < CH * 16; i += 32 * TEAM)       // keys nobody sees
       if (c0 + (i >> 4) >= keys) *reinterpret_cast<uint4 *>(smem + (team * CH + (i >> 4)) * ROWB + ((i & 15) << 4)) = make_uint4(0, 0, 0, 0);
   }
+  TRACE(1);
   pdl_wait();
+  TRACE(2);
   float s[4][4];
 #pragma unroll
   for (int n = 0; n < 4; ++n) s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f;
@@ -155,6 +174,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_few_kernel(const FewParams p)
 #pragma unroll
       for (int n = 0; n < 4; ++n) mma16(s[n], a, kf[n][st].x, kf[n][st].y);
     }
+    TRACE(3);
     // ---- this warp's row maxima
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -237,6 +257,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_few_kernel(const FewParams p)
         *reinterpret_cast<float2 *>(fl + ((lane >> 2) + 8 * i) * O_PITCH + tw * 32 + 8 * n + 2 * t4) = make_float2(o[n][2 * i], o[n][2 * i + 1]);
   }
   __syncthreads();
+  TRACE(4);
   // ---- the span's piece: a warp per row, four dims a lane
   {
     const int row = tid >> 5, d = 4 * lane;
@@ -265,6 +286,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_few_kernel(const FewParams p)
       *reinterpret_cast<float4 *>(dst + 4 + d) = o;
     }
   }
+  TRACE(5);
 }
 
 }  // namespace

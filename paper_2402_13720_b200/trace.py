@@ -2,10 +2,10 @@
 
     python -m paper_2402_13720_b200.trace [--config C2] [--cache-len 4096] [--rows 37] [--which target|draft]
 
-Builds libouro_trace.so (the library compiled with -DOURO_TRACE: selected threads of every CTA of the weight GEMM
-and of the tcgen05 attention stamp the GPU's nanosecond timer at fixed points), runs a few forwards of the chosen
+Builds libouro_trace.so (the library compiled with -DOURO_TRACE: selected threads of every CTA of the weight GEMMs
+and of the attention kernels stamp the GPU's nanosecond timer at fixed points), runs a few forwards of the chosen
 configuration and prints, per kernel of the last forward, when its CTAs reached each point, relative to the moment
-the kernel's dependency wait returned (= the previous kernel had completed).  The regular library is not touched.
+the kernel's dependency wait returned (= the previous kernel had completed) or its activations arrived.  The regular library is not touched.
 """
 from __future__ import annotations
 
@@ -15,6 +15,60 @@ import os
 import sys
 
 import numpy as np
+
+
+GEMMS = ["q,k,v", "o-proj", "gate,up", "down", "LM head"]
+# What the stamps of a GEMM mean, in the order of time: gemm_tc_kernel, and gemm_rows_kernel (single rows of small layers).  A GEMM
+# begins with the first CTA's BEGIN (CTAs that had nothing to do in the GEMM before ask for a single row's activations long before they
+# are there) and ends with the last stamp of END.
+POINTS_TILES = [(0, "CTA entry"), (8, "last weight load issued"), (2, "first stage full"), (3, "last MMA issued"),
+                (4, "last accumulator complete"), (5, "whole tiles done / fix-up begins"), (12, "  group 0: last batch added up"),
+                (10, "  group 0: its tokens finished"), (11, "  group 0: counted"), (7, "fix-up done")]
+BEGIN_TILES, END_TILES = 1, (7, 5)
+POINTS_ROWS = [(0, "CTA entry"), (8, "last weight load issued"), (1, "activations asked for"), (4, "activations there"),
+               (2, "first stage full"), (3, "sums of warp 0 complete"), (5, "sums of all warps and the factor there"), (10, "outputs written")]
+BEGIN_ROWS, END_ROWS = 4, (10,)
+POINTS_ATTN = [(0, "CTA entry"), (1, "set-up done, waiting"), (2, "dependency wait over"), (3, "first scores"),
+               (6, "(head dim 64) second chunk begins"), (7, "(head dim 64) third chunk begins"), (4, "last pass accumulated"), (5, "CTA done")]
+
+
+def _stats(x):
+    return "min %6.1f  med %6.1f  max %6.1f" % (x.min(), np.median(x), x.max()) if len(x) else "-"
+
+
+def report(gemm, attn, single_row):
+    """The lines that describe the stamps `gemm` [8][160][16] and `attn` [512][8] (nanoseconds, 0: not stamped); `single_row`: the
+    GEMMs ran on gemm_rows_kernel."""
+    lines, spans = [], []
+    points, begin, end = (POINTS_ROWS, BEGIN_ROWS, END_ROWS) if single_row else (POINTS_TILES, BEGIN_TILES, END_TILES)
+    since = "the first activations' arrival" if single_row else "the end of the dependency wait"
+    for kind, name in enumerate(GEMMS):
+        t = gemm[kind]
+        live = t[:, 1] > 0                       # stamped by every GEMM of a chained launch (slot 0: by its first only)
+        if not live.any():
+            continue
+        t = t[live]
+        t0 = t[:, begin].min()
+        lines.append(f"{name}  ({live.sum()} CTAs; us relative to {since})")
+        for col, nm in points:
+            x = t[:, col][t[:, col] > 0]
+            lines.append("   %-38s %s" % (nm, _stats((x - t0) / 1e3)))
+        spans.append((name, t0, max(t[:, col].max() for col in end)))
+    live = attn[:, 0] > 0
+    if live.any():
+        t = attn[live]
+        t0 = t[:, 2][t[:, 2] > 0].min()
+        lines.append(f"attention  ({live.sum()} CTAs)")
+        for col, nm in POINTS_ATTN:
+            x = t[:, col][t[:, col] > 0]
+            lines.append("   %-38s %s" % (nm, _stats((x - t0) / 1e3)))
+        spans.append(("attention", t0, t[:, 5].max()))
+    spans.sort(key=lambda s: s[1])
+    lines.append("in launch order: kernel, begun at (us), last CTA done at (us), length")
+    for nm, t0, t1 in spans:
+        base = spans[0][1]
+        lines.append("   %-10s %8.1f %8.1f %8.1f" % (nm, (t0 - base) / 1e3, (t1 - base) / 1e3, (t1 - t0) / 1e3))
+    return lines
 
 
 def main():
@@ -55,49 +109,15 @@ def main():
     torch.cuda.synchronize()
     lib = binding.lib()
     g = (C.c_ulonglong * (8 * 160 * 16))()
-    a = (C.c_ulonglong * (512 * 8))()
-    assert lib.ouro_trace_read_gemm(g) == 0 and lib.ouro_trace_read_attn(a) == 0
+    assert lib.ouro_trace_read_gemm(g) == 0
     g = np.array(g[:], dtype=np.int64).reshape(8, 160, 16)
-    a = np.array(a[:], dtype=np.int64).reshape(512, 8)
-    if not (a[:, 0] > 0).any():                  # head dim 64: the mma.sync attention kernel keeps a timeline of its own
-        assert lib.ouro_trace_read_attn_tc(a.ctypes.data_as(C.POINTER(C.c_ulonglong))) == 0
-
-    def stats(x):
-        return "min %6.1f  med %6.1f  max %6.1f" % (x.min(), np.median(x), x.max()) if len(x) else "-"
-
-    names = ["q,k,v", "o-proj", "gate,up", "down", "LM head"]
-    points = [(0, "CTA entry"), (8, "last weight load issued"), (2, "first stage full"), (3, "last MMA issued"),
-              (4, "last accumulator complete"), (5, "whole tiles done / fix-up begins"), (12, "  group 0: last batch added up"),
-              (10, "  group 0: its tokens finished"), (11, "  group 0: counted"),
-              (7, "fix-up done")]
-    spans = []
-    for kind in range(5):
-        t = g[kind]
-        live = t[:, 1] > 0                       # stamped by every GEMM of a chained launch (slot 0: by its first only)
-        if not live.any():
-            continue
-        t = t[live]
-        t0 = t[:, 1].min()
-        print(f"{names[kind]}  ({live.sum()} CTAs; us relative to the end of the dependency wait)")
-        for col, nm in points:
-            x = t[:, col][t[:, col] > 0]
-            print("   %-34s %s" % (nm, stats((x - t0) / 1e3)))
-        spans.append((names[kind], t0, max(t[:, 7].max(), t[:, 5].max())))
-    live = a[:, 0] > 0
-    if live.any():
-        t = a[live]
-        t0 = t[:, 2].min()
-        print(f"attention  ({live.sum()} CTAs)")
-        for col, nm in [(0, "CTA entry"), (1, "set-up done, waiting"), (2, "dependency wait over"), (3, "first scores"), (6, "(head dim 64) second chunk begins"), (7, "(head dim 64) third chunk begins"),
-                        (4, "last pass accumulated"), (5, "CTA done")]:
-            x = t[:, col][t[:, col] > 0]
-            print("   %-34s %s" % (nm, stats((x - t0) / 1e3)))
-        spans.append(("attention", t0, t[:, 5].max()))
-    spans.sort(key=lambda s: s[1])
-    print("in launch order: kernel, dependency wait over at (us), last CTA done at (us), length")
-    base = spans[0][1]
-    for nm, t0, t1 in spans:
-        print("   %-10s %8.1f %8.1f %8.1f" % (nm, (t0 - base) / 1e3, (t1 - base) / 1e3, (t1 - t0) / 1e3))
+    for read in (lib.ouro_trace_read_attn, lib.ouro_trace_read_attn_few, lib.ouro_trace_read_attn_tc):   # the kernel that ran has stamped
+        a = (C.c_ulonglong * (512 * 8))()
+        assert read(a) == 0
+        a = np.array(a[:], dtype=np.int64).reshape(512, 8)
+        if (a[:, 0] > 0).any():
+            break
+    print("\n".join(report(g, a, eng.debug_counts()["rows_launches"] > 0)))
     eng.close()
 
 
