@@ -939,8 +939,10 @@ struct ouro_fast { FastState s; };
 size_t ouro_scratch_bytes(const ouro_model_desc *t, const ouro_model_desc *d) {
   size_t attn = attention_tc_scratch_bytes(*t);
   if (d && attention_tc_scratch_bytes(*d) > attn) attn = attention_tc_scratch_bytes(*d);
-  const size_t packets = std::max(packets_bytes(*t), d ? packets_bytes(*d) : 0);
-  return slots_bytes() + CHAIN_BYTES + 2 * tile_best_bytes() + ss_bytes() + squares_bytes() + packets + attn;
+  return slots_bytes() + CHAIN_BYTES + 2 * tile_best_bytes() + ss_bytes() + attn;
+}
+size_t ouro_single_bytes(const ouro_model_desc *t, const ouro_model_desc *d) {
+  return squares_bytes() + std::max(packets_bytes(*t), d ? packets_bytes(*d) : 0);
 }
 
 static bool shape_ok(const ouro_model_desc &d) {
@@ -1080,13 +1082,10 @@ int ouro_fast_setup(ouro_ctx *c) {
   f->s.tile_arg = (int *)((char *)f->s.tile_max + tile_best_bytes());
   f->s.ss = (float *)((char *)f->s.tile_arg + tile_best_bytes());
   f->s.attn_part = (float *)((char *)f->s.ss + ss_bytes());
-  size_t attn = 0, packets = 0;                                 // (one model computes at a time)
+  size_t packets = 0;                                           // (one model computes at a time)
   for (auto &M : c->m)
-    if (M.present) {
-      attn = std::max(attn, attention_tc_scratch_bytes(M.d));
-      packets = std::max(packets, packets_bytes(M.d));
-    }
-  f->s.squares = (float *)((char *)f->s.attn_part + attn);
+    if (M.present) packets = std::max(packets, packets_bytes(M.d));
+  f->s.squares = c->a.single;
   f->s.packets = (uint4 *)((char *)f->s.squares + squares_bytes());
   f->s.packets_size = packets;
   if (cudaMemsetAsync(f->s.slots, 0xff, slots_bytes(), c->stream) != cudaSuccess ||

@@ -120,6 +120,7 @@ struct Activations {  // sized for OURO_MAX_ROWS rows of the larger model, 16-bi
   int32_t *argmax; // [rows]
   float *scratch;  // split-K partial sums / split-KV partial softmax states
   size_t scratch_bytes;
+  float *single;   // single rows: squares, then packets
 };
 
 struct ouro_fast;   // tensor maps and launch state of the tensor-core paths (gemm_tc.cu)
