@@ -1,12 +1,12 @@
 // Weight-streaming GEMMs for one token (plain decoding, drafting) of a model with small layers: part of gemm_tc.cu, which has the
-// chain and the schedule that says where a tile is cut along K.
+// chain, the schedule that says where a tile is cut along K, and the rules that say which models run here (rows_x_bytes, rows_pay).
 //
 // At one token a GEMM of gemm_tc_kernel is latency: a tile of 128 weight rows is cut along K among several CTAs, whose
 // partial sums cross the chip before anybody can finish the token (3 us of the 5 to 10 of a GEMM of the 1.1B shape), and
 // the outputs cross it again behind a fence and a counter (2 us).  Here a CTA owns its weight rows for the whole of K: groups of 16
 // (a unit), as many per CTA as an equal split over the SMs gives, so that only finished activations leave it.  They travel
 // in packets that say themselves that they are there (row_ops.cuh), and every CTA gathers all of them into its shared memory.
-// 1.1B draft, four forwards behind 389 keys: 3156 -> 2510 us; a layer 36 -> 28 us, of which 13.5 are its 88 MB at the copy peak and
+// 1.1B draft, four forwards behind 389 keys: 3156 -> 2497 us; a layer 36 -> 28 us, of which 13.5 are its 88 MB at the copy peak and
 // the rest four hand-overs, the attention and two launches.
 //
 // The tensor cores are used through mma.sync (16 weight rows x 8 tokens x 16 values of K, operands by ldmatrix): its fragments

@@ -1624,7 +1624,7 @@ def test_groups_shared_by_several_ctas_are_bit_identical_to_plain_decoding(kv, K
 ])
 def test_few_rows_are_bit_identical_to_wider_blocks(d, heads, kv, hd, ffn, vocab):
     """A single row of a model of small layers runs on GEMM kernels of its own, and up to 16 query rows of a kv head without
-    candidates on attention of their own (head dim 128, in one span or in front of those kernels).  A token's logits,
+    candidates on attention of their own (head dim 128), both where they are faster.  A token's logits,
     choice, keys and values must not show which: blocks of 1, 2, 5, 8, 9 and 16 rows against one block of 40, behind 490 keys, so
     that the rows pass the end of a span."""
     desc = synth.ModelDesc(1 if d > 2048 else 2, d, heads, kv, hd, ffn, vocab, 640, "bf16")
