@@ -988,8 +988,8 @@ static rows_gemm::Plan rows_plan(int kind, int units, int kb, int tiles, int gri
 //   head dim 64: 2048 x 5632 1.2 / 1.2 (0, 1.3), 256 x 1600 1.13 / 1.09 (2.5, 2.7), 2240 x 768 1.00 / 1.01 (3.1, 3.6), 384 x 3200 1.06 / 1.07 (4.7, 5.4), 384
 //   x 1024 with 3072 query columns 0.95 / 0.96 (4.5, 4.8), 320 x 1600 0.97 / 0.96 (5.0, 5.2), 1984 x 256 0.88 / 0.90 (5.6, 6.0); 4096 x 4096 with 512
 //   query columns 0.96 / 0.97 (0, 2.9): the worst that is let in
-// The head costs 1 us more in each of its passes than it does there (one layer of 512 in front of 65536 / 262144 logits 44 / 79 us
-// and 42 / 86), which each layer's saving makes up for a few of.
+// The head costs up to 1 us more in each of its passes than it does there, which a layer's saving makes up for four of: one layer in front of 3 / 6
+// passes 1.02 to 1.19 / 0.96 to 1.05, two in front of 6 / 12 1.01 to 1.16 / 0.96 to 1.05, three in front of 12 1.005 to 1.09 (256 to 2048 wide, 150 keys).
 static bool rows_pay(const rows_gemm::Plan *plan, const int *kb, int head_dim, int n_layers) {
   double beyond = 0, late = 0;
   for (int k = 0; k < 4; ++k) {
@@ -1000,7 +1000,7 @@ static bool rows_pay(const rows_gemm::Plan *plan, const int *kb, int head_dim, i
     beyond += std::max(0.0, walk - stream);
     late += std::max(0.0, walk - 0.4 * stream);
   }
-  return beyond <= (head_dim == 128 ? 4.4 : 3.3) && late <= 6.0 && plan[G_HEAD].passes <= 3 * n_layers;
+  return beyond <= (head_dim == 128 ? 4.4 : 3.3) && late <= 6.0 && plan[G_HEAD].passes <= 4 * n_layers;
 }
 static bool rows_setup(int grid, int smem_max, const ModelRt &M, RowsModel &rm) {
   const ouro_model_desc &d = M.d;

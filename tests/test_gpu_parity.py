@@ -1707,8 +1707,8 @@ def test_single_rows_with_a_late_warp(monkeypatch, fuse):
     (1, 1536, 12, 3, 128, 16896, 1000, False),     # 88 k-blocks of the down projection, 48 of gate and up, in 152 MB
     (1, 2048, 32, 4, 64, 5632, 32000, True),
     (1, 2560, 20, 5, 128, 10240, 1000, False),     # beyond 160 MB
-    (3, 256, 2, 1, 128, 256, 262144, False),       # twelve passes of the head behind three layers
-    (4, 256, 2, 1, 128, 256, 262144, True),        # ... and four
+    (2, 256, 2, 1, 128, 256, 262144, False),       # twelve passes of the head behind two layers
+    (3, 256, 2, 1, 128, 256, 262144, True),        # ... and three
     (1, 512, 4, 4, 96, 512, 1000, False),          # another head dim
 ])
 def test_single_rows_take_the_kernel_that_is_faster(layers, d, heads, kv, hd, ffn, vocab, owned):
